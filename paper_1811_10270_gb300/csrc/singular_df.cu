@@ -33,9 +33,18 @@ __device__ __forceinline__ void st(float2* p, int64_t i, df v) { p[i] = make_flo
 
 __device__ __forceinline__ int tri_off_i(int p, int m) { return m * (p + 1) - m * (m - 1) / 2; }
 
-__global__ void k_to_df(const double* __restrict__ x, int64_t n, float2* __restrict__ out) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < n) st(out, e, dfl::from_double(x[e]));
+struct Centre {
+  double c[3];
+};
+
+// position coefficients relative to the drop's centre: the kernels see differences of positions only, and a
+// double-float holds them to 2^-48 of the drop's size instead of its distance from the origin
+__global__ void k_to_df(const double* __restrict__ x, int nc, Centre C, float2* __restrict__ out) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 3 * nc) return;
+  double v = x[e];
+  if (e % nc == 0) v -= C.c[e / nc] * 3.5449077018110320546;   // sqrt(4 pi): the degree-0 harmonic of a constant
+  st(out, e, dfl::from_double(v));
 }
 
 // Rotation of all components of TPB targets per CTA, degree by degree (degrees n_begin .. p; the lower
@@ -137,181 +146,218 @@ k_rotate_deg_df(const float2* __restrict__ vin, int64_t in_stride, int nc, int p
   }
 }
 
-// Four-longitude Fourier synthesis (the parity folding of synth4) in double-float.
-__device__ void synth4_df(const float2* __restrict__ a, const float2* __restrict__ b, df a0, float beta, int p,
-                          int k, int N, const float2* __restrict__ tc, const float2* __restrict__ ts,
-                          float2* __restrict__ dst) {
-  dfl::acc ce, co, se, so;
+// Four-longitude Fourier synthesis (the parity folding of synth4) of the three components of one kind in
+// double-float: a and b hold the cosine and sine coefficients of component f at f * fs. One pass over the orders
+// serves the three components, so a pair of trig values is read once for six multiply-adds.
+__device__ __forceinline__ void synth4_df3(const float2* __restrict__ a, const float2* __restrict__ b, int fs, bool dphi,
+                                           int p, int k, int N, const float2* __restrict__ tc,
+                                           const float2* __restrict__ ts, float2* __restrict__ dst, int ds) {
+  dfl::acc ce[3], co[3], se[3], so[3];
   int id = 0;
+  auto next = [&](int m, dfl::acc (&c3)[3], dfl::acc (&s3)[3]) {
+    id += k;
+    if (id >= N) id -= N;
+    const df c = ld(tc, id), s = ld(ts, id);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      c3[f].add_prod(ld(a, f * fs + m), c);
+      s3[f].add_prod(ld(b, f * fs + m), s);
+    }
+  };
   int m = 1;
   for (; m + 1 <= p; m += 2) {
-    id += k;
-    if (id >= N) id -= N;
-    co.add_prod(ld(a, m), ld(tc, id));
-    so.add_prod(ld(b, m), ld(ts, id));
-    id += k;
-    if (id >= N) id -= N;
-    ce.add_prod(ld(a, m + 1), ld(tc, id));
-    se.add_prod(ld(b, m + 1), ld(ts, id));
+    next(m, co, so);
+    next(m + 1, ce, se);
   }
-  if (m <= p) {
-    id += k;
-    if (id >= N) id -= N;
-    co.add_prod(ld(a, m), ld(tc, id));
-    so.add_prod(ld(b, m), ld(ts, id));
-  }
+  if (m <= p) next(m, co, so);
   const df s2{1.41421353816986084f, 2.4203234971764687e-08f};  // sqrt(2) as hi + lo
-  const df CE = ce.value(), CO = co.value();
-  df SE = se.value(), SO = so.value();
-  if (beta < 0) {
-    SE = dfl::neg(SE);
-    SO = dfl::neg(SO);
-  } else if (beta == 0) {
-    SE = df{0.f, 0.f};
-    SO = df{0.f, 0.f};
-  }
-  const df c1 = dfl::add(CE, CO), s1 = dfl::add(SE, SO);
-  const df c2 = dfl::sub(CE, CO), s2v = dfl::sub(SO, SE);
   const int h = N >> 1;
-  st(dst, k, dfl::add(a0, dfl::mul(s2, dfl::add(c1, s1))));
-  st(dst, (N - k) % N, dfl::add(a0, dfl::mul(s2, dfl::sub(c1, s1))));
-  st(dst, h - k, dfl::add(a0, dfl::mul(s2, dfl::add(c2, s2v))));
-  st(dst, h + k, dfl::add(a0, dfl::mul(s2, dfl::sub(c2, s2v))));
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    const df CE = ce[f].value(), CO = co[f].value();
+    df SE = se[f].value(), SO = so[f].value();
+    if (dphi) {
+      SE = dfl::neg(SE);
+      SO = dfl::neg(SO);
+    }
+    const df a0 = dphi ? df{0.f, 0.f} : ld(a, f * fs);
+    const df c1 = dfl::add(CE, CO), s1 = dfl::add(SE, SO);
+    const df c2 = dfl::sub(CE, CO), s2v = dfl::sub(SO, SE);
+    float2* o = dst + f * ds;
+    st(o, k, dfl::add(a0, dfl::mul(s2, dfl::add(c1, s1))));
+    st(o, (N - k) % N, dfl::add(a0, dfl::mul(s2, dfl::sub(c1, s1))));
+    st(o, h - k, dfl::add(a0, dfl::mul(s2, dfl::add(c2, s2v))));
+    st(o, h + k, dfl::add(a0, dfl::mul(s2, dfl::sub(c2, s2v))));
+  }
 }
 
-// For target blockIdx.x (chunk-local) and up-grid latitude blockIdx.y: synthesise the rotated
-// position and tangents, then the 14 kernel weights of every node of the latitude.
-__global__ void k_self_weights_df(const float2* __restrict__ rot, int p, int q, const float2* __restrict__ alf,
-                                  const float2* __restrict__ trig, const double* __restrict__ mu,
-                                  const double* __restrict__ tgt, int64_t ntarget, int64_t tgt0,
-                                  float2* __restrict__ wbuf, int* __restrict__ rexp) {
+// float2 between the coefficient sets of two (latitude, kind) pairs: 6 (p + 1), padded so that the six pairs that
+// neighbouring lanes read start in different banks (12 words apart modulo 32)
+__host__ __device__ __forceinline__ int weights_set(int p) {
+  const int w = 12 * (p + 1);
+  return (w + ((12 - w) % 32 + 32) % 32) / 2;
+}
+
+// For target blockIdx.x (chunk-local) and the up-grid latitudes j = blockIdx.y and q - j: synthesise the rotated
+// position and tangents, then the 14 kernel weights of every node of the two latitudes.
+// FP32-pipe bound. The two latitudes mirror each other, P_n^m(-t) = (-1)^(n+m) P_n^m(t): sums over even and odd
+// n - m serve both, half the Legendre multiply-adds and table reads of one latitude at a time. A thread carries the
+// three kinds of one coefficient pair through the Legendre sums (one coefficient read for three multiply-adds) and
+// the three components of one kind through the Fourier sums. Four drops of degree 16, 31, 48 and 64: 169 ms with one
+// latitude and one field per thread, 94 ms so (about 45 ms of FP32 issue slots; the rest is shared-memory reads and sums
+// of uneven length in a warp).
+__global__ void __launch_bounds__(288)
+k_self_weights_df(const float2* __restrict__ rot, int p, int q, const float2* __restrict__ alf,
+                  const float2* __restrict__ trig, const double* __restrict__ mu,
+                  const double* __restrict__ tgt, int64_t ntarget, int64_t tgt0, Centre C,
+                  float2* __restrict__ wbuf, int* __restrict__ rexp) {
   extern __shared__ float2 smf[];
   const int t = blockIdx.x;
-  const int j = blockIdx.y;
   const int N = 2 * q + 2;
   const int P1 = p + 1;
   const int nc = P1 * P1;
   const int nt = P1 * (p + 2) / 2;
-  float2* A = smf;            // [3 f][3 kind][2][P1]
-  float2* tc = A + 18 * P1;
+  const int set = weights_set(p);
+  float2* A = smf;            // [latitude, kind][f][cos, sin][P1], sets `set` apart
+  float2* tc = A + 6 * set;
   float2* ts = tc + N;
-  float2* V = ts + N;         // [9][N]
+  float2* V = ts + N;         // [latitude][f][kind][N]
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     tc[i] = trig[i];
     ts[i] = trig[N + i];
   }
-  const float2* T = alf + (int64_t)j * 3 * nt;
+  const float2* T = alf + (int64_t)blockIdx.y * 3 * nt;
   const float2* cf = rot + (int64_t)t * 3 * nc;
   // order m-major, so that the 32 lanes of a warp hold sums of (nearly) equal length p + 1 - m
-  for (int task = threadIdx.x; task < 18 * P1; task += blockDim.x) {
-    const int m = task / 18;
-    const int r = task - m * 18;
-    const int fk = r >> 1;
+  for (int task = threadIdx.x; task < 6 * P1; task += blockDim.x) {
+    const int m = task / 6;
+    const int r = task - m * 6;
+    const int f = r >> 1;
     const int cs = r & 1;
-    const int f = fk / 3, kind = fk - f * 3;
-    dfl::acc acc;
+    dfl::acc e[3], o[3];
     if (!(cs == 1 && m == 0)) {
-      const float2* col = T + kind * nt + tri_off_i(p, m);
-      const float2* c = cf + f * nc;
-      const int sg = cs ? -m : m;
-      for (int n = m; n <= p; ++n) acc.add_prod(ld(c, n * n + n + sg), ld(col, n - m));
+      const float2* col = T + tri_off_i(p, m) - m;
+      const float2* c = cf + f * nc + (cs ? -m : m);
+      int n = m;
+      for (; n < p; n += 2) {
+        const df x = ld(c, n * n + n), y = ld(c, n * n + 3 * n + 2);   // degrees n and n + 1
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          e[k].add_prod(x, ld(col, k * nt + n));
+          o[k].add_prod(y, ld(col, k * nt + n + 1));
+        }
+      }
+      if (n == p) {
+        const df x = ld(c, n * n + n);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) e[k].add_prod(x, ld(col, k * nt + n));
+      }
     }
-    st(A, (fk * 2 + cs) * P1 + m, acc.value());
+    // even and odd parts swap signs between the latitudes; the theta derivative once more
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const df E = e[k].value(), O = o[k].value();
+      const int at = (f * 2 + cs) * P1 + m;
+      st(A, k * set + at, dfl::add(E, O));
+      st(A, (3 + k) * set + at, k == 1 ? dfl::sub(O, E) : dfl::sub(E, O));
+    }
   }
   __syncthreads();
   const int Q4 = N >> 2;
-  // field fastest: the lanes of a warp read the same few trig entries (broadcasts) instead of
+  // (latitude, kind) fastest: the lanes of a warp read the same few trig entries (broadcasts) instead of
   // entries m k apart (bank conflicts)
-  for (int task = threadIdx.x; task < 9 * (Q4 + 1); task += blockDim.x) {
-    const int k = task / 9;
-    const int fk = task - k * 9;
-    const float2* Ac = A + (fk * 2) * P1;
+  for (int task = threadIdx.x; task < 6 * (Q4 + 1); task += blockDim.x) {
+    const int k = task / 6;
+    const int lk = task - k * 6;
+    const int kind = lk % 3;
+    const float2* Ac = A + lk * set;
     const float2* As = Ac + P1;
     // the phi-derivative kind swaps the cos / sin roles: selected per lane, one code path
-    const bool dphi = fk % 3 == 2;
-    synth4_df(dphi ? As : Ac, dphi ? Ac : As, dphi ? df{0.f, 0.f} : ld(Ac, 0), dphi ? -1.f : 1.f, p, k, N, tc, ts,
-              V + fk * N);
+    const bool dphi = kind == 2;
+    synth4_df3(dphi ? As : Ac, dphi ? Ac : As, 2 * P1, dphi, p, k, N, tc, ts, V + ((lk / 3) * 9 + kind) * N, 3 * N);
   }
-  __syncthreads();
-  // the target's position and normal and mu_j / (4 pi) as double-float, converted once per block
-  // (FP64 conversions run on the FP64 pipe)
-  __shared__ float2 tv[7];
-  if (threadIdx.x < 7) {
+  // the target's position and normal and mu_j / (4 pi) of the two latitudes as double-float, converted once per
+  // block (FP64 conversions run on the FP64 pipe)
+  __shared__ float2 tv[8];
+  if (threadIdx.x < 8) {
     const int64_t tg = tgt0 + t;
-    const double v = threadIdx.x < 6 ? tgt[threadIdx.x * ntarget + tg] : mu[j] * 0.07957747154594766788;
-    st(tv, threadIdx.x, dfl::from_double(v));
+    const int jj = threadIdx.x == 6 ? blockIdx.y : q - blockIdx.y;
+    const double v = threadIdx.x < 6 ? tgt[threadIdx.x * ntarget + tg] : mu[jj] * 0.07957747154594766788;
+    const double c = threadIdx.x < 3 ? C.c[threadIdx.x] : 0.0;
+    st(tv, threadIdx.x, dfl::from_double(v - c));
   }
   __syncthreads();
-  const df x0 = ld(tv, 0), y0 = ld(tv, 1), z0 = ld(tv, 2);
-  const df n0x = ld(tv, 3), n0y = ld(tv, 4), n0z = ld(tv, 5);
-  const df w0 = ld(tv, 6);
   const int64_t Ns = (int64_t)(q + 1) * N;
-  float mx[14];
+  for (int half = 0; half < 2; ++half) {
+    const int j = half == 0 ? blockIdx.y : q - blockIdx.y;
+    const float2* W = V + half * 9 * N;
+    float mx[14];
 #pragma unroll
-  for (int c = 0; c < 14; ++c) mx[c] = 0.f;
-  for (int k = threadIdx.x; k < N; k += blockDim.x) {
-    const df xt0 = ld(V, 1 * N + k), xt1 = ld(V, 4 * N + k), xt2 = ld(V, 7 * N + k);
-    const df xp0 = ld(V, 2 * N + k), xp1 = ld(V, 5 * N + k), xp2 = ld(V, 8 * N + k);
-    const df c0 = dfl::sub(dfl::mul(xt1, xp2), dfl::mul(xt2, xp1));
-    const df c1 = dfl::sub(dfl::mul(xt2, xp0), dfl::mul(xt0, xp2));
-    const df c2 = dfl::sub(dfl::mul(xt0, xp1), dfl::mul(xt1, xp0));
-    const df J2 = dfl::dot3(c0, c1, c2, c0, c1, c2);
-    const df rJ = dfl::rsqrt(J2);
-    const df J = dfl::mul(J2, rJ);
-    const df nx = dfl::mul(c0, rJ), ny = dfl::mul(c1, rJ), nz = dfl::mul(c2, rJ);
-    const df hx = dfl::diff(x0, ld(V, k)), hy = dfl::diff(y0, ld(V, 3 * N + k)), hz = dfl::diff(z0, ld(V, 6 * N + k));
-    const df r2 = dfl::dot3(hx, hy, hz, hx, hy, hz);
-    const df ri = dfl::rsqrt(r2);
-    const df ri2 = dfl::sqr(ri);
-    const df ri3 = dfl::mul(ri2, ri);
-    const df w = dfl::mul(w0, J);
-    const df hn = dfl::dot3(hx, hy, hz, nx, ny, nz);
-    const df d5 = dfl::mul(dfl::mul(dfl::mul_f(w, -6.f), hn), dfl::mul(ri3, ri2));
-    const df s3 = dfl::mul(w, ri3);
-    const df wr = dfl::mul(w, ri);
-    df out[14];
-    out[0] = dfl::mul(dfl::mul(w, dfl::dot3(hx, hy, hz, n0x, n0y, n0z)), ri3);
-    out[1] = wr;
-    const df sx = dfl::mul(s3, hx), sy = dfl::mul(s3, hy), sz = dfl::mul(s3, hz);
-    out[2] = dfl::add(wr, dfl::mul(sx, hx));
-    out[3] = dfl::mul(sx, hy);
-    out[4] = dfl::mul(sx, hz);
-    out[5] = dfl::add(wr, dfl::mul(sy, hy));
-    out[6] = dfl::mul(sy, hz);
-    out[7] = dfl::add(wr, dfl::mul(sz, hz));
-    const df dx = dfl::mul(d5, hx), dy = dfl::mul(d5, hy), dz = dfl::mul(d5, hz);
-    out[8] = dfl::mul(dx, hx);
-    out[9] = dfl::mul(dx, hy);
-    out[10] = dfl::mul(dx, hz);
-    out[11] = dfl::mul(dy, hy);
-    out[12] = dfl::mul(dy, hz);
-    out[13] = dfl::mul(dz, hz);
-    const int64_t node = (int64_t)j * N + k;
-#pragma unroll
-    for (int c = 0; c < 14; ++c) {
-      st(wbuf, ((int64_t)t * 14 + c) * Ns + node, out[c]);
-      mx[c] = fmaxf(mx[c], fabsf(out[c].hi));
+    for (int c = 0; c < 14; ++c) mx[c] = 0.f;
+    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+      const df x0 = ld(tv, 0), y0 = ld(tv, 1), z0 = ld(tv, 2);
+      const df xt0 = ld(W, 1 * N + k), xt1 = ld(W, 4 * N + k), xt2 = ld(W, 7 * N + k);
+      const df xp0 = ld(W, 2 * N + k), xp1 = ld(W, 5 * N + k), xp2 = ld(W, 8 * N + k);
+      const df c0 = dfl::sub(dfl::mul(xt1, xp2), dfl::mul(xt2, xp1));
+      const df c1 = dfl::sub(dfl::mul(xt2, xp0), dfl::mul(xt0, xp2));
+      const df c2 = dfl::sub(dfl::mul(xt0, xp1), dfl::mul(xt1, xp0));
+      const df J2 = dfl::dot3(c0, c1, c2, c0, c1, c2);
+      const df rJ = dfl::rsqrt(J2);
+      const df J = dfl::mul(J2, rJ);
+      const df nx = dfl::mul(c0, rJ), ny = dfl::mul(c1, rJ), nz = dfl::mul(c2, rJ);
+      const df hx = dfl::diff(x0, ld(W, k)), hy = dfl::diff(y0, ld(W, 3 * N + k)), hz = dfl::diff(z0, ld(W, 6 * N + k));
+      const df r2 = dfl::dot3(hx, hy, hz, hx, hy, hz);
+      const df ri = dfl::rsqrt(r2);
+      const df ri2 = dfl::sqr(ri);
+      const df ri3 = dfl::mul(ri2, ri);
+      const df w = dfl::mul(ld(tv, 6 + half), J);
+      const df hn = dfl::dot3(hx, hy, hz, nx, ny, nz);
+      const df d5 = dfl::mul(dfl::mul(dfl::mul_f(w, -6.f), hn), dfl::mul(ri3, ri2));
+      const df s3 = dfl::mul(w, ri3);
+      const df wr = dfl::mul(w, ri);
+      float2* dst = wbuf + (int64_t)t * 14 * Ns + (int64_t)j * N + k;
+      auto put = [&](int c, df v) {
+        st(dst, c * Ns, v);
+        mx[c] = fmaxf(mx[c], fabsf(v.hi));
+      };
+      put(0, dfl::mul(dfl::mul(w, dfl::dot3(hx, hy, hz, ld(tv, 3), ld(tv, 4), ld(tv, 5))), ri3));
+      put(1, wr);
+      const df sx = dfl::mul(s3, hx), sy = dfl::mul(s3, hy), sz = dfl::mul(s3, hz);
+      put(2, dfl::add(wr, dfl::mul(sx, hx)));
+      put(3, dfl::mul(sx, hy));
+      put(4, dfl::mul(sx, hz));
+      put(5, dfl::add(wr, dfl::mul(sy, hy)));
+      put(6, dfl::mul(sy, hz));
+      put(7, dfl::add(wr, dfl::mul(sz, hz)));
+      const df dx = dfl::mul(d5, hx), dy = dfl::mul(d5, hy), dz = dfl::mul(d5, hz);
+      put(8, dfl::mul(dx, hx));
+      put(9, dfl::mul(dx, hy));
+      put(10, dfl::mul(dx, hz));
+      put(11, dfl::mul(dy, hy));
+      put(12, dfl::mul(dy, hz));
+      put(13, dfl::mul(dz, hz));
     }
-  }
-  // power-of-two scale of each (component, latitude) row for the tensor-core analysis: max |hi|
-  // < 2^e over the row's N nodes
-  if (rexp) {
-    __shared__ float red[4][14];   // blockDim.x <= 128
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    // power-of-two scale of each (component, latitude) row for the tensor-core analysis: max |hi|
+    // < 2^e over the row's N nodes
+    if (rexp) {
+      __shared__ float red[9][14];   // blockDim.x <= 288
+      const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+      if (half) __syncthreads();     // the first latitude's values have been read
 #pragma unroll
-    for (int c = 0; c < 14; ++c) {
-      float v = mx[c];
+      for (int c = 0; c < 14; ++c) {
+        float v = mx[c];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-      if (lane == 0) red[wp][c] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 14) {
-      float v = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmaxf(v, red[w][threadIdx.x]);
-      int e = 0;
-      frexpf(v, &e);
-      rexp[((int64_t)t * 14 + threadIdx.x) * (q + 1) + j] = max(e, -120);
+        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+        if (lane == 0) red[wp][c] = v;
+      }
+      __syncthreads();
+      if (threadIdx.x < 14) {
+        float v = 0.f;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmaxf(v, red[w][threadIdx.x]);
+        int e = 0;
+        frexpf(v, &e);
+        rexp[((int64_t)t * 14 + threadIdx.x) * (q + 1) + j] = max(e, -120);
+      }
     }
   }
 }
@@ -502,6 +548,7 @@ int build_singular_rows_df(shbim_ctx* ctx, cudaStream_t s, const double* xcoef) 
     const GridTables& up = d.tab->up;
     const int64_t Ns = d.ns;
     const int nc = d.nc;
+    const Centre ctr{{d.centre[0], d.centre[1], d.centre[2]}};
     const int N = 2 * d.q + 2;
     const int CT = chunk_of(d);
     const int wmax = 2 * d.p + 1;
@@ -516,7 +563,9 @@ int build_singular_rows_df(shbim_ctx* ctx, cudaStream_t s, const double* xcoef) 
     const int deg_smem14 = dq_bytes + tpb14 * per_t14;
     SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_deg_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, deg_smem3));
     SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_deg_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, deg_smem14));
-    const size_t w_smem = (size_t)(18 * (d.p + 1) + 11 * N) * sizeof(float2);
+    const int w_threads = (N + 31) / 32 * 32;   // one node of a latitude per thread (N <= 260)
+    const size_t w_smem = (size_t)(6 * weights_set(d.p) + 20 * N) * sizeof(float2);
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_self_weights_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w_smem));
     const int budget = 46 * 1024 / (int)sizeof(float2) - 2 * N;
     const int rows = std::max(1, std::min(8, budget / (2 * N)));
     const size_t f_smem = (size_t)(2 * N + rows * 2 * N) * sizeof(float2);
@@ -541,7 +590,7 @@ int build_singular_rows_df(shbim_ctx* ctx, cudaStream_t s, const double* xcoef) 
       // row exponents of the weights for the tensor-core analysis, written by the weights kernel
       int* rexp = dft_tc ? reinterpret_cast<int*>(L.rexp) : nullptr;
       if (L.xdrop != (int)di) {
-        k_to_df<<<(unsigned)((3 * nc + 255) / 256), 256, 0, st>>>(xcoef + 3 * d.coef_off, 3 * nc, xc);
+        k_to_df<<<(unsigned)((3 * nc + 255) / 256), 256, 0, st>>>(xcoef + 3 * d.coef_off, nc, ctr, xc);
         SHBIM_CHECK_LAUNCH(ctx, "k_to_df");
         L.xdrop = (int)di;
       }
@@ -560,8 +609,8 @@ int build_singular_rows_df(shbim_ctx* ctx, cudaStream_t s, const double* xcoef) 
       }
       {
         TimeScope ts(ctx, SHBIM_K_SELF_WEIGHTS, st);
-        k_self_weights_df<<<dim3(ct, d.q + 1), 128, w_smem, st>>>(rot, d.p, d.q, d.tab->up_alf_df, d.tab->up_trig_df,
-                                                                  up.mu, ctx->geo.tgt, ctx->ntarget, d.tgt_off + t0, wb,
+        k_self_weights_df<<<dim3(ct, (d.q + 1) / 2), w_threads, w_smem, st>>>(rot, d.p, d.q, d.tab->up_alf_df, d.tab->up_trig_df,
+                                                                  up.mu, ctx->geo.tgt, ctx->ntarget, d.tgt_off + t0, ctr, wb,
                                                                   rexp);
         SHBIM_CHECK_LAUNCH(ctx, "k_self_weights_df");
       }
