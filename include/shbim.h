@@ -54,7 +54,9 @@ extern "C" {
 #define SHBIM_CONVERGED 1           /* shbim_gmres_step: relative residual <= tol */
 
 /* Arithmetic of the all-pairs sums (the singular self rows, the transforms and GMRES are
- * always FP64). */
+ * always FP64). Where it pays, the sums between drops far enough apart go through multipole and local
+ * expansions of the same quadrature rule, in FP64 or double-float arithmetic, truncated below the rounding of
+ * the mode (3e-15 of a pair's sum of magnitudes, 1e-8 in FP32 mode); the others are formed pair by pair. */
 #define SHBIM_PREC_FP64 0           /* FP64 sums */
 #define SHBIM_PREC_FP32_COMP 1      /* FP32 pair arithmetic, positions relative to the drop
                                        centres, compensated (two-sum) accumulation */
@@ -591,7 +593,8 @@ int shbim_kernel_stats(shbim_ctx* ctx, int kernel_class, double* ms_host, int64_
 /* Algorithmic work of the bracketed launches of one class since timing was (re)enabled, in
  * floating-point operations of the method's formulas (an add or a multiply is 1, a fused
  * multiply-add 2, a reciprocal square root 1), whatever arithmetic the kernel uses to carry them out:
- * for the all-pairs classes, target-source pairs of other drops times the operations of one kernel
+ * for the all-pairs classes, the target-source pairs of other drops that are summed directly (all of them,
+ * or those of drops too close for the expansions below) times the operations of one kernel
  * term (Laplace single layer 11, target-normal double layer 19, Stokeslet 29, stresslet 30, both
  * Stokes terms 42); 0 for the other classes. Synchronises the device like shbim_kernel_stats. */
 int shbim_kernel_work(shbim_ctx* ctx, int kernel_class, double* flops_host);

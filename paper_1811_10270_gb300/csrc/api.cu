@@ -4,6 +4,7 @@
 #include <cstring>
 #include <set>
 
+#include "far.h"
 #include "internal.h"
 
 namespace shbim {
@@ -42,7 +43,7 @@ int rebuild_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
   SHBIM_CUDA(ctx, cudaMemcpy(ctx->drops_dev, dd.data(), dd.size() * sizeof(DropDev), cudaMemcpyHostToDevice));
   int rc;
   if ((rc = build_geometry(ctx, xcoef_dev, s))) return rc;
-  if ((rc = build_quantized_sources(ctx, s))) return rc;
+  if ((rc = build_pair_lists(ctx, s))) return rc;
   if ((rc = build_stokes_preconditioner(ctx, xcoef_dev, s))) return rc;
   if ((rc = ctx->rows_prec == SHBIM_PREC_DF64 ? build_singular_rows_df(ctx, s, xcoef_dev)
                                               : build_singular_rows(ctx, xcoef_dev, s)))
@@ -153,6 +154,7 @@ int shbim_destroy(shbim_ctx* ctx) {
   free_drop_state(ctx);
   for (auto& kv : ctx->tables) free_degree_tables(kv.second);
   cudaFree(ctx->sht_scratch);
+  far_free(ctx);
   cudaFree(ctx->dq_ext_dev);
   cudaFree(ctx->dq_far);
   cudaFree(ctx->rot_coef);
@@ -488,8 +490,6 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
     if ((rc = dalloc(ctx, &ctx->tiles_dev, ctx->tiles.size(), "tiles"))) return rc;
     SHBIM_CUDA(ctx, cudaMemcpy(ctx->tiles_dev, ctx->tiles.data(), ctx->tiles.size() * sizeof(PairTile),
                                cudaMemcpyHostToDevice));
-    ctx->cross_pairs = 0;
-    for (const Drop& d : ctx->drops) ctx->cross_pairs += (int64_t)d.nt * (so - d.ns);
     ctx->split_max = (int)std::max<int64_t>(1, std::min<int64_t>(4 * splits, std::max<int64_t>(1, min_other / 64)));
     ctx->split_max = std::min(ctx->split_max, 256);
     ctx->pair_splits = std::min(ctx->pair_splits, ctx->split_max);

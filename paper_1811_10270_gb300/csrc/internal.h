@@ -158,6 +158,8 @@ struct Geometry {
   int64_t* src_start = nullptr;  // [n_drops+1]
 };
 
+struct FarState;             // expansions between well-separated drops (far.h)
+
 }  // namespace shbim
 
 struct shbim_ctx {
@@ -215,6 +217,7 @@ struct shbim_ctx {
   unsigned* dq_ext_dev = nullptr; // [n_drops] largest |x - c| over each drop's sources (float bits)
   unsigned char* dq_far = nullptr; // [n_drops][n_drops]: the drop pair uses the quantised form
   int dq_cap = 0;                 // drops the two tables above hold
+  shbim::FarState* far = nullptr; // lists of direct and far drop pairs, workspaces of the expansions
   int eos = SHBIM_EOS_LANGMUIR;      // tension law of shbim_rates / shbim_step (shbim_set_equation_of_state)
   bool refine_direct[2] = {true, true};     // refined solves (electric, Stokes): first inner solve aims at the end
   shbim_mlp* warm_net = nullptr;  // learned initial guesses of shbim_rates (shbim_set_warm_start), not owned
@@ -368,7 +371,6 @@ struct shbim_ctx {
   double class_ms[SHBIM_K_COUNT] = {0};
   int64_t class_launches[SHBIM_K_COUNT] = {0};
   double class_work[SHBIM_K_COUNT] = {0};
-  int64_t cross_pairs = 0;        // target-source pairs of different drops per all-pairs launch
 };
 
 namespace shbim {
@@ -471,8 +473,9 @@ int rotate_tc(shbim_ctx* ctx, const DegreeTables& T, bool adjoint, const float2*
               int t_begin, int ct, int ncomp, float2* vout, float* rows_lap, float* rows_sto, int nt_drop,
               cudaStream_t s);
 int dft_tc_digits(shbim_ctx* ctx, int p, DegreeTables& T);
-// the kernel holds a 128-row tile of W in shared memory: degrees up to 34
 bool dft_tc_fits(int p);
+// degrees above 39: the folded kernel, whose output is order-major (for the tensor-core Legendre stage)
+bool dft_tc_omajor_only(int p);
 int analysis_fourier_tc(shbim_ctx* ctx, const DegreeTables& T, const float2* W, int64_t rows, const int* rexp,
                         float2* F, cudaStream_t s, bool omajor = false);
 bool leg_tc_fits(int p);
@@ -488,12 +491,13 @@ int rebuild_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s);
 // added into out_accum
 // Stokes preconditioner basis and factors of the current geometry (gmres.cu)
 int build_stokes_preconditioner(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s);
-// quantised source positions of the FP64-class pair sums (once per geometry)
-int build_quantized_sources(shbim_ctx* ctx, cudaStream_t s);
+// extents of the drops, quantised source positions of the FP64-class pair sums and the lists of direct and
+// far drop pairs (once per geometry)
+int build_pair_lists(shbim_ctx* ctx, cudaStream_t s);
 int pairs_laplace(shbim_ctx* ctx, int which, double* out_accum, cudaStream_t s, cudaEvent_t before_reduce = nullptr);
 int pairs_stokes(shbim_ctx* ctx, bool has_f, bool has_u, double* out_accum, cudaStream_t s,
                  cudaEvent_t before_reduce = nullptr);
-// algorithmic flops of one all-pairs launch: cross pairs times the operations of one kernel term
+// algorithmic flops of one launch's direct sums: target-source pairs times the operations of one kernel term
 // (kind 0 Laplace DL, 1 SL, 2 Stokes S + D, 3 S, 4 D)
 double pairs_work(const shbim_ctx* ctx, int kind);
 

@@ -1,11 +1,12 @@
 // Tiled all-pairs sums of the regular rule (Eq. reg_quadrature) between different drops:
 // Laplace single layer and target-normal double layer (Eqs. E_n, dl_op_laplace), Stokeslet and
 // stresslet (Eqs. GandT, op_stokes). Same-drop pairs are excluded: those targets get the
-// singular self rows instead.
+// singular self rows instead. Pairs of drops far enough apart may go through expansions (far.cu); the kernels
+// here sum over each target drop's list of the others (NearList), which is every other drop where they do not pay.
 //
 // Work decomposition: the target list is cut into tiles of 512 targets of one drop; a CTA owns
 // 128 threads x TPT targets of a tile (register blocking, TPT = 1, 2 or 4, so a tile takes 4/TPT
-// CTAs) and one split of the other drops' sources; sources are staged through shared memory in
+// CTAs) and one split of the listed drops' sources; sources are staged through shared memory in
 // tiles of 256 and read as warp-wide broadcasts. Each split writes its own partial sums; a second
 // kernel adds the splits in a fixed order (deterministic). TPT, the split count and the launch
 // form (a CTA per unit, or persistent CTAs on an atomic work counter) are chosen per kernel kind
@@ -27,6 +28,7 @@
 #include <vector>
 
 #include "dfloat.cuh"
+#include "far.h"
 #include "internal.h"
 #include "pair_df.cuh"
 #include "pair_dq.cuh"
@@ -53,19 +55,34 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float a) {
   lo += e;
 }
 
-// virtual source index v in [0, nsource - ns_i) skips drop i's own sources
+// virtual source index v in [0, total): the sources of the target drop's direct list (NearList), one listed
+// drop after the other
 struct SrcRange {
   int64_t a, b;
 };
 
-__device__ __forceinline__ SrcRange drop_range(const DropDev& Di, const DropDev& Dj, int i, int j,
-                                               int64_t v0, int64_t v1) {
-  const int64_t shift = (j > i) ? Di.ns : 0;
-  const int64_t vs = Dj.src_off - shift;
-  const int64_t ve = vs + Dj.ns;
+// sources of drop j, at pre in the list, that fall in [v0, v1)
+__device__ __forceinline__ SrcRange drop_range(const DropDev& Dj, int64_t pre, int64_t v0, int64_t v1) {
   SrcRange r;
-  r.a = max(v0, vs) + shift;
-  r.b = min(v1, ve) + shift;
+  r.a = Dj.src_off + max(v0 - pre, (int64_t)0);
+  r.b = Dj.src_off + min(v1 - pre, (int64_t)Dj.ns);
+  return r;
+}
+
+// split `by` of `nsplit` of the target drop's list: [v0, v1) and the list's entries
+struct ListSplit {
+  int e0, e1;
+  int64_t v0, v1;
+};
+
+__device__ __forceinline__ ListSplit list_split(const NearList& nl, int i, int by, int nsplit) {
+  ListSplit r;
+  r.e0 = nl.off[i];
+  r.e1 = nl.off[i + 1] - 1;
+  const int64_t total = nl.pre[r.e1];
+  const int64_t chunk = (total + nsplit - 1) / nsplit;
+  r.v0 = (int64_t)by * chunk;
+  r.v1 = min(total, r.v0 + chunk);
   return r;
 }
 
@@ -86,7 +103,7 @@ __device__ __forceinline__ bool sub_tile(const PairTile* __restrict__ tiles, Pai
 // (uniformly for the CTA) for an empty sub-tile.
 template <int KIND, int kTPT>
 __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __restrict__ tiles,
-                                             const DropDev* __restrict__ drops, int n_drops,
+                                             const DropDev* __restrict__ drops, NearList nl,
                                              const double* __restrict__ tgt, int64_t ntarget,
                                              const float* __restrict__ src32, int64_t nsource,
                                              const float* __restrict__ dens32, int nsplit, int has_f, int has_u,
@@ -97,10 +114,7 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
   if (!sub_tile<kTPT>(tiles, tile, bx)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const int64_t other = nsource - Di.ns;
-  const int64_t chunk = (other + nsplit - 1) / nsplit;
-  const int64_t v0 = (int64_t)by * chunk;
-  const int64_t v1 = min(other, v0 + chunk);
+  const ListSplit ls = list_split(nl, i, by, nsplit);
 
   int64_t tg[kTPT];
   bool ok[kTPT];
@@ -123,10 +137,10 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
 #pragma unroll
     for (int c = 0; c < NC; ++c) hi[k][c] = lo[k][c] = 0.f;
 
-  for (int j = 0; j < n_drops; ++j) {
-    if (j == i) continue;
+  for (int en = ls.e0; en < ls.e1; ++en) {
+    const int j = nl.drop[en];
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Di, Dj, i, j, v0, v1);
+    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     float th[kTPT][3], tl[kTPT][3];
     const double cj[3] = {Dj.cx, Dj.cy, Dj.cz};
@@ -243,14 +257,14 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
 // one CTA per work unit (grid = sub-tiles x splits)
 template <int KIND, int kTPT>
 __global__ void __launch_bounds__(kThreads)
-k_pairs32(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, int n_drops,
+k_pairs32(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, NearList nl,
           const double* __restrict__ tgt, int64_t ntarget, const float* __restrict__ src32,
           int64_t nsource, const float* __restrict__ dens32, int nsplit, int has_f, int has_u,
           double* __restrict__ part) {
   __shared__ float4 sh0[kTile];
   __shared__ float4 sh1[stokes_kind(KIND) ? kTile : 1];
   __shared__ float4 sh2[stokes_kind(KIND) ? kTile : 1];
-  pairs32_unit<KIND, kTPT>(blockIdx.x, blockIdx.y, tiles, drops, n_drops, tgt, ntarget, src32, nsource, dens32,
+  pairs32_unit<KIND, kTPT>(blockIdx.x, blockIdx.y, tiles, drops, nl, tgt, ntarget, src32, nsource, dens32,
                            nsplit, has_f, has_u, part, sh0, sh1, sh2);
 }
 
@@ -259,7 +273,7 @@ k_pairs32(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
 // finish puts the counter back to zero for the next launch on the stream. No CTA waits on another.
 template <int KIND, int kTPT>
 __global__ void __launch_bounds__(kThreads)
-k_pairs32_queue(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, int n_drops,
+k_pairs32_queue(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, NearList nl,
                 const double* __restrict__ tgt, int64_t ntarget, const float* __restrict__ src32,
                 int64_t nsource, const float* __restrict__ dens32, int nsplit, int has_f, int has_u,
                 double* __restrict__ part, int nunits, int* __restrict__ queue) {
@@ -273,7 +287,7 @@ k_pairs32_queue(const PairTile* __restrict__ tiles, const DropDev* __restrict__ 
     __syncthreads();
     const int u = s_unit;
     if (u >= nunits) break;
-    pairs32_unit<KIND, kTPT>(u / nsplit, u - (u / nsplit) * nsplit, tiles, drops, n_drops, tgt, ntarget, src32,
+    pairs32_unit<KIND, kTPT>(u / nsplit, u - (u / nsplit) * nsplit, tiles, drops, nl, tgt, ntarget, src32,
                              nsource, dens32, nsplit, has_f, has_u, part, sh0, sh1, sh2);
   }
   if (threadIdx.x == 0) {
@@ -288,7 +302,7 @@ k_pairs32_queue(const PairTile* __restrict__ tiles, const DropDev* __restrict__ 
 
 template <int KIND>
 __global__ void __launch_bounds__(kThreads)
-k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, int n_drops,
+k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, NearList nl,
            const double* __restrict__ tgt, int64_t ntarget, const float* __restrict__ src32,
            const float* __restrict__ src32lo, int64_t nsource, const float* __restrict__ dens32,
            const float* __restrict__ dens32lo, int nsplit, int has_f, int has_u, double* __restrict__ part) {
@@ -300,10 +314,7 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   if (!sub_tile<1>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const int64_t other = nsource - Di.ns;
-  const int64_t chunk = (other + nsplit - 1) / nsplit;
-  const int64_t v0 = (int64_t)blockIdx.y * chunk;
-  const int64_t v1 = min(other, v0 + chunk);
+  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
   const int64_t tg = tile.t0 + threadIdx.x;
   const bool ok = (int)threadIdx.x < tile.nt;
   const int64_t t = ok ? tg : tile.t0;
@@ -315,10 +326,10 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
     N0[c] = dfl::from_double(tgt[(3 + c) * ntarget + t]);
   }
   dfl::acc A[NC];
-  for (int j = 0; j < n_drops; ++j) {
-    if (j == i) continue;
+  for (int en = ls.e0; en < ls.e1; ++en) {
+    const int j = nl.drop[en];
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Di, Dj, i, j, v0, v1);
+    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     const df T[3] = {dfl::from_double(X0[0] - Dj.cx), dfl::from_double(X0[1] - Dj.cy),
                      dfl::from_double(X0[2] - Dj.cz)};
@@ -378,11 +389,11 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
 // qs = 2^Q, qi = 2^-Q.
 template <int KIND>
 __global__ void __launch_bounds__(kThreads)
-k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, int n_drops,
+k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, NearList nl,
            const double* __restrict__ tgt, int64_t ntarget, const float* __restrict__ srcq,
            const float* __restrict__ src32, const float* __restrict__ src32lo, int64_t nsource,
            const float* __restrict__ dens32, const float* __restrict__ dens32lo, int nsplit, int has_f, int has_u,
-           double qs, double qi, const unsigned char* __restrict__ dq_far, double* __restrict__ part) {
+           double qs, double qi, const unsigned char* __restrict__ dq_far, int n_drops, double* __restrict__ part) {
   using dfl::df;
   constexpr int NC = stokes_kind(KIND) ? 3 : 1;
   constexpr int NV = stokes_kind(KIND) ? 6 : 2;   // float4 per staged source
@@ -391,10 +402,7 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   if (!sub_tile<1>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const int64_t other = nsource - Di.ns;
-  const int64_t chunk = (other + nsplit - 1) / nsplit;
-  const int64_t v0 = (int64_t)blockIdx.y * chunk;
-  const int64_t v1 = min(other, v0 + chunk);
+  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
   const int64_t tg = tile.t0 + threadIdx.x;
   const bool ok = (int)threadIdx.x < tile.nt;
   const int64_t t = ok ? tg : tile.t0;
@@ -406,10 +414,10 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
     N0[c] = dfl::from_double(tgt[(3 + c) * ntarget + t]);
   }
   dfl::acc A[NC];
-  for (int j = 0; j < n_drops; ++j) {
-    if (j == i) continue;
+  for (int en = ls.e0; en < ls.e1; ++en) {
+    const int j = nl.drop[en];
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Di, Dj, i, j, v0, v1);
+    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     const bool far = dq_far[(int64_t)i * n_drops + j] != 0;
     const double cj[3] = {Dj.cx, Dj.cy, Dj.cz};
@@ -482,7 +490,7 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
 
 template <int KIND, int kTPT>
 __global__ void __launch_bounds__(kThreads)
-k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, int n_drops,
+k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, NearList nl,
           const double* __restrict__ tgt, int64_t ntarget, const double* __restrict__ src,
           int64_t nsource, const double* __restrict__ dens, int nsplit, int has_f, int has_u,
           double* __restrict__ part) {
@@ -493,10 +501,7 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
   if (!sub_tile<kTPT>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const int64_t other = nsource - Di.ns;
-  const int64_t chunk = (other + nsplit - 1) / nsplit;
-  const int64_t v0 = (int64_t)blockIdx.y * chunk;
-  const int64_t v1 = min(other, v0 + chunk);
+  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
   int64_t tg[kTPT];
   bool ok[kTPT];
   double X0[kTPT][3], N0[kTPT][3], acc[kTPT][NC];
@@ -513,10 +518,10 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
 #pragma unroll
     for (int c = 0; c < NC; ++c) acc[k][c] = 0.0;
   }
-  for (int j = 0; j < n_drops; ++j) {
-    if (j == i) continue;
+  for (int en = ls.e0; en < ls.e1; ++en) {
+    const int j = nl.drop[en];
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Di, Dj, i, j, v0, v1);
+    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     for (int64_t base = rg.a; base < rg.b; base += kTile) {
       const int cnt = (int)min((int64_t)kTile, rg.b - base);
@@ -608,41 +613,41 @@ int queue_grid() {
 }
 
 template <int KIND, int TPT>
-void launch_shape(shbim_ctx* ctx, bool has_f, bool has_u, int splits, bool queue, cudaStream_t s) {
+void launch_shape(shbim_ctx* ctx, const NearList& nl, bool has_f, bool has_u, int splits, bool queue, cudaStream_t s) {
   dim3 grid((unsigned)(ctx->tiles.size() * (kMaxTPT / TPT)), splits);
   if (queue && ctx->opts.precision == SHBIM_PREC_FP32_COMP) {
     const int nunits = (int)(grid.x * grid.y);
     const int g = std::min(nunits, queue_grid<KIND, TPT>());
-    k_pairs32_queue<KIND, TPT><<<g, kThreads, 0, s>>>(ctx->tiles_dev, ctx->drops_dev, ctx->n_drops, ctx->geo.tgt,
+    k_pairs32_queue<KIND, TPT><<<g, kThreads, 0, s>>>(ctx->tiles_dev, ctx->drops_dev, nl, ctx->geo.tgt,
                                                        ctx->ntarget, ctx->geo.src32, ctx->nsource, ctx->dens_up32,
                                                        splits, has_f, has_u, ctx->part, nunits, ctx->pair_queue);
     return;
   }
   if (ctx->opts.precision == SHBIM_PREC_DF64 && ctx->dq_pairs && ctx->dq_scale > 0.0) {
     k_pairs_dq<KIND><<<dim3((unsigned)(ctx->tiles.size() * kMaxTPT), splits), kThreads, 0, s>>>(
-        ctx->tiles_dev, ctx->drops_dev, ctx->n_drops, ctx->geo.tgt, ctx->ntarget, ctx->geo.srcq, ctx->geo.src32,
+        ctx->tiles_dev, ctx->drops_dev, nl, ctx->geo.tgt, ctx->ntarget, ctx->geo.srcq, ctx->geo.src32,
         ctx->geo.src32lo, ctx->nsource, ctx->dens_up32, ctx->dens_up32lo, splits, has_f, has_u, ctx->dq_scale,
-        1.0 / ctx->dq_scale, ctx->dq_far, ctx->part);
+        1.0 / ctx->dq_scale, ctx->dq_far, ctx->n_drops, ctx->part);
   } else if (ctx->opts.precision == SHBIM_PREC_DF64) {
     k_pairs_df<KIND><<<dim3((unsigned)(ctx->tiles.size() * kMaxTPT), splits), kThreads, 0, s>>>(
-        ctx->tiles_dev, ctx->drops_dev, ctx->n_drops, ctx->geo.tgt, ctx->ntarget, ctx->geo.src32,
+        ctx->tiles_dev, ctx->drops_dev, nl, ctx->geo.tgt, ctx->ntarget, ctx->geo.src32,
         ctx->geo.src32lo, ctx->nsource, ctx->dens_up32, ctx->dens_up32lo, splits, has_f, has_u, ctx->part);
   } else if (ctx->opts.precision == SHBIM_PREC_FP32_COMP) {
-    k_pairs32<KIND, TPT><<<grid, kThreads, 0, s>>>(ctx->tiles_dev, ctx->drops_dev, ctx->n_drops, ctx->geo.tgt,
+    k_pairs32<KIND, TPT><<<grid, kThreads, 0, s>>>(ctx->tiles_dev, ctx->drops_dev, nl, ctx->geo.tgt,
                                                    ctx->ntarget, ctx->geo.src32, ctx->nsource, ctx->dens_up32,
                                                    splits, has_f, has_u, ctx->part);
   } else {
-    k_pairs64<KIND, TPT><<<grid, kThreads, 0, s>>>(ctx->tiles_dev, ctx->drops_dev, ctx->n_drops, ctx->geo.tgt,
+    k_pairs64<KIND, TPT><<<grid, kThreads, 0, s>>>(ctx->tiles_dev, ctx->drops_dev, nl, ctx->geo.tgt,
                                                    ctx->ntarget, ctx->geo.src, ctx->nsource, ctx->dens_up,
                                                    splits, has_f, has_u, ctx->part);
   }
 }
 
 template <int KIND>
-void launch_raw(shbim_ctx* ctx, bool has_f, bool has_u, int tpt, int splits, bool queue, cudaStream_t s) {
-  if (tpt == 4) launch_shape<KIND, 4>(ctx, has_f, has_u, splits, queue, s);
-  else if (tpt == 2) launch_shape<KIND, 2>(ctx, has_f, has_u, splits, queue, s);
-  else launch_shape<KIND, 1>(ctx, has_f, has_u, splits, queue, s);
+void launch_raw(shbim_ctx* ctx, const NearList& nl, bool has_f, bool has_u, int tpt, int splits, bool queue, cudaStream_t s) {
+  if (tpt == 4) launch_shape<KIND, 4>(ctx, nl, has_f, has_u, splits, queue, s);
+  else if (tpt == 2) launch_shape<KIND, 2>(ctx, nl, has_f, has_u, splits, queue, s);
+  else launch_shape<KIND, 1>(ctx, nl, has_f, has_u, splits, queue, s);
 }
 
 // Choose the register blocking (targets per thread), the source-split count and the launch form
@@ -651,7 +656,7 @@ void launch_raw(shbim_ctx* ctx, bool has_f, bool has_u, int tpt, int splits, boo
 // layout's default (times 1/4 ... 4, at most the partial-buffer capacity), in both forms, is
 // launched twice and the second launch timed with CUDA events; the fastest is kept.
 template <int KIND>
-int autotune(shbim_ctx* ctx, bool has_f, bool has_u, cudaStream_t s) {
+int autotune(shbim_ctx* ctx, const NearList& nl, bool has_f, bool has_u, cudaStream_t s) {
   auto& C = ctx->pair_cfg[KIND];
   C.tuned = true;
   if (ctx->timing || ctx->opts.precision != SHBIM_PREC_FP32_COMP) return SHBIM_OK;
@@ -672,9 +677,9 @@ int autotune(shbim_ctx* ctx, bool has_f, bool has_u, cudaStream_t s) {
   for (int q = 0; q < 2; ++q)
     for (int tpt = 1; tpt <= kMaxTPT; tpt *= 2) {
       for (int sp = sp0; sp <= hi; sp *= 2) {
-        launch_raw<KIND>(ctx, has_f, has_u, tpt, sp, q != 0, s);  // warm
+        launch_raw<KIND>(ctx, nl, has_f, has_u, tpt, sp, q != 0, s);  // warm
         cudaEventRecord(a, s);
-        launch_raw<KIND>(ctx, has_f, has_u, tpt, sp, q != 0, s);
+        launch_raw<KIND>(ctx, nl, has_f, has_u, tpt, sp, q != 0, s);
         cudaEventRecord(b, s);
         cudaEventSynchronize(b);
         float ms = 0.f;
@@ -734,40 +739,52 @@ int launch_pairs(shbim_ctx* ctx, bool has_f, bool has_u, double* out, cudaStream
     if (before_reduce) SHBIM_CUDA(ctx, cudaStreamWaitEvent(s, before_reduce, 0));
     return SHBIM_OK;
   }
-  auto& C = ctx->pair_cfg[KIND];
-  if (!C.tuned) {
-    int rc = autotune<KIND>(ctx, has_f, has_u, s);
-    if (rc) return rc;
+  // well-separated drop pairs through expansions (far.cu), where they pay; the rest directly
+  const FarPlan* far = far_plan(ctx, KIND);
+  if (!ctx->far) return fail(ctx, SHBIM_ERR_ARG, "no drop pair lists: the last shbim_set_drops failed");
+  const FarPlan& plan = far ? *far : far_all(ctx);
+  const NearList& nl = plan.near;
+  if (!nl.off) return fail(ctx, SHBIM_ERR_ARG, "no drop pair lists: the last shbim_set_drops failed");
+  int rc;
+  if (far && (rc = far_expand(ctx, *far, KIND, s))) return rc;
+  if (plan.direct_pairs == 0.0) {
+    if (before_reduce) SHBIM_CUDA(ctx, cudaStreamWaitEvent(s, before_reduce, 0));
+    return far ? far_evaluate(ctx, *far, KIND, out, s) : SHBIM_OK;
   }
+  auto& C = ctx->pair_cfg[KIND];
+  if (!C.tuned && (rc = autotune<KIND>(ctx, nl, has_f, has_u, s))) return rc;
   // the FP64 kernels keep the layout's default shape; the FP64-class kernel (4 CTAs per tile, one target
   // per thread) takes the split count fp64class_splits chooses for its occupancy
   const bool fp32 = ctx->opts.precision == SHBIM_PREC_FP32_COMP;
   const bool df = ctx->opts.precision == SHBIM_PREC_DF64;
   const int tpt = fp32 ? C.tpt : (df ? 1 : 2);
   const int splits = fp32 ? C.splits : (df ? fp64class_splits<KIND>(ctx) : ctx->pair_splits);
-  launch_raw<KIND>(ctx, has_f, has_u, tpt, splits, fp32 && C.queue, s);
+  launch_raw<KIND>(ctx, nl, has_f, has_u, tpt, splits, fp32 && C.queue, s);
   SHBIM_CHECK_LAUNCH(ctx, "k_pairs");
   if (before_reduce) SHBIM_CUDA(ctx, cudaStreamWaitEvent(s, before_reduce, 0));
   const int64_t n = NC * ctx->ntarget;
   k_reduce_parts<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ctx->part, splits, n, out);
   SHBIM_CHECK_LAUNCH(ctx, "k_reduce_parts");
-  return SHBIM_OK;
+  return far ? far_evaluate(ctx, *far, KIND, out, s) : SHBIM_OK;
 }
 
-// Largest |x - c| (Euclidean) over the sources of every drop: one CTA row per drop; the maximum goes to
-// out[drop] as the bit pattern of a non-negative float (integer order = float order), rounded up.
-__global__ void k_src_extent(const double* __restrict__ src, int64_t nsource, const DropDev* __restrict__ drops,
-                             unsigned* __restrict__ out) {
+// Largest |x - c| (Euclidean) over the sources (blockIdx.z 0) and the targets (1) of every drop: one CTA row per
+// drop; the maximum goes to out[drop], out[n + drop] as the bit pattern of a non-negative float (integer order =
+// float order), rounded up.
+__global__ void k_extent(const double* __restrict__ src, int64_t nsource, const double* __restrict__ tgt,
+                         int64_t ntarget, const DropDev* __restrict__ drops, unsigned* __restrict__ out) {
   const DropDev D = drops[blockIdx.y];
+  const bool t = blockIdx.z != 0;
+  const double* pos = t ? tgt + D.tgt_off : src + D.src_off;
+  const int64_t ld = t ? ntarget : nsource, n = t ? D.nt : D.ns;
   float m = 0.0f;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < D.ns; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t sI = D.src_off + e;
-    const double dx = src[sI] - D.cx, dy = src[nsource + sI] - D.cy, dz = src[2 * nsource + sI] - D.cz;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const double dx = pos[e] - D.cx, dy = pos[ld + e] - D.cy, dz = pos[2 * ld + e] - D.cz;
     m = fmaxf(m, __double2float_ru(sqrt(dx * dx + dy * dy + dz * dz)));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out + blockIdx.y, __float_as_uint(m));
+  if ((threadIdx.x & 31) == 0) atomicMax(out + (t ? gridDim.y : 0) + blockIdx.y, __float_as_uint(m));
 }
 
 // v = x - c split as the multiple vq of qi = 2^-Q nearest to v and the FP32 remainder vl = v - vq
@@ -802,6 +819,7 @@ int pairs_stokes(shbim_ctx* ctx, bool has_f, bool has_u, double* out, cudaStream
 
 int pairs_tile_targets() { return kTileTargets; }
 
+// Extents of the drops, then:
 // Quantum of the FP64-class pair sums for the current geometry (pair_dq.cuh) and the drop pairs that
 // use it. With ext_j the largest |x - c_j| of drop j's nodes, B = max over pairs of drops of
 // |c_i - c_j| (per component) + 1.01 ext_i + ext_j bounds every target offset |x0 - c_j|, every source
@@ -811,7 +829,7 @@ int pairs_tile_targets() { return kTileTargets; }
 // remainders below the quantum are good to ~2^-(Q+23) absolute, ~2^-42 relative to r for r >= 2^(19-Q):
 // the quantised form is used for drop pairs whose surfaces are at least that far apart,
 // |c_i - c_j| - 1.01 ext_i - ext_j >= 2^(19-Q); closer pairs keep the general double-float form.
-int build_quantized_sources(shbim_ctx* ctx, cudaStream_t s) {
+int build_pair_lists(shbim_ctx* ctx, cudaStream_t s) {
   ctx->dq_scale = 0.0;
   const int nd = ctx->n_drops;
   if (nd < 2 || !ctx->geo.srcq) return SHBIM_OK;
@@ -820,7 +838,7 @@ int build_quantized_sources(shbim_ctx* ctx, cudaStream_t s) {
     cudaFree(ctx->dq_far);
     ctx->dq_ext_dev = nullptr;
     ctx->dq_far = nullptr;
-    if (cudaMalloc(&ctx->dq_ext_dev, (size_t)nd * sizeof(unsigned)) != cudaSuccess ||
+    if (cudaMalloc(&ctx->dq_ext_dev, (size_t)2 * nd * sizeof(unsigned)) != cudaSuccess ||
         cudaMalloc(&ctx->dq_far, (size_t)nd * nd) != cudaSuccess)
       return fail(ctx, SHBIM_ERR_NOMEM, "cudaMalloc quantisation tables");
     ctx->dq_cap = nd;
@@ -828,18 +846,21 @@ int build_quantized_sources(shbim_ctx* ctx, cudaStream_t s) {
   int maxns = 0;
   for (const auto& d : ctx->drops) maxns = std::max(maxns, d.ns);
   const dim3 grid((unsigned)std::min(64, (maxns + 255) / 256), (unsigned)nd);
-  SHBIM_CUDA(ctx, cudaMemsetAsync(ctx->dq_ext_dev, 0, (size_t)nd * sizeof(unsigned), s));
-  k_src_extent<<<grid, 256, 0, s>>>(ctx->geo.src, ctx->nsource, ctx->drops_dev, ctx->dq_ext_dev);
-  SHBIM_CHECK_LAUNCH(ctx, "k_src_extent");
-  std::vector<unsigned> bits(nd);
-  SHBIM_CUDA(ctx, cudaMemcpyAsync(bits.data(), ctx->dq_ext_dev, (size_t)nd * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+  SHBIM_CUDA(ctx, cudaMemsetAsync(ctx->dq_ext_dev, 0, (size_t)2 * nd * sizeof(unsigned), s));
+  k_extent<<<dim3(grid.x, grid.y, 2), 256, 0, s>>>(ctx->geo.src, ctx->nsource, ctx->geo.tgt, ctx->ntarget,
+                                                  ctx->drops_dev, ctx->dq_ext_dev);
+  SHBIM_CHECK_LAUNCH(ctx, "k_extent");
+  std::vector<unsigned> bits(2 * nd);
+  SHBIM_CUDA(ctx, cudaMemcpyAsync(bits.data(), ctx->dq_ext_dev, (size_t)2 * nd * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
   SHBIM_CUDA(ctx, cudaStreamSynchronize(s));
-  std::vector<double> ext(nd);
-  for (int i = 0; i < nd; ++i) {
+  std::vector<double> ext(2 * nd);
+  for (int i = 0; i < 2 * nd; ++i) {
     float e;
     std::memcpy(&e, &bits[i], sizeof(e));
     ext[i] = (double)e;
   }
+  // the lists stand for any extents (a non-finite one makes every pair of its drop direct)
+  if (int rc = build_far(ctx, ext, s)) return rc;
   double B = 0.0;
   for (int i = 0; i < nd; ++i)
     for (int j = 0; j < nd; ++j) {
@@ -867,7 +888,6 @@ int build_quantized_sources(shbim_ctx* ctx, cudaStream_t s) {
   k_quantize_src<<<grid, 256, 0, s>>>(ctx->geo.src, ctx->nsource, ctx->drops_dev, ctx->dq_scale,
                                       std::ldexp(1.0, -Q), ctx->geo.srcq);
   SHBIM_CHECK_LAUNCH(ctx, "k_quantize_src");
-  ctx->launches += 2;
   return SHBIM_OK;
 }
 
@@ -882,7 +902,9 @@ int build_quantized_sources(shbim_ctx* ctx, cudaStream_t s) {
 // (the 1/(4 pi) and the stresslet's -6 (lambda - 1) are applied per target or folded into strengths)
 double pairs_work(const shbim_ctx* ctx, int kind) {
   static const double kFlops[5] = {19.0, 11.0, 42.0, 29.0, 30.0};
-  return kind >= 0 && kind < 5 ? kFlops[kind] * (double)ctx->cross_pairs : 0.0;
+  if (kind < 0 || kind > 4 || ctx->n_drops < 2 || !ctx->far) return 0.0;
+  const FarPlan* far = far_plan(ctx, kind);
+  return kFlops[kind] * (far ? far->direct_pairs : far_all(ctx).direct_pairs);
 }
 
 }  // namespace shbim
