@@ -111,6 +111,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&a)[16]) {
       : "r"(addr));
 }
 
+// 4 consecutive FP32 columns of the warp's 32 tensor-memory lanes
+__device__ __forceinline__ void tmem_ld4(uint32_t addr, uint32_t (&a)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+               : "r"(addr));
+}
+
 // 8 consecutive FP32 columns of the warp's 32 tensor-memory lanes
 __device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t (&a)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
