@@ -575,8 +575,9 @@ int build_singular_rows_df(shbim_ctx* ctx, cudaStream_t s, const double* xcoef) 
     const int df_n0 = rot_n + 1;
     const int leg_smem = (d.q + 1) * 2 * (d.p + 1) * (int)sizeof(float2);
     SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_analysis_leg_item_df, cudaFuncAttributeMaxDynamicSharedMemorySize, leg_smem));
-    const bool dft_tc = ctx->tc_rows && dft_tc_fits(d.p);
-    const bool leg_tc = dft_tc && ctx->tc_leg && leg_tc_fits(d.p);   // reads the order-major Fourier output
+    const bool leg_fits = ctx->tc_leg && leg_tc_fits(d.p);
+    const bool dft_tc = ctx->tc_rows && dft_tc_fits(d.p) && (leg_fits || !dft_tc_omajor_only(d.p));
+    const bool leg_tc = dft_tc && leg_fits;   // reads the order-major Fourier output
     for (int t0 = 0; t0 < d.nt; t0 += CT, ++c) {
       const int ct = std::min(CT, d.nt - t0);
       const int lane = two ? (c & 1) : 0;
