@@ -18,8 +18,13 @@
 // fill one of two stages and one thread issues the 21 digit products as 9 MMAs (one row digit
 // against up to three table digits, N <= 240); the epilogue combines the six
 // accumulators in double-float. Every wait is bounded; a timeout sets the error flag and the CTA
-// stops. Degree blocks with 2n+1 <= 80 (n <= 39) only: for drops of higher degree (whose shared memory
-// still fits, p <= 48) the degrees above 39 use the FP32-pipe kernel (singular_df.cu).
+// stops.
+//
+// Degrees 40 to 63 (SPLIT): M couples neither cosine orders with sine orders nor the reverse (a rotation about y commutes
+// with the reflection y -> -y), so the block is two blocks of n (sine) and n + 1 (cosine) rows, contiguous in the
+// coefficient order: two GEMMs of half the size each, a quarter of the products, that fit tensor memory with seven
+// digits (these degrees were double-float before and keep that accuracy). Angles come from L1 there: the value block
+// takes the shared memory. Degree 64 (65 cosine rows) stays on the FP32-pipe kernel (singular_df.cu).
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -42,6 +47,10 @@ static_assert(diag_sums_exact(kNmax), "rotations: digit sums must stay exact in 
 constexpr int kPlaneA = kMT * kKS;                          // bf16 per row-digit plane
 constexpr int kPlaneBmax = kNmax * kKS;                     // bf16 per table-digit plane
 constexpr int kStageBytes = kDig * (kPlaneA + kPlaneBmax) * 2;
+constexpr int kSplitNmax = 64;                              // largest padded half block
+constexpr int kSplitFirst = 40, kSplitLast = 63;            // degrees of the split form
+static_assert(diag_sums_exact7(kSplitNmax), "split rotations: digit sums must stay exact in FP32");
+constexpr int kStageSplit = kDig7 * (kPlaneA + kSplitNmax * kKS) * 2;
 constexpr uint32_t kTmemCols = 512;
 
 __device__ __forceinline__ df lds(const float2* p, int i) {
@@ -67,17 +76,17 @@ __device__ __forceinline__ void cp_async_wait_all() {
 __host__ __device__ inline int max_targets(int ncomp) { return kMT / ncomp + 2; }
 
 // The items of one launch: latitudes lat0 .. lat0 + L - 1 of the chunk, T tiles of 128 vectors per
-// latitude, degrees nmax .. 0 (nmax <= p: the higher degrees of a drop whose blocks exceed kNmax are
+// latitude, degrees nmax .. nmin (nmax <= p: the higher degrees of a drop whose blocks exceed kNmax are
 // rotated by the double-float kernel).
 struct Items {
-  int p, nmax, nlon, ncomp, t_begin, ct, lat0, L, T;
+  int p, nmax, nmin, nlon, ncomp, t_begin, ct, lat0, L, T;
   int64_t total;
-  __host__ __device__ Items(int p_, int nmax_, int ncomp_, int t_begin_, int ct_)
-      : p(p_), nmax(nmax_), nlon(2 * p_ + 2), ncomp(ncomp_), t_begin(t_begin_), ct(ct_) {
+  __host__ __device__ Items(int p_, int nmax_, int nmin_, int ncomp_, int t_begin_, int ct_)
+      : p(p_), nmax(nmax_), nmin(nmin_), nlon(2 * p_ + 2), ncomp(ncomp_), t_begin(t_begin_), ct(ct_) {
     lat0 = t_begin / nlon;
     L = (t_begin + ct - 1) / nlon - lat0 + 1;
     T = (nlon * ncomp + kMT - 1) / kMT;
-    total = (int64_t)(nmax + 1) * L * T;
+    total = (int64_t)(nmax + 1 - nmin) * L * T;
   }
   // degree, latitude and chunk-local vector range [va, vb) of an item (empty if va >= vb)
   __device__ void decode(int64_t it, int& n, int& lat, int& va, int& vb) const {
@@ -101,27 +110,34 @@ struct Items {
   }
 };
 
-template <bool ADJ>
+// parts of a degree block: one of 2n + 1 rows, or (SPLIT) the sine rows [0, n) and the cosine rows [n, 2n + 1)
+__host__ __device__ inline int part_len(bool split, int n, int part) { return split ? n + part : 2 * n + 1; }
+__host__ __device__ inline int part_off(bool split, int n, int part) { return split ? part * n : 0; }
+
+template <bool ADJ, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
-k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, int nmax, int t_begin, int ct, int ncomp,
+k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, int nmax, int nmin, int t_begin, int ct, int ncomp,
             const float2* __restrict__ cs_phi, const uint4* __restrict__ tdig, const int* __restrict__ toff,
             const signed char* __restrict__ texp, float2* __restrict__ vout, float* __restrict__ rows_lap,
             float* __restrict__ rows_sto, int nt_drop, int* __restrict__ err, uint64_t wlim) {
-  // dynamic shared memory: [two MMA stages][value block 128 x (2p+1)][(cos, sin)(m phi) of the
-  // item's targets, 2 (p+1) each]
+  constexpr int ND = SPLIT ? kDig7 : kDig;
+  constexpr int kParts = SPLIT ? 2 : 1;
+  constexpr int kStage = SPLIT ? kStageSplit : kStageBytes;
+  // dynamic shared memory: [two MMA stages][value block 128 x (2 nmax + 1)][(cos, sin)(m phi) of the
+  // item's targets, 2 (p+1) each, unless SPLIT]
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ __align__(8) uint64_t bbar[2];
   __shared__ uint32_t tmem_base;
   __shared__ int rowexp[kMT];
   __shared__ int rowtgt[kMT];
-  __shared__ int colexp[kNmax];
-  const int WS = 2 * p + 1;   // row stride of the value block (odd: conflict-free column access)
+  __shared__ int colexp[SPLIT ? 2 * kSplitNmax : kNmax];
+  const int WS = 2 * nmax + 1;   // row stride of the value block (odd: conflict-free column access)
   const int CS = 2 * (p + 1); // one angle table
-  float2* sX = reinterpret_cast<float2*>(smem + 2 * kStageBytes);
+  float2* sX = reinterpret_cast<float2*>(smem + 2 * kStage);
   float2* sCS = sX + kMT * WS;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const Items I(p, nmax, ncomp, t_begin, ct);
+  const Items I(p, nmax, nmin, ncomp, t_begin, ct);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_base)),
                  "r"(kTmemCols));
@@ -144,20 +160,24 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
   bool abort_all = false;
   const int r_loc = tid & (kMT - 1), qt = tid >> 7;   // row of the tile, quarter of a K step
   // table planes of (latitude, degree), K step ks, into stage st (thread 0)
-  auto issue_b = [&](int lat, int n, int ks, int st) {
-    const int Np = padded(2 * n + 1);
-    const uint32_t bytes = (uint32_t)(kDig * Np * kKS * 2);
-    const int64_t o = toff[((ADJ ? 1 : 0) * (p + 1) + lat) * (p + 1) + n];
-    bulk_load(smem + st * kStageBytes + kDig * kPlaneA * 2, tdig + o + (int64_t)ks * (bytes / 16), bytes, &bbar[st]);
+  auto issue_b = [&](int lat, int n, int part, int ks, int st) {
+    const int Np = padded(part_len(SPLIT, n, part));
+    const uint32_t bytes = (uint32_t)(ND * Np * kKS * 2);
+    int64_t o = toff[((ADJ ? 1 : 0) * (p + 1) + lat) * (p + 1) + n];
+    if (part) {
+      const int N0 = padded(part_len(SPLIT, n, 0));
+      o += (int64_t)(N0 / kKS) * (ND * N0 * kKS * 2 / 16);
+    }
+    bulk_load(smem + st * kStage + ND * kPlaneA * 2, tdig + o + (int64_t)ks * (bytes / 16), bytes, &bbar[st]);
   };
-  // the first two K steps' table planes of item `it` (both stages free)
-  auto prefetch = [&](int64_t it) {
+  // the first two K steps' table planes of a part of item `it` (both stages free)
+  auto prefetch = [&](int64_t it, int part) {
     int n, lat, va, vb;
     I.decode(it, n, lat, va, vb);
-    const bool two = padded(2 * n + 1) > kKS;
+    const bool two = padded(part_len(SPLIT, n, part)) > kKS;
     if (tid == 0) {
-      issue_b(lat, n, 0, 0);
-      if (two) issue_b(lat, n, 1, 1);
+      issue_b(lat, n, part, 0, 0);
+      if (two) issue_b(lat, n, part, 1, 1);
     }
     bpend[0] = true;
     bpend[1] = two;
@@ -166,7 +186,7 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
   auto dz = [&](int n, bool neg) {
     const int rt = rowtgt[r_loc];
     if (rt < 0) return;
-    const float2* cs = sCS + rt * CS;
+    const float2* cs = SPLIT ? cs_phi + (int64_t)rt * CS : sCS + rt * CS;
     float2* x = sX + r_loc * WS;
     for (int m = 1 + qt; m <= n; m += 4) {
       const float2 c2 = cs[m], s2 = cs[p + 1 + m];
@@ -179,23 +199,22 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
   };
 
   int64_t item = I.next(blockIdx.x, gridDim.x);
-  if (item < I.total) prefetch(item);
+  if (item < I.total) prefetch(item, 0);
   while (item < I.total && !abort_all) {
     int n, lat, va, vb;
     I.decode(item, n, lat, va, vb);
     const int w = 2 * n + 1;
-    const int Np = padded(w);
-    const int ksteps = Np / kKS;
     const int b_lo = va / ncomp;
     const int nb = (vb - 1) / ncomp - b_lo + 1;
     // rows of the item (vector v = chunk-local target b, component c), their targets' phi tables
     // and degree blocks: asynchronous copies, one wait
     if (tid < kMT) {
       const int v = va + tid;
-      rowtgt[tid] = v < vb ? v / ncomp - b_lo : -1;
+      // index of the row's angle table: among the item's targets, or (SPLIT) its longitude
+      rowtgt[tid] = v < vb ? (SPLIT ? (t_begin + v / ncomp) % I.nlon : v / ncomp - b_lo) : -1;
     }
     if (tid < w) colexp[tid] = texp[((int64_t)(ADJ ? 1 : 0) * (p + 1) + lat) * (p + 1) * (p + 1) + n * n + tid];
-    for (int e = tid; e < nb * (CS / 2); e += kThreads) {
+    for (int e = tid; !SPLIT && e < nb * (CS / 2); e += kThreads) {
       const int bt = e / (CS / 2), k2 = e - bt * (CS / 2);   // target, 16-byte piece of its table
       const int tl = t_begin + b_lo + bt;
       const float2* src = cs_phi + (int64_t)(tl % I.nlon) * CS;
@@ -217,19 +236,24 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
       dz(n, true);
       __syncthreads();
     }
+    int64_t next = item;
+    for (int part = 0; part < kParts; ++part) {
+    const int wp = part_len(SPLIT, n, part), o0 = part_off(SPLIT, n, part);
+    const int Np = padded(wp);
+    const int ksteps = Np / kKS;
     // per-row power-of-two scale, max |hi| < 2^e: one thread per row (odd row stride: no bank
     // conflicts)
     if (tid < kMT) {
       float mx = 0.f;
-      const float2* xr = sX + tid * WS;
-      for (int k = 0; k < w; ++k) mx = fmaxf(mx, fabsf(xr[k].x));
+      const float2* xr = sX + tid * WS + o0;
+      for (int k = 0; k < wp; ++k) mx = fmaxf(mx, fabsf(xr[k].x));
       int e = 0;
       frexpf(mx, &e);
       rowexp[tid] = max(e, -120);
     }
     __syncthreads();
     const int e_r = rowexp[r_loc];
-    const float2* xrow = sX + r_loc * WS;
+    const float2* xrow = sX + r_loc * WS + o0;
     for (int ks = 0; ks < ksteps; ++ks) {
       const int st = ks & 1;
       if (pending[st]) {
@@ -241,22 +265,22 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
           break;
         }
       }
-      uint8_t* base = smem + st * kStageBytes;
+      uint8_t* base = smem + st * kStage;
       {
         const float sc = __int_as_float((127 + 7 - e_r) << 23);   // 2^(7 - e), exact
-        float d[kDig][4];
+        float d[ND][4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int k = ks * kKS + qt * 4 + i;
-          const float2 v = k < w ? xrow[k] : make_float2(0.f, 0.f);
-          float dd[kDig];
-          digits6(v.x * sc, v.y * sc, dd);
+          const float2 v = k < wp ? xrow[k] : make_float2(0.f, 0.f);
+          float dd[ND];
+          digits_n<ND>(v.x * sc, v.y * sc, dd);
 #pragma unroll
-          for (int j = 0; j < kDig; ++j) d[j][i] = dd[j];
+          for (int j = 0; j < ND; ++j) d[j][i] = dd[j];
         }
         const int off = canon16(r_loc, qt * 4) * 2;   // bytes; 8-byte aligned
 #pragma unroll
-        for (int j = 0; j < kDig; ++j) {
+        for (int j = 0; j < ND; ++j) {
           uint2 q;
           q.x = pack_bf16f(d[j][0], d[j][1]);
           q.y = pack_bf16f(d[j][2], d[j][3]);
@@ -270,26 +294,25 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
         // caller sees the error flag)
         if (!mbar_wait(&bbar[st], bphase[st], wlim)) atomicExch(err, 1);
         asm volatile("tcgen05.fence::after_thread_sync;\n");
-        const uint32_t a0 = smem_u32(base), b0 = smem_u32(base + kDig * kPlaneA * 2);
-        // row digit j_a against up to three consecutive table digits in one MMA of N = Np g (the
+        const uint32_t a0 = smem_u32(base), b0 = smem_u32(base + ND * kPlaneA * 2);
+        // row digit j_a against as many consecutive table digits as N <= 256 allows in one MMA (the
         // planes lie one after the other like the rows of one operand; their products go to the
-        // consecutive accumulators j_a + j_b - 5 ..); j_a = 5 first, overwriting all six in step 0
-#pragma unroll
-        for (int ja = kDig - 1; ja >= 0; --ja)
-#pragma unroll
-          for (int jb0 = kDig - 1 - ja; jb0 < kDig; jb0 += 3) {
-            const int g = min(3, kDig - jb0);
-            const int dgl = ja + jb0 - (kDig - 1);
-            const uint32_t acc = (ks > 0 || ja != kDig - 1) ? 1u : 0u;
-            mma_bf16(tmem + (uint32_t)(dgl * Np), desc_k16(a0 + ja * kPlaneA * 2), desc_k16(b0 + jb0 * Np * kKS * 2),
-                     idesc_bf16(Np * g), acc);
+        // consecutive accumulators j_a + j_b - ND + 1 ..); the top row digit first, overwriting all of them in step 0
+        const int gmax = 256 / Np;
+        for (int ja = ND - 1; ja >= 0; --ja)
+          for (int jb = ND - 1 - ja; jb < ND;) {
+            const int g = min(gmax, ND - jb);
+            const uint32_t acc = (ks > 0 || ja != ND - 1) ? 1u : 0u;
+            mma_bf16(tmem + (uint32_t)((ja + jb - (ND - 1)) * Np), desc_k16(a0 + ja * kPlaneA * 2),
+                     desc_k16(b0 + jb * Np * kKS * 2), idesc_bf16(Np * g), acc);
+            jb += g;
           }
         mma_commit(&mbar[st]);
         // the table planes of K step ks + 1 go to the other stage once its products are done
         // (step 1's planes were issued with step 0's)
         if (ks >= 1 && ks + 1 < ksteps) {
           mbar_wait(&mbar[st ^ 1], phase[st ^ 1], wlim);
-          issue_b(lat, n, ks + 1, st ^ 1);
+          issue_b(lat, n, part, ks + 1, st ^ 1);
         }
       }
       bphase[st] ^= 1u;
@@ -309,9 +332,13 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
       abort_all = true;
       break;
     }
-    // both stages are free: the next item's first table planes travel during the epilogue
-    const int64_t next = I.next(item + gridDim.x, gridDim.x);
-    if (next < I.total) prefetch(next);
+    // both stages are free: the next part's or item's first table planes travel during the epilogue
+    if (part + 1 < kParts) {
+      prefetch(item, part + 1);
+    } else {
+      next = I.next(item + gridDim.x, gridDim.x);
+      if (next < I.total) prefetch(next, 0);
+    }
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     // epilogue: warp w reads lanes 32 (w % 4) .. +31; column blocks of 8 split among w, w+4, w+8, w+12
     {
@@ -319,18 +346,19 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
       const int rl = 32 * lq + lane;
       const int ee = rowexp[rl];
       for (int cb = wq; cb < Np / 8; cb += 4) {
-        uint32_t a[kDig][8];
+        uint32_t a[ND][8];
 #pragma unroll
-        for (int dg = 0; dg < kDig; ++dg)
+        for (int dg = 0; dg < ND; ++dg)
           tmem_ld8(tmem + ((uint32_t)(32 * lq) << 16) + (uint32_t)(dg * Np + cb * 8), a[dg]);
         asm volatile("tcgen05.wait::ld.sync.aligned;\n");
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int o = cb * 8 + j;
-          if (o < w) {
-            const df r = combine6(__uint_as_float(a[5][j]), __uint_as_float(a[4][j]), __uint_as_float(a[3][j]),
-                                  __uint_as_float(a[2][j]), __uint_as_float(a[1][j]), __uint_as_float(a[0][j]));
-            sX[rl * WS + o] = scale2(r, ee + colexp[o] - 14);
+          if (o < wp) {
+            float s[ND];
+#pragma unroll
+            for (int dg = 0; dg < ND; ++dg) s[dg] = __uint_as_float(a[dg][j]);
+            sX[rl * WS + o0 + o] = scale2(combine_n<ND>(s), ee + colexp[o0 + o] - 14);
           }
         }
       }
@@ -339,6 +367,8 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n");
+    }  // parts
+    if (abort_all) break;
     if (ADJ) {
       dz(n, false);
       __syncthreads();
@@ -376,21 +406,24 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
 }
 
-int rot_tc_smem(int p, int ncomp) {
-  return 2 * kStageBytes + (kMT * (2 * p + 1) + max_targets(ncomp) * 2 * (p + 1)) * (int)sizeof(float2);
+int rot_tc_smem(int p, int nmax, int ncomp) {
+  return 2 * kStageBytes + (kMT * (2 * nmax + 1) + max_targets(ncomp) * 2 * (p + 1)) * (int)sizeof(float2);
 }
 
-}  // namespace
+int rot_split_smem(int nmax) { return 2 * kStageSplit + kMT * (2 * nmax + 1) * (int)sizeof(float2); }
 
-// Highest degree the tensor-core rotations take for drops of degree p (blocks up to kNmax), or -1 where
-// the shared memory of degree p does not fit (the forward rotation, 3 components per target, needs the
-// most angle tables); the degrees above it go to the double-float kernel.
-int rot_tc_nmax(int p) {
-  if (rot_tc_smem(p, 3) + 4096 > 227 * 1024) return -1;
+// highest degree of the whole-block form: blocks up to kNmax
+int rot_whole_nmax(int p) {
   int n = p;
   while (n >= 0 && padded(2 * n + 1) > kNmax) --n;
   return n;
 }
+
+}  // namespace
+
+// Highest degree the tensor-core rotations take for drops of degree p: all of them up to 63 (whole blocks to degree
+// 39, split blocks above); degree 64 goes to the double-float kernel.
+int rot_tc_nmax(int p) { return std::min(p, kSplitLast); }
 
 // Digit planes of M = Dq_n^T Dz(-theta_j) Dq_n (forward, dir 0) and Dq_n^T Dz(theta_j) Dq_n
 // (adjoint, dir 1) for every base-grid latitude j and degree n, as the B operand B[m][k] = M[m][k]:
@@ -408,8 +441,11 @@ int rot_tc_digits(shbim_ctx* ctx, int p, const std::vector<double>& D, const std
     for (int j = 0; j < P1; ++j)
       for (int n = 0; n <= nmax; ++n) {
         off[((size_t)dir * P1 + j) * P1 + n] = total / 8;
-        const int Np = padded(2 * n + 1);
-        total += (int64_t)(Np / kKS) * kDig * Np * kKS;
+        const bool split = n >= kSplitFirst;
+        for (int part = 0; part < (split ? 2 : 1); ++part) {
+          const int Np = padded(part_len(split, n, part));
+          total += (int64_t)(Np / kKS) * (split ? kDig7 : kDig) * Np * kKS;
+        }
       }
   if (total / 8 > INT_MAX) return fail(ctx, SHBIM_ERR_ARG, "rotation digit table too large");
   std::vector<uint16_t> h((size_t)total, 0);
@@ -437,8 +473,9 @@ int rot_tc_digits(shbim_ctx* ctx, int p, const std::vector<double>& D, const std
       for (int k = 0; k < w; ++k)
         for (int r = 0; r < w; ++r) {
           const double dkr = Dn[(size_t)k * w + r];
-          if (dkr == 0.0) continue;
-          for (int c2 = 0; c2 < w; ++c2) M[(size_t)r * w + c2] += dkr * Z[(size_t)k * w + c2];
+          if (std::fabs(dkr) < 1e-16) continue;
+          // sine rows couple to sine columns, cosine rows to cosine columns
+          for (int c2 = r < n ? 0 : n; c2 < (r < n ? n : w); ++c2) M[(size_t)r * w + c2] += dkr * Z[(size_t)k * w + c2];
         }
       // a power-of-two scale per row m of M (max_k |M[m][k]| < 2^e_m), undone per output column
       std::vector<int> em(Np, 0);
@@ -451,16 +488,22 @@ int rot_tc_digits(shbim_ctx* ctx, int p, const std::vector<double>& D, const std
         ex[((size_t)dj * P1) * P1 + (size_t)n * n + m] = (signed char)em[m];
       }
       uint16_t* dst = h.data() + off[(size_t)dj * P1 + n] * 8;
-      for (int ks = 0; ks < Np / kKS; ++ks)
-        for (int m = 0; m < Np; ++m)
-          for (int kk = 0; kk < kKS; ++kk) {
-            const int k = ks * kKS + kk;
-            const double v = (m < w && k < w) ? M[(size_t)m * w + k] : 0.0;
-            int dg[kDig];
-            digits_host(v, em[m], dg);
-            for (int jd = 0; jd < kDig; ++jd)
-              dst[((size_t)ks * kDig + jd) * Np * kKS + canon16(m, kk)] = bf16_int(dg[jd]);
-          }
+      const bool split = n >= kSplitFirst;
+      const int nd = split ? kDig7 : kDig;
+      for (int part = 0; part < (split ? 2 : 1); ++part) {
+        const int len = part_len(split, n, part), o0 = part_off(split, n, part), Nq = padded(len);
+        for (int ks = 0; ks < Nq / kKS; ++ks)
+          for (int m = 0; m < Nq; ++m)
+            for (int kk = 0; kk < kKS; ++kk) {
+              const int k = ks * kKS + kk;
+              const double v = (m < len && k < len) ? M[(size_t)(o0 + m) * w + o0 + k] : 0.0;
+              int dg[kDig7];
+              digits_host_n(v, m < len ? em[o0 + m] : 0, nd, dg);
+              for (int jd = 0; jd < nd; ++jd)
+                dst[((size_t)ks * nd + jd) * Nq * kKS + canon16(m, kk)] = bf16_int(dg[jd]);
+            }
+        dst += (size_t)(Nq / kKS) * nd * Nq * kKS;
+      }
     }
   }
   std::vector<int> off32(off.begin(), off.end());
@@ -486,28 +529,26 @@ int rotate_tc(shbim_ctx* ctx, const DegreeTables& T, bool adjoint, const float2*
     SHBIM_CUDA(ctx, cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), s));
   }
   const int p = T.p;
-  const int nmax = rot_tc_nmax(p);
-  if (nmax < 0) return fail(ctx, SHBIM_ERR_ARG, "degree too large for the tensor-core rotations");
-  const int smem = rot_tc_smem(p, ncomp);
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const Items I(p, nmax, ncomp, t_begin, ct);
-  const unsigned grid = (unsigned)std::min<int64_t>(I.total, nsm);
   const uint4* tdig = reinterpret_cast<const uint4*>(T.rot_digits);
-  if (adjoint) {
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_rotate_tc<true><<<grid, kThreads, smem, s>>>(vin, in_stride, nc, p, nmax, t_begin, ct, ncomp, T.cs_phi_df, tdig,
-                                                   T.rot_toff, T.rot_exp, vout, rows_lap, rows_sto, nt_drop,
-                                                   ctx->tc_err, ctx->wait_ns);
-  } else {
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_rotate_tc<false><<<grid, kThreads, smem, s>>>(vin, in_stride, nc, p, nmax, t_begin, ct, ncomp, T.cs_phi_df, tdig,
-                                                    T.rot_toff, T.rot_exp, vout, rows_lap, rows_sto, nt_drop,
-                                                   ctx->tc_err, ctx->wait_ns);
-  }
-  SHBIM_CHECK_LAUNCH(ctx, "k_rotate_tc");
-  return SHBIM_OK;
+  auto launch = [&](auto kernel, int smem, int nmax, int nmin) -> int {
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const Items I(p, nmax, nmin, ncomp, t_begin, ct);
+    kernel<<<(unsigned)std::min<int64_t>(I.total, nsm), kThreads, smem, s>>>(
+        vin, in_stride, nc, p, nmax, nmin, t_begin, ct, ncomp, T.cs_phi_df, tdig, T.rot_toff, T.rot_exp, vout, rows_lap,
+        rows_sto, nt_drop, ctx->tc_err, ctx->wait_ns);
+    SHBIM_CHECK_LAUNCH(ctx, "k_rotate_tc");
+    return SHBIM_OK;
+  };
+  const int nw = rot_whole_nmax(p), ns = rot_tc_nmax(p);
+  if (ns >= kSplitFirst)
+    if (int rc = adjoint ? launch(k_rotate_tc<true, true>, rot_split_smem(ns), ns, kSplitFirst)
+                         : launch(k_rotate_tc<false, true>, rot_split_smem(ns), ns, kSplitFirst))
+      return rc;
+  return adjoint ? launch(k_rotate_tc<true, false>, rot_tc_smem(p, nw, ncomp), nw, 0)
+                 : launch(k_rotate_tc<false, false>, rot_tc_smem(p, nw, ncomp), nw, 0);
 }
 
 }  // namespace shbim
