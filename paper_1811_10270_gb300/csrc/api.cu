@@ -38,7 +38,7 @@ int rebuild_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
   for (int i = 0; i < ctx->n_drops; ++i) {
     const Drop& d = ctx->drops[i];
     dd[i] = DropDev{d.p, d.q, d.nt, d.ns, d.nc, d.coef_off, d.tgt_off, d.src_off, d.lam,
-                    d.centre[0], d.centre[1], d.centre[2], d.rows_lap, d.rows_sto};
+                    d.centre[0], d.centre[1], d.centre[2], d.rows_lap, d.rows_sto, d.pad_off};
   }
   SHBIM_CUDA(ctx, cudaMemcpy(ctx->drops_dev, dd.data(), dd.size() * sizeof(DropDev), cudaMemcpyHostToDevice));
   int rc;
@@ -375,7 +375,7 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
   }
   // layout
   ctx->drops.resize(n_drops);
-  int64_t co = 0, to = 0, so = 0;
+  int64_t co = 0, to = 0, so = 0, po = 0;
   for (int i = 0; i < n_drops; ++i) {
     Drop& d = ctx->drops[i];
     d.p = p_host[i];
@@ -388,10 +388,13 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
     d.src_off = so;
     d.lam = lambda_host ? lambda_host[i] : 1.0;
     d.tab = ctx->tables[d.p];
+    d.pad_off = po;
+    po += padded_nc(d.nc);
     co += d.nc;
     to += d.nt;
     so += d.ns;
   }
+  ctx->npad = po;
   ctx->n_drops = n_drops;
   ctx->ncoef = co;
   ctx->ntarget = to;
@@ -411,9 +414,12 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
       (rc = dalloc(ctx, &ctx->xup, 3 * (size_t)kNumTab * so, "position derivatives")))
     return rc;
   for (auto& d : ctx->drops) {
-    if ((rc = dalloc(ctx, &d.rows_lap, 2 * (size_t)d.nt * kNumLap * d.nc, "laplace rows")) ||
-        (rc = dalloc(ctx, &d.rows_sto, 2 * (size_t)d.nt * kNumSto * d.nc, "stokes rows")))
+    const size_t lap = 2 * (size_t)d.nt * kNumLap * padded_nc(d.nc), sto = 2 * (size_t)d.nt * kNumSto * padded_nc(d.nc);
+    if ((rc = dalloc(ctx, &d.rows_lap, lap, "laplace rows")) || (rc = dalloc(ctx, &d.rows_sto, sto, "stokes rows")))
       return rc;
+    // the padding stays zero: the builds write the rows' coefficients only
+    SHBIM_CUDA(ctx, cudaMemsetAsync(d.rows_lap, 0, lap * sizeof(float), s));
+    SHBIM_CUDA(ctx, cudaMemsetAsync(d.rows_sto, 0, sto * sizeof(float), s));
   }
   // drops grouped by degree: the transforms of an operator application take one launch per degree
   {

@@ -22,6 +22,9 @@ inline int ntri(int p) { return (p + 1) * (p + 2) / 2; }
 inline int nlat(int q) { return q + 1; }
 inline int nlon(int q) { return 2 * q + 2; }
 inline int npts(int q) { return (q + 1) * (2 * q + 2); }
+// coefficients of one singular row or density component as the self products read them: padded with zeros to
+// whole 16-byte loads
+__host__ __device__ inline int padded_nc(int nc) { return (nc + 3) & ~3; }
 
 // Number of Laplace / Stokes weight components in the singular self rows.
 constexpr int kNumLap = 2;        // 0: double layer (target normal), 1: single layer
@@ -73,13 +76,13 @@ struct DegreeTables {
   uint16_t* dft_digits = nullptr;
   int dft_ntiles = 0, dft_ksteps = 0;
   // digit planes of Dq_n^T Dz(-+theta_j) Dq_n per base-grid latitude for the tensor-core rotations
-  // (rot_tc.cu), p <= 39: [2][p+1][p+1][K step][digit][Np x 16], with per-(direction, latitude,
+  // (rot_tc.cu): [2][p+1][p+1][part][K step][digit][Np x 16], with per-(direction, latitude,
   // degree) offsets in 16-byte units
   uint16_t* rot_digits = nullptr;
   int* rot_toff = nullptr;
   signed char* rot_exp = nullptr;   // [2][p+1][(p+1)^2] row exponents of the tables
   // digit planes of Pbar_n^m at the degree 2p+1 grid latitudes for the tensor-core Legendre stage
-  // (leg_tc.cu), p <= 39: [m][K step][digit][Np x 16], offsets per m, row exponents [m][p+1]
+  // (leg_tc.cu): [m][K step][digit][Np x 16], offsets per m and tile of 64 degrees, row exponents
   uint16_t* leg_digits = nullptr;
   int* leg_toff = nullptr;
   signed char* leg_exp = nullptr;
@@ -96,8 +99,10 @@ struct Drop {
   DegreeTables* tab = nullptr;
   // singular rows as two FP32 planes (hi, then lo = value - hi): the FP32 path reads the hi plane
   // only, the FP64-class path both (double-float); same bytes as FP64 storage
-  float* rows_lap = nullptr;    // [2][nt][kNumLap][nc]
-  float* rows_sto = nullptr;    // [2][nt][kNumSto][nc]
+  // (rows padded_nc(nc) apart, the padding zero)
+  float* rows_lap = nullptr;    // [2][nt][kNumLap][padded nc]
+  float* rows_sto = nullptr;    // [2][nt][kNumSto][padded nc]
+  int64_t pad_off = 0;          // into the padded density copies of the self products
 };
 
 // The drops of one degree, wherever they lie in the layout: transforms over a list take one launch per
@@ -115,8 +120,9 @@ struct DropDev {
   int64_t coef_off, tgt_off, src_off;
   double lam;
   double cx, cy, cz;
-  const float* rows_lap;        // [2][nt][kNumLap][nc] (hi plane, lo plane)
-  const float* rows_sto;        // [2][nt][kNumSto][nc]
+  const float* rows_lap;        // [2][nt][kNumLap][padded nc] (hi plane, lo plane)
+  const float* rows_sto;        // [2][nt][kNumSto][padded nc]
+  int64_t pad_off;
 };
 
 // Target tile of the all-pairs kernels: targets [t0, t0+nt) of one drop.
@@ -197,7 +203,8 @@ struct shbim_ctx {
     size_t rot_n = 0, w_n = 0, F_n = 0, v_n = 0, xdf_n = 0, rexp_n = 0;
     int xdrop = -1;
   } lanes[2];
-  float* dens_split = nullptr;    // [2][3 ncoef] hi / lo planes of a density for the self GEMV
+  float* dens_split = nullptr;    // [2][3 npad] hi / lo planes of a density for the self GEMV
+  int64_t npad = 0;               // sum of the drops' padded coefficient counts
   size_t dens_split_cap = 0;
   int outer_prec = SHBIM_PREC_DF64;  // FP64-class applications: refinement residuals, one-shot sums
   int rows_prec = SHBIM_PREC_DF64;   // arithmetic of the singular-row build (FP64 or double-float)

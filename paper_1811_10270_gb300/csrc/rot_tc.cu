@@ -383,8 +383,9 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
         for (int k = lane; k < w; k += 32) dst[k] = sX[r * WS + k];
       } else {
         const int64_t tl = (int64_t)t_begin + b;
-        float* dst = c < kNumLap ? rows_lap + (tl * kNumLap + c) * nc : rows_sto + (tl * kNumSto + (c - kNumLap)) * nc;
-        const int64_t plane = (int64_t)nt_drop * (c < kNumLap ? kNumLap : kNumSto) * nc;
+        float* dst = c < kNumLap ? rows_lap + (tl * kNumLap + c) * padded_nc(nc)
+                                 : rows_sto + (tl * kNumSto + (c - kNumLap)) * padded_nc(nc);
+        const int64_t plane = (int64_t)nt_drop * (c < kNumLap ? kNumLap : kNumSto) * padded_nc(nc);
         for (int k = lane; k < w; k += 32) {
           const float2 x = sX[r * WS + k];
           dst[n * n + k] = x.x;

@@ -224,9 +224,9 @@ __global__ void k_rotate_adj(const double* __restrict__ vbuf, int nc, int p, int
   __syncthreads();
   dz_apply(b0, p, cp, sp, 1.0);
   __syncthreads();
-  float* dst = c < kNumLap ? rows_lap + ((int64_t)tl * kNumLap + c) * nc
-                           : rows_sto + ((int64_t)tl * kNumSto + (c - kNumLap)) * nc;
-  const int64_t plane = (int64_t)nt_drop * (c < kNumLap ? kNumLap : kNumSto) * nc;
+  float* dst = c < kNumLap ? rows_lap + ((int64_t)tl * kNumLap + c) * padded_nc(nc)
+                           : rows_sto + ((int64_t)tl * kNumSto + (c - kNumLap)) * padded_nc(nc);
+  const int64_t plane = (int64_t)nt_drop * (c < kNumLap ? kNumLap : kNumSto) * padded_nc(nc);
   for (int o = threadIdx.x; o < nc; o += blockDim.x) {
     const float h = (float)b0[o];
     dst[o] = h;
@@ -400,15 +400,23 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // Self GEMVs over the FP32 row planes. FP32 path (DF = false): hi plane and the FP32 copy of the
 // density, FP32 accumulation. FP64-class path (DF = true): both planes and both density planes,
-// double-float accumulation. One warp per target; HBM-bound in both forms (in FP64 arithmetic the
-// GEMV would be bound by the FP64 pipe: 2 flops per 8 bytes is above this GPU's FP64 balance).
-__global__ void k_split_density(const double* __restrict__ x, int64_t n, float* __restrict__ hi,
-                                float* __restrict__ lo) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  const float h = (float)x[e];
-  hi[e] = h;
-  lo[e] = (float)(x[e] - (double)h);
+// double-float accumulation (in FP64 arithmetic the GEMV would be bound by the FP64 pipe: 2 flops per 8 bytes
+// is above this GPU's FP64 balance). One warp per target; HBM-bound in both forms: a lane reads four coefficients
+// of every plane by 16-byte loads (rows and density copies padded to whole loads), so twelve 512-byte pieces per
+// warp are in flight. The stresslet product of 64 drops of degree 16 to 48 (11.4 GB): 3.76 ms by 4-byte loads, 2.19 ms
+// (5.2 TB/s) so; the Laplace product 0.46 and 0.30 ms.
+// density planes of ncomp components per drop, each component padded: hi / lo [ncomp pad_off + c padded_nc + k]
+__global__ void k_split_density(const double* __restrict__ x, const DropDev* __restrict__ drops, int ncomp,
+                                float* __restrict__ hi, float* __restrict__ lo) {
+  const DropDev D = drops[blockIdx.y];
+  const int ncp = padded_nc(D.nc);
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ncomp * ncp; e += gridDim.x * blockDim.x) {
+    const int c = e / ncp, k = e - c * ncp;
+    const double v = k < D.nc ? x[ncomp * D.coef_off + (int64_t)c * D.nc + k] : 0.0;
+    const float h = (float)v;
+    hi[ncomp * D.pad_off + e] = h;
+    lo[ncomp * D.pad_off + e] = (float)(v - (double)h);
+  }
 }
 
 __device__ __forceinline__ float warp_sum_f(float v) {
@@ -417,8 +425,12 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float at4(const float4& v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w)); }
+
 template <bool DF>
-__global__ void k_self_lap(const DropDev* __restrict__ drops, const int* __restrict__ tgt_drop,
+__global__ void __launch_bounds__(256)
+k_self_lap(const DropDev* __restrict__ drops, const int* __restrict__ tgt_drop,
                            int64_t ntarget, int which, const float* __restrict__ xh,
                            const float* __restrict__ xl, double* __restrict__ out) {
   const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -426,26 +438,37 @@ __global__ void k_self_lap(const DropDev* __restrict__ drops, const int* __restr
   if (t >= ntarget) return;
   const DropDev D = drops[tgt_drop[t]];
   const int64_t tl = t - D.tgt_off;
-  const int64_t plane = (int64_t)D.nt * kNumLap * D.nc;
-  const float* rh = D.rows_lap + (tl * kNumLap + which) * D.nc;
-  const float* x = xh + D.coef_off;
+  const int ncp = padded_nc(D.nc);
+  const int64_t plane = (int64_t)D.nt * kNumLap * ncp;
+  const float* rh = D.rows_lap + (tl * kNumLap + which) * ncp;
+  const float* x = xh + D.pad_off;
   double v;
   if (!DF) {
     float acc = 0.f;
-    for (int e = lane; e < D.nc; e += 32) acc = fmaf(rh[e], x[e], acc);
+#pragma unroll 2
+    for (int e = 4 * lane; e < ncp; e += 128) {
+      const float4 r = ld4(rh + e), y = ld4(x + e);
+      acc = fmaf(r.x, y.x, fmaf(r.y, y.y, fmaf(r.z, y.z, fmaf(r.w, y.w, acc))));
+    }
     v = (double)warp_sum_f(acc);
   } else {
     const float* rl = rh + plane;
-    const float* x2 = xl + D.coef_off;
+    const float* x2 = xl + D.pad_off;
     dfl::acc acc;
-    for (int e = lane; e < D.nc; e += 32) acc.add_prod(dfl::df{rh[e], rl[e]}, dfl::df{x[e], x2[e]});
+#pragma unroll 2
+    for (int e = 4 * lane; e < ncp; e += 128) {
+      const float4 r = ld4(rh + e), q = ld4(rl + e), y = ld4(x + e), z = ld4(x2 + e);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc.add_prod(dfl::df{at4(r, k), at4(q, k)}, dfl::df{at4(y, k), at4(z, k)});
+    }
     v = warp_sum(dfl::to_double(acc.value()));
   }
   if (lane == 0) out[t] = v;
 }
 
 template <bool DF>
-__global__ void k_self_sto(const DropDev* __restrict__ drops, const int* __restrict__ tgt_drop,
+__global__ void __launch_bounds__(256)
+k_self_sto(const DropDev* __restrict__ drops, const int* __restrict__ tgt_drop,
                            int64_t ntarget, const float* __restrict__ fh, const float* __restrict__ fl,
                            const float* __restrict__ uh, const float* __restrict__ ul, double* __restrict__ out) {
   const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -453,7 +476,7 @@ __global__ void k_self_sto(const DropDev* __restrict__ drops, const int* __restr
   if (t >= ntarget) return;
   const DropDev D = drops[tgt_drop[t]];
   const int64_t tl = t - D.tgt_off;
-  const int nc = D.nc;
+  const int nc = padded_nc(D.nc);
   const int64_t plane = (int64_t)D.nt * kNumSto * nc;
   const float* rows = D.rows_sto + tl * kNumSto * nc;
   double res[3] = {0.0, 0.0, 0.0};
@@ -462,39 +485,58 @@ __global__ void k_self_sto(const DropDev* __restrict__ drops, const int* __restr
     if (!vh || (part == 1 && D.lam == 1.0)) continue;
     const float* vl = part == 0 ? fl : ul;
     const float* r = rows + part * 6 * nc;
-    const float* Xh = vh + 3 * D.coef_off;
+    const float* Xh = vh + 3 * D.pad_off;
     double s3[3];
     if (!DF) {
       float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-      for (int e = lane; e < nc; e += 32) {
-        const float X = Xh[e], Y = Xh[nc + e], Z = Xh[2 * nc + e];
-        const float xx = r[e], xy = r[nc + e], xz = r[2 * nc + e];
-        const float yy = r[3 * nc + e], yz = r[4 * nc + e], zz = r[5 * nc + e];
-        a0 = fmaf(xx, X, fmaf(xy, Y, fmaf(xz, Z, a0)));
-        a1 = fmaf(xy, X, fmaf(yy, Y, fmaf(yz, Z, a1)));
-        a2 = fmaf(xz, X, fmaf(yz, Y, fmaf(zz, Z, a2)));
+      for (int e = 4 * lane; e < nc; e += 128) {
+        float4 m[6], X[3];   // xx, xy, xz, yy, yz, zz
+#pragma unroll
+        for (int c = 0; c < 6; ++c) m[c] = ld4(r + c * nc + e);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) X[c] = ld4(Xh + c * nc + e);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float x = at4(X[0], k), y = at4(X[1], k), z = at4(X[2], k);
+          a0 = fmaf(at4(m[0], k), x, fmaf(at4(m[1], k), y, fmaf(at4(m[2], k), z, a0)));
+          a1 = fmaf(at4(m[1], k), x, fmaf(at4(m[3], k), y, fmaf(at4(m[4], k), z, a1)));
+          a2 = fmaf(at4(m[2], k), x, fmaf(at4(m[4], k), y, fmaf(at4(m[5], k), z, a2)));
+        }
       }
       s3[0] = warp_sum_f(a0);
       s3[1] = warp_sum_f(a1);
       s3[2] = warp_sum_f(a2);
     } else {
-      const float* Xl = vl + 3 * D.coef_off;
+      const float* Xl = vl + 3 * D.pad_off;
       const float* q = r + plane;
       dfl::acc a0, a1, a2;
-      for (int e = lane; e < nc; e += 32) {
-        const dfl::df X{Xh[e], Xl[e]}, Y{Xh[nc + e], Xl[nc + e]}, Z{Xh[2 * nc + e], Xl[2 * nc + e]};
-        const dfl::df xx{r[e], q[e]}, xy{r[nc + e], q[nc + e]}, xz{r[2 * nc + e], q[2 * nc + e]};
-        const dfl::df yy{r[3 * nc + e], q[3 * nc + e]}, yz{r[4 * nc + e], q[4 * nc + e]};
-        const dfl::df zz{r[5 * nc + e], q[5 * nc + e]};
-        a0.add_prod(xx, X);
-        a0.add_prod(xy, Y);
-        a0.add_prod(xz, Z);
-        a1.add_prod(xy, X);
-        a1.add_prod(yy, Y);
-        a1.add_prod(yz, Z);
-        a2.add_prod(xz, X);
-        a2.add_prod(yz, Y);
-        a2.add_prod(zz, Z);
+      for (int e = 4 * lane; e < nc; e += 128) {
+        float4 m[6], l[6], X[3], Y[3];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          m[c] = ld4(r + c * nc + e);
+          l[c] = ld4(q + c * nc + e);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          X[c] = ld4(Xh + c * nc + e);
+          Y[c] = ld4(Xl + c * nc + e);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const dfl::df x{at4(X[0], k), at4(Y[0], k)}, y{at4(X[1], k), at4(Y[1], k)}, z{at4(X[2], k), at4(Y[2], k)};
+          const dfl::df xx{at4(m[0], k), at4(l[0], k)}, xy{at4(m[1], k), at4(l[1], k)}, xz{at4(m[2], k), at4(l[2], k)};
+          const dfl::df yy{at4(m[3], k), at4(l[3], k)}, yz{at4(m[4], k), at4(l[4], k)}, zz{at4(m[5], k), at4(l[5], k)};
+          a0.add_prod(xx, x);
+          a0.add_prod(xy, y);
+          a0.add_prod(xz, z);
+          a1.add_prod(xy, x);
+          a1.add_prod(yy, y);
+          a1.add_prod(yz, z);
+          a2.add_prod(xz, x);
+          a2.add_prod(yz, y);
+          a2.add_prod(zz, z);
+        }
       }
       s3[0] = warp_sum(dfl::to_double(a0.value()));
       s3[1] = warp_sum(dfl::to_double(a1.value()));
@@ -512,9 +554,9 @@ __global__ void k_self_sto(const DropDev* __restrict__ drops, const int* __restr
 }
 
 namespace {
-// hi / lo planes of n doubles into slot 0 or 1 (3 ncoef floats each) of the context's split buffer
-int split_density(shbim_ctx* ctx, const double* x, int64_t n, int slot, float** hi, float** lo, cudaStream_t s) {
-  const size_t need = (size_t)12 * ctx->ncoef;   // [hi, lo][slot 0, slot 1][3 ncoef]
+// hi / lo planes of a density of ncomp components into slot 0 or 1 (3 npad floats each) of the context's split buffer
+int split_density(shbim_ctx* ctx, const double* x, int ncomp, int slot, float** hi, float** lo, cudaStream_t s) {
+  const size_t need = (size_t)12 * ctx->npad;   // [hi, lo][slot 0, slot 1][3 npad]
   if (ctx->dens_split_cap < need) {
     cudaFree(ctx->dens_split);
     ctx->dens_split = nullptr;
@@ -524,9 +566,12 @@ int split_density(shbim_ctx* ctx, const double* x, int64_t n, int slot, float** 
     ctx->dens_split_cap = need;
     ctx->geom_version++;  // captured operator graphs referenced the old buffer
   }
-  *hi = ctx->dens_split + (int64_t)slot * 3 * ctx->ncoef;
-  *lo = *hi + 6 * ctx->ncoef;
-  k_split_density<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, n, *hi, *lo);
+  *hi = ctx->dens_split + (int64_t)slot * 3 * ctx->npad;
+  *lo = *hi + 6 * ctx->npad;
+  int most = 0;
+  for (const auto& d : ctx->drops) most = std::max(most, padded_nc(d.nc));
+  k_split_density<<<dim3((unsigned)((ncomp * most + 255) / 256), (unsigned)ctx->n_drops), 256, 0, s>>>(
+      x, ctx->drops_dev, ncomp, *hi, *lo);
   SHBIM_CHECK_LAUNCH(ctx, "k_split_density");
   return SHBIM_OK;
 }
@@ -534,7 +579,7 @@ int split_density(shbim_ctx* ctx, const double* x, int64_t n, int slot, float** 
 
 int apply_self_laplace(shbim_ctx* ctx, int which, const double* dens, double* out, cudaStream_t s) {
   float *xh, *xl;
-  int rc = split_density(ctx, dens, ctx->ncoef, 0, &xh, &xl, s);
+  int rc = split_density(ctx, dens, 1, 0, &xh, &xl, s);
   if (rc) return rc;
   const int64_t threads = ctx->ntarget * 32;
   const unsigned g = (unsigned)((threads + 255) / 256);
@@ -549,9 +594,8 @@ int apply_self_laplace(shbim_ctx* ctx, int which, const double* dens, double* ou
 int apply_self_stokes(shbim_ctx* ctx, const double* f, const double* u, double* out, cudaStream_t s) {
   float *fh = nullptr, *fl = nullptr, *uh = nullptr, *ul = nullptr;
   int rc;
-  const int64_t n3 = 3 * ctx->ncoef;
-  if (f && (rc = split_density(ctx, f, n3, 0, &fh, &fl, s))) return rc;
-  if (u && (rc = split_density(ctx, u, n3, 1, &uh, &ul, s))) return rc;
+  if (f && (rc = split_density(ctx, f, 3, 0, &fh, &fl, s))) return rc;
+  if (u && (rc = split_density(ctx, u, 3, 1, &uh, &ul, s))) return rc;
   const int64_t threads = ctx->ntarget * 32;
   const unsigned g = (unsigned)((threads + 255) / 256);
   if (ctx->opts.precision == SHBIM_PREC_FP32_COMP && ctx->self_prec == SHBIM_PREC_FP32_COMP)

@@ -11,7 +11,7 @@
 // The rotations of steps 1 and 4 run on the tensor cores (rot_tc.cu) where the degree fits.
 // Every sum and every pointwise operation here is double-float (hi + lo FP32 pairs; Dekker
 // products, Knuth sums, Newton square roots), ~2^-44 relative per operation; the tensor-core stages
-// split their operands into exact digit products (~2^-40 of the sum of magnitudes). The rows agree
+// split their operands into exact digit products (~2^-40 of the sum of magnitudes, 2^-47 from degree 40 on). The rows agree
 // with the FP64 build to rounding level while the FP64 pipe (1/64 of the FP32 rate here) stays idle.
 #include <algorithm>
 
@@ -136,9 +136,9 @@ k_rotate_deg_df(const float2* __restrict__ vin, int64_t in_stride, int nc, int p
         vout[((int64_t)(b0 + b) * ncomp + c) * nc + n * n + k] = make_float2(x.hi, x.lo);
       } else {
         const int tl = t_begin + b0 + b;
-        float* dst = c < kNumLap ? rows_lap + ((int64_t)tl * kNumLap + c) * nc
-                                 : rows_sto + ((int64_t)tl * kNumSto + (c - kNumLap)) * nc;
-        const int64_t plane = (int64_t)nt_drop * (c < kNumLap ? kNumLap : kNumSto) * nc;
+        float* dst = c < kNumLap ? rows_lap + ((int64_t)tl * kNumLap + c) * padded_nc(nc)
+                                 : rows_sto + ((int64_t)tl * kNumSto + (c - kNumLap)) * padded_nc(nc);
+        const int64_t plane = (int64_t)nt_drop * (c < kNumLap ? kNumLap : kNumSto) * padded_nc(nc);
         dst[n * n + k] = x.hi;
         dst[plane + n * n + k] = x.lo;
       }
@@ -569,7 +569,7 @@ int build_singular_rows_df(shbim_ctx* ctx, cudaStream_t s, const double* xcoef) 
     const int budget = 46 * 1024 / (int)sizeof(float2) - 2 * N;
     const int rows = std::max(1, std::min(8, budget / (2 * N)));
     const size_t f_smem = (size_t)(2 * N + rows * 2 * N) * sizeof(float2);
-    // tensor-core rotations for degrees 0 .. rot_n (all of them up to p = 39), the FP32-pipe kernel above
+    // tensor-core rotations for degrees 0 .. rot_n (all of them up to 63), the FP32-pipe kernel above
     const int rot_n = ctx->tc_rot ? rot_tc_nmax(d.p) : -1;
     const bool rot_tc = rot_n >= 0;
     const int df_n0 = rot_n + 1;
