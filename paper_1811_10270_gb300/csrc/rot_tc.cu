@@ -20,10 +20,10 @@
 // accumulators in double-float. Every wait is bounded; a timeout sets the error flag and the CTA
 // stops.
 //
-// Degrees 40 to 63 (SPLIT): M couples neither cosine orders with sine orders nor the reverse (a rotation about y commutes
+// Drops of degree 40 and more (SPLIT), degrees up to 63: M couples neither cosine orders with sine orders nor the reverse (a rotation about y commutes
 // with the reflection y -> -y), so the block is two blocks of n (sine) and n + 1 (cosine) rows, contiguous in the
 // coefficient order: two GEMMs of half the size each, a quarter of the products, that fit tensor memory with seven
-// digits (these degrees were double-float before and keep that accuracy). Angles come from L1 there: the value block
+// digits (2^-47: as close as the double-float kernel). Angles come from L1 there: the value block
 // takes the shared memory. Degree 64 (65 cosine rows) stays on the FP32-pipe kernel (singular_df.cu).
 #include <algorithm>
 #include <climits>
@@ -48,7 +48,8 @@ constexpr int kPlaneA = kMT * kKS;                          // bf16 per row-digi
 constexpr int kPlaneBmax = kNmax * kKS;                     // bf16 per table-digit plane
 constexpr int kStageBytes = kDig * (kPlaneA + kPlaneBmax) * 2;
 constexpr int kSplitNmax = 64;                              // largest padded half block
-constexpr int kSplitFirst = 40, kSplitLast = 63;            // degrees of the split form
+constexpr int kSplitFirst = 40;                             // smallest drop degree of the split form
+constexpr int kSplitLast = 63;                              // its highest degree block
 static_assert(diag_sums_exact7(kSplitNmax), "split rotations: digit sums must stay exact in FP32");
 constexpr int kStageSplit = kDig7 * (kPlaneA + kSplitNmax * kKS) * 2;
 constexpr uint32_t kTmemCols = 512;
@@ -76,17 +77,17 @@ __device__ __forceinline__ void cp_async_wait_all() {
 __host__ __device__ inline int max_targets(int ncomp) { return kMT / ncomp + 2; }
 
 // The items of one launch: latitudes lat0 .. lat0 + L - 1 of the chunk, T tiles of 128 vectors per
-// latitude, degrees nmax .. nmin (nmax <= p: the higher degrees of a drop whose blocks exceed kNmax are
+// latitude, degrees nmax .. 0 (nmax <= p: the higher degrees of a drop whose blocks exceed kNmax are
 // rotated by the double-float kernel).
 struct Items {
-  int p, nmax, nmin, nlon, ncomp, t_begin, ct, lat0, L, T;
+  int p, nmax, nlon, ncomp, t_begin, ct, lat0, L, T;
   int64_t total;
-  __host__ __device__ Items(int p_, int nmax_, int nmin_, int ncomp_, int t_begin_, int ct_)
-      : p(p_), nmax(nmax_), nmin(nmin_), nlon(2 * p_ + 2), ncomp(ncomp_), t_begin(t_begin_), ct(ct_) {
+  __host__ __device__ Items(int p_, int nmax_, int ncomp_, int t_begin_, int ct_)
+      : p(p_), nmax(nmax_), nlon(2 * p_ + 2), ncomp(ncomp_), t_begin(t_begin_), ct(ct_) {
     lat0 = t_begin / nlon;
     L = (t_begin + ct - 1) / nlon - lat0 + 1;
     T = (nlon * ncomp + kMT - 1) / kMT;
-    total = (int64_t)(nmax + 1 - nmin) * L * T;
+    total = (int64_t)(nmax + 1) * L * T;
   }
   // degree, latitude and chunk-local vector range [va, vb) of an item (empty if va >= vb)
   __device__ void decode(int64_t it, int& n, int& lat, int& va, int& vb) const {
@@ -116,7 +117,7 @@ __host__ __device__ inline int part_off(bool split, int n, int part) { return sp
 
 template <bool ADJ, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
-k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, int nmax, int nmin, int t_begin, int ct, int ncomp,
+k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, int nmax, int t_begin, int ct, int ncomp,
             const float2* __restrict__ cs_phi, const uint4* __restrict__ tdig, const int* __restrict__ toff,
             const signed char* __restrict__ texp, float2* __restrict__ vout, float* __restrict__ rows_lap,
             float* __restrict__ rows_sto, int nt_drop, int* __restrict__ err, uint64_t wlim) {
@@ -137,7 +138,7 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
   float2* sX = reinterpret_cast<float2*>(smem + 2 * kStage);
   float2* sCS = sX + kMT * WS;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const Items I(p, nmax, nmin, ncomp, t_begin, ct);
+  const Items I(p, nmax, ncomp, t_begin, ct);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_base)),
                  "r"(kTmemCols));
@@ -407,23 +408,16 @@ k_rotate_tc(const float2* __restrict__ vin, int64_t in_stride, int nc, int p, in
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
 }
 
-int rot_tc_smem(int p, int nmax, int ncomp) {
-  return 2 * kStageBytes + (kMT * (2 * nmax + 1) + max_targets(ncomp) * 2 * (p + 1)) * (int)sizeof(float2);
+int rot_tc_smem(int p, int ncomp) {
+  return 2 * kStageBytes + (kMT * (2 * p + 1) + max_targets(ncomp) * 2 * (p + 1)) * (int)sizeof(float2);
 }
 
 int rot_split_smem(int nmax) { return 2 * kStageSplit + kMT * (2 * nmax + 1) * (int)sizeof(float2); }
 
-// highest degree of the whole-block form: blocks up to kNmax
-int rot_whole_nmax(int p) {
-  int n = p;
-  while (n >= 0 && padded(2 * n + 1) > kNmax) --n;
-  return n;
-}
-
 }  // namespace
 
-// Highest degree the tensor-core rotations take for drops of degree p: all of them up to 63 (whole blocks to degree
-// 39, split blocks above); degree 64 goes to the double-float kernel.
+// Highest degree the tensor-core rotations take for drops of degree p: all of them up to 63 (whole blocks for drops of
+// degree 39 and less, split blocks otherwise); degree 64 goes to the double-float kernel.
 int rot_tc_nmax(int p) { return std::min(p, kSplitLast); }
 
 // Digit planes of M = Dq_n^T Dz(-theta_j) Dq_n (forward, dir 0) and Dq_n^T Dz(theta_j) Dq_n
@@ -434,7 +428,8 @@ int rot_tc_nmax(int p) { return std::min(p, kSplitLast); }
 int rot_tc_digits(shbim_ctx* ctx, int p, const std::vector<double>& D, const std::vector<double>& theta,
                   DegreeTables& T) {
   const int nmax = rot_tc_nmax(p);
-  if (nmax < 0) return SHBIM_OK;
+  const bool split = p >= kSplitFirst;
+  const int nd = split ? kDig7 : kDig;
   const int P1 = p + 1;
   std::vector<int64_t> off((size_t)2 * P1 * P1, 0);
   int64_t total = 0;   // uint16 elements
@@ -442,10 +437,9 @@ int rot_tc_digits(shbim_ctx* ctx, int p, const std::vector<double>& D, const std
     for (int j = 0; j < P1; ++j)
       for (int n = 0; n <= nmax; ++n) {
         off[((size_t)dir * P1 + j) * P1 + n] = total / 8;
-        const bool split = n >= kSplitFirst;
         for (int part = 0; part < (split ? 2 : 1); ++part) {
           const int Np = padded(part_len(split, n, part));
-          total += (int64_t)(Np / kKS) * (split ? kDig7 : kDig) * Np * kKS;
+          total += (int64_t)(Np / kKS) * nd * Np * kKS;
         }
       }
   if (total / 8 > INT_MAX) return fail(ctx, SHBIM_ERR_ARG, "rotation digit table too large");
@@ -489,8 +483,6 @@ int rot_tc_digits(shbim_ctx* ctx, int p, const std::vector<double>& D, const std
         ex[((size_t)dj * P1) * P1 + (size_t)n * n + m] = (signed char)em[m];
       }
       uint16_t* dst = h.data() + off[(size_t)dj * P1 + n] * 8;
-      const bool split = n >= kSplitFirst;
-      const int nd = split ? kDig7 : kDig;
       for (int part = 0; part < (split ? 2 : 1); ++part) {
         const int len = part_len(split, n, part), o0 = part_off(split, n, part), Nq = padded(len);
         for (int ks = 0; ks < Nq / kKS; ++ks)
@@ -534,22 +526,21 @@ int rotate_tc(shbim_ctx* ctx, const DegreeTables& T, bool adjoint, const float2*
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const uint4* tdig = reinterpret_cast<const uint4*>(T.rot_digits);
-  auto launch = [&](auto kernel, int smem, int nmax, int nmin) -> int {
+  const int nmax = rot_tc_nmax(p);
+  auto launch = [&](auto kernel, int smem) -> int {
     SHBIM_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    const Items I(p, nmax, nmin, ncomp, t_begin, ct);
+    const Items I(p, nmax, ncomp, t_begin, ct);
     kernel<<<(unsigned)std::min<int64_t>(I.total, nsm), kThreads, smem, s>>>(
-        vin, in_stride, nc, p, nmax, nmin, t_begin, ct, ncomp, T.cs_phi_df, tdig, T.rot_toff, T.rot_exp, vout, rows_lap,
+        vin, in_stride, nc, p, nmax, t_begin, ct, ncomp, T.cs_phi_df, tdig, T.rot_toff, T.rot_exp, vout, rows_lap,
         rows_sto, nt_drop, ctx->tc_err, ctx->wait_ns);
     SHBIM_CHECK_LAUNCH(ctx, "k_rotate_tc");
     return SHBIM_OK;
   };
-  const int nw = rot_whole_nmax(p), ns = rot_tc_nmax(p);
-  if (ns >= kSplitFirst)
-    if (int rc = adjoint ? launch(k_rotate_tc<true, true>, rot_split_smem(ns), ns, kSplitFirst)
-                         : launch(k_rotate_tc<false, true>, rot_split_smem(ns), ns, kSplitFirst))
-      return rc;
-  return adjoint ? launch(k_rotate_tc<true, false>, rot_tc_smem(p, nw, ncomp), nw, 0)
-                 : launch(k_rotate_tc<false, false>, rot_tc_smem(p, nw, ncomp), nw, 0);
+  if (p >= kSplitFirst)
+    return adjoint ? launch(k_rotate_tc<true, true>, rot_split_smem(nmax))
+                   : launch(k_rotate_tc<false, true>, rot_split_smem(nmax));
+  return adjoint ? launch(k_rotate_tc<true, false>, rot_tc_smem(p, ncomp))
+                 : launch(k_rotate_tc<false, false>, rot_tc_smem(p, ncomp));
 }
 
 }  // namespace shbim
