@@ -11,7 +11,9 @@
 //     sum over upsampled nodes of K(x0, y) s(y)  -  sum over degree-q nodes of K(x0, y) s(y)
 // to the all-pairs result, replacing the degree-q regular value by the upsampled one. The
 // FP32 variant uses the same centre-relative coordinates, (hi, lo) target offsets and two-sum
-// accumulation as the all-pairs kernel; the FP64 variant plain FP64.
+// accumulation as the all-pairs kernel; the FP64 variant plain FP64. The Stokes kinds are the all-pairs kernels'
+// (both terms, f alone, u alone): two drops of degree 32, 0.1 apart, u alone: FP32 140 -> 111 us, double-float
+// 1.05 -> 0.81 ms against the kernel of both terms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -166,46 +168,10 @@ __device__ __forceinline__ double block_sum_near(double v) {
 }
 
 // Sum over one grid of drop j of K(x0, y) s(y) for kernel KIND (0 DL target normal, 1 SL,
-// 2 Stokes with f and u strengths) into acc[3]. FP32: positions relative to drop j's centre
-// (pos32, [x y z nx ny nz][stride]), strengths str32 [comp][sstride]; FP64: absolute.
-template <int KIND>
-__device__ void near_sum32(const float* __restrict__ pos, int64_t stride, const float* __restrict__ str,
-                           int64_t sstride, int64_t n, const float th[3], const float tl[3], const float nv[3],
-                           int has_f, int has_u, double acc[3]) {
-  float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f};
-  for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-    const float dx = (th[0] - pos[e]) + tl[0];
-    const float dy = (th[1] - pos[stride + e]) + tl[1];
-    const float dz = (th[2] - pos[2 * stride + e]) + tl[2];
-    const float ri = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-    if (KIND == 1) {
-      two_sum_f(hi[0], lo[0], str[e] * ri);
-    } else if (KIND == 0) {
-      const float dn = fmaf(dx, nv[0], fmaf(dy, nv[1], dz * nv[2]));
-      two_sum_f(hi[0], lo[0], str[e] * ri * ri * ri * dn);
-    } else {
-      const float fx = has_f ? str[e] : 0.f, fy = has_f ? str[sstride + e] : 0.f, fz = has_f ? str[2 * sstride + e] : 0.f;
-      const float ux = has_u ? str[3 * sstride + e] : 0.f, uy = has_u ? str[4 * sstride + e] : 0.f,
-                  uz = has_u ? str[5 * sstride + e] : 0.f;
-      const float nx = pos[3 * stride + e], ny = pos[4 * stride + e], nz = pos[5 * stride + e];
-      const float ri2 = ri * ri, ri3 = ri2 * ri;
-      const float hf = fmaf(dx, fx, fmaf(dy, fy, dz * fz));
-      const float hu = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
-      const float hn = fmaf(dx, nx, fmaf(dy, ny, dz * nz));
-      const float t = ri3 * fmaf(hu * hn, ri2, hf);
-      two_sum_f(hi[0], lo[0], fmaf(fx, ri, dx * t));
-      two_sum_f(hi[1], lo[1], fmaf(fy, ri, dy * t));
-      two_sum_f(hi[2], lo[2], fmaf(fz, ri, dz * t));
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) acc[c] = (double)hi[c] + (double)lo[c];
-}
-
+// 2 Stokes with f and u strengths, 3 f alone, 4 u alone) into acc[3], in FP64 on absolute positions.
 template <int KIND>
 __device__ void near_sum64(const double* __restrict__ pos, int64_t stride, const double* __restrict__ str,
-                           int64_t sstride, int64_t n, const double x0[3], const double nv[3], int has_f,
-                           int has_u, double acc[3]) {
+                           int64_t sstride, int64_t n, const double x0[3], const double nv[3], double acc[3]) {
   double a[3] = {0.0, 0.0, 0.0};
   for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
     const double dx = x0[0] - pos[e], dy = x0[1] - pos[stride + e], dz = x0[2] - pos[2 * stride + e];
@@ -215,66 +181,29 @@ __device__ void near_sum64(const double* __restrict__ pos, int64_t stride, const
     } else if (KIND == 0) {
       a[0] = fma(str[e] * ri * ri * ri, dx * nv[0] + dy * nv[1] + dz * nv[2], a[0]);
     } else {
-      const double fx = has_f ? str[e] : 0.0, fy = has_f ? str[sstride + e] : 0.0, fz = has_f ? str[2 * sstride + e] : 0.0;
-      const double ux = has_u ? str[3 * sstride + e] : 0.0, uy = has_u ? str[4 * sstride + e] : 0.0,
-                   uz = has_u ? str[5 * sstride + e] : 0.0;
       const double ri2 = ri * ri, ri3 = ri2 * ri;
-      const double hf = dx * fx + dy * fy + dz * fz;
-      const double hu = dx * ux + dy * uy + dz * uz;
-      const double hn = dx * pos[3 * stride + e] + dy * pos[4 * stride + e] + dz * pos[5 * stride + e];
-      const double t = ri3 * (hf + hu * hn * ri2);
-      a[0] += fx * ri + dx * t;
-      a[1] += fy * ri + dy * t;
-      a[2] += fz * ri + dz * t;
+      double t = 0.0;
+      if (KIND != 3) {
+        const double hu = dx * str[3 * sstride + e] + dy * str[4 * sstride + e] + dz * str[5 * sstride + e];
+        const double hn = dx * pos[3 * stride + e] + dy * pos[4 * stride + e] + dz * pos[5 * stride + e];
+        t = hu * hn * ri2;
+      }
+      if (KIND != 4) {
+        const double fx = str[e], fy = str[sstride + e], fz = str[2 * sstride + e];
+        t = ri3 * (dx * fx + dy * fy + dz * fz + t);
+        a[0] += fx * ri + dx * t;
+        a[1] += fy * ri + dy * t;
+        a[2] += fz * ri + dz * t;
+      } else {
+        t *= ri3;
+        a[0] += dx * t;
+        a[1] += dy * t;
+        a[2] += dz * t;
+      }
     }
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) acc[c] = a[c];
-}
-
-// Double-float version (FP64-class accuracy on the FP32 pipe): positions, normals and strengths
-// are (FP32 copy, low part) pairs relative to drop j's centre; T is the target offset.
-template <int KIND>
-__device__ void near_sum_df(const float* __restrict__ pos, const float* __restrict__ poslo, int64_t stride,
-                            const float* __restrict__ str, const float* __restrict__ strlo, int64_t sstride,
-                            int64_t n, const dfl::df T[3], const dfl::df nv[3], int has_f, int has_u,
-                            double acc[3]) {
-  using dfl::df;
-  dfl::acc A[3];
-  for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-    const df dx = dfl::diff(T[0], df{pos[e], poslo[e]});
-    const df dy = dfl::diff(T[1], df{pos[stride + e], poslo[stride + e]});
-    const df dz = dfl::diff(T[2], df{pos[2 * stride + e], poslo[2 * stride + e]});
-    const df ri = dfl::rsqrt(dfl::dot3(dx, dy, dz, dx, dy, dz));
-    if (KIND == 1) {
-      A[0].add_prod(df{str[e], strlo[e]}, ri);
-    } else if (KIND == 0) {
-      const df dn = dfl::dot3(dx, dy, dz, nv[0], nv[1], nv[2]);
-      A[0].add_prod(dfl::mul(df{str[e], strlo[e]}, dfl::mul(dfl::sqr(ri), ri)), dn);
-    } else {
-      df f[3], u[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        f[c] = has_f ? df{str[c * sstride + e], strlo[c * sstride + e]} : df{0.f, 0.f};
-        u[c] = has_u ? df{str[(3 + c) * sstride + e], strlo[(3 + c) * sstride + e]} : df{0.f, 0.f};
-      }
-      const df nx{pos[3 * stride + e], poslo[3 * stride + e]}, ny{pos[4 * stride + e], poslo[4 * stride + e]},
-          nz{pos[5 * stride + e], poslo[5 * stride + e]};
-      const df hf = dfl::dot3(dx, dy, dz, f[0], f[1], f[2]);
-      const df hu = dfl::dot3(dx, dy, dz, u[0], u[1], u[2]);
-      const df hn = dfl::dot3(dx, dy, dz, nx, ny, nz);
-      const df ri2 = dfl::sqr(ri);
-      const df tt = dfl::mul(dfl::mul(ri2, ri), dfl::add(hf, dfl::mul(dfl::mul(hu, hn), ri2)));
-      const df d[3] = {dx, dy, dz};
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        A[c].add_prod(f[c], ri);
-        A[c].add_prod(d[c], tt);
-      }
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) acc[c] = dfl::to_double(A[c].value());
 }
 
 struct NearArgs {
@@ -300,14 +229,12 @@ struct NearArgs {
   const float* fstr32lo;
   const float* src32lo;
   const float* sstr32lo;
-  int has_f, has_u;
   double* out;
 };
 
-// MODE 0: FP64, 1: FP32 compensated, 2: double-float
-template <int KIND, int MODE>
+// FP64: one CTA per near pair and chunk of nodes
+template <int KIND>
 __global__ void __launch_bounds__(256) k_near_direct(NearArgs A) {
-  constexpr bool F32 = MODE == 1;
   const int pr = blockIdx.x;
   const int64_t t = A.pair_t[pr];
   const int j = A.pair_j[pr];
@@ -325,50 +252,14 @@ __global__ void __launch_bounds__(256) k_near_direct(NearArgs A) {
     nv[c] = A.tgt[(3 + c) * A.ntarget + t];
   }
   double af[3], au[3];
-  if (F32) {
-    const double cj[3] = {D.cx, D.cy, D.cz};
-    float th[3], tl[3], n32[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double d = x0[c] - cj[c];
-      th[c] = (float)d;
-      tl[c] = (float)(d - (double)th[c]);
-      n32[c] = (float)nv[c];
-    }
-    near_sum32<KIND>(A.fpos32 + fo, A.nfine, A.fstr32 + fo, A.nfine, fn, th, tl, n32, A.has_f, A.has_u, af);
-    near_sum32<KIND>(A.src32 + so, A.nsource, A.sstr32 + so, A.nsource, sn, th, tl, n32,
-                     A.has_f, A.has_u, au);
-  } else if (MODE == 2) {
-    // the target offset and normal as double-float, converted once per block (FP64 pipe)
-    __shared__ float2 tv[6];
-    if (threadIdx.x < 6) {
-      const double cj[3] = {D.cx, D.cy, D.cz};
-      const int c = threadIdx.x % 3;
-      const dfl::df v = dfl::from_double(threadIdx.x < 3 ? x0[c] - cj[c] : nv[c]);
-      tv[threadIdx.x] = make_float2(v.hi, v.lo);
-    }
-    __syncthreads();
-    dfl::df T[3], nd[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      T[c] = dfl::df{tv[c].x, tv[c].y};
-      nd[c] = dfl::df{tv[3 + c].x, tv[3 + c].y};
-    }
-    near_sum_df<KIND>(A.fpos32 + fo, A.fpos32lo + fo, A.nfine, A.fstr32 + fo, A.fstr32lo + fo, A.nfine, fn, T, nd,
-                      A.has_f, A.has_u, af);
-    near_sum_df<KIND>(A.src32 + so, A.src32lo + so, A.nsource, A.sstr32 + so, A.sstr32lo + so, A.nsource, sn, T,
-                      nd, A.has_f, A.has_u, au);
-  } else {
-    near_sum64<KIND>(A.fpos + fo, A.nfine, A.fstr + fo, A.nfine, fn, x0, nv, A.has_f, A.has_u, af);
-    near_sum64<KIND>(A.src + so, A.nsource, A.sstr + so, A.nsource, sn, x0, nv, A.has_f,
-                     A.has_u, au);
-  }
-  const int nc = KIND == 2 ? 3 : 1;
+  near_sum64<KIND>(A.fpos + fo, A.nfine, A.fstr + fo, A.nfine, fn, x0, nv, af);
+  near_sum64<KIND>(A.src + so, A.nsource, A.sstr + so, A.nsource, sn, x0, nv, au);
+  const int nc = KIND >= 2 ? 3 : 1;
   for (int c = 0; c < nc; ++c) {
     const double v = block_sum_near(af[c] - au[c]);
     if (threadIdx.x == 0) {
       const double val = 0.07957747154594766788 * v;
-      if (KIND != 2) {
+      if (KIND < 2) {
         atomicAdd(A.out + t, val);
       } else {
         const DropDev Di = A.drops[A.tgt_drop[t]];
@@ -382,23 +273,40 @@ __global__ void __launch_bounds__(256) k_near_direct(NearArgs A) {
 // target per thread) and a chunk of the concatenated node list [drop j's upsampled nodes, then
 // its degree-q nodes with the strengths negated]; nodes are staged through shared memory in
 // tiles and read as broadcasts (as in the all-pairs kernels), sums compensated by two-sum, each
-// chunk's result added to the target's output with an FP64 atomic.
+// chunk's result added to the target's output with an FP64 atomic. A group of 64 or fewer targets needs one or two
+// warps; the CTA's others take every second or fourth node of the tile (40 drops of degree 11, 20 to 60 near targets
+// each: 0.42 -> 0.20 ms in double-float).
+struct NearSlot {
+  int t, slice, slices;   // target of the group (-1: none), this warp's share of the nodes
+};
+__device__ __forceinline__ NearSlot near_slot(int targets) {
+  const int warps = kNearGroup / 32, need = (targets + 31) / 32, w = threadIdx.x >> 5;
+  NearSlot r;
+  r.slices = warps / need;
+  r.slice = w / need;
+  const int t = (w % need) * 32 + (threadIdx.x & 31);
+  r.t = r.slice < r.slices && t < targets ? t : -1;
+  return r;
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(kNearGroup)
 k_near_tiled32(NearArgs A, const int4* __restrict__ groups) {
-  constexpr int NC = KIND == 2 ? 3 : 1;
+  constexpr bool STO = KIND >= 2;
+  constexpr int NC = STO ? 3 : 1;
   constexpr int TILE = 256;
   __shared__ float4 sp[TILE];                  // x y z (relative to drop j's centre), strength 0
-  __shared__ float4 sq[KIND == 2 ? TILE : 1];  // strengths 1..4
-  __shared__ float4 sr[KIND == 2 ? TILE : 1];  // strength 5, normal
+  __shared__ float4 sq[STO ? TILE : 1];  // strengths 1..4
+  __shared__ float4 sr[KIND == 2 || KIND == 4 ? TILE : 1];  // strength 5, normal
   const int4 g = groups[blockIdx.x];
   const int j = g.z;
   const DropDev D = A.drops[j];
   const int64_t fo = A.fine_off[j], fn = A.fine_n[j];
   const int64_t ntot = fn + D.ns;
   const int64_t c0 = ntot * blockIdx.y / gridDim.y, c1 = ntot * (blockIdx.y + 1) / gridDim.y;
-  const bool act = (int)threadIdx.x < g.y;
-  const int64_t t = A.pair_t[g.x + (act ? threadIdx.x : 0)];
+  const NearSlot sl = near_slot(g.y);
+  const bool act = sl.t >= 0;
+  const int64_t t = A.pair_t[g.x + (act ? sl.t : 0)];
   float th[3], tl[3], nv[3];
   {
     const double cj[3] = {D.cx, D.cy, D.cz};
@@ -423,15 +331,15 @@ k_near_tiled32(NearArgs A, const int4* __restrict__ groups) {
       const float* str = fine ? A.fstr32 + fo + v : A.sstr32 + D.src_off + (v - fn);
       const int64_t ps = fine ? A.nfine : A.nsource;
       const float sg = fine ? 1.f : -1.f;
-      if (KIND != 2) {
+      if (!STO) {
         sp[e] = make_float4(pos[0], pos[ps], pos[2 * ps], sg * str[0]);
       } else {
-        const float f0 = A.has_f ? sg * str[0] : 0.f, f1 = A.has_f ? sg * str[ps] : 0.f, f2 = A.has_f ? sg * str[2 * ps] : 0.f;
-        const float u0 = A.has_u ? sg * str[3 * ps] : 0.f, u1 = A.has_u ? sg * str[4 * ps] : 0.f,
-                    u2 = A.has_u ? sg * str[5 * ps] : 0.f;
+        const bool F = KIND != 4, U = KIND != 3;
+        const float f0 = F ? sg * str[0] : 0.f, f1 = F ? sg * str[ps] : 0.f, f2 = F ? sg * str[2 * ps] : 0.f;
+        const float u0 = U ? sg * str[3 * ps] : 0.f, u1 = U ? sg * str[4 * ps] : 0.f, u2 = U ? sg * str[5 * ps] : 0.f;
         sp[e] = make_float4(pos[0], pos[ps], pos[2 * ps], f0);
         sq[e] = make_float4(f1, f2, u0, u1);
-        sr[e] = make_float4(u2, pos[3 * ps], pos[4 * ps], pos[5 * ps]);
+        if (U) sr[e] = make_float4(u2, pos[3 * ps], pos[4 * ps], pos[5 * ps]);
       }
     }
     __syncthreads();
@@ -439,7 +347,7 @@ k_near_tiled32(NearArgs A, const int4* __restrict__ groups) {
 #pragma unroll
     for (int c = 0; c < NC; ++c) acc[c] = 0.f;
 #pragma unroll 4
-    for (int e = 0; e < cnt; ++e) {
+    for (int e = sl.slice; e < cnt; e += sl.slices) {
       const float4 P = sp[e];
       const float dx = (th[0] - P.x) + tl[0];
       const float dy = (th[1] - P.y) + tl[1];
@@ -451,15 +359,26 @@ k_near_tiled32(NearArgs A, const int4* __restrict__ groups) {
         const float dn = fmaf(dx, nv[0], fmaf(dy, nv[1], dz * nv[2]));
         acc[0] = fmaf(P.w * ri * ri * ri, dn, acc[0]);
       } else {
-        const float4 Q = sq[e], R = sr[e];
+        const float4 Q = sq[e];
         const float ri2 = ri * ri, ri3 = ri2 * ri;
-        const float hf = fmaf(dx, P.w, fmaf(dy, Q.x, dz * Q.y));
-        const float hu = fmaf(dx, Q.z, fmaf(dy, Q.w, dz * R.x));
-        const float hn = fmaf(dx, R.y, fmaf(dy, R.z, dz * R.w));
-        const float tt = ri3 * fmaf(hu * hn, ri2, hf);
-        acc[0] = fmaf(P.w, ri, fmaf(dx, tt, acc[0]));
-        acc[1] = fmaf(Q.x, ri, fmaf(dy, tt, acc[1]));
-        acc[2] = fmaf(Q.y, ri, fmaf(dz, tt, acc[2]));
+        float tt = 0.f;
+        if (KIND != 3) {
+          const float4 R = sr[e];
+          const float hu = fmaf(dx, Q.z, fmaf(dy, Q.w, dz * R.x));
+          const float hn = fmaf(dx, R.y, fmaf(dy, R.z, dz * R.w));
+          tt = KIND == 4 ? (hu * hn) * (ri3 * ri2) : hu * hn;
+        }
+        if (KIND != 4) {
+          const float hf = fmaf(dx, P.w, fmaf(dy, Q.x, dz * Q.y));
+          tt = KIND == 3 ? ri3 * hf : ri3 * fmaf(tt, ri2, hf);
+          acc[0] = fmaf(P.w, ri, fmaf(dx, tt, acc[0]));
+          acc[1] = fmaf(Q.x, ri, fmaf(dy, tt, acc[1]));
+          acc[2] = fmaf(Q.y, ri, fmaf(dz, tt, acc[2]));
+        } else {
+          acc[0] = fmaf(dx, tt, acc[0]);
+          acc[1] = fmaf(dy, tt, acc[1]);
+          acc[2] = fmaf(dz, tt, acc[2]);
+        }
       }
     }
 #pragma unroll
@@ -469,7 +388,7 @@ k_near_tiled32(NearArgs A, const int4* __restrict__ groups) {
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
     const double val = 0.07957747154594766788 * ((double)hi[c] + (double)lo[c]);
-    if (KIND != 2) {
+    if (!STO) {
       atomicAdd(A.out + t, val);
     } else {
       const DropDev Di = A.drops[A.tgt_drop[t]];
@@ -483,8 +402,9 @@ k_near_tiled32(NearArgs A, const int4* __restrict__ groups) {
 template <int KIND>
 __global__ void __launch_bounds__(kNearGroup)
 k_near_tiled_df(NearArgs A, const int4* __restrict__ groups) {
-  constexpr int NC = KIND == 2 ? 3 : 1;
-  constexpr int NV = KIND == 2 ? 6 : 2;
+  constexpr bool STO = KIND >= 2;
+  constexpr int NC = STO ? 3 : 1;
+  constexpr int NV = STO ? 6 : 2;
   constexpr int TILE = 128;
   __shared__ float4 sh[NV][TILE];
   __shared__ float2 tv[kNearGroup][6];   // per target: offset from drop j's centre, normal
@@ -494,8 +414,9 @@ k_near_tiled_df(NearArgs A, const int4* __restrict__ groups) {
   const int64_t fo = A.fine_off[j], fn = A.fine_n[j];
   const int64_t ntot = fn + D.ns;
   const int64_t c0 = ntot * blockIdx.y / gridDim.y, c1 = ntot * (blockIdx.y + 1) / gridDim.y;
-  const bool act = (int)threadIdx.x < g.y;
-  const int64_t t = A.pair_t[g.x + (act ? threadIdx.x : 0)];
+  const NearSlot sl = near_slot(g.y);
+  const bool act = sl.t >= 0;
+  const int64_t t = A.pair_t[g.x + (act ? sl.t : 0)];
   {
     const double cj[3] = {D.cx, D.cy, D.cz};
 #pragma unroll
@@ -527,16 +448,16 @@ k_near_tiled_df(NearArgs A, const int4* __restrict__ groups) {
       const int64_t ps = fine ? A.nfine : A.nsource;
       const float sg = fine ? 1.f : -1.f;
       sh[0][e] = make_float4(ph[o], ph[ps + o], ph[2 * ps + o], pl[o]);
-      if constexpr (KIND != 2) {
+      if constexpr (!STO) {
         sh[1][e] = make_float4(pl[ps + o], pl[2 * ps + o], sg * qh[o], sg * ql[o]);
       } else {
         float fv[6], uv[6];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          fv[2 * c] = A.has_f ? sg * qh[c * ps + o] : 0.f;
-          fv[2 * c + 1] = A.has_f ? sg * ql[c * ps + o] : 0.f;
-          uv[2 * c] = A.has_u ? sg * qh[(3 + c) * ps + o] : 0.f;
-          uv[2 * c + 1] = A.has_u ? sg * ql[(3 + c) * ps + o] : 0.f;
+          fv[2 * c] = KIND != 4 ? sg * qh[c * ps + o] : 0.f;
+          fv[2 * c + 1] = KIND != 4 ? sg * ql[c * ps + o] : 0.f;
+          uv[2 * c] = KIND != 3 ? sg * qh[(3 + c) * ps + o] : 0.f;
+          uv[2 * c + 1] = KIND != 3 ? sg * ql[(3 + c) * ps + o] : 0.f;
         }
         sh[1][e] = make_float4(pl[ps + o], pl[2 * ps + o], fv[0], fv[1]);
         sh[2][e] = make_float4(fv[2], fv[3], fv[4], fv[5]);
@@ -547,8 +468,8 @@ k_near_tiled_df(NearArgs A, const int4* __restrict__ groups) {
     }
     __syncthreads();
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int e = 0; e < cnt; ++e) {
-      if constexpr (KIND != 2)
+    for (int e = sl.slice; e < cnt; e += sl.slices) {
+      if constexpr (!STO)
         df_term<KIND>(T, N0, sh[0][e], sh[1][e], z4, z4, z4, z4, acc);
       else
         df_term<KIND>(T, N0, sh[0][e], sh[1][e], sh[2][e], sh[3][e], sh[4][e], sh[5][e], acc);
@@ -558,7 +479,7 @@ k_near_tiled_df(NearArgs A, const int4* __restrict__ groups) {
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
     const double val = 0.07957747154594766788 * dfl::to_double(acc[c].value());
-    if (KIND != 2) {
+    if (!STO) {
       atomicAdd(A.out + t, val);
     } else {
       const DropDev Di = A.drops[A.tgt_drop[t]];
@@ -754,54 +675,36 @@ int build_near(shbim_ctx* ctx, const double* xcoef, cudaStream_t s) {
 
 namespace {
 
-int launch_direct(shbim_ctx* ctx, int kind, bool has_f, bool has_u, double* out, cudaStream_t s) {
+template <int KIND>
+int launch_direct(shbim_ctx* ctx, double* out, cudaStream_t s) {
   auto& N = ctx->near;
   NearArgs A{N.pair_t, N.pair_j, N.foff_dev, N.foff_dev + ctx->n_drops, ctx->drops_dev, ctx->geo.tgt_drop,
              ctx->geo.tgt, ctx->ntarget, N.fgeo, N.fgeo32, N.fstr, N.fstr32, N.nfine, ctx->geo.src,
              ctx->geo.src32, ctx->dens_up, ctx->dens_up32, ctx->nsource, N.fgeo32lo, N.fstr32lo,
-             ctx->geo.src32lo, ctx->dens_up32lo, has_f ? 1 : 0, has_u ? 1 : 0, out};
-  const int mode = ctx->opts.precision == SHBIM_PREC_FP32_COMP ? 1 : (ctx->opts.precision == SHBIM_PREC_DF64 ? 2 : 0);
-  // enough CTAs for ~8 per SM: each near pair's sums are split into chunks of both grids
+             ctx->geo.src32lo, ctx->dens_up32lo, out};
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(32, (8ll * nsm + N.npairs - 1) / N.npairs));
-  const dim3 g((unsigned)N.npairs, (unsigned)chunks);
-  if (mode != 0) {
-    // FP32 and double-float: tiled over groups of targets sharing a source drop
-    // chunks of at least 512 nodes, enough CTAs for ~8 per SM
-    int64_t nmax = 0;
-    for (int j = 0; j < ctx->n_drops; ++j)
-      if (N.fine_off_h[j] >= 0) nmax = std::max<int64_t>(nmax, N.fine_n_h[j] + ctx->drops[j].ns);
-    const int gc = (int)std::max<int64_t>(
-        1, std::min<int64_t>(std::max<int64_t>(1, nmax / 512), (8ll * nsm + N.ngroups - 1) / N.ngroups));
-    const dim3 gg((unsigned)N.ngroups, (unsigned)gc);
-    if (mode == 1) {
-      if (kind == 0) k_near_tiled32<0><<<gg, kNearGroup, 0, s>>>(A, N.groups);
-      else if (kind == 1) k_near_tiled32<1><<<gg, kNearGroup, 0, s>>>(A, N.groups);
-      else k_near_tiled32<2><<<gg, kNearGroup, 0, s>>>(A, N.groups);
-    } else {
-      if (kind == 0) k_near_tiled_df<0><<<gg, kNearGroup, 0, s>>>(A, N.groups);
-      else if (kind == 1) k_near_tiled_df<1><<<gg, kNearGroup, 0, s>>>(A, N.groups);
-      else k_near_tiled_df<2><<<gg, kNearGroup, 0, s>>>(A, N.groups);
-    }
-    SHBIM_CHECK_LAUNCH(ctx, "k_near_tiled");
+  if (ctx->opts.precision == SHBIM_PREC_FP64) {
+    // enough CTAs for ~8 per SM: each near pair's sums are split into chunks of both grids
+    const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(32, (8ll * nsm + N.npairs - 1) / N.npairs));
+    k_near_direct<KIND><<<dim3((unsigned)N.npairs, (unsigned)chunks), 256, 0, s>>>(A);
+    SHBIM_CHECK_LAUNCH(ctx, "k_near_direct");
     return SHBIM_OK;
   }
-  if (kind == 0) {
-    if (mode == 1) k_near_direct<0, 1><<<g, 256, 0, s>>>(A);
-    else if (mode == 2) k_near_direct<0, 2><<<g, 256, 0, s>>>(A);
-    else k_near_direct<0, 0><<<g, 256, 0, s>>>(A);
-  } else if (kind == 1) {
-    if (mode == 1) k_near_direct<1, 1><<<g, 256, 0, s>>>(A);
-    else if (mode == 2) k_near_direct<1, 2><<<g, 256, 0, s>>>(A);
-    else k_near_direct<1, 0><<<g, 256, 0, s>>>(A);
-  } else {
-    if (mode == 1) k_near_direct<2, 1><<<g, 256, 0, s>>>(A);
-    else if (mode == 2) k_near_direct<2, 2><<<g, 256, 0, s>>>(A);
-    else k_near_direct<2, 0><<<g, 256, 0, s>>>(A);
-  }
-  SHBIM_CHECK_LAUNCH(ctx, "k_near_direct");
+  // FP32 and double-float: tiled over groups of targets sharing a source drop, chunks of at least 512 nodes, enough
+  // CTAs for ~8 per SM
+  int64_t nmax = 0;
+  for (int j = 0; j < ctx->n_drops; ++j)
+    if (N.fine_off_h[j] >= 0) nmax = std::max<int64_t>(nmax, N.fine_n_h[j] + ctx->drops[j].ns);
+  const int gc = (int)std::max<int64_t>(
+      1, std::min<int64_t>(std::max<int64_t>(1, nmax / 512), (8ll * nsm + N.ngroups - 1) / N.ngroups));
+  const dim3 gg((unsigned)N.ngroups, (unsigned)gc);
+  if (ctx->opts.precision == SHBIM_PREC_FP32_COMP)
+    k_near_tiled32<KIND><<<gg, kNearGroup, 0, s>>>(A, N.groups);
+  else
+    k_near_tiled_df<KIND><<<gg, kNearGroup, 0, s>>>(A, N.groups);
+  SHBIM_CHECK_LAUNCH(ctx, "k_near_tiled");
   return SHBIM_OK;
 }
 
@@ -820,7 +723,7 @@ int apply_near_laplace(shbim_ctx* ctx, int which, const double* dens, double* ou
     if (rc) return rc;
   }
   if (before_sums) SHBIM_CUDA(ctx, cudaStreamWaitEvent(s, before_sums, 0));
-  return launch_direct(ctx, which == SHBIM_LAPLACE_SL ? 1 : 0, false, false, out, s);
+  return which == SHBIM_LAPLACE_SL ? launch_direct<1>(ctx, out, s) : launch_direct<0>(ctx, out, s);
 }
 
 int apply_near_stokes(shbim_ctx* ctx, const double* f, const double* u, double* out, cudaStream_t s,
@@ -844,7 +747,8 @@ int apply_near_stokes(shbim_ctx* ctx, const double* f, const double* u, double* 
       return rc;
   }
   if (before_sums) SHBIM_CUDA(ctx, cudaStreamWaitEvent(s, before_sums, 0));
-  return launch_direct(ctx, 2, f != nullptr, u != nullptr, out, s);
+  // the kernels of one term alone (KIND 3, 4) skip the other's arithmetic and strengths
+  return f && u ? launch_direct<2>(ctx, out, s) : (f ? launch_direct<3>(ctx, out, s) : launch_direct<4>(ctx, out, s));
 }
 
 }  // namespace shbim
