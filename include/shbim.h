@@ -197,7 +197,7 @@ int shbim_electric_rhs(shbim_ctx* ctx, const double* E_u_host, double E_q, doubl
  *                  or grid values (inverse output, forward input), each field's block after the
  *                  previous one's; must not alias
  * SHBIM_ERR_ARG for a drop index out of range, a bad direction or grid, or null pointers with
- * n_fields > 0. Consecutive fields of one drop are transformed by one launch. */
+ * n_fields > 0. Fields on grids of one degree are transformed together (up to 128 per launch). */
 int shbim_sht(shbim_ctx* ctx, int dir, int grid, int n_fields, const int32_t* field_drop_host,
               const double* in_dev, double* out_dev, void* stream);
 

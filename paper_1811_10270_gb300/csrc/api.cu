@@ -529,37 +529,34 @@ int shbim_sht(shbim_ctx* ctx, int dir, int grid, int n_fields, const int32_t* fi
     if (field_drop_host[f] < 0 || field_drop_host[f] >= ctx->n_drops)
       return fail(ctx, SHBIM_ERR_ARG, "field_drop: drop index out of range");
   cudaStream_t s = (cudaStream_t)stream;
-  // fields are concatenated, each with its own drop's coefficient count and grid size; a run of
-  // consecutive fields of one drop is one transform launch
-  int64_t in_off = 0, out_off = 0;
-  for (int f = 0, g; f < n_fields; f = g) {
-    g = f + 1;
-    while (g < n_fields && field_drop_host[g] == field_drop_host[f]) ++g;
+  // fields are concatenated, each with its own drop's coefficient count and grid size; those of one degree go together
+  struct Group {
+    const GridTables* tab;
+    std::vector<int64_t> coef, val;
+  };
+  std::vector<Group> groups;
+  int64_t co = 0, vo = 0;
+  for (int f = 0; f < n_fields; ++f) {
     const Drop& d = ctx->drops[field_drop_host[f]];
-    const GridTables& T = grid == SHBIM_GRID_BASE ? d.tab->base : d.tab->up;
-    const int64_t n = npts(T.q);
-    const int nf = g - f;
-    int rc;
-    if (dir == SHBIM_SHT_INVERSE) {
-      rc = sht_synth(ctx, T, nf, in_dev + in_off, d.nc, 1, out_dev + out_off, n, 0, nullptr, nullptr, s);
-      in_off += (int64_t)nf * d.nc;
-      out_off += (int64_t)nf * n;
-    } else {
-      rc = sht_analysis(ctx, T, nf, in_dev + in_off, n, true, out_dev + out_off, d.nc, s);
-      in_off += (int64_t)nf * n;
-      out_off += (int64_t)nf * d.nc;
-    }
-    if (rc) return rc;
+    const GridTables* T = grid == SHBIM_GRID_BASE ? &d.tab->base : &d.tab->up;
+    size_t k = 0;
+    while (k < groups.size() && groups[k].tab != T) ++k;
+    if (k == groups.size()) groups.push_back(Group{T, {}, {}});
+    groups[k].coef.push_back(co);
+    groups[k].val.push_back(vo);
+    co += d.nc;
+    vo += npts(T->q);
   }
+  for (const Group& g : groups)
+    if (int rc = sht_fields(ctx, *g.tab, dir == SHBIM_SHT_FORWARD, (int)g.coef.size(), g.coef.data(), g.val.data(), in_dev,
+                            out_dev, s))
+      return rc;
   return SHBIM_OK;
 }
 
 }  // extern "C"
 
 namespace shbim {
-namespace {
-
-}  // namespace
 
 int ensure_side_stream(shbim_ctx* ctx) {
   if (ctx->side) return SHBIM_OK;

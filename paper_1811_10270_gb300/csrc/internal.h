@@ -442,6 +442,11 @@ int sht_analysis(shbim_ctx* ctx, const GridTables& g, int n_items, const double*
                  int64_t val_stride, bool weighted, double* coef, int64_t coef_stride,
                  cudaStream_t s, int kpd = 1, const DropList* L = nullptr);
 
+// Transforms of n single fields of one degree, field f's coefficients at coef_off[f] and grid values at val_off[f] (host
+// arrays), values only, weighted analysis.
+int sht_fields(shbim_ctx* ctx, const GridTables& g, bool forward, int n, const int64_t* coef_off, const int64_t* val_off,
+               const double* in, double* out, cudaStream_t s);
+
 // ---- geometry / singular rows (singular.cu)
 int build_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s);
 int build_singular_rows(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s);

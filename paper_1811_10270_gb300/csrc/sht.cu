@@ -14,6 +14,27 @@ namespace shbim {
 
 __device__ __forceinline__ int tri_off_d(int p, int m) { return m * (p + 1) - m * (m - 1) / 2; }
 
+// Where the items of a launch lie. DropList: device arrays, kpd items per drop; FieldList: up to kMaxFields single fields
+// of one degree, their offsets in the kernel's parameters (calls on fields of several drops need no list in memory).
+constexpr int kMaxFields = 128;
+struct FieldList {
+  int64_t coef[kMaxFields];
+  int64_t val[kMaxFields];
+};
+struct ItemAt {
+  int64_t coef, val;
+  int drop;           // for the per-drop factor
+};
+__device__ __forceinline__ ItemAt item_at(const DropList& L, int item, int kpd, int64_t coef_stride, int64_t val_stride,
+                                          int64_t drop_stride) {
+  const int dl = item / kpd, ci = item - dl * kpd;
+  if (!L.idx) return ItemAt{(int64_t)item * coef_stride, (int64_t)dl * drop_stride + (int64_t)ci * val_stride, dl};
+  return ItemAt{(int64_t)kpd * L.coef_off[dl] + (int64_t)ci * coef_stride, L.val_off[dl] + (int64_t)ci * val_stride, L.idx[dl]};
+}
+__device__ __forceinline__ ItemAt item_at(const FieldList& L, int item, int, int64_t, int64_t, int64_t) {
+  return ItemAt{L.coef[item], L.val[item], 0};
+}
+
 // kinds bitmask -> table index of the slot-th set bit
 __device__ __forceinline__ int kind_of_slot(int kinds, int slot) {
   int k = 0;
@@ -29,19 +50,18 @@ __device__ __forceinline__ int kind_of_slot(int kinds, int slot) {
 // Items are (drop d, component c) with item = d kpd + c: coefficients at item * coef_stride,
 // values at d drop_stride + c item_stride (+ kind slot * kind_stride), the per-node scale at
 // d drop_stride, the factor alpha (times alpha_drop[d] when given).
+template <class List>
 __global__ void k_synth(const double* __restrict__ coef, int64_t coef_stride, int p, int q,
                         const double* __restrict__ alf, const double* __restrict__ trig, int kinds,
                         double* __restrict__ out, int64_t item_stride, int64_t kind_stride,
                         const double* __restrict__ scale, double alpha, float* __restrict__ out32,
                         float* __restrict__ out32lo, int kpd, int64_t drop_stride,
-                        const double* __restrict__ alpha_drop, DropList L) {
+                        const double* __restrict__ alpha_drop, const __grid_constant__ List L) {
   extern __shared__ double sm[];
-  const int item = blockIdx.x;
-  const int dl = item / kpd, ci = item - dl * kpd;
-  const int64_t dbase = L.idx ? L.val_off[dl] : (int64_t)dl * drop_stride;
-  const int64_t obase = dbase + (int64_t)ci * item_stride;
-  if (scale) scale += dbase;
-  if (alpha_drop) alpha *= alpha_drop[L.idx ? L.idx[dl] : dl];
+  const ItemAt at = item_at(L, blockIdx.x, kpd, coef_stride, item_stride, drop_stride);
+  const int64_t obase = at.val;
+  if (scale) scale += at.val - (int64_t)(blockIdx.x % kpd) * item_stride;   // one scale per drop, not per component
+  if (alpha_drop) alpha *= alpha_drop[at.drop];
   const int j = blockIdx.y;
   const int nk = __popc(kinds);
   const int N = 2 * q + 2;
@@ -53,8 +73,7 @@ __global__ void k_synth(const double* __restrict__ coef, int64_t coef_stride, in
     tc[i] = trig[i];
     ts[i] = trig[N + i];
   }
-  const double* c = coef + (L.idx ? (int64_t)kpd * L.coef_off[dl] + (int64_t)ci * coef_stride
-                                   : (int64_t)item * coef_stride);
+  const double* c = coef + at.coef;
   const int nt = (p + 1) * (p + 2) / 2;
   const double* T = alf + (int64_t)j * kNumTab * nt;
   const int ntask = nk * 2 * P1;
@@ -146,7 +165,8 @@ __global__ void k_synth(const double* __restrict__ coef, int64_t coef_stride, in
 int synth_smem_ok(shbim_ctx* ctx, size_t smem) {
   if (smem <= 48 * 1024) return SHBIM_OK;
   if (smem > 227 * 1024) return fail(ctx, SHBIM_ERR_ARG, "synthesis grid too large for shared memory");
-  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_synth, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_synth<DropList>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_synth<FieldList>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   return SHBIM_OK;
 }
 
@@ -159,7 +179,7 @@ int sht_synth(shbim_ctx* ctx, const GridTables& g, int n_items, const double* co
   const size_t smem = (size_t)(nk * 2 * (g.p + 1) + (2 + nk) * (2 * g.q + 2)) * sizeof(double);
   if (int rc = synth_smem_ok(ctx, smem)) return rc;
   dim3 grid(n_items, g.q + 1);
-  k_synth<<<grid, 128, smem, s>>>(coef, coef_stride, g.p, g.q, g.alf, g.trig, kinds, out,
+  k_synth<DropList><<<grid, 128, smem, s>>>(coef, coef_stride, g.p, g.q, g.alf, g.trig, kinds, out,
                                   item_stride, kind_stride, scale, 1.0, out32, nullptr, L ? kpd : n_items, 0, nullptr,
                                   L ? *L : DropList{});
   SHBIM_CHECK_LAUNCH(ctx, "k_synth");
@@ -268,7 +288,7 @@ int sht_synth_drops(shbim_ctx* ctx, const GridTables& g, int nb, int kpd, const 
   const size_t smem = (size_t)(2 * (g.p + 1) + 3 * (2 * g.q + 2)) * sizeof(double);
   if (int rc = synth_smem_ok(ctx, smem)) return rc;
   dim3 grid(n_items, g.q + 1);
-  k_synth<<<grid, 128, smem, s>>>(coef, coef_stride, g.p, g.q, g.alf, g.trig, 1, out, item_stride,
+  k_synth<DropList><<<grid, 128, smem, s>>>(coef, coef_stride, g.p, g.q, g.alf, g.trig, 1, out, item_stride,
                                   0, scale, alpha, out32, out32 ? out32lo : nullptr, kpd, drop_stride, alpha_drop,
                                   list);
   SHBIM_CHECK_LAUNCH(ctx, "k_synth");
@@ -276,9 +296,10 @@ int sht_synth_drops(shbim_ctx* ctx, const GridTables& g, int nb, int kpd, const 
 }
 
 // Fourier stage of the analysis: F[item][j][cs][m] = (omega_j) sum_k v[j][k] (cos|sin)(m phi_k)
+template <class List>
 __global__ void k_analysis_fourier(const double* __restrict__ vals, int64_t val_stride, int p, int q,
                                    const double* __restrict__ trig, const double* __restrict__ omega,
-                                   int weighted, double* __restrict__ F, int kpd, DropList L) {
+                                   int weighted, double* __restrict__ F, int kpd, const __grid_constant__ List L) {
   extern __shared__ double sm[];
   const int item = blockIdx.x;
   const int j = blockIdx.y;
@@ -287,8 +308,7 @@ __global__ void k_analysis_fourier(const double* __restrict__ vals, int64_t val_
   double* row = sm;
   double* tc = row + N;
   double* ts = tc + N;
-  const int64_t ib = L.idx ? L.val_off[item / kpd] + (int64_t)(item % kpd) * val_stride : (int64_t)item * val_stride;
-  const double* v = vals + ib + (int64_t)j * N;
+  const double* v = vals + item_at(L, item, kpd, 0, val_stride, (int64_t)kpd * val_stride).val + (int64_t)j * N;
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     row[i] = v[i];
     tc[i] = trig[i];
@@ -315,10 +335,11 @@ __global__ void k_analysis_fourier(const double* __restrict__ vals, int64_t val_
 // Fourier stage for N divisible by 4, `rows` (item, latitude) rows per block. Each row is
 // folded twice -- k with N-k (even / odd part in phi) and k with N/2-k (parity of m) -- so every
 // output sums N/4-1 terms instead of N: four times fewer FP64 FMAs than the plain sum.
+template <class List>
 __global__ void k_analysis_fourier4(const double* __restrict__ vals, int64_t val_stride, int p, int q,
                                     const double* __restrict__ trig, const double* __restrict__ omega,
                                     int weighted, int64_t nrows, int rows, double* __restrict__ F, int kpd,
-                                    DropList L) {
+                                    const __grid_constant__ List L) {
   extern __shared__ double sm[];
   const int N = 2 * q + 2;
   const int P1 = p + 1;
@@ -337,7 +358,7 @@ __global__ void k_analysis_fourier4(const double* __restrict__ vals, int64_t val
     const int r = e / N, k = e - r * N;
     const int64_t row = r0 + r;
     const int64_t item = row / (q + 1), j = row - item * (q + 1);
-    const int64_t ib = L.idx ? L.val_off[item / kpd] + (item % kpd) * val_stride : item * val_stride;
+    const int64_t ib = item_at(L, (int)item, kpd, 0, val_stride, (int64_t)kpd * val_stride).val;
     R[r * 2 * N + k] = vals[ib + j * N + k];
   }
   __syncthreads();
@@ -390,9 +411,10 @@ __global__ void k_analysis_fourier4(const double* __restrict__ vals, int64_t val
 }
 
 // Legendre stage: coef[item][n^2+n+-m] = s_m sum_j F[item][j][cs][m] Pbar_n^m(t_j)
+template <class List>
 __global__ void k_analysis_legendre(const double* __restrict__ F, int p, int q,
                                     const double* __restrict__ alf, double* __restrict__ coef,
-                                    int64_t coef_stride, int kpd, DropList L) {
+                                    int64_t coef_stride, int kpd, const __grid_constant__ List L) {
   const int item = blockIdx.x;
   const int nt = (p + 1) * (p + 2) / 2;
   const int o = blockIdx.y * blockDim.x + threadIdx.x;
@@ -408,8 +430,7 @@ __global__ void k_analysis_legendre(const double* __restrict__ F, int p, int q,
     ac = fma(Fi[(int64_t)j * 2 * P1 + m], a, ac);
     as = fma(Fi[(int64_t)j * 2 * P1 + P1 + m], a, as);
   }
-  double* c = coef + (L.idx ? (int64_t)kpd * L.coef_off[item / kpd] + (int64_t)(item % kpd) * coef_stride
-                             : (int64_t)item * coef_stride);
+  double* c = coef + item_at(L, item, kpd, coef_stride, 0, 0).coef;
   if (m == 0) {
     c[n * n + n] = ac;
   } else {
@@ -419,11 +440,10 @@ __global__ void k_analysis_legendre(const double* __restrict__ F, int p, int q,
   }
 }
 
-int sht_analysis(shbim_ctx* ctx, const GridTables& g, int n_items, const double* vals,
-                 int64_t val_stride, bool weighted, double* coef, int64_t coef_stride,
-                 cudaStream_t s, int kpd, const DropList* L) {
-  if (n_items <= 0) return SHBIM_OK;
-  const DropList list = L ? *L : DropList{};
+namespace {
+template <class List>
+int analysis(shbim_ctx* ctx, const GridTables& g, int n_items, const double* vals, int64_t val_stride, bool weighted,
+             double* coef, int64_t coef_stride, cudaStream_t s, int kpd, const List& list) {
   const size_t need = (size_t)n_items * (g.q + 1) * 2 * (g.p + 1);
   if (need > ctx->sht_scratch_elems) {
     // growing scratch: wait for queued users of the old buffer before freeing it
@@ -443,20 +463,52 @@ int sht_analysis(shbim_ctx* ctx, const GridTables& g, int n_items, const double*
     const int rows = std::max(1, std::min(8, budget / (2 * N)));
     const int64_t nrows = (int64_t)n_items * (g.q + 1);
     const size_t smem = (size_t)(2 * N + rows * 2 * N) * sizeof(double);
-    k_analysis_fourier4<<<(unsigned)((nrows + rows - 1) / rows), 128, smem, s>>>(
+    k_analysis_fourier4<List><<<(unsigned)((nrows + rows - 1) / rows), 128, smem, s>>>(
         vals, val_stride, g.p, g.q, g.trig, g.omega, weighted ? 1 : 0, nrows, rows, ctx->sht_scratch, kpd, list);
     SHBIM_CHECK_LAUNCH(ctx, "k_analysis_fourier4");
   } else {
     dim3 g1(n_items, g.q + 1);
-    k_analysis_fourier<<<g1, 64, 3 * N * sizeof(double), s>>>(vals, val_stride, g.p, g.q, g.trig,
+    k_analysis_fourier<List><<<g1, 64, 3 * N * sizeof(double), s>>>(vals, val_stride, g.p, g.q, g.trig,
                                                               g.omega, weighted ? 1 : 0,
                                                               ctx->sht_scratch, kpd, list);
     SHBIM_CHECK_LAUNCH(ctx, "k_analysis_fourier");
   }
   const int nt = ntri(g.p);
   dim3 g2(n_items, (nt + 127) / 128);
-  k_analysis_legendre<<<g2, 128, 0, s>>>(ctx->sht_scratch, g.p, g.q, g.alf, coef, coef_stride, kpd, list);
+  k_analysis_legendre<List><<<g2, 128, 0, s>>>(ctx->sht_scratch, g.p, g.q, g.alf, coef, coef_stride, kpd, list);
   SHBIM_CHECK_LAUNCH(ctx, "k_analysis_legendre");
+  return SHBIM_OK;
+}
+}  // namespace
+
+int sht_analysis(shbim_ctx* ctx, const GridTables& g, int n_items, const double* vals,
+                 int64_t val_stride, bool weighted, double* coef, int64_t coef_stride,
+                 cudaStream_t s, int kpd, const DropList* L) {
+  if (n_items <= 0) return SHBIM_OK;
+  return analysis(ctx, g, n_items, vals, val_stride, weighted, coef, coef_stride, s, kpd, L ? *L : DropList{});
+}
+
+// Transforms of n single fields on one degree's grid, each at its own place: as many launches as kMaxFields asks for.
+// One launch per drop and direction is what fields of many drops cost otherwise (16 drops of four degrees, three
+// fields each, both ways: 48 launches, 0.70 ms; 12 launches, 0.23 ms so).
+int sht_fields(shbim_ctx* ctx, const GridTables& g, bool forward, int n, const int64_t* coef_off, const int64_t* val_off,
+               const double* in, double* out, cudaStream_t s) {
+  const size_t smem = (size_t)(2 * (g.p + 1) + 3 * (2 * g.q + 2)) * sizeof(double);
+  if (!forward)
+    if (int rc = synth_smem_ok(ctx, smem)) return rc;
+  for (int f = 0; f < n; f += kMaxFields) {
+    const int m = std::min(kMaxFields, n - f);
+    FieldList L{};
+    std::copy(coef_off + f, coef_off + f + m, L.coef);
+    std::copy(val_off + f, val_off + f + m, L.val);
+    if (forward) {
+      if (int rc = analysis(ctx, g, m, in, 0, true, out, 0, s, 1, L)) return rc;
+    } else {
+      k_synth<FieldList><<<dim3(m, g.q + 1), 128, smem, s>>>(in, 0, g.p, g.q, g.alf, g.trig, 1, out, 0, 0, nullptr, 1.0,
+                                                             nullptr, nullptr, 1, 0, nullptr, L);
+      SHBIM_CHECK_LAUNCH(ctx, "k_synth");
+    }
+  }
   return SHBIM_OK;
 }
 
