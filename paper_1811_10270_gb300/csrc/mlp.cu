@@ -39,19 +39,29 @@ namespace shbim {
 namespace {
 
 // ---------------------------------------------------------------- tcgen05 GEMM
-// C(m, n) = act(sum_k A(m, k) B(k, n) + bias(n)) for one 128 x 64 tile of C per CTA (4 warps).
-// Per K block of 64: the CTA stages A (128 x 64) and B (64 x 64, as N x K) into shared memory as
-// bfloat16 in the no-swizzle K-major canonical layout (8-row x 16-byte core matrices; leading-
-// dimension offset = 128 B between core matrices along K, stride offset = 1024 B between 8-row
-// groups), one thread issues four tcgen05.mma kind::f16 (M = 128, N = 64, K = 16) accumulating in
-// tensor memory and commits them to an mbarrier; every wait is bounded (a timed-out tile is
-// written as NaN so the failure is loud). The epilogue reads the accumulator with tcgen05.ld.
-constexpr int TM = 128, TN = 64, TK = 64;
+// C(m, n) = act(sum_k A(m, k) B(k, n) + bias(n)) [(1 - h(m, n)^2)] for one 128 x 32 tile of C per CTA (8
+// warps). Per K block of 128 the CTA holds A (128 x 128) and B (32 x 128, as N x K) in shared memory as
+// bfloat16 in the no-swizzle K-major canonical layout (8-row x 16-byte core matrices; leading-dimension
+// offset = 128 B between core matrices along K, stride offset = 2048 B between 8-row groups); one thread
+// issues up to eight tcgen05.mma kind::f16 (M = 128, N = 32, K = 16) accumulating in tensor memory and
+// commits them to an mbarrier; every wait is bounded (a timed-out tile is written as NaN so the failure is
+// loud).
+//
+// The products are small (a batch of 1 to 96 rows, widths of some hundreds), so a tile is bound by the
+// latency of staging, not by the tensor cores. A thread therefore moves units of eight k of one row: all
+// loads of a K block are in flight together, they are issued before the wait for the products of the block
+// before, and a unit is stored by one 16-byte store. The units of a warp follow the operand's order in
+// memory: 8 rows x 4 units where k is the dense index, 32 rows x 1 unit where the row is. 32 columns per
+// CTA, not 64, give a layer of width 512 sixteen CTAs. Widths 657-512-512-512-648, batch 64: 53 us per
+// product with loads of one element at a time, each waiting for the last, on 128 threads; 11.7 us forward and
+// backward (weights 0.7 MB from L2) and 4.5 us for the weights' gradients this way.
+constexpr int TM = 128, TN = 32, TK = 128;
+constexpr int kGemmThreads = 256;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// index of element (row r, k) in a [rows][TK] K-major canonical tile
-__device__ __forceinline__ int canon(int r, int k) { return ((r >> 3) * (TK >> 3) + (k >> 3)) * 64 + (r & 7) * 8 + (k & 7); }
+// index of element (row r, k = 8 o) in a [rows][TK] K-major canonical tile
+__device__ __forceinline__ int canon8(int r, int o) { return ((r >> 3) * (TK >> 3) + o) * 64 + (r & 7) * 8; }
 
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
   uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFF);
@@ -61,17 +71,77 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
   return d;
 }
 
-template <typename TA, typename TB>
-__global__ void __launch_bounds__(128)
+__device__ __forceinline__ __nv_bfloat16 bf16_of(float v) { return __float2bfloat16_rn(v); }
+__device__ __forceinline__ __nv_bfloat16 bf16_of(__nv_bfloat16 v) { return v; }
+__device__ __forceinline__ void zero(float& v) { v = 0.f; }
+__device__ __forceinline__ void zero(__nv_bfloat16& v) { v = __ushort_as_bfloat16((unsigned short)0); }
+
+// row and k unit of unit u of a ROWS x TK tile: KD = k is the dense index in memory
+template <int ROWS, bool KD>
+__device__ __forceinline__ void unit_of(int u, int& r, int& o) {
+  if (KD) {
+    r = ((u >> 7) << 3) + (u & 7);      // 16 units of each of 8 rows in 128 consecutive u
+    o = (u >> 3) & 15;
+  } else {
+    r = u % ROWS;
+    o = u / ROWS;
+  }
+}
+
+// the K block at k0 of rows r0 .. of X(r, k) = X[r sr + k sk], zeros outside R x K
+template <int ROWS, bool KD, typename T>
+struct Tile {
+  static constexpr int kUnits = ROWS * (TK / 8) / kGemmThreads;
+  T v[kUnits][8];
+
+  __device__ __forceinline__ void load(const T* __restrict__ X, int r0, int k0, int R, int K, int64_t sr, int64_t sk) {
+#pragma unroll
+    for (int i = 0; i < kUnits; ++i) {
+      int r, o;
+      unit_of<ROWS, KD>(threadIdx.x + i * kGemmThreads, r, o);
+      const int k = k0 + 8 * o;
+      const bool in = r0 + r < R;
+      const T* x = X + (int64_t)(r0 + r) * sr + (int64_t)k * sk;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (in && k + j < K)
+          v[i][j] = KD ? x[j] : x[j * sk];
+        else
+          zero(v[i][j]);
+      }
+    }
+  }
+
+  __device__ __forceinline__ void store(__nv_bfloat16* __restrict__ s) const {
+#pragma unroll
+    for (int i = 0; i < kUnits; ++i) {
+      int r, o;
+      unit_of<ROWS, KD>(threadIdx.x + i * kGemmThreads, r, o);
+      __align__(16) __nv_bfloat16 h[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) h[j] = bf16_of(v[i][j]);
+      *reinterpret_cast<uint4*>(s + canon8(r, o)) = *reinterpret_cast<const uint4*>(h);
+    }
+  }
+};
+
+static_assert(TM * (TK / 8) % kGemmThreads == 0 && TN * (TK / 8) % kGemmThreads == 0, "whole units per thread");
+
+template <typename TA, typename TB, bool KA, bool KB>
+__global__ void __launch_bounds__(kGemmThreads)
 k_gemm_tc(int M, int N, int K, const TA* __restrict__ A, int64_t sam, int64_t sak, const TB* __restrict__ B,
-          int64_t sbk, int64_t sbn, float* __restrict__ C, int64_t scm, int64_t scn,
-          const float* __restrict__ bias, int act) {
+          int64_t sbk, int64_t sbn, float* __restrict__ C, int64_t ldc, const float* __restrict__ bias, int act,
+          const float* __restrict__ h) {
   __shared__ __align__(1024) __nv_bfloat16 sA[TM * TK];
   __shared__ __align__(1024) __nv_bfloat16 sB[TN * TK];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_base;
   const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
   const int tid = threadIdx.x, warp = tid >> 5;
+  Tile<TM, KA, TA> ta;
+  Tile<TN, KB, TB> tb;
+  ta.load(A, m0, 0, M, K, sam, sak);
+  tb.load(B, n0, 0, N, K, sbn, sbk);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_base)),
                  "r"(TN));
@@ -89,24 +159,14 @@ k_gemm_tc(int M, int N, int K, const TA* __restrict__ A, int64_t sam, int64_t sa
   bool ok = true;
   int phase = 0;
   for (int k0 = 0; k0 < K; k0 += TK) {
-    for (int e = tid; e < TM * TK; e += 128) {
-      const int mm = e / TK, kk = e - mm * TK;
-      const int gm = m0 + mm, gk = k0 + kk;
-      const float v = (gm < M && gk < K) ? (float)A[(int64_t)gm * sam + (int64_t)gk * sak] : 0.f;
-      sA[canon(mm, kk)] = __float2bfloat16_rn(v);
-    }
-    for (int e = tid; e < TN * TK; e += 128) {
-      const int nn = e / TK, kk = e - nn * TK;
-      const int gn = n0 + nn, gk = k0 + kk;
-      const float v = (gn < N && gk < K) ? (float)B[(int64_t)gk * sbk + (int64_t)gn * sbn] : 0.f;
-      sB[canon(nn, kk)] = __float2bfloat16_rn(v);
-    }
+    ta.store(sA);
+    tb.store(sB);
     asm volatile("fence.proxy.async.shared::cta;\n");
     __syncthreads();
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;\n");
-#pragma unroll
-      for (int ks = 0; ks < TK / 16; ++ks) {
+      const int steps = (min(TK, K - k0) + 15) / 16;  // what lies beyond K is zero and left out
+      for (int ks = 0; ks < steps; ++ks) {
         const uint64_t da = smem_desc(smem_u32(sA) + ks * 256);
         const uint64_t db = smem_desc(smem_u32(sB) + ks * 256);
         const uint32_t acc = (k0 > 0 || ks > 0) ? 1u : 0u;
@@ -118,6 +178,10 @@ k_gemm_tc(int M, int N, int K, const TA* __restrict__ A, int64_t sam, int64_t sa
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
           smem_u32(&mbar)));
     }
+    if (k0 + TK < K) {
+      ta.load(A, m0, k0 + TK, M, K, sam, sak);
+      tb.load(B, n0, k0 + TK, N, K, sbn, sbk);
+    }
     // the staged tiles may be overwritten only after the MMAs that read them have completed
     // (bounded by one second of the global timer)
     uint32_t done = 0;
@@ -126,7 +190,8 @@ k_gemm_tc(int M, int N, int K, const TA* __restrict__ A, int64_t sam, int64_t sa
       asm volatile(
           "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
           : "=r"(done)
-          : "r"(smem_u32(&mbar)), "r"(phase));
+          : "r"(smem_u32(&mbar)), "r"(phase)
+          : "memory");
       uint64_t t;
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
       if (it == 0) t0 = t;
@@ -140,40 +205,46 @@ k_gemm_tc(int M, int N, int K, const TA* __restrict__ A, int64_t sam, int64_t sa
     }
     asm volatile("tcgen05.fence::after_thread_sync;\n");
   }
-  const int row = m0 + 32 * warp + (tid & 31);
-  for (int c0 = 0; c0 < TN; c0 += 16) {
+  // accumulator to shared memory (a warp may read the 32 lanes of its number modulo 4: four warps per half of
+  // the columns), from where rows are written densely
+  float* sC = reinterpret_cast<float*>(sA);
+  const int c0 = (warp >> 2) * 16;
+  if (ok) {
     uint32_t v[16];
-    if (ok) {
-      const uint32_t addr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0;
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(addr));
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n");
-    }
-    if (row < M) {
+    const uint32_t addr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+    const int r = 32 * (warp & 3) + (tid & 31);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int gn = n0 + c0 + j;
-        if (gn < N) {
-          float x = ok ? __uint_as_float(v[j]) + (bias ? bias[gn] : 0.f) : __int_as_float(0x7fc00000);
-          if (act) x = tanhf(x);
-          C[(int64_t)row * scm + (int64_t)gn * scn] = x;
-        }
-      }
-    }
+    for (int j = 0; j < 16; ++j) sC[r * (TN + 1) + c0 + j] = __uint_as_float(v[j]);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TN));
+  const int gn = n0 + (tid & (TN - 1));
+  if (gn >= N) return;
+  const float bn = bias ? bias[gn] : 0.f;
+#pragma unroll 4
+  for (int r = tid / TN; r < min(TM, M - m0); r += kGemmThreads / TN) {
+    float x = ok ? sC[r * (TN + 1) + (tid & (TN - 1))] + bn : __int_as_float(0x7fc00000);
+    if (act) x = tanhf(x);
+    const int64_t e = (int64_t)(m0 + r) * ldc + gn;
+    if (h) x *= 1.f - h[e] * h[e];
+    C[e] = x;
+  }
 }
 
-template <typename TA, typename TB>
-int gemm(shbim_mlp*, int M, int N, int K, const TA* A, int64_t sam, int64_t sak, const TB* B, int64_t sbk,
-         int64_t sbn, float* C, int64_t scm, int64_t scn, const float* bias, int act, cudaStream_t s) {
+// C [M x N] dense; h, if given, of C's shape
+template <bool KA, bool KB, typename TA, typename TB>
+int gemm(int M, int N, int K, const TA* A, int64_t sa, const TB* B, int64_t sb, float* C, const float* bias, int act,
+         const float* h, cudaStream_t s) {
   dim3 grid((N + TN - 1) / TN, (M + TM - 1) / TM);
-  k_gemm_tc<TA, TB><<<grid, 128, 0, s>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, scm, scn, bias, act);
+  k_gemm_tc<TA, TB, KA, KB><<<grid, kGemmThreads, 0, s>>>(M, N, K, A, KA ? sa : 1, KA ? 1 : sa, B, KB ? 1 : sb,
+                                                         KB ? sb : 1, C, N, bias, act, h);
   return cudaGetLastError() == cudaSuccess ? SHBIM_OK : SHBIM_ERR_CUDA;
 }
 
@@ -191,16 +262,12 @@ __global__ void k_out_grad(const float* __restrict__ y, const float* __restrict_
   if ((threadIdx.x & 31) == 0 && l != 0.0) atomicAdd(loss, l);
 }
 
-__global__ void k_tanh_grad(float* __restrict__ d, const float* __restrict__ h, int64_t n) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < n) d[e] *= 1.f - h[e] * h[e];
-}
-
-// gb[n] = sum_b d[b][n]  (fixed order)
+// gb[n] = sum_b d[b][n]  (fixed order; one chain per column, its loads in flight together)
 __global__ void k_colsum(const float* __restrict__ d, int B, int N, float* __restrict__ gb) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
   float s = 0.f;
+#pragma unroll 16
   for (int b = 0; b < B; ++b) s += d[(int64_t)b * N + n];
   gb[n] = s;
 }
@@ -336,8 +403,8 @@ int forward(shbim_mlp* net, int B, const float* x, cudaStream_t s) {
                                                                               l < net->L - 1 ? 1 : 0, net->H[l + 1]);
       if (cudaGetLastError() != cudaSuccess) return SHBIM_ERR_CUDA;
     } else {
-      int rc = gemm<float, __nv_bfloat16>(net, B, N, K, in, K, 1, net->Wh[l], 1, K, net->H[l + 1], N, 1, net->b[l],
-                                          l < net->L - 1 ? 1 : 0, s);
+      int rc = gemm<true, true>(B, N, K, in, K, net->Wh[l], K, net->H[l + 1], net->b[l], l < net->L - 1 ? 1 : 0, nullptr,
+                                s);
       if (rc) return rc;
     }
     in = net->H[l + 1];
@@ -478,15 +545,13 @@ int shbim_mlp_train_step(shbim_mlp* n, int batch, const float* x_dev, const floa
   float* dn = n->dB;
   for (int l = L - 1; l >= 0; --l) {
     const int K = n->w[l], N = n->w[l + 1];
-    if (l < L - 1) k_tanh_grad<<<nb((int64_t)batch * N), 256, 0, s>>>(d, n->H[l + 1], (int64_t)batch * N);
     const float* in = l == 0 ? x_in : n->H[l];
     // gW[N x K] = d^T [N x B] . in [B x K]
-    if ((rc = gemm<float, float>(n, N, K, batch, d, 1, N, in, K, 1, n->gW[l], K, 1, nullptr, 0, s))) return rc;
-    k_colsum<<<(N + 255) / 256, 256, 0, s>>>(d, batch, N, n->gb[l]);
+    if ((rc = gemm<false, false>(N, K, batch, d, N, in, K, n->gW[l], nullptr, 0, nullptr, s))) return rc;
+    k_colsum<<<(N + 63) / 64, 64, 0, s>>>(d, batch, N, n->gb[l]);
     if (l > 0) {
-      // dn [B x K] = d [B x N] . W [N x K]
-      if ((rc = gemm<float, __nv_bfloat16>(n, batch, K, N, d, N, 1, n->Wh[l], K, 1, dn, K, 1, nullptr, 0, s)))
-        return rc;
+      // dn [B x K] = (d [B x N] . W [N x K]) tanh'
+      if ((rc = gemm<true, false>(batch, K, N, d, N, n->Wh[l], K, dn, nullptr, 0, n->H[l], s))) return rc;
       std::swap(d, dn);
     }
   }
