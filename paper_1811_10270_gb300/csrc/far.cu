@@ -1104,7 +1104,7 @@ int upload_tables(shbim_ctx* ctx) {
 // issue slots per instruction), by kind DL, SL, S + D, S, D
 constexpr double kDirect32[5] = {25.0, 18.0, 45.0, 35.0, 37.0};
 constexpr double kDirectDf[5] = {121.0, 78.0, 260.0, 187.0, 195.0};
-constexpr double kDirect64[5] = {1400.0, 1030.0, 2600.0, 2130.0, 1940.0};
+constexpr double kDirect64[5] = {1060.0, 740.0, 1980.0, 1540.0, 1470.0};
 constexpr int kSets[5] = {3, 1, 12, 12, 12};
 constexpr int kCharges[5] = {1, 1, 13, 4, 9};
 // derivatives taken of 1/r in the truncation bound
@@ -1327,17 +1327,18 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
   return SHBIM_OK;
 }
 
-// The estimate in FP32 instructions of the expansions' inner steps (doubled for latency and reads, plus 75 us of
-// launches and short kernels) against the direct sums they replace. 40 drops of degree 11, single layer in double-float
-// (5.2e8 pairs): 1.80 ms directly, 1.11 with expansions; six drops of degree 16 in FP64 (4e7): 2.4 and 2.2 ms per
-// application; two drops, or 1e8 pairs in FP32, stay direct.
+// The estimate in FP32 instructions of the expansions' inner steps (half as much again for latency and reads, twice
+// in FP64, plus 75 us of launches and short kernels) against the direct sums they replace. 40 drops of degree 11,
+// single layer in double-float (5.2e8 pairs): 1.48 ms directly, 1.03 with expansions; six drops of degree 16 in
+// FP64 (4e7 pairs, a third far), eight applications: 14.2 ms directly, 16.9 with expansions, and left direct; two
+// drops, or 1e8 pairs in FP32, stay direct.
 bool far_worth(const FarPlan& P, int precision, int kind) {
   const double* direct = precision == SHBIM_PREC_FP32_COMP ? kDirect32 : (precision == SHBIM_PREC_DF64 ? kDirectDf : kDirect64);
   const double unit = precision == SHBIM_PREC_FP64 ? 64.0 / 12.0 : 1.0;
   const int npot = stokes_like(kind) ? 4 : 1;
   const double cost = unit * (P.src_work * (45.0 + 26.0 * kCharges[kind]) + P.tgt_work * (30.0 + 26.0 * kSets[kind]) +
                               P.pair_work * npot * 30.0);
-  return P.npairs > 0 && 1.5 * cost + 3e9 < P.far_pairs * direct[kind];
+  return P.npairs > 0 && (precision == SHBIM_PREC_FP64 ? 2.0 : 1.5) * cost + 3e9 < P.far_pairs * direct[kind];
 }
 
 const FarPlan* far_plan(const shbim_ctx* ctx, int kind) {

@@ -20,6 +20,7 @@
 
 #include "dfloat.cuh"
 #include "internal.h"
+#include "inv64.cuh"
 #include "pair_df.cuh"
 
 namespace shbim {
@@ -175,27 +176,29 @@ __device__ void near_sum64(const double* __restrict__ pos, int64_t stride, const
   double a[3] = {0.0, 0.0, 0.0};
   for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
     const double dx = x0[0] - pos[e], dy = x0[1] - pos[stride + e], dz = x0[2] - pos[2 * stride + e];
-    const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
+    const double r2 = dx * dx + dy * dy + dz * dz;
     if (KIND == 1) {
-      a[0] = fma(str[e], ri, a[0]);
+      a[0] = fma(str[e], inv_r(r2), a[0]);
     } else if (KIND == 0) {
-      a[0] = fma(str[e] * ri * ri * ri, dx * nv[0] + dy * nv[1] + dz * nv[2], a[0]);
+      a[0] = fma(str[e] * inv_r3(r2), dx * nv[0] + dy * nv[1] + dz * nv[2], a[0]);
     } else {
-      const double ri2 = ri * ri, ri3 = ri2 * ri;
-      double t = 0.0;
+      double hh = 0.0;
       if (KIND != 3) {
         const double hu = dx * str[3 * sstride + e] + dy * str[4 * sstride + e] + dz * str[5 * sstride + e];
         const double hn = dx * pos[3 * stride + e] + dy * pos[4 * stride + e] + dz * pos[5 * stride + e];
-        t = hu * hn * ri2;
+        hh = hu * hn;
       }
       if (KIND != 4) {
+        const double ri = inv_r(r2), ri2 = ri * ri;
         const double fx = str[e], fy = str[sstride + e], fz = str[2 * sstride + e];
-        t = ri3 * (dx * fx + dy * fy + dz * fz + t);
+        double t = dx * fx + dy * fy + dz * fz;
+        if (KIND == 2) t = fma(hh, ri2, t);
+        t *= ri2 * ri;
         a[0] += fx * ri + dx * t;
         a[1] += fy * ri + dy * t;
         a[2] += fz * ri + dz * t;
       } else {
-        t *= ri3;
+        const double t = hh * inv_r5(r2);
         a[0] += dx * t;
         a[1] += dy * t;
         a[2] += dz * t;

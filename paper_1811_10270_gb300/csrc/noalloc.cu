@@ -12,6 +12,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "inv64.cuh"
 
 namespace shbim {
 namespace {
@@ -76,12 +77,12 @@ k_pairs_noalloc(const double* __restrict__ tgt, int64_t nt, const double* __rest
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const double dx = X[k][0] - sh[0][e], dy = X[k][1] - sh[1][e], dz = X[k][2] - sh[2][e];
-        const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
+        const double r2 = dx * dx + dy * dy + dz * dz;
         if (KIND == 1) {
-          acc[k] = fma(sh[3][e], ri, acc[k]);
+          acc[k] = fma(sh[3][e], inv_r(r2), acc[k]);
         } else {
           const double dn = dx * Nn[k][0] + dy * Nn[k][1] + dz * Nn[k][2];
-          acc[k] = fma(sh[3][e] * ri * ri * ri, dn, acc[k]);
+          acc[k] = fma(sh[3][e] * inv_r3(r2), dn, acc[k]);
         }
       }
     }

@@ -30,6 +30,7 @@
 #include "dfloat.cuh"
 #include "far.h"
 #include "internal.h"
+#include "inv64.cuh"
 #include "pair_df.cuh"
 #include "pair_dq.cuh"
 
@@ -549,28 +550,31 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
         for (int k = 0; k < kTPT; ++k) {
           const double dx = X0[k][0] - sx, dy = X0[k][1] - sy, dz = X0[k][2] - sz;
           const double r2 = dx * dx + dy * dy + dz * dz;
-          const double ri = rsqrt(r2);
           if (KIND == LSL) {
-            acc[k][0] = fma(sh[3][e], ri, acc[k][0]);
+            acc[k][0] = fma(sh[3][e], inv_r(r2), acc[k][0]);
           } else if (KIND == LDL) {
             const double dn = dx * N0[k][0] + dy * N0[k][1] + dz * N0[k][2];
-            acc[k][0] = fma(sh[3][e] * ri * ri * ri, dn, acc[k][0]);
+            acc[k][0] = fma(sh[3][e] * inv_r3(r2), dn, acc[k][0]);
+          } else if (KIND == STD) {
+            const double hu = dx * sh[6][e] + dy * sh[7][e] + dz * sh[8][e];
+            const double hn = dx * sh[9][e] + dy * sh[10][e] + dz * sh[11][e];
+            const double t = hu * hn * inv_r5(r2);
+            acc[k][0] += dx * t;
+            acc[k][1] += dy * t;
+            acc[k][2] += dz * t;
           } else {
-            const double ri2 = ri * ri, ri3 = ri2 * ri;
+            const double ri = inv_r(r2), ri2 = ri * ri;
             const double fx = sh[3][e], fy = sh[4][e], fz = sh[5][e];
-            const double hf = KIND == STD ? 0.0 : dx * fx + dy * fy + dz * fz;
-            const double hu = KIND == STS ? 0.0 : dx * sh[6][e] + dy * sh[7][e] + dz * sh[8][e];
-            const double hn = KIND == STS ? 0.0 : dx * sh[9][e] + dy * sh[10][e] + dz * sh[11][e];
-            const double t = ri3 * (hf + hu * hn * ri2);
-            if (KIND == STD) {
-              acc[k][0] += dx * t;
-              acc[k][1] += dy * t;
-              acc[k][2] += dz * t;
-            } else {
-              acc[k][0] += fx * ri + dx * t;
-              acc[k][1] += fy * ri + dy * t;
-              acc[k][2] += fz * ri + dz * t;
+            double t = dx * fx + dy * fy + dz * fz;
+            if (KIND == STO) {
+              const double hu = dx * sh[6][e] + dy * sh[7][e] + dz * sh[8][e];
+              const double hn = dx * sh[9][e] + dy * sh[10][e] + dz * sh[11][e];
+              t = fma(hu * hn, ri2, t);
             }
+            t *= ri2 * ri;
+            acc[k][0] += fx * ri + dx * t;
+            acc[k][1] += fy * ri + dy * t;
+            acc[k][2] += fz * ri + dz * t;
           }
         }
       }
