@@ -21,26 +21,39 @@ int cuda_fail(shbim_ctx* ctx, cudaError_t e, const char* what) {
 
 int pairs_tile_targets();
 
+// drop centres into the drop table and centres[3 i + c]
+__global__ void k_centres(const double* __restrict__ x, int nd, double s4pi, DropDev* __restrict__ drops,
+                          double* __restrict__ centres) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nd) return;
+  const double* c = x + 3 * drops[i].coef_off;
+  const int64_t nc = drops[i].nc;
+  drops[i].cx = centres[3 * i] = c[0] / s4pi;
+  drops[i].cy = centres[3 * i + 1] = c[nc] / s4pi;
+  drops[i].cz = centres[3 * i + 2] = c[2 * nc] / s4pi;
+}
+
 // Shape-dependent state for the current layout: drop centres (x_00 / sqrt(4 pi), the mean
 // position over the parameter sphere), the device drop table, geometry and singular rows.
 int rebuild_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
-  SHBIM_CUDA(ctx, cudaStreamSynchronize(s));
   ctx->geom_version++;  // invalidates captured operator graphs
   ctx->xcoef_cur = xcoef_dev;
-  for (auto& d : ctx->drops) {
-    double c00[3];
-    for (int c = 0; c < 3; ++c)
-      SHBIM_CUDA(ctx, cudaMemcpy(&c00[c], xcoef_dev + 3 * d.coef_off + (int64_t)c * d.nc, sizeof(double),
-                                 cudaMemcpyDeviceToHost));
-    for (int c = 0; c < 3; ++c) d.centre[c] = c00[c] / std::sqrt(4.0 * kPi);
-  }
   std::vector<DropDev> dd(ctx->n_drops);
   for (int i = 0; i < ctx->n_drops; ++i) {
     const Drop& d = ctx->drops[i];
     dd[i] = DropDev{d.p, d.q, d.nt, d.ns, d.nc, d.coef_off, d.tgt_off, d.src_off, d.lam,
-                    d.centre[0], d.centre[1], d.centre[2], d.rows_lap, d.rows_sto, d.pad_off};
+                    0.0, 0.0, 0.0, d.rows_lap, d.rows_sto, d.pad_off};
   }
-  SHBIM_CUDA(ctx, cudaMemcpy(ctx->drops_dev, dd.data(), dd.size() * sizeof(DropDev), cudaMemcpyHostToDevice));
+  SHBIM_CUDA(ctx, cudaMemcpyAsync(ctx->drops_dev, dd.data(), dd.size() * sizeof(DropDev), cudaMemcpyHostToDevice, s));
+  // the centres in one launch and one read-back, however many drops there are (a copy takes about 10 us)
+  std::vector<double> c3(3 * (size_t)ctx->n_drops);
+  k_centres<<<(unsigned)((ctx->n_drops + 127) / 128), 128, 0, s>>>(xcoef_dev, ctx->n_drops, std::sqrt(4.0 * kPi),
+                                                                  ctx->drops_dev, ctx->centres_dev);
+  SHBIM_CHECK_LAUNCH(ctx, "k_centres");
+  SHBIM_CUDA(ctx, cudaMemcpyAsync(c3.data(), ctx->centres_dev, c3.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+  SHBIM_CUDA(ctx, cudaStreamSynchronize(s));
+  for (int i = 0; i < ctx->n_drops; ++i)
+    for (int c = 0; c < 3; ++c) ctx->drops[i].centre[c] = c3[3 * i + c];
   int rc;
   if ((rc = build_geometry(ctx, xcoef_dev, s))) return rc;
   if ((rc = build_pair_lists(ctx, s))) return rc;
@@ -72,6 +85,8 @@ void free_drop_state(shbim_ctx* ctx) {
   ctx->tiles_dev = nullptr;
   cudaFree(ctx->drops_dev);
   ctx->drops_dev = nullptr;
+  cudaFree(ctx->centres_dev);
+  ctx->centres_dev = nullptr;
   cudaFree(ctx->lamm1_dev);
   ctx->lamm1_dev = nullptr;
   cudaFree(ctx->prec_basis);
@@ -211,6 +226,7 @@ int shbim_destroy(shbim_ctx* ctx) {
     cudaFree(L.rexp);
   }
   cudaFree(ctx->tc_err);
+  cudaFree(ctx->geo_tmp);
   cudaFree(ctx->gm.xr);
   cudaFree(ctx->gm.rr);
   cudaFree(ctx->gm.dr);
@@ -355,11 +371,15 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
   if (same) {
     // same layout: keep every allocation, refresh the shape-dependent state only
     std::vector<double> lm1(n_drops);
+    bool moved = false;
     for (int i = 0; i < n_drops; ++i) {
-      ctx->drops[i].lam = lambda_host ? lambda_host[i] : 1.0;
-      lm1[i] = ctx->drops[i].lam - 1.0;
+      const double lam = lambda_host ? lambda_host[i] : 1.0;
+      moved = moved || lam != ctx->drops[i].lam;
+      ctx->drops[i].lam = lam;
+      lm1[i] = lam - 1.0;
     }
-    SHBIM_CUDA(ctx, cudaMemcpy(ctx->lamm1_dev, lm1.data(), n_drops * sizeof(double), cudaMemcpyHostToDevice));
+    if (moved || !ctx->lamm1_dev)
+      SHBIM_CUDA(ctx, cudaMemcpy(ctx->lamm1_dev, lm1.data(), n_drops * sizeof(double), cudaMemcpyHostToDevice));
     return rebuild_geometry(ctx, xcoef_dev, s);
   }
   free_drop_state(ctx);
@@ -463,7 +483,9 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
       std::fill(tdrop.begin() + ctx->drops[i].tgt_off,
                 tdrop.begin() + ctx->drops[i].tgt_off + ctx->drops[i].nt, i);
     SHBIM_CUDA(ctx, cudaMemcpy(ctx->geo.tgt_drop, tdrop.data(), to * sizeof(int), cudaMemcpyHostToDevice));
-    if ((rc = dalloc(ctx, &ctx->drops_dev, n_drops, "drop table"))) return rc;
+    if ((rc = dalloc(ctx, &ctx->drops_dev, n_drops, "drop table")) ||
+        (rc = dalloc(ctx, &ctx->centres_dev, 3 * (size_t)n_drops, "drop centres")))
+      return rc;
     std::vector<double> lm1(n_drops);
     for (int i = 0; i < n_drops; ++i) lm1[i] = ctx->drops[i].lam - 1.0;
     if ((rc = dalloc(ctx, &ctx->lamm1_dev, n_drops, "viscosity contrasts"))) return rc;

@@ -277,6 +277,147 @@ __global__ void k_xupdate_k(double* __restrict__ x, const double* __restrict__ V
 // maps those outlying eigenvalues to 1 and the cluster near 1 (P_i is the same form with the inverse
 // factors). GMRES iterates y = P x and applies A P^{-1}; the solution is x = P^{-1} y.
 
+// One drop per block: the translations e_k (constant fields, coefficient sqrt(4 pi) on Y_00), the rotations
+// e_k x x (from the position coefficients) and the parameter sphere's radial field r^ (degree 1),
+// orthonormalised in that order in FP64; factors from the drop's viscosity ratio.
+// The translations are unit vectors of the Y_00 coefficients, and what they project out of the others is just those.
+// The other four take the Cholesky factor of their Gram matrix, twice (CholeskyQR2: orthonormal to rounding where the
+// condition is below 1e7): two reductions instead of 21. Where a pivot has lost six digits the vectors go through
+// Gram-Schmidt one by one (twice), which also finds shapes without a basis. Bound by the latency of FP64 reductions:
+// 126 us with Gram-Schmidt throughout, 35 us so at degree 16; on the host it took 0.07 ms for a drop of degree 16
+// and 1 ms for one of degree 64, one drop after the other, with the GPU waiting.
+constexpr int kPrecThreads = 256;
+__global__ void __launch_bounds__(kPrecThreads)
+k_prec_basis(const double* __restrict__ x, const DropDev* __restrict__ drops, double* __restrict__ basis,
+             double* __restrict__ fac, int* __restrict__ bad) {
+  __shared__ double red[10][kPrecThreads / 32], tot[10];
+  const DropDev D = drops[blockIdx.x];
+  const int nc = D.nc, n3 = 3 * nc;
+  const double* xc = x + 3 * D.coef_off;
+  double* b = basis + 21 * D.coef_off;
+  const double s4pi3 = 2.0466534158929769770;    // sqrt(4 pi / 3)
+  // entry e of vector k; a thread reads and writes its own entries only
+  auto start = [&](int k, int e) {
+    const int c = e / nc, j = e - c * nc;
+    if (k < 3) return c == k && j == 0 ? 1.0 : 0.0;
+    if (j == 0) return 0.0;
+    if (k == 6)   // radial field: x on the (1, 1), y on the (1, -1) and z on the (1, 0) harmonic
+      return c == 0 && j == 3 ? -s4pi3 : (c == 1 && j == 1 ? -s4pi3 : (c == 2 && j == 2 ? s4pi3 : 0.0));
+    // (e_k x x)_{k1} = -x_{k2}, (e_k x x)_{k2} = x_{k1}
+    const int r = k - 3, k1 = (r + 1) % 3, k2 = (r + 2) % 3;
+    return c == k1 ? -xc[k2 * nc + j] : (c == k2 ? xc[k1 * nc + j] : 0.0);
+  };
+  for (int e = threadIdx.x; e < n3; e += kPrecThreads)
+#pragma unroll
+    for (int k = 0; k < 7; ++k) b[k * n3 + e] = start(k, e);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // sums over the block of a[0 .. n) into tot
+  auto sums = [&](const double (&a)[10], int n) {
+    __syncthreads();
+#pragma unroll
+    for (int l = 0; l < 10; ++l) {
+      if (l >= n) break;
+      double v = a[l];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) red[l][warp] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < n) {
+      double v = 0.0;
+#pragma unroll
+      for (int w = 0; w < kPrecThreads / 32; ++w) v += red[threadIdx.x][w];
+      tot[threadIdx.x] = v;
+    }
+    __syncthreads();
+  };
+  double a[10];
+  bool fine = true;
+  for (int pass = 0; pass < 2 && fine; ++pass) {
+#pragma unroll
+    for (int l = 0; l < 10; ++l) a[l] = 0.0;
+    for (int e = threadIdx.x; e < n3; e += kPrecThreads) {
+      double v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = b[(3 + i) * n3 + e];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int l = 0; l <= i; ++l) a[i * (i + 1) / 2 + l] = fma(v[i], v[l], a[i * (i + 1) / 2 + l]);
+    }
+    sums(a, 10);
+    double R[10];   // lower factor of the Gram matrix, its diagonal inverted (every thread the same)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int l = 0; l <= i; ++l) {
+        double v = tot[i * (i + 1) / 2 + l];
+#pragma unroll
+        for (int m = 0; m < l; ++m) v = fma(-R[i * (i + 1) / 2 + m], R[l * (l + 1) / 2 + m], v);
+        if (l < i) {
+          R[i * (i + 1) / 2 + l] = v * R[l * (l + 1) / 2 + l];
+        } else {
+          fine = fine && v > 1e-6 * tot[i * (i + 1) / 2 + i] && v > 1e-24;
+          R[i * (i + 1) / 2 + i] = 1.0 / sqrt(v);
+        }
+      }
+    if (!fine) break;
+    for (int e = threadIdx.x; e < n3; e += kPrecThreads) {
+      double v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        v[i] = b[(3 + i) * n3 + e];
+#pragma unroll
+        for (int l = 0; l < i; ++l) v[i] = fma(-R[i * (i + 1) / 2 + l], v[l], v[i]);
+        v[i] *= R[i * (i + 1) / 2 + i];
+        b[(3 + i) * n3 + e] = v[i];
+      }
+    }
+  }
+  if (!fine) {   // the same for every thread
+    for (int k = 3; k < 7; ++k) {
+      double* v = b + k * n3;
+      for (int e = threadIdx.x; e < n3; e += kPrecThreads) v[e] = start(k, e);
+      for (int pass = 0; pass < 2 && k > 3; ++pass) {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) a[l] = 0.0;
+        for (int e = threadIdx.x; e < n3; e += kPrecThreads) {
+#pragma unroll
+          for (int l = 0; l < 3; ++l)
+            if (3 + l < k) a[l] = fma(b[(3 + l) * n3 + e], v[e], a[l]);
+        }
+        sums(a, k - 3);
+        for (int e = threadIdx.x; e < n3; e += kPrecThreads) {
+          double y = v[e];
+#pragma unroll
+          for (int l = 0; l < 3; ++l)
+            if (3 + l < k) y = fma(-tot[l], b[(3 + l) * n3 + e], y);
+          v[e] = y;
+        }
+      }
+      a[0] = 0.0;
+      for (int e = threadIdx.x; e < n3; e += kPrecThreads) a[0] = fma(v[e], v[e], a[0]);
+      sums(a, 1);
+      const double nrm = sqrt(tot[0]);
+      if (!(nrm > 1e-12)) {
+        if (threadIdx.x == 0) atomicOr(bad, 1);
+        return;
+      }
+      for (int e = threadIdx.x; e < n3; e += kPrecThreads) v[e] /= nrm;
+    }
+  }
+  if (threadIdx.x == 0) {
+    const double lam = D.lam, h = 1.0 / (lam + 1.0);
+    double* f = fac + 6 * blockIdx.x;
+    f[0] = h;
+    f[1] = 0.5 - h;
+    f[2] = 0.5 / lam - h;
+    f[3] = lam + 1.0;
+    f[4] = 2.0 - (lam + 1.0);
+    f[5] = 2.0 * lam - (lam + 1.0);
+  }
+}
+
 // dots[drop][k] = basis_k . v over the drop's 3 nc coefficients (one block per drop, fixed order)
 __global__ void k_prec_dots(const double* __restrict__ v, const double* __restrict__ basis,
                             const DropDev* __restrict__ drops, double* __restrict__ dots) {
@@ -581,11 +722,14 @@ int device_cycles(shbim_ctx* ctx, cudaStream_t s, bool* done) {
   double* sc_h = G.h_host + 2 * (G.m + 2);
   int* is_h = reinterpret_cast<int*>(sc_h + 4);
   for (;;) {
-    // the host's state of the current cycle
-    SHBIM_CUDA(ctx, cudaMemcpyAsync(C.H, G.H.data(), G.H.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-    SHBIM_CUDA(ctx, cudaMemcpyAsync(C.cs, G.cs.data(), G.m * sizeof(double), cudaMemcpyHostToDevice, s));
-    SHBIM_CUDA(ctx, cudaMemcpyAsync(C.sn, G.sn.data(), G.m * sizeof(double), cudaMemcpyHostToDevice, s));
-    SHBIM_CUDA(ctx, cudaMemcpyAsync(C.g, G.g.data(), (G.m + 1) * sizeof(double), cudaMemcpyHostToDevice, s));
+    // the host's state of the current cycle: columns and rotations of the steps so far (a step writes its own
+    // before it reads them), then g
+    if (G.k > 0) {
+      SHBIM_CUDA(ctx, cudaMemcpyAsync(C.H, G.H.data(), (size_t)G.k * (G.m + 1) * sizeof(double), cudaMemcpyHostToDevice, s));
+      SHBIM_CUDA(ctx, cudaMemcpyAsync(C.cs, G.cs.data(), G.k * sizeof(double), cudaMemcpyHostToDevice, s));
+      SHBIM_CUDA(ctx, cudaMemcpyAsync(C.sn, G.sn.data(), G.k * sizeof(double), cudaMemcpyHostToDevice, s));
+    }
+    SHBIM_CUDA(ctx, cudaMemcpyAsync(C.g, G.g.data(), (G.k + 1) * sizeof(double), cudaMemcpyHostToDevice, s));
     sc_h[0] = G.resid;
     sc_h[1] = G.bnorm;
     sc_h[2] = ctx->opts.gmres_tol;
@@ -642,67 +786,24 @@ int update_x(shbim_ctx* ctx, cudaStream_t s) {
 
 }  // namespace
 
-// Basis of the Stokes preconditioner for the current geometry: per drop the translations e_k (constant
-// fields, coefficient sqrt(4 pi) on Y_00), the rotations e_k x x (from the position coefficients) and
-// the parameter sphere's radial field r^ (degree 1), orthonormalised in that order in FP64 (modified
-// Gram-Schmidt, twice); factors from the drop's viscosity ratio.
+// Basis of the Stokes preconditioner for the current geometry (k_prec_basis). A shape whose modes are linearly
+// dependent or not finite is refused before anything else is built from it.
 int build_stokes_preconditioner(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
   const int64_t nc_all = ctx->ncoef;
   if (!ctx->prec_basis) {
     if (cudaMalloc(&ctx->prec_basis, (size_t)21 * nc_all * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&ctx->prec_dots, (size_t)7 * ctx->n_drops * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&ctx->prec_fac, (size_t)6 * ctx->n_drops * sizeof(double)) != cudaSuccess)
+        cudaMalloc(&ctx->prec_fac, ((size_t)6 * ctx->n_drops + 1) * sizeof(double)) != cudaSuccess)
       return fail(ctx, SHBIM_ERR_NOMEM, "Stokes preconditioner allocation failed");
   }
-  std::vector<double> x((size_t)3 * nc_all), B((size_t)21 * nc_all, 0.0), F((size_t)6 * ctx->n_drops);
-  SHBIM_CUDA(ctx, cudaMemcpyAsync(x.data(), xcoef_dev, x.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+  int* bad = reinterpret_cast<int*>(ctx->prec_fac + 6 * (size_t)ctx->n_drops);
+  SHBIM_CUDA(ctx, cudaMemsetAsync(bad, 0, sizeof(int), s));
+  k_prec_basis<<<ctx->n_drops, kPrecThreads, 0, s>>>(xcoef_dev, ctx->drops_dev, ctx->prec_basis, ctx->prec_fac, bad);
+  SHBIM_CHECK_LAUNCH(ctx, "k_prec_basis");
+  int h = 0;
+  SHBIM_CUDA(ctx, cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
   SHBIM_CUDA(ctx, cudaStreamSynchronize(s));
-  const double s4pi = std::sqrt(4.0 * kPi), s4pi3 = std::sqrt(4.0 * kPi / 3.0);
-  for (int i = 0; i < ctx->n_drops; ++i) {
-    const Drop& d = ctx->drops[i];
-    const int64_t nc = d.nc, n3 = 3 * nc;
-    const double* xc = x.data() + 3 * d.coef_off;
-    double* b = B.data() + 21 * d.coef_off;
-    for (int k = 0; k < 3; ++k) b[k * n3 + k * nc] = s4pi;
-    for (int k = 0; k < 3; ++k) {
-      double* v = b + (3 + k) * n3;
-      const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
-      // (e_k x x)_{k1} = -x_{k2}, (e_k x x)_{k2} = x_{k1}
-      for (int64_t j = 0; j < nc; ++j) {
-        v[k1 * nc + j] = -xc[k2 * nc + j];
-        v[k2 * nc + j] = xc[k1 * nc + j];
-      }
-    }
-    double* r = b + 6 * n3;
-    r[0 * nc + 3] = -s4pi3;   // x: -sqrt(4 pi/3) on the (1, 1) harmonic
-    r[1 * nc + 1] = -s4pi3;   // y: -sqrt(4 pi/3) on the (1, -1) harmonic
-    r[2 * nc + 2] = s4pi3;    // z:  sqrt(4 pi/3) on the (1, 0) harmonic
-    for (int k = 0; k < 7; ++k) {
-      double* v = b + k * n3;
-      for (int pass = 0; pass < 2; ++pass)
-        for (int l = 0; l < k; ++l) {
-          const double* u = b + l * n3;
-          double dot = 0.0;
-          for (int64_t j = 0; j < n3; ++j) dot += u[j] * v[j];
-          for (int64_t j = 0; j < n3; ++j) v[j] -= dot * u[j];
-        }
-      double nrm = 0.0;
-      for (int64_t j = 0; j < n3; ++j) nrm += v[j] * v[j];
-      nrm = std::sqrt(nrm);
-      if (!(nrm > 1e-12)) return fail(ctx, SHBIM_ERR_ARG, "degenerate drop shape for the Stokes preconditioner");
-      for (int64_t j = 0; j < n3; ++j) v[j] /= nrm;
-    }
-    const double lam = d.lam, a = 1.0 / (lam + 1.0);
-    double* f = F.data() + 6 * i;
-    f[0] = a;
-    f[1] = 0.5 - a;
-    f[2] = 0.5 / lam - a;
-    f[3] = lam + 1.0;
-    f[4] = 2.0 - (lam + 1.0);
-    f[5] = 2.0 * lam - (lam + 1.0);
-  }
-  SHBIM_CUDA(ctx, cudaMemcpy(ctx->prec_basis, B.data(), B.size() * sizeof(double), cudaMemcpyHostToDevice));
-  SHBIM_CUDA(ctx, cudaMemcpy(ctx->prec_fac, F.data(), F.size() * sizeof(double), cudaMemcpyHostToDevice));
+  if (h) return fail(ctx, SHBIM_ERR_ARG, "degenerate drop shape for the Stokes preconditioner");
   return SHBIM_OK;
 }
 

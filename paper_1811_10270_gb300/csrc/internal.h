@@ -181,6 +181,7 @@ struct shbim_ctx {
   shbim::PairTile* tiles_dev = nullptr;
   double* lamm1_dev = nullptr;    // lambda_j - 1 per drop
   shbim::DropDev* drops_dev = nullptr;
+  double* centres_dev = nullptr;  // [n_drops][3]
   int pair_splits = 1;            // default source-split count of the layout
   int split_max = 1;              // capacity of the partial-sum buffer in splits
   // shape of the FP32 all-pairs launches per kernel kind (Laplace DL, Laplace SL, Stokes S + D, Stokes S,
@@ -218,7 +219,8 @@ struct shbim_ctx {
   bool stokes_prec = true;
   double* prec_basis = nullptr;
   double* prec_dots = nullptr;    // [n_drops][7]
-  double* prec_fac = nullptr;     // [n_drops][6]: inverse (1/(lam+1), 1/2 - ., 1/(2 lam) - .), forward (lam+1, ...)
+  double* prec_fac = nullptr;     // [n_drops][6]: inverse (1/(lam+1), 1/2 - ., 1/(2 lam) - .), forward (lam+1, ...),
+                                  // then an int: a shape without a basis
   bool dq_pairs = true;           // FP64-class pair sums on quantised positions (k_pairs_dq) or general double-float
   double dq_scale = 0.0;          // 2^Q of the quantised positions (0: not built for this geometry)
   unsigned* dq_ext_dev = nullptr; // [n_drops] largest |x - c| over each drop's sources (float bits)
@@ -241,6 +243,8 @@ struct shbim_ctx {
   double* part = nullptr;         // [pair_splits][3][ntarget] partial sums
   double* grid_out = nullptr;     // [3][ntarget] operator values before projection
   double* xup = nullptr;          // per drop [3][kNumTab][ns]: position and derivatives on the up grid
+  double* geo_tmp = nullptr;      // synthesised fields of one grid while the geometry is set up
+  size_t geo_tmp_n = 0;
   double* sht_scratch = nullptr;  // Fourier stage of forward transforms
   size_t sht_scratch_elems = 0;
   // singular-row build workspace
@@ -502,6 +506,8 @@ int rebuild_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s);
 // the sums go to partial buffers; `before_reduce` (optional) is waited for before they are
 // added into out_accum
 // Stokes preconditioner basis and factors of the current geometry (gmres.cu)
+// ctx->geo_tmp with room for n doubles
+int geometry_scratch(shbim_ctx* ctx, size_t n);
 int build_stokes_preconditioner(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s);
 // extents of the drops, quantised source positions of the FP64-class pair sums and the lists of direct and
 // far drop pairs (once per geometry)

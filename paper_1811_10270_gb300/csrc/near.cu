@@ -636,8 +636,8 @@ int build_near(shbim_ctx* ctx, const double* xcoef, cudaStream_t s) {
   }
   int64_t maxn = 0;
   for (int j = 0; j < nd; ++j) maxn = std::max(maxn, N.fine_n_h[j]);
-  double* tmp = nullptr;
-  if (cudaMalloc(&tmp, sizeof(double) * 9 * maxn) != cudaSuccess) return fail(ctx, SHBIM_ERR_NOMEM, "fine scratch");
+  if ((rc = geometry_scratch(ctx, (size_t)9 * maxn))) return rc;
+  double* tmp = ctx->geo_tmp;
   for (int j = 0; j < nd && rc == SHBIM_OK; ++j) {
     if (N.fine_off_h[j] < 0) continue;
     const Drop& d = ctx->drops[j];
@@ -671,8 +671,6 @@ int build_near(shbim_ctx* ctx, const double* xcoef, cudaStream_t s) {
       N.min_ratio = std::sqrt((double)r2);
     }
   }
-  cudaStreamSynchronize(s);
-  cudaFree(tmp);
   return rc;
 }
 

@@ -79,14 +79,24 @@ int geometry_kernel32(shbim_ctx* ctx, const double* buf, int64_t n, int nkind, c
   return SHBIM_OK;
 }
 
+int geometry_scratch(shbim_ctx* ctx, size_t n) {
+  if (n <= ctx->geo_tmp_n) return SHBIM_OK;
+  cudaFree(ctx->geo_tmp);
+  ctx->geo_tmp = nullptr;
+  ctx->geo_tmp_n = 0;
+  if (cudaMalloc(&ctx->geo_tmp, n * sizeof(double)) != cudaSuccess)
+    return fail(ctx, SHBIM_ERR_NOMEM, "cudaMalloc geometry scratch");
+  ctx->geo_tmp_n = n;
+  return SHBIM_OK;
+}
+
 int build_geometry(shbim_ctx* ctx, const double* xcoef, cudaStream_t s) {
   // scratch for the 9 synthesised fields of the largest grid
   int64_t maxn = 0;
   for (auto& d : ctx->drops) maxn = std::max<int64_t>(maxn, d.nt);
-  double* tmp = nullptr;
-  if (cudaMalloc(&tmp, (size_t)9 * maxn * sizeof(double)) != cudaSuccess)
-    return fail(ctx, SHBIM_ERR_NOMEM, "cudaMalloc geometry scratch");
-  int rc = SHBIM_OK;
+  int rc = geometry_scratch(ctx, (size_t)9 * maxn);
+  if (rc) return rc;
+  double* tmp = ctx->geo_tmp;
   for (auto& d : ctx->drops) {
     const double* xc = xcoef + 3 * d.coef_off;
     for (int pass = 0; pass < 2 && rc == SHBIM_OK; ++pass) {
@@ -110,8 +120,6 @@ int build_geometry(shbim_ctx* ctx, const double* xcoef, cudaStream_t s) {
     }
     if (rc) break;
   }
-  cudaStreamSynchronize(s);
-  cudaFree(tmp);
   return rc;
 }
 
