@@ -83,6 +83,8 @@ void free_drop_state(shbim_ctx* ctx) {
   ctx->geo = Geometry{};
   cudaFree(ctx->tiles_dev);
   ctx->tiles_dev = nullptr;
+  cudaFree(ctx->tgt_order);
+  ctx->tgt_order = nullptr;
   cudaFree(ctx->drops_dev);
   ctx->drops_dev = nullptr;
   cudaFree(ctx->centres_dev);
@@ -490,6 +492,18 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
     for (int i = 0; i < n_drops; ++i) lm1[i] = ctx->drops[i].lam - 1.0;
     if ((rc = dalloc(ctx, &ctx->lamm1_dev, n_drops, "viscosity contrasts"))) return rc;
     SHBIM_CUDA(ctx, cudaMemcpy(ctx->lamm1_dev, lm1.data(), n_drops * sizeof(double), cudaMemcpyHostToDevice));
+  }
+  // order of a drop's targets in the pair sums: bands of six latitudes, longitude by longitude, so that 32 in a row
+  // are a patch about as wide as it is high
+  {
+    std::vector<int> order;
+    order.reserve(to);
+    for (const auto& d : ctx->drops)
+      for (int r0 = 0; r0 <= d.p; r0 += 6)
+        for (int c = 0; c < 2 * d.p + 2; ++c)
+          for (int r = r0; r <= std::min(r0 + 5, d.p); ++r) order.push_back((int)d.tgt_off + r * (2 * d.p + 2) + c);
+    if ((rc = dalloc(ctx, &ctx->tgt_order, (size_t)to, "target order"))) return rc;
+    SHBIM_CUDA(ctx, cudaMemcpy(ctx->tgt_order, order.data(), to * sizeof(int), cudaMemcpyHostToDevice));
   }
   // all-pairs tiling: tiles never cross a drop; sources split so that the grid fills the GPU
   {

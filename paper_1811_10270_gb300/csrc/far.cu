@@ -107,6 +107,9 @@ __device__ __forceinline__ void t_ld2(const df* p, int64_t i, df& a, df& b) {
   b = df{v.z, v.w};
 }
 
+__device__ __forceinline__ double t_rsqrt(double a) { return rsqrt(a); }
+__device__ __forceinline__ df t_rsqrt(df a) { return dfl::rsqrt(a); }
+
 template <class T>
 struct Acc;
 template <>
@@ -137,6 +140,19 @@ __device__ __forceinline__ T warp_total(T v) {
 
 __host__ __device__ __forceinline__ int tri_n(int L) { return (L + 1) * (L + 2) / 2; }
 __host__ __device__ __forceinline__ int tri_o(int L, int m) { return m * (L + 1) - m * (m - 1) / 2; }
+
+// the entry whose groups hold flat group f
+__device__ __forceinline__ int entry_of(const int64_t* __restrict__ goff, int nent, int64_t f) {
+  int a = 0, b = nent;                    // goff[a] <= f < goff[b]
+  while (b - a > 1) {
+    const int c = (a + b) >> 1;
+    if (goff[c] <= f)
+      a = c;
+    else
+      b = c;
+  }
+  return a;
+}
 
 // (x + i y)^m by binary powers
 template <class T>
@@ -732,27 +748,13 @@ __global__ void k_far_lset(const FarTgtDrop* __restrict__ td, const float* __res
 // moments. Up to nfull FP32-pipe bound (35 + 24 NS instructions per target and (n, m) in double-float); splitting
 // the orders keeps every SM busy from a few thousand targets on.
 template <class T, int NS>
-__global__ void __launch_bounds__(32 * kL2pWarps, 2)
-k_far_l2p(const FarTgtDrop* __restrict__ td, const int2* __restrict__ blocks, const DropDev* __restrict__ drops,
-          const float* __restrict__ inv_scale, int nfull, const T* __restrict__ rec, const T* __restrict__ set,
-          const double* __restrict__ tgt, int64_t ntarget, double* __restrict__ out) {
+__device__ __forceinline__ void eval_sets(T x, T y, T z, int L, int Ls, int nfull, const T* __restrict__ rec,
+                                          const T* __restrict__ set, T* __restrict__ red, unsigned char* slot_raw) {
   constexpr int VB = 2 * NS;               // coefficients of one (n, m)
   constexpr int NB = 32 / VB;              // degrees per slot
-  __shared__ __align__(16) unsigned char red_raw[kL2pWarps * NS * 32 * 8];
-  __shared__ __align__(16) unsigned char slot_raw[kL2pWarps * 2 * 32 * 8];
-  T* red = reinterpret_cast<T*>(red_raw);
-  const int2 b = blocks[blockIdx.x];                    // drop, first target within the drop
-  const FarTgtDrop d = td[b.x];
-  const DropDev D = drops[b.x];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool ok = b.y + lane < D.nt;
-  const int64_t t = D.tgt_off + (ok ? b.y + lane : 0);
-  const float inv = inv_scale[b.x];
-  const T x = t_pow2(from_d<T>(tgt[t] - D.cx), inv), y = t_pow2(from_d<T>(tgt[ntarget + t] - D.cy), inv),
-          z = t_pow2(from_d<T>(tgt[2 * ntarget + t] - D.cz), inv);
   const T z2 = t_pow2(z, 2.f);
   const T r2 = t_add(t_add(t_mul(x, x), t_mul(y, y)), t_mul(z, z));
-  const int L = d.L;
   T* slot = reinterpret_cast<T*>(slot_raw) + warp * 64;
   float* fslot = reinterpret_cast<float*>(slot);
   T* tot = red + (warp * NS) * 32 + lane;               // [NS] with stride 32: this thread's own totals
@@ -764,7 +766,7 @@ k_far_l2p(const FarTgtDrop* __restrict__ td, const int2* __restrict__ blocks, co
   int buf = 0;
   for (int m = warp; m <= L; m += kL2pWarps) {
     T q1 = from_d<T>(1.0), q2 = from_d<T>(0.0);
-    const T* c = set + (int64_t)VB * (d.tri + tri_o(L, m));
+    const T* c = set + (int64_t)VB * tri_o(Ls, m);
     const T* rc = rec + tri_o(kFarLmax, m) - m;
     const int left = (L - m + 1) * VB;
     int o = 0, n = m;
@@ -855,6 +857,26 @@ k_far_l2p(const FarTgtDrop* __restrict__ td, const int2* __restrict__ blocks, co
     t_st(red, k * 32 + lane, s.value());    // slot (0, k) is read by this thread only
   }
   __syncthreads();
+}
+
+template <class T, int NS>
+__global__ void __launch_bounds__(32 * kL2pWarps, 2)
+k_far_l2p(const FarTgtDrop* __restrict__ td, const int2* __restrict__ blocks, const DropDev* __restrict__ drops,
+          const float* __restrict__ inv_scale, int nfull, const T* __restrict__ rec, const T* __restrict__ set,
+          const double* __restrict__ tgt, int64_t ntarget, double* __restrict__ out) {
+  __shared__ __align__(16) unsigned char red_raw[kL2pWarps * NS * 32 * 8];
+  __shared__ __align__(16) unsigned char slot_raw[kL2pWarps * 2 * 32 * 8];
+  T* red = reinterpret_cast<T*>(red_raw);
+  const int2 b = blocks[blockIdx.x];                    // drop, first target within the drop
+  const FarTgtDrop d = td[b.x];
+  const DropDev D = drops[b.x];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool ok = b.y + lane < D.nt;
+  const int64_t t = D.tgt_off + (ok ? b.y + lane : 0);
+  const float inv = inv_scale[b.x];
+  const T x = t_pow2(from_d<T>(tgt[t] - D.cx), inv), y = t_pow2(from_d<T>(tgt[ntarget + t] - D.cy), inv),
+          z = t_pow2(from_d<T>(tgt[2 * ntarget + t] - D.cz), inv);
+  eval_sets<T, NS>(x, y, z, d.L, d.L, nfull, rec, set + (int64_t)2 * NS * d.tri, red, slot_raw);
   if (!ok) return;
   const double w4 = 0.07957747154594766788;
   if (NS == 1) {
@@ -876,6 +898,180 @@ k_far_l2p(const FarTgtDrop* __restrict__ td, const int2* __restrict__ blocks, co
     const double v = t_double(t_ld(red, c * 32 + lane)) - B * t_double(g.value());
     out[3 * D.tgt_off + (int64_t)c * D.nt + (t - D.tgt_off)] += w4 * v;
   }
+}
+
+
+// ---- 5. close pairs: targets far enough from the source drop's centre take its multipole expansion itself,
+// Phi = 1/r sum_nm c_nm R_nm(x A / r^2), the regular harmonics at the inverted point, so the sets and the
+// evaluation are those of the local expansions. A drop's neighbours at gaps of 0.2 to 1 have half to two thirds of
+// their targets beyond 1.7 to 2 radii, and a value of order 45 costs a seventh to a thirtieth of a sum over the
+// 5e3 to 2e4 sources of a drop of degree 24 to 48.
+
+// order at which the targets of a group may take the expansion of an entry's drop: a warp per group
+__global__ void k_far_reach(int nent, const int* __restrict__ ent_tgt, NearList nl, int64_t ngroup,
+                            const DropDev* __restrict__ drops, const unsigned* __restrict__ ext,
+                            const int* __restrict__ Lsrc, const float* __restrict__ rho_max,
+                            const double* __restrict__ tgt, int64_t ntarget, unsigned char* __restrict__ order) {
+  const int64_t f = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (f >= ngroup) return;
+  const int en = entry_of(nl.goff, nent, f), lane = threadIdx.x & 31;
+  const int j = nl.drop[en];
+  const DropDev Di = drops[ent_tgt[en]], Dj = drops[j];
+  const int64_t sl = (f - nl.goff[en]) * kFarGroup + lane;
+  double d2 = INFINITY;
+  if (sl < Di.nt) {
+    const int64_t t = nl.tgt[Di.tgt_off + sl];
+    const double dx = tgt[t] - Dj.cx, dy = tgt[ntarget + t] - Dj.cy, dz = tgt[2 * ntarget + t] - Dj.cz;
+    d2 = dx * dx + dy * dy + dz * dz;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) d2 = fmin(d2, __shfl_xor_sync(0xffffffffu, d2, o));
+  if (lane) return;
+  const float rho = (float)((double)__uint_as_float(ext[j]) / sqrt(d2)) * 1.000001f;
+  int L = 2;
+  while (L <= Lsrc[j] && !(rho <= rho_max[L])) ++L;
+  order[f] = (unsigned char)(L <= Lsrc[j] ? L : kNoReach);
+}
+
+// coefficient (n, mm) of the derivative along axis ax of the multipole expansion v, times -A (a dipole along ax)
+template <class T>
+__device__ T multi_grad(const T* __restrict__ v, int n, int mm, int ax, const T* __restrict__ la,
+                        const T* __restrict__ lp, const T* __restrict__ lq) {
+  Acc<T> a;
+  if (n == 0) return a.value();
+  const int m = abs(mm), sg = mm < 0 ? -1 : 1, k = n - 1;
+  const int t = tri_o(kFarLmax, m) + n - m;
+  if (ax == 2) {
+    if (m <= k) a.add_prod(t_ld(la, t), coef_at(v, k, mm));
+    return a.value();
+  }
+  const T Pv = t_ld(lp, t), Q = t_ld(lq, t);
+  if (mm == 0) {
+    if (k >= 1) a.add_prod(Pv, coef_at(v, k, ax == 0 ? 1 : -1));
+    return a.value();
+  }
+  if (ax == 0) {
+    if (m + 1 <= k) a.add_prod(Pv, coef_at(v, k, sg * (m + 1)));
+    if (sg > 0 || m >= 2) a.add_prod(t_neg(Q), coef_at(v, k, sg * (m - 1)));
+  } else {
+    if (m + 1 <= k) a.add_prod(sg > 0 ? Pv : t_neg(Pv), coef_at(v, k, -sg * (m + 1)));
+    if (sg < 0)
+      a.add_prod(t_neg(Q), coef_at(v, k, m - 1));
+    else if (m >= 2)
+      a.add_prod(Q, coef_at(v, k, -(m - 1)));
+  }
+  return a.value();
+}
+
+// the sets of k_far_lset of a source drop's multipole expansion
+template <class T, int NS>
+__global__ void k_far_mset(const FarSrcDrop* __restrict__ sd, const int* __restrict__ Lsrc,
+                           const float* __restrict__ inv_scale, FarTab<T> tab, int npot, const T* __restrict__ mom,
+                           T* __restrict__ set) {
+  const int j = blockIdx.y;
+  const int L = Lsrc[j];
+  if (L < 0) return;
+  const FarSrcDrop d = sd[j];
+  const int nc = (L + 1) * (L + 1), ntri = tri_n(L);
+  const T* l = mom + npot * d.coef;
+  const T inv = from_d<T>(-(double)inv_scale[j]);
+  T* out = set + (int64_t)2 * NS * d.tri;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ntri * 2 * NS; e += gridDim.x * blockDim.x) {
+    const int o = e / (2 * NS), r = e - o * 2 * NS;
+    const int st = r >> 1, cs = r & 1;
+    int m = 0;
+    while (m < L && tri_o(L, m + 1) <= o) ++m;
+    const int n = m + (o - tri_o(L, m));
+    T v = from_d<T>(0.0);
+    if (!(cs == 1 && m == 0)) {
+      const int mu = cs ? -m : m;
+      if (NS == 1) {
+        v = coef_at(l, n, mu);
+      } else if (NS == 3) {
+        v = t_mul(inv, multi_grad(l, n, mu, st, tab.la, tab.lp, tab.lq));
+      } else if (st < 3) {
+        v = t_add(coef_at(l + (int64_t)st * nc, n, mu),
+                  t_mul(inv, multi_grad(l + (int64_t)3 * nc, n, mu, st, tab.la, tab.lp, tab.lq)));
+      } else {
+        const int k = (st - 3) / 3, ax = (st - 3) - 3 * k;
+        v = t_mul(inv, multi_grad(l + (int64_t)k * nc, n, mu, ax, tab.la, tab.lp, tab.lq));
+      }
+      v = t_mul(v, t_mul(t_ld(tab.kap, tri_o(kFarLmax, m) + n - m), from_d<T>(12.566370614359172954 / (2 * n + 1))));
+    }
+    t_st(out, e, v);
+  }
+}
+
+// values of one entry's expansion at one group of targets, [group][component][32]; bound as k_far_l2p
+template <class T, int NS>
+__global__ void __launch_bounds__(32 * kL2pWarps, 2)
+k_far_m2p(int nent, const int* __restrict__ ent_tgt, NearList nl, const FarSrcDrop* __restrict__ sd,
+          const int* __restrict__ Lsrc, const DropDev* __restrict__ drops, const float* __restrict__ inv_scale, int nfull,
+          const T* __restrict__ rec, const T* __restrict__ set, const double* __restrict__ tgt, int64_t ntarget,
+          double* __restrict__ part) {
+  constexpr int NC = NS == 12 ? 3 : 1;
+  __shared__ __align__(16) unsigned char red_raw[kL2pWarps * NS * 32 * 8];
+  __shared__ __align__(16) unsigned char slot_raw[kL2pWarps * 2 * 32 * 8];
+  T* red = reinterpret_cast<T*>(red_raw);
+  const int64_t f = blockIdx.x;
+  const int en = entry_of(nl.goff, nent, f);
+  const int j = nl.drop[en];
+  const DropDev Dj = drops[j];
+  const int g = (int)(f - nl.goff[en]);
+  if (nl.direct(en, g, Dj.ns)) return;                  // uniform over the CTA
+  const DropDev Di = drops[ent_tgt[en]];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int sl = g * kFarGroup + lane;
+  const int64_t t = nl.tgt[Di.tgt_off + min(sl, Di.nt - 1)];
+  const float inv = inv_scale[j];
+  const T x = t_pow2(from_d<T>(tgt[t] - Dj.cx), inv), y = t_pow2(from_d<T>(tgt[ntarget + t] - Dj.cy), inv),
+          z = t_pow2(from_d<T>(tgt[2 * ntarget + t] - Dj.cz), inv);
+  const T ri = t_rsqrt(t_add(t_add(t_mul(x, x), t_mul(y, y)), t_mul(z, z)));
+  const T ri2 = t_mul(ri, ri);
+  eval_sets<T, NS>(t_mul(x, ri2), t_mul(y, ri2), t_mul(z, ri2), nl.order[f], Lsrc[j], nfull, rec,
+                   set + (int64_t)2 * NS * sd[j].tri, red, slot_raw);
+  const double w = 0.07957747154594766788 * (double)inv * t_double(ri);
+  double* o = part + f * NC * 32 + lane;
+  if (NS == 1) {
+    if (warp == 0) o[0] = w * t_double(t_ld(red, lane));
+  } else if (NS == 3) {
+    if (warp == 0) {
+      double v = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v = fma(tgt[(3 + k) * ntarget + t], t_double(t_ld(red, k * 32 + lane)), v);
+      o[0] = -w * v;
+    }
+  } else if (warp < 3) {
+    const int c = warp;
+    const T xs[3] = {x, y, z};
+    Acc<T> a;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) a.add_prod(xs[k], t_ld(red, (3 + 3 * k + c) * 32 + lane));
+    o[32 * c] = w * (t_double(t_ld(red, c * 32 + lane)) - t_double(a.value()) / (double)inv);
+  }
+}
+
+// a drop's targets: the entries' values in order
+template <int NC>
+__global__ void k_far_msum(NearList nl, const DropDev* __restrict__ drops, const double* __restrict__ part,
+                           double* __restrict__ out) {
+  const int i = blockIdx.y;
+  const DropDev D = drops[i];
+  const int sl = blockIdx.x * blockDim.x + threadIdx.x;
+  if (sl >= D.nt) return;
+  const int g = sl / kFarGroup;
+  double s[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) s[c] = 0.0;
+  for (int en = nl.off[i]; en < nl.off[i + 1] - 1; ++en) {
+    if (nl.direct(en, g, drops[nl.drop[en]].ns)) continue;
+    const double* p = part + (nl.goff[en] + g) * NC * 32 + (sl & 31);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) s[c] += p[32 * c];
+  }
+  const int64_t t = nl.tgt[D.tgt_off + sl] - D.tgt_off;
+#pragma unroll
+  for (int c = 0; c < NC; ++c) out[(int64_t)NC * D.tgt_off + (int64_t)c * D.nt + t] += s[c];
 }
 
 // ---- constants (host, once per process; copied to each context's device memory)
@@ -1125,6 +1321,9 @@ void far_free(shbim_ctx* ctx) {
   cudaFree(F.lpair);
   cudaFree(F.loc);
   cudaFree(F.set);
+  cudaFree(F.mset);
+  cudaFree(F.order);
+  cudaFree(F.mpart);
   delete ctx->far;
   ctx->far = nullptr;
 }
@@ -1144,7 +1343,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     return o;
   };
   struct Offsets {
-    size_t nb_off, nb_drop, nb_pre, pairs, lsrc, sd, td, chunks, blocks;
+    size_t nb_off, nb_drop, nb_pre, pairs, lsrc, sd, td, chunks, blocks, goff, ent_tgt, rho;
   } off[kFarPlans + 1] = {};
   std::vector<float> inv(2 * nd, 1.f);
   for (int i = 0; i < 2 * nd; ++i) {
@@ -1153,7 +1352,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     inv[i] = (float)std::ldexp(1.0, -e);
   }
   const size_t inv_off = put(inv.data(), inv.size() * sizeof(float));
-  size_t max_part = 0, max_v = 0, max_mom = 0, max_lp = 0, max_loc = 0, max_set = 0, max_ang = 0;
+  size_t max_part = 0, max_v = 0, max_mom = 0, max_lp = 0, max_loc = 0, max_set = 0, max_ang = 0, max_mset = 0, max_mpart = 0;
   bool any = false;
   for (int pl = 0; pl <= kFarPlans; ++pl) {
     FarPlan& P = F.plan[pl];
@@ -1165,8 +1364,10 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     // rho_max[L]: largest ratio order L serves
     std::vector<double> rho_max(cap + 1);
     for (int L = 0; L <= cap; ++L) rho_max[L] = std::pow(eps / std::pow(L + 1.0, g), 1.0 / (L + 1));
-    std::vector<int> Lsrc(nd, -1), nb_off(nd + 1, 0), nb_drop;
-    std::vector<int64_t> nb_pre;
+    std::vector<int> Lsrc(nd, -1), nb_off(nd + 1, 0), nb_drop, ent_tgt;
+    std::vector<int64_t> nb_pre, goff;
+    std::vector<float> rho_f(cap + 1);
+    for (int L = 0; L <= cap; ++L) rho_f[L] = std::nextafterf((float)rho_max[L], 0.f);
     std::vector<FarPair> pairs;
     std::vector<FarTgtDrop> td(nd);
     for (int i = 0; i < nd; ++i) {
@@ -1193,6 +1394,9 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
         if (L < 0) {
           nb_drop.push_back(j);
           nb_pre.push_back(pre);
+          ent_tgt.push_back(i);
+          goff.push_back(P.ngroup);
+          P.ngroup += (ctx->drops[i].nt + kFarGroup - 1) / kFarGroup;
           pre += ctx->drops[j].ns;
           P.direct_pairs += (double)ctx->drops[i].nt * ctx->drops[j].ns;
         } else {
@@ -1205,6 +1409,8 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
       }
       nb_drop.push_back(-1);                // end of the list, with the total
       nb_pre.push_back(pre);
+      ent_tgt.push_back(-1);
+      goff.push_back(P.ngroup);
       nb_off[i + 1] = (int)nb_drop.size();
       td[i].pair1 = (int)pairs.size();
     }
@@ -1214,7 +1420,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     std::vector<int2> blocks;
     int64_t part = 0, coef = 0, lout = 0, ang = 0, loc = 0, tri = 0;
     for (int j = 0; j < nd; ++j) {
-      sd[j] = FarSrcDrop{part, coef, 0};
+      sd[j] = FarSrcDrop{part, coef, P.stri, 0};
       if (Lsrc[j] < 0) continue;
       const int L = Lsrc[j];
       for (int f = 0; f < ctx->drops[j].ns; f += kP2mSrc) {
@@ -1223,6 +1429,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
         sd[j].nchunk++;
       }
       coef += (int64_t)(L + 1) * (L + 1);
+      P.stri += tri_n(L);
       P.src_work += (double)ctx->drops[j].ns * tri_n(L);
     }
     for (auto& p : pairs) {
@@ -1264,6 +1471,8 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
         max_loc = std::max(max_loc, npot * (size_t)loc);
         max_set = std::max(max_set, (size_t)2 * kSets[k] * tri);
         max_ang = std::max(max_ang, (size_t)ang);
+        max_mset = std::max(max_mset, (size_t)2 * kSets[k] * P.stri);
+        max_mpart = std::max(max_mpart, (size_t)(stokes_like(k) ? 96 : 32) * P.ngroup);
         F.max_charges = std::max(F.max_charges, kCharges[k]);
       }
     Offsets& o = off[pl];
@@ -1276,6 +1485,14 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     o.td = put(td.data(), td.size() * sizeof(FarTgtDrop));
     o.chunks = put(chunks.data(), chunks.size() * sizeof(FarChunk));
     o.blocks = put(blocks.data(), blocks.size() * sizeof(int2));
+    goff.push_back(P.ngroup);
+    P.nent = (int)nb_drop.size();
+    o.goff = put(goff.data(), goff.size() * sizeof(int64_t));
+    o.ent_tgt = put(ent_tgt.data(), ent_tgt.size() * sizeof(int));
+    o.rho = put(rho_f.data(), rho_f.size() * sizeof(float));
+    P.h_drop = std::move(nb_drop);
+    P.h_tgt = std::move(ent_tgt);
+    P.h_goff = std::move(goff);
   }
   int rc;
   if ((rc = far_grow(ctx, (void**)&F.blob, &F.blob_cap, blob.size(), "expansion plans"))) return rc;
@@ -1287,7 +1504,10 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     FarPlan& P = F.plan[pl];
     const Offsets& o = off[pl];
     P.near = NearList{reinterpret_cast<const int*>(F.blob + o.nb_off), reinterpret_cast<const int*>(F.blob + o.nb_drop),
-                      reinterpret_cast<const int64_t*>(F.blob + o.nb_pre)};
+                      reinterpret_cast<const int64_t*>(F.blob + o.nb_pre), ctx->tgt_order,
+                      reinterpret_cast<const int64_t*>(F.blob + o.goff), nullptr, FarReach{}};
+    P.ent_tgt = reinterpret_cast<const int*>(F.blob + o.ent_tgt);
+    P.rho_max = reinterpret_cast<const float*>(F.blob + o.rho);
     P.pairs = reinterpret_cast<const FarPair*>(F.blob + o.pairs);
     P.Lsrc = reinterpret_cast<const int*>(F.blob + o.lsrc);
     P.sd = reinterpret_cast<const FarSrcDrop*>(F.blob + o.sd);
@@ -1296,8 +1516,11 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     P.blocks = reinterpret_cast<const int2*>(F.blob + o.blocks);
   }
   if (!any) return SHBIM_OK;
-  size_t ang_total = 0;
-  for (int pl = 0; pl < kFarPlans; ++pl) ang_total += (size_t)F.plan[pl].ang;
+  size_t ang_total = 0, group_total = 0;
+  for (int pl = 0; pl < kFarPlans; ++pl) {
+    ang_total += (size_t)F.plan[pl].ang;
+    group_total += (size_t)F.plan[pl].ngroup;
+  }
   if ((rc = upload_tables(ctx)) ||
       (rc = far_grow(ctx, (void**)&F.ang, &F.ang_cap, ang_total * 8, "expansion angles")) ||
       (rc = far_grow(ctx, &F.q, &F.q_cap, (size_t)F.max_charges * ctx->nsource * 8, "expansion charges")) ||
@@ -1306,23 +1529,34 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
       (rc = far_grow(ctx, &F.mom, &F.mom_cap, max_mom * 8, "expansion dipole moments")) ||
       (rc = far_grow(ctx, &F.lpair, &F.lpair_cap, max_lp * 8, "expansion pair terms")) ||
       (rc = far_grow(ctx, &F.loc, &F.loc_cap, max_loc * 8, "local expansions")) ||
-      (rc = far_grow(ctx, &F.set, &F.set_cap, max_set * 8, "local expansions of derivatives"))) {
+      (rc = far_grow(ctx, &F.set, &F.set_cap, max_set * 8, "local expansions of derivatives")) ||
+      (rc = far_grow(ctx, &F.order, &F.order_cap, std::max<size_t>(group_total, 1), "orders of close pairs")) ||
+      (rc = far_grow(ctx, &F.mset, &F.mset_cap, max_mset * 8, "multipole expansions of derivatives")) ||
+      (rc = far_grow(ctx, &F.mpart, &F.mpart_cap, max_mpart * 8, "values of multipole expansions"))) {
     // no room for the expansions: every pair directly
     for (auto& P : F.plan) std::memset(P.use, 0, sizeof(P.use));
     ctx->err.clear();
     return SHBIM_OK;
   }
-  size_t ao = 0;
+  size_t ao = 0, go = 0;
   for (int pl = 0; pl < kFarPlans; ++pl) {
     FarPlan& P = F.plan[pl];
     P.ang_dev = F.ang + ao;
     ao += (size_t)P.ang;
+    P.order = static_cast<unsigned char*>(F.order) + go;
+    go += (size_t)P.ngroup;
     bool used = false;
     for (auto& r : P.use)
       for (bool u : r) used = used || u;
     if (!used || P.npairs == 0) continue;
     k_far_angles<<<P.npairs, 64, 0, s>>>(P.pairs, ctx->drops_dev, F.inv_src, F.inv_tgt, P.ang_dev);
     SHBIM_CHECK_LAUNCH(ctx, "k_far_angles");
+    if (P.ngroup == 0) continue;
+    k_far_reach<<<(unsigned)((P.ngroup * 32 + 255) / 256), 256, 0, s>>>(
+        P.nent, P.ent_tgt, P.near, P.ngroup, ctx->drops_dev, ctx->dq_ext_dev, P.Lsrc, P.rho_max, ctx->geo.tgt,
+        ctx->ntarget, P.order);
+    SHBIM_CHECK_LAUNCH(ctx, "k_far_reach");
+    P.near.order = P.order;
   }
   return SHBIM_OK;
 }
@@ -1330,7 +1564,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
 // The estimate in FP32 instructions of the expansions' inner steps (half as much again for latency and reads, twice
 // in FP64, plus 75 us of launches and short kernels) against the direct sums they replace. 40 drops of degree 11,
 // single layer in double-float (5.2e8 pairs): 1.48 ms directly, 1.03 with expansions; six drops of degree 16 in
-// FP64 (4e7 pairs, a third far), eight applications: 14.2 ms directly, 16.9 with expansions, and left direct; two
+// FP64 (4e7 pairs, a third far), eight applications: 14.2 ms directly, 15.7 with expansions, and left direct; two
 // drops, or 1e8 pairs in FP32, stay direct.
 bool far_worth(const FarPlan& P, int precision, int kind) {
   const double* direct = precision == SHBIM_PREC_FP32_COMP ? kDirect32 : (precision == SHBIM_PREC_DF64 ? kDirectDf : kDirect64);
@@ -1349,6 +1583,43 @@ const FarPlan* far_plan(const shbim_ctx* ctx, int kind) {
 }
 
 const FarPlan& far_all(const shbim_ctx* ctx) { return ctx->far->plan[kFarPlans]; }
+
+// Instructions of an expansion's value: recurrence and 2 NS multiply-adds per (n, m), half as much again for reads
+// and orders of uneven length; `base` for the powers of x + iy and the sums over warps. In FP64 four times that: six
+// drops of degree 16, double layer, solve of eight applications: 16.9 ms without these expansions, 16.3 at one
+// time, 15.7 at four. 64 drops of degree 16 to 48, without and with them: Stokeslet in double-float 35.5 and 24.2 ms,
+// stresslet FP32 10.2 and 9.0, double layer FP32 3.83 and 2.88; twice the instructions here change nothing.
+NearList far_near(const shbim_ctx* ctx, const FarPlan& P, int kind) {
+  NearList nl = P.near;
+  const int ns = kSets[kind], pr = ctx->opts.precision;
+  FarReach& r = nl.reach;
+  if (pr == SHBIM_PREC_FP64) {
+    r = FarReach{kFarLmax, 384 * (3 + 2 * ns), 0, 120000, (int)kDirect64[kind]};
+  } else {
+    const bool fp32 = pr == SHBIM_PREC_FP32_COMP;
+    r = FarReach{fp32 ? 12 : 36, 50 + 36 * ns, 9 + 6 * ns, 15000, (int)(fp32 ? kDirect32 : kDirectDf)[kind]};
+  }
+  return nl;
+}
+
+double far_direct_pairs(const shbim_ctx* ctx, const FarPlan& P, int kind) {
+  const NearList nl = far_near(ctx, P, kind);
+  if (!nl.order) return P.direct_pairs;
+  std::vector<unsigned char> L((size_t)P.ngroup);
+  if (cudaMemcpy(L.data(), nl.order, L.size(), cudaMemcpyDeviceToHost) != cudaSuccess) {
+    cudaGetLastError();
+    return P.direct_pairs;
+  }
+  double n = 0.0;
+  for (int en = 0; en < P.nent; ++en) {
+    if (P.h_drop[en] < 0) continue;
+    const int ns = ctx->drops[P.h_drop[en]].ns, nt = ctx->drops[P.h_tgt[en]].nt;
+    for (int64_t f = P.h_goff[en]; f < P.h_goff[en + 1]; ++f)
+      if (L[f] == kNoReach || !nl.reach.worth(L[f], ns))
+        n += (double)ns * std::min<int64_t>(kFarGroup, nt - (f - P.h_goff[en]) * kFarGroup);
+  }
+  return n;
+}
 
 namespace {
 
@@ -1412,6 +1683,34 @@ int expand(shbim_ctx* ctx, const FarPlan& P, int kind, cudaStream_t s) {
   else
     k_far_lset<T, 12><<<dim3(lb, nd), 128, 0, s>>>(P.td, F.inv_tgt, tab, npot, loc, set);
   SHBIM_CHECK_LAUNCH(ctx, "k_far_lset");
+  if (P.near.order) {
+    T* ms = static_cast<T*>(F.mset);
+    if (kind == 1)
+      k_far_mset<T, 1><<<dim3(lb, nd), 128, 0, s>>>(P.sd, P.Lsrc, F.inv_src, tab, npot, mom, ms);
+    else if (kind == 0)
+      k_far_mset<T, 3><<<dim3(lb, nd), 128, 0, s>>>(P.sd, P.Lsrc, F.inv_src, tab, npot, mom, ms);
+    else
+      k_far_mset<T, 12><<<dim3(lb, nd), 128, 0, s>>>(P.sd, P.Lsrc, F.inv_src, tab, npot, mom, ms);
+    SHBIM_CHECK_LAUNCH(ctx, "k_far_mset");
+  }
+  return SHBIM_OK;
+}
+
+template <class T, int NS>
+int evaluate_multi(shbim_ctx* ctx, const FarPlan& P, int kind, double* out, cudaStream_t s) {
+  constexpr int NC = NS == 12 ? 3 : 1;
+  FarState& F = *ctx->far;
+  const NearList nl = far_near(ctx, P, kind);
+  if (!nl.order) return SHBIM_OK;
+  double* part = static_cast<double*>(F.mpart);
+  k_far_m2p<T, NS><<<(unsigned)P.ngroup, 32 * kL2pWarps, 0, s>>>(P.nent, P.ent_tgt, nl, P.sd, P.Lsrc, ctx->drops_dev, F.inv_src,
+                                                               far_full(ctx), tab_of<T>(F).rec, static_cast<const T*>(F.mset),
+                                                               ctx->geo.tgt, ctx->ntarget, part);
+  SHBIM_CHECK_LAUNCH(ctx, "k_far_m2p");
+  int maxnt = 0;
+  for (const auto& d : ctx->drops) maxnt = std::max(maxnt, d.nt);
+  k_far_msum<NC><<<dim3((unsigned)((maxnt + 127) / 128), (unsigned)ctx->n_drops), 128, 0, s>>>(nl, ctx->drops_dev, part, out);
+  SHBIM_CHECK_LAUNCH(ctx, "k_far_msum");
   return SHBIM_OK;
 }
 
@@ -1436,7 +1735,9 @@ int evaluate_kind(shbim_ctx* ctx, const FarPlan& P, int kind, double* out, cudaS
   else
     k_far_l2p<T, 12><<<g, b, 0, s>>>(P.td, P.blocks, ctx->drops_dev, F.inv_tgt, far_full(ctx), tab.rec, set, ctx->geo.tgt, ctx->ntarget, out);
   SHBIM_CHECK_LAUNCH(ctx, "k_far_l2p");
-  return SHBIM_OK;
+  return kind == 1   ? evaluate_multi<T, 1>(ctx, P, kind, out, s)
+         : kind == 0 ? evaluate_multi<T, 3>(ctx, P, kind, out, s)
+                     : evaluate_multi<T, 12>(ctx, P, kind, out, s);
 }
 
 }  // namespace

@@ -181,6 +181,7 @@ struct shbim_ctx {
   shbim::PairTile* tiles_dev = nullptr;
   double* lamm1_dev = nullptr;    // lambda_j - 1 per drop
   shbim::DropDev* drops_dev = nullptr;
+  int* tgt_order = nullptr;       // [ntarget] targets of each drop, patch by patch
   double* centres_dev = nullptr;  // [n_drops][3]
   int pair_splits = 1;            // default source-split count of the layout
   int split_max = 1;              // capacity of the partial-sum buffer in splits

@@ -87,6 +87,18 @@ __device__ __forceinline__ ListSplit list_split(const NearList& nl, int i, int b
   return r;
 }
 
+// which of the warp's groups of 32 targets (slots s0 + 32 k of a drop of nt targets) entry en is summed for directly
+template <int TPT>
+__device__ __forceinline__ bool warp_near(const NearList& nl, int en, int ns, int s0, int nt, bool (&nr)[TPT]) {
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < TPT; ++k) {
+    nr[k] = s0 + 32 * k < nt && nl.direct(en, s0 / kFarGroup + k, ns);
+    any = any || nr[k];
+  }
+  return any;
+}
+
 // bx = tile * (kMaxTPT / TPT) + sub-tile; returns false for a sub-tile past the tile's last
 // target (the whole CTA then skips it, before any barrier)
 template <int TPT>
@@ -117,15 +129,17 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
   const DropDev Di = drops[i];
   const ListSplit ls = list_split(nl, i, by, nsplit);
 
+  // a warp's targets are neighbours: groups of 32 side by side
+  const int s0 = (threadIdx.x >> 5) * 32 * kTPT;
   int64_t tg[kTPT];
   bool ok[kTPT];
   double X0[kTPT][3];
   float N0[kTPT][3];
 #pragma unroll
   for (int k = 0; k < kTPT; ++k) {
-    tg[k] = tile.t0 + threadIdx.x + k * kThreads;
-    ok[k] = tg[k] < (int64_t)tile.t0 + tile.nt;
-    const int64_t t = ok[k] ? tg[k] : tile.t0;
+    const int sl = s0 + 32 * k + (threadIdx.x & 31);
+    ok[k] = sl < tile.nt;
+    const int64_t t = tg[k] = nl.tgt[tile.t0 + (ok[k] ? sl : 0)];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       X0[k][c] = tgt[c * ntarget + t];
@@ -143,6 +157,9 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
     const DropDev Dj = drops[j];
     const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
+    bool nr[kTPT];
+    const bool mine = warp_near<kTPT>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
+    if (!__syncthreads_or(mine)) continue;
     float th[kTPT][3], tl[kTPT][3];
     const double cj[3] = {Dj.cx, Dj.cy, Dj.cz};
 #pragma unroll
@@ -176,6 +193,7 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
         }
       }
       __syncthreads();
+      if (!mine) continue;
       float acc[kTPT][NC];
 #pragma unroll
       for (int k = 0; k < kTPT; ++k)
@@ -239,7 +257,8 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
 #pragma unroll
       for (int k = 0; k < kTPT; ++k)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) two_sum_acc(hi[k][c], lo[k][c], acc[k][c]);
+        for (int c = 0; c < NC; ++c)
+          if (nr[k]) two_sum_acc(hi[k][c], lo[k][c], acc[k][c]);
     }
   }
   double* P = part + (int64_t)by * NC * ntarget;
@@ -316,9 +335,9 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   const int i = tile.drop;
   const DropDev Di = drops[i];
   const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
-  const int64_t tg = tile.t0 + threadIdx.x;
+  const int s0 = (int)threadIdx.x & ~31;
   const bool ok = (int)threadIdx.x < tile.nt;
-  const int64_t t = ok ? tg : tile.t0;
+  const int64_t tg = nl.tgt[tile.t0 + (ok ? (int)threadIdx.x : 0)], t = tg;
   double X0[3];
   df N0[3];
 #pragma unroll
@@ -332,6 +351,9 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
     const DropDev Dj = drops[j];
     const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
+    bool nr[1];
+    const bool mine = warp_near<1>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
+    if (!__syncthreads_or(mine)) continue;
     const df T[3] = {dfl::from_double(X0[0] - Dj.cx), dfl::from_double(X0[1] - Dj.cy),
                      dfl::from_double(X0[2] - Dj.cz)};
     for (int64_t base = rg.a; base < rg.b; base += kTile) {
@@ -363,6 +385,7 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
         }
       }
       __syncthreads();
+      if (!mine) continue;
       for (int e = 0; e < cnt; ++e) {
         const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
         if constexpr (!stokes_kind(KIND))
@@ -404,9 +427,9 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   const int i = tile.drop;
   const DropDev Di = drops[i];
   const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
-  const int64_t tg = tile.t0 + threadIdx.x;
+  const int s0 = (int)threadIdx.x & ~31;
   const bool ok = (int)threadIdx.x < tile.nt;
-  const int64_t t = ok ? tg : tile.t0;
+  const int64_t tg = nl.tgt[tile.t0 + (ok ? (int)threadIdx.x : 0)], t = tg;
   double X0[3];
   df N0[3];
 #pragma unroll
@@ -420,6 +443,9 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
     const DropDev Dj = drops[j];
     const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
+    bool nr[1];
+    const bool mine = warp_near<1>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
+    if (!__syncthreads_or(mine)) continue;
     const bool far = dq_far[(int64_t)i * n_drops + j] != 0;
     const double cj[3] = {Dj.cx, Dj.cy, Dj.cz};
     float Th[3], Tl[3];
@@ -461,6 +487,7 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
         }
       }
       __syncthreads();
+      if (!mine) continue;
       const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
       if (far) {
         for (int e = 0; e < cnt; ++e) {
@@ -503,14 +530,15 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
   const int i = tile.drop;
   const DropDev Di = drops[i];
   const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
+  const int s0 = (threadIdx.x >> 5) * 32 * kTPT;
   int64_t tg[kTPT];
   bool ok[kTPT];
   double X0[kTPT][3], N0[kTPT][3], acc[kTPT][NC];
 #pragma unroll
   for (int k = 0; k < kTPT; ++k) {
-    tg[k] = tile.t0 + threadIdx.x + k * kThreads;
-    ok[k] = tg[k] < (int64_t)tile.t0 + tile.nt;
-    const int64_t t = ok[k] ? tg[k] : tile.t0;
+    const int sl = s0 + 32 * k + (threadIdx.x & 31);
+    ok[k] = sl < tile.nt;
+    const int64_t t = tg[k] = nl.tgt[tile.t0 + (ok[k] ? sl : 0)];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       X0[k][c] = tgt[c * ntarget + t];
@@ -524,6 +552,9 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
     const DropDev Dj = drops[j];
     const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
+    bool nr[kTPT];
+    const bool mine = warp_near<kTPT>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
+    if (!__syncthreads_or(mine)) continue;
     for (int64_t base = rg.a; base < rg.b; base += kTile) {
       const int cnt = (int)min((int64_t)kTile, rg.b - base);
       __syncthreads();
@@ -544,10 +575,12 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
         }
       }
       __syncthreads();
+      if (!mine) continue;
       for (int e = 0; e < cnt; ++e) {
         const double sx = sh[0][e], sy = sh[1][e], sz = sh[2][e];
 #pragma unroll
         for (int k = 0; k < kTPT; ++k) {
+          if (!nr[k]) continue;              // uniform over the warp
           const double dx = X0[k][0] - sx, dy = X0[k][1] - sy, dz = X0[k][2] - sz;
           const double r2 = dx * dx + dy * dy + dz * dz;
           if (KIND == LSL) {
@@ -747,7 +780,7 @@ int launch_pairs(shbim_ctx* ctx, bool has_f, bool has_u, double* out, cudaStream
   const FarPlan* far = far_plan(ctx, KIND);
   if (!ctx->far) return fail(ctx, SHBIM_ERR_ARG, "no drop pair lists: the last shbim_set_drops failed");
   const FarPlan& plan = far ? *far : far_all(ctx);
-  const NearList& nl = plan.near;
+  const NearList nl = far ? far_near(ctx, plan, KIND) : plan.near;
   if (!nl.off) return fail(ctx, SHBIM_ERR_ARG, "no drop pair lists: the last shbim_set_drops failed");
   int rc;
   if (far && (rc = far_expand(ctx, *far, KIND, s))) return rc;
@@ -908,7 +941,7 @@ double pairs_work(const shbim_ctx* ctx, int kind) {
   static const double kFlops[5] = {19.0, 11.0, 42.0, 29.0, 30.0};
   if (kind < 0 || kind > 4 || ctx->n_drops < 2 || !ctx->far) return 0.0;
   const FarPlan* far = far_plan(ctx, kind);
-  return kFlops[kind] * (far ? far->direct_pairs : far_all(ctx).direct_pairs);
+  return kFlops[kind] * (far ? far_direct_pairs(ctx, *far, kind) : far_all(ctx).direct_pairs);
 }
 
 }  // namespace shbim
