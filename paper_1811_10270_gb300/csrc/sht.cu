@@ -21,19 +21,22 @@ struct FieldList {
   int64_t coef[kMaxFields];
   int64_t val[kMaxFields];
 };
-struct ItemAt {
-  int64_t coef, val;
-  int drop;           // for the per-drop factor
-};
-__device__ __forceinline__ ItemAt item_at(const DropList& L, int item, int kpd, int64_t coef_stride, int64_t val_stride,
-                                          int64_t drop_stride) {
-  const int dl = item / kpd, ci = item - dl * kpd;
-  if (!L.idx) return ItemAt{(int64_t)item * coef_stride, (int64_t)dl * drop_stride + (int64_t)ci * val_stride, dl};
-  return ItemAt{(int64_t)kpd * L.coef_off[dl] + (int64_t)ci * coef_stride, L.val_off[dl] + (int64_t)ci * val_stride, L.idx[dl]};
+// Each offset where it is used, so that the loads of a list do not stand before those of the tables.
+__device__ __forceinline__ int64_t item_coef(const DropList& L, int item, int kpd, int64_t coef_stride) {
+  return L.idx ? (int64_t)kpd * L.coef_off[item / kpd] + (int64_t)(item % kpd) * coef_stride : (int64_t)item * coef_stride;
 }
-__device__ __forceinline__ ItemAt item_at(const FieldList& L, int item, int, int64_t, int64_t, int64_t) {
-  return ItemAt{L.coef[item], L.val[item], 0};
+__device__ __forceinline__ int64_t item_coef(const FieldList& L, int item, int, int64_t) { return L.coef[item]; }
+// values of a drop's first component; component c lies c strides on
+__device__ __forceinline__ int64_t drop_val(const DropList& L, int dl, int64_t drop_stride) {
+  return L.idx ? L.val_off[dl] : (int64_t)dl * drop_stride;
 }
+__device__ __forceinline__ int64_t drop_val(const FieldList& L, int dl, int64_t) { return L.val[dl]; }
+__device__ __forceinline__ int64_t item_val(const DropList& L, int64_t item, int kpd, int64_t val_stride) {
+  return L.idx ? L.val_off[item / kpd] + (item % kpd) * val_stride : item * val_stride;
+}
+__device__ __forceinline__ int64_t item_val(const FieldList& L, int64_t item, int, int64_t) { return L.val[item]; }
+__device__ __forceinline__ int drop_index(const DropList& L, int dl) { return L.idx ? L.idx[dl] : dl; }
+__device__ __forceinline__ int drop_index(const FieldList&, int) { return 0; }
 
 // kinds bitmask -> table index of the slot-th set bit
 __device__ __forceinline__ int kind_of_slot(int kinds, int slot) {
@@ -58,10 +61,12 @@ __global__ void k_synth(const double* __restrict__ coef, int64_t coef_stride, in
                         float* __restrict__ out32lo, int kpd, int64_t drop_stride,
                         const double* __restrict__ alpha_drop, const __grid_constant__ List L) {
   extern __shared__ double sm[];
-  const ItemAt at = item_at(L, blockIdx.x, kpd, coef_stride, item_stride, drop_stride);
-  const int64_t obase = at.val;
-  if (scale) scale += at.val - (int64_t)(blockIdx.x % kpd) * item_stride;   // one scale per drop, not per component
-  if (alpha_drop) alpha *= alpha_drop[at.drop];
+  const int item = blockIdx.x;
+  const int dl = item / kpd, ci = item - dl * kpd;
+  const int64_t dbase = drop_val(L, dl, drop_stride);
+  const int64_t obase = dbase + (int64_t)ci * item_stride;
+  if (scale) scale += dbase;        // one scale per drop, not per component
+  if (alpha_drop) alpha *= alpha_drop[drop_index(L, dl)];
   const int j = blockIdx.y;
   const int nk = __popc(kinds);
   const int N = 2 * q + 2;
@@ -73,7 +78,7 @@ __global__ void k_synth(const double* __restrict__ coef, int64_t coef_stride, in
     tc[i] = trig[i];
     ts[i] = trig[N + i];
   }
-  const double* c = coef + at.coef;
+  const double* c = coef + item_coef(L, item, kpd, coef_stride);
   const int nt = (p + 1) * (p + 2) / 2;
   const double* T = alf + (int64_t)j * kNumTab * nt;
   const int ntask = nk * 2 * P1;
@@ -308,7 +313,7 @@ __global__ void k_analysis_fourier(const double* __restrict__ vals, int64_t val_
   double* row = sm;
   double* tc = row + N;
   double* ts = tc + N;
-  const double* v = vals + item_at(L, item, kpd, 0, val_stride, (int64_t)kpd * val_stride).val + (int64_t)j * N;
+  const double* v = vals + item_val(L, item, kpd, val_stride) + (int64_t)j * N;
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     row[i] = v[i];
     tc[i] = trig[i];
@@ -358,7 +363,7 @@ __global__ void k_analysis_fourier4(const double* __restrict__ vals, int64_t val
     const int r = e / N, k = e - r * N;
     const int64_t row = r0 + r;
     const int64_t item = row / (q + 1), j = row - item * (q + 1);
-    const int64_t ib = item_at(L, (int)item, kpd, 0, val_stride, (int64_t)kpd * val_stride).val;
+    const int64_t ib = item_val(L, item, kpd, val_stride);
     R[r * 2 * N + k] = vals[ib + j * N + k];
   }
   __syncthreads();
@@ -430,7 +435,7 @@ __global__ void k_analysis_legendre(const double* __restrict__ F, int p, int q,
     ac = fma(Fi[(int64_t)j * 2 * P1 + m], a, ac);
     as = fma(Fi[(int64_t)j * 2 * P1 + P1 + m], a, as);
   }
-  double* c = coef + item_at(L, item, kpd, coef_stride, 0, 0).coef;
+  double* c = coef + item_coef(L, item, kpd, coef_stride);
   if (m == 0) {
     c[n * n + n] = ac;
   } else {
