@@ -675,7 +675,7 @@ int shbim_eval_electric(shbim_ctx* ctx, int which, const double* dens_dev, doubl
   if (br.join) SHBIM_CUDA(ctx, cudaEventRecord(br.join, br.side));
   {
     TimeScope ts(ctx, pair_class(ctx), s);
-    ts.work = pairs_work(ctx, which == SHBIM_LAPLACE_SL ? 1 : 0);
+    if (ts.b) ts.work = pairs_work(ctx, which == SHBIM_LAPLACE_SL ? 1 : 0);
     if ((rc = pairs_laplace(ctx, which, vals, s, br.join))) return rc;
   }
   if (out_kind == SHBIM_OUT_COEF) {
@@ -736,7 +736,7 @@ int shbim_eval_stokes(shbim_ctx* ctx, const double* f_dev, const double* u_dev, 
   if (br.join) SHBIM_CUDA(ctx, cudaEventRecord(br.join, br.side));
   {
     TimeScope ts(ctx, pair_class(ctx), s);
-    ts.work = pairs_work(ctx, f_dev && u_dev ? 2 : (f_dev ? 3 : 4));
+    if (ts.b) ts.work = pairs_work(ctx, f_dev && u_dev ? 2 : (f_dev ? 3 : 4));
     if ((rc = pairs_stokes(ctx, f_dev != nullptr, u_dev != nullptr, vals, s, br.join))) return rc;
   }
   if (out_kind == SHBIM_OUT_COEF) {

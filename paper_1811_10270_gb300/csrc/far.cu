@@ -1588,16 +1588,19 @@ const FarPlan& far_all(const shbim_ctx* ctx) { return ctx->far->plan[kFarPlans];
 // and orders of uneven length; `base` for the powers of x + iy and the sums over warps. In FP64 four times that: six
 // drops of degree 16, double layer, solve of eight applications: 16.9 ms without these expansions, 16.3 at one
 // time, 15.7 at four. 64 drops of degree 16 to 48, without and with them: Stokeslet in double-float 35.5 and 24.2 ms,
-// stresslet FP32 10.2 and 9.0, double layer FP32 3.83 and 2.88; twice the instructions here change nothing.
+// stresslet FP32 10.2 and 9.0, double layer FP32 3.83 and 2.88; twice the instructions here change nothing. Below 0.1 ms
+// of direct sums the three launches cost more than they give (40 drops of degree 11, 3e9: 1.00 and 1.03 ms).
 NearList far_near(const shbim_ctx* ctx, const FarPlan& P, int kind) {
   NearList nl = P.near;
   const int ns = kSets[kind], pr = ctx->opts.precision;
+  const double direct = (pr == SHBIM_PREC_FP64 ? kDirect64 : (pr == SHBIM_PREC_DF64 ? kDirectDf : kDirect32))[kind];
+  if (P.direct_pairs * direct < 4e9) nl.order = nullptr;
   FarReach& r = nl.reach;
   if (pr == SHBIM_PREC_FP64) {
-    r = FarReach{kFarLmax, 384 * (3 + 2 * ns), 0, 120000, (int)kDirect64[kind]};
+    r = FarReach{kFarLmax, 384 * (3 + 2 * ns), 0, 120000, (int)direct};
   } else {
     const bool fp32 = pr == SHBIM_PREC_FP32_COMP;
-    r = FarReach{fp32 ? 12 : 36, 50 + 36 * ns, 9 + 6 * ns, 15000, (int)(fp32 ? kDirect32 : kDirectDf)[kind]};
+    r = FarReach{fp32 ? 12 : 36, 50 + 36 * ns, 9 + 6 * ns, 15000, (int)direct};
   }
   return nl;
 }
@@ -1683,7 +1686,7 @@ int expand(shbim_ctx* ctx, const FarPlan& P, int kind, cudaStream_t s) {
   else
     k_far_lset<T, 12><<<dim3(lb, nd), 128, 0, s>>>(P.td, F.inv_tgt, tab, npot, loc, set);
   SHBIM_CHECK_LAUNCH(ctx, "k_far_lset");
-  if (P.near.order) {
+  if (far_near(ctx, P, kind).order) {
     T* ms = static_cast<T*>(F.mset);
     if (kind == 1)
       k_far_mset<T, 1><<<dim3(lb, nd), 128, 0, s>>>(P.sd, P.Lsrc, F.inv_src, tab, npot, mom, ms);
