@@ -14,7 +14,8 @@ residuals). Every operator application is one launch per kernel kind over all dr
 drops of uneven degree), and every GMRES operator application a replayed CUDA graph.
 
 Metric: target-source kernel pairs per second = operator applications in the step x
-sum_i N_t(i) x sum_j N_s(j) / step time (self pairs counted as N_t N_s rotated pairs), and the time to a
+sum_i N_t(i) x sum_j N_s(j) / step time (self pairs counted as N_t N_s rotated pairs; pairs of drops far
+enough apart count as well, though their sums are formed by expansions and not pair by pair), and the time to a
 1e-8 residual of the electric and Stokes solves, mixed precision against plain FP64 GMRES.
 
 --impl reference times the FP64 CPU oracle on a bounded sample of the same workload.
@@ -43,12 +44,12 @@ UNIT = "pairs/s"
 FP64_NOMINAL_TFLOPS = 1.25      # GB300 FP64 rate (vector and tensor), 1/64 of the FP32 lane rate
 # DRAM bytes (read + write) per launch of the pair kernel classes from one single-pass ncu capture of the
 # same kernels on this workload (profiles/); None where the kernel has changed since its capture.
-TRAFFIC = {"pairs_fp32": 11.9e6, "pairs_fp64class": None}
+TRAFFIC = {"pairs_fp32": None, "pairs_fp64class": None}
 # the last capture of a class whose kernel has changed since (reported beside the null, not as traffic)
 TRAFFIC_BEFORE_CHANGE = {"pairs_fp64class": {
     "bytes_per_launch": 46.3e6,
-    "changed_since": "k_pairs_dq's powers of 1/r now come from the renormalised pair (arithmetic only, the "
-                     "same loads); counters not taken again"}}
+    "changed_since": "far drops and far sides of close drops now go through expansions, whose kernels the class's "
+                     "time includes; counters not taken again"}}
 WORKLOAD_NAME = ("config 3: 64 drops, p in {16,24,32,48} (seed 3), radii U(0.8,1.2), 12^3 box, gaps >= 0.2, "
                  "lambda U(0.5,10), R=2, Q=0.5, Ca_E=0.1, Langmuir beta=0.2 x_s=0.5, E=z; one midpoint time "
                  "step (Algorithm 1) = 2 x (geometry + singular rows + electric solve + potential + forces + "
@@ -178,7 +179,8 @@ def roofline(cls_ms, cls_n, cls_work, cfg, peaks, dom=None):
                     "peak_source": "FP32 FMA rate measured by this run's probe (shbim_probe_peak, 2 flops per FMA; "
                                    "MEASURED_PEAKS.json has no FP32 figure): of measured",
                     "work": "flops of the kernel formulas per target-source pair (Laplace SL 11, DL 19, Stokeslet 29, "
-                            "stresslet 30, both 42) x pairs of different drops per launch",
+                            "stresslet 30, both 42) x pairs summed directly; the time includes the expansions "
+                            "that take the other pairs",
                     "kernel": "k_pairs32 / k_pairs32_queue (FP32, compensated)" if dom == "pairs_fp32"
                               else "k_pairs_dq (double-float terms on quantised positions, FP32 pipe)"})
         if dom == "pairs_fp64class":
@@ -361,7 +363,7 @@ def run_own(args):
                    "sources": sum((2 * p + 2) * (4 * p + 4) for p in ps),
                    "dt": args.dt, "precision": "mixed: FP32 compensated pair sums inside GMRES, double-float (FP64-class) "
                    "residuals and one-shot applications, FP64 Arnoldi",
-                   "pairs_per_application": P,
+                   "pairs_per_application": P, "pairs_of_far_drops": "through multipole and local expansions",
                    "applications_per_step": apps_total / max(1, args.steps) / max(1, world),
                    "gmres_iters_per_step": stats[-1][2], "step_error_estimate": stats[-1][1],
                    "l2": "inputs larger than L2: the singular rows alone are ~10 GB, no flush needed",

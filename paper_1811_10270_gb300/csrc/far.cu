@@ -13,17 +13,19 @@
 //      Dq the fixed matrix of Rx(pi/2)), translated along it order by order, rotated back;
 //   3. k_far_lsum, k_far_lset: a drop's local expansion (sum over its far drops in a fixed order) and the
 //      expansions of the derivatives its targets need;
-//   4. k_far_l2p: values at the targets, added to the operator values.
+//   4. k_far_l2p: values at the targets, added to the operator values;
+//   5. k_far_mset, k_far_m2p, k_far_msum: drops too close for this, whose targets far enough from the source drop's
+//      centre take its multipole expansion itself; the direct sums of pairs.cu leave those targets out.
 // What it costs: O(L^2) per source and target and O(L^3) per pair of drops instead of the product of
-// their node counts. Whole operator applications at 64 drops of degree 16 to 48 (7.8e10 pairs, 95 % of them far), every
-// pair directly -> expansions: Laplace double layer FP32 50.4 -> 4.2 ms, stresslet FP32 73.7 -> 11.5 ms, Stokeslet
-// double-float 432 -> 38.8 ms; what remains is the direct sums of close drops (25 ms of the 38.8, 3.6 of the 11.5), the
-// singular rows (3.8) and k_far_p2m (4.6, 2.6). Against native FP64 direct sums the double-float results are 4 to 60
+// their node counts. Whole operator applications at 64 drops of degree 16 to 48 (6.6e10 pairs, 95 % of them far), every
+// pair directly -> expansions: Laplace double layer FP32 50.4 -> 3.2 ms, stresslet FP32 73.7 -> 9.7 ms, Stokeslet
+// double-float 432 -> 27.6 ms; what remains is the direct sums (10.7 ms of the 27.6, 1.8 of the 9.7), the singular
+// rows (2.2) and k_far_p2m (4.6, 2.6). Against native FP64 direct sums the double-float results are 4 to 60
 // times closer than the direct double-float sums, the FP32 ones as close or closer.
 //
 // Orders: the truncation error of a pair with source radius a, target radius b and centre distance D is at
 // most sum|q| (L+1)^g rho^(L+1) / (D-a-b), rho = max(a/(D-b), b/(D-a)), g the number of derivatives taken; L is
-// the smallest order that puts it below 3e-15 (FP64 and double-float sums) or 1e-9 (FP32 sums, whose own
+// the smallest order that puts it below 3e-15 (FP64 and double-float sums) or 1e-8 (FP32 sums, whose own
 // error is 3e-8). A pair that would need more than the level's largest order is summed directly.
 //
 // Arithmetic: native FP64 in FP64 mode, double-float on the FP32 pipe otherwise (a multiply-add costs 12
