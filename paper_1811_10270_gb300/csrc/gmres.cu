@@ -787,8 +787,12 @@ int update_x(shbim_ctx* ctx, cudaStream_t s) {
 }  // namespace
 
 // Basis of the Stokes preconditioner for the current geometry (k_prec_basis). A shape whose modes are linearly
-// dependent or not finite is refused before anything else is built from it.
+// dependent or not finite is refused before anything else is built from it; the modes do not hold the degree-0
+// coefficients (the translations are projected out of them), so these are looked at as the drop's centre.
 int build_stokes_preconditioner(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
+  for (const Drop& d : ctx->drops)
+    if (!std::isfinite(d.centre[0]) || !std::isfinite(d.centre[1]) || !std::isfinite(d.centre[2]))
+      return fail(ctx, SHBIM_ERR_ARG, "degenerate drop shape for the Stokes preconditioner: its centre is not finite");
   const int64_t nc_all = ctx->ncoef;
   if (!ctx->prec_basis) {
     if (cudaMalloc(&ctx->prec_basis, (size_t)21 * nc_all * sizeof(double)) != cudaSuccess ||

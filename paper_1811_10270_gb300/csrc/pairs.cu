@@ -899,7 +899,8 @@ int build_pair_lists(shbim_ctx* ctx, cudaStream_t s) {
     std::memcpy(&e, &bits[i], sizeof(e));
     ext[i] = (double)e;
   }
-  // the lists stand for any extents (a non-finite one makes every pair of its drop direct)
+  // the lists stand for any extents: a NaN node does not count in them (k_extent) and an infinite one makes every pair
+  // of its drop direct; such a shape is refused by build_stokes_preconditioner, or below
   if (int rc = build_far(ctx, ext, s)) return rc;
   double B = 0.0;
   for (int i = 0; i < nd; ++i)
