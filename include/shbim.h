@@ -121,7 +121,9 @@ int shbim_set_R(shbim_ctx* ctx, double R);
  * Allocates device memory (SHBIM_ERR_NOMEM on failure). Synchronises `stream` on entry,
  * reads the degree-0 position coefficients back to the host (the drop centres) and
  * synchronises again while building; the last kernels it queues on `stream` may still be
- * running when it returns. Replaces any previous drop set of the context. */
+ * running when it returns. A call that fails after its arguments have been checked leaves no drops set
+ * if it was for other degrees than the one before, and else a context that refuses sums between
+ * drops until a call succeeds. Replaces any previous drop set of the context. */
 int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const double* lambda_host,
                     const double* xcoef_dev, void* stream);
 

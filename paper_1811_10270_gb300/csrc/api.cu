@@ -33,11 +33,8 @@ __global__ void k_centres(const double* __restrict__ x, int nd, double s4pi, Dro
   drops[i].cz = centres[3 * i + 2] = c[2 * nc] / s4pi;
 }
 
-// Shape-dependent state for the current layout: drop centres (x_00 / sqrt(4 pi), the mean
-// position over the parameter sphere), the device drop table, geometry and singular rows.
-int rebuild_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
-  ctx->geom_version++;  // invalidates captured operator graphs
-  ctx->xcoef_cur = xcoef_dev;
+namespace {
+int build_shapes(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
   std::vector<DropDev> dd(ctx->n_drops);
   for (int i = 0; i < ctx->n_drops; ++i) {
     const Drop& d = ctx->drops[i];
@@ -64,10 +61,29 @@ int rebuild_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
   if ((rc = build_near(ctx, xcoef_dev, s))) return rc;
   return SHBIM_OK;
 }
+}  // namespace
+
+// Shape-dependent state for the current layout: drop centres (x_00 / sqrt(4 pi), the mean
+// position over the parameter sphere), the device drop table, geometry and singular rows. Where a step fails, part
+// of the state is of these shapes and part of earlier ones: the sums between drops are refused until a call succeeds.
+int rebuild_geometry(shbim_ctx* ctx, const double* xcoef_dev, cudaStream_t s) {
+  ctx->geom_version++;  // invalidates captured operator graphs
+  ctx->xcoef_cur = xcoef_dev;
+  far_forget(ctx);
+  const int rc = build_shapes(ctx, xcoef_dev, s);
+  if (rc) {
+    far_forget(ctx);
+    ctx->near.npairs = 0;
+  }
+  return rc;
+}
 
 namespace {
 
 void free_drop_state(shbim_ctx* ctx) {
+  ctx->geom_version++;   // captured operator graphs, drop pair lists and near pairs refer to the buffers freed here
+  far_forget(ctx);
+  ctx->near.npairs = 0;
   for (auto& d : ctx->drops) {
     cudaFree(d.rows_lap);
     cudaFree(d.rows_sto);
@@ -357,6 +373,16 @@ int shbim_sizes(shbim_ctx* ctx, int64_t* nc, int64_t* nt, int64_t* ns) {
   return SHBIM_OK;
 }
 
+}  // extern "C"
+
+namespace shbim {
+namespace {
+int new_layout(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const double* lambda_host, cudaStream_t s);
+}  // namespace
+}  // namespace shbim
+
+extern "C" {
+
 int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const double* lambda_host,
                     const double* xcoef_dev, void* stream) {
   if (!ctx) return SHBIM_ERR_ARG;
@@ -385,6 +411,19 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
     return rebuild_geometry(ctx, xcoef_dev, s);
   }
   free_drop_state(ctx);
+  int rc = new_layout(ctx, n_drops, p_host, lambda_host, s);
+  if (!rc) rc = rebuild_geometry(ctx, xcoef_dev, s);
+  if (rc) free_drop_state(ctx);   // no half-made layout stays behind: no drops are set
+  return rc;
+}
+
+}  // extern "C"
+
+namespace shbim {
+namespace {
+
+// Buffers and tables of a layout, in a context without drops
+int new_layout(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const double* lambda_host, cudaStream_t s) {
   int rc;
   // tables per distinct degree (kept across calls)
   for (int i = 0; i < n_drops; ++i) {
@@ -542,8 +581,13 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
       SHBIM_CUDA(ctx, cudaMemset(ctx->pair_queue, 0, 2 * sizeof(int)));
     }
   }
-  return rebuild_geometry(ctx, xcoef_dev, s);
+  return SHBIM_OK;
 }
+
+}  // namespace
+}  // namespace shbim
+
+extern "C" {
 
 int shbim_target_geometry(shbim_ctx* ctx, double* out_dev, void* stream) {
   if (!ctx || !out_dev) return SHBIM_ERR_ARG;
@@ -616,6 +660,8 @@ struct Branches {
   cudaEvent_t coarse = nullptr, join = nullptr;
 };
 
+constexpr const char* kNoLists = "no drop pair lists: the last shbim_set_drops failed";
+
 // timing class of the all-pairs sums at the context's precision
 int pair_class(const shbim_ctx* ctx) {
   return ctx->opts.precision == SHBIM_PREC_FP32_COMP ? SHBIM_K_PAIRS : SHBIM_K_PAIRS_FP64CLASS;
@@ -642,6 +688,7 @@ int shbim_eval_electric(shbim_ctx* ctx, int which, const double* dens_dev, doubl
                         void* stream) {
   if (!ctx) return SHBIM_ERR_ARG;
   if (ctx->n_drops == 0) return fail(ctx, SHBIM_ERR_ARG, "no drops set");
+  if (!far_ready(ctx)) return fail(ctx, SHBIM_ERR_ARG, kNoLists);
   if (which != SHBIM_LAPLACE_DL && which != SHBIM_LAPLACE_SL) return fail(ctx, SHBIM_ERR_ARG, "bad kernel");
   if (out_kind != SHBIM_OUT_GRID && out_kind != SHBIM_OUT_COEF) return fail(ctx, SHBIM_ERR_ARG, "bad out kind");
   if (!dens_dev || !out_dev) return fail(ctx, SHBIM_ERR_ARG, "null pointer");
@@ -693,6 +740,7 @@ int shbim_eval_stokes(shbim_ctx* ctx, const double* f_dev, const double* u_dev, 
                       int out_kind, void* stream) {
   if (!ctx) return SHBIM_ERR_ARG;
   if (ctx->n_drops == 0) return fail(ctx, SHBIM_ERR_ARG, "no drops set");
+  if (!far_ready(ctx)) return fail(ctx, SHBIM_ERR_ARG, kNoLists);
   if (!f_dev && !u_dev) return fail(ctx, SHBIM_ERR_ARG, "need f or u");
   if (out_kind != SHBIM_OUT_GRID && out_kind != SHBIM_OUT_COEF) return fail(ctx, SHBIM_ERR_ARG, "bad out kind");
   if (!out_dev) return fail(ctx, SHBIM_ERR_ARG, "null output");

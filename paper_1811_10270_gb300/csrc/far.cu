@@ -1330,6 +1330,11 @@ void far_free(shbim_ctx* ctx) {
   ctx->far = nullptr;
 }
 
+void far_forget(shbim_ctx* ctx) {
+  if (!ctx->far) return;
+  for (auto& P : ctx->far->plan) P = FarPlan{};
+}
+
 // Lists of direct and far drop pairs of the current geometry, per truncation level and number of
 // derivatives, and the workspaces of their expansions. ext holds per drop the largest |x - c| of the
 // sources, then of the targets.
@@ -1585,6 +1590,8 @@ const FarPlan* far_plan(const shbim_ctx* ctx, int kind) {
 }
 
 const FarPlan& far_all(const shbim_ctx* ctx) { return ctx->far->plan[kFarPlans]; }
+
+bool far_ready(const shbim_ctx* ctx) { return ctx->n_drops < 2 || (ctx->far && far_all(ctx).near.off); }
 
 // Instructions of an expansion's value: recurrence and 2 NS multiply-adds per (n, m), half as much again for reads
 // and orders of uneven length; `base` for the powers of x + iy and the sums over warps. In FP64 four times that: six

@@ -124,11 +124,15 @@ struct FarState {
 
 int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s);
 void far_free(shbim_ctx* ctx);
+// empties every plan (the workspaces stay): what comes before build_far may fail
+void far_forget(shbim_ctx* ctx);
 // whether the expansions pay for this kind of sum at this precision
 bool far_worth(const FarPlan& P, int precision, int kind);
 // the plan of a kind (0 DL, 1 SL, 2 S + D, 3 S, 4 D) at the context's precision, null: all pairs directly
 const FarPlan* far_plan(const shbim_ctx* ctx, int kind);
 const FarPlan& far_all(const shbim_ctx* ctx);
+// the lists of the current shapes have been made (or none are needed)
+bool far_ready(const shbim_ctx* ctx);
 // the plan's lists with the rule of a kind at the context's precision
 NearList far_near(const shbim_ctx* ctx, const FarPlan& P, int kind);
 // target-source pairs of the plan that the kind sums directly (reads the orders back)

@@ -781,10 +781,8 @@ int launch_pairs(shbim_ctx* ctx, bool has_f, bool has_u, double* out, cudaStream
   }
   // well-separated drop pairs through expansions (far.cu), where they pay; the rest directly
   const FarPlan* far = far_plan(ctx, KIND);
-  if (!ctx->far) return fail(ctx, SHBIM_ERR_ARG, "no drop pair lists: the last shbim_set_drops failed");
   const FarPlan& plan = far ? *far : far_all(ctx);
   const NearList nl = far ? far_near(ctx, plan, KIND) : plan.near;
-  if (!nl.off) return fail(ctx, SHBIM_ERR_ARG, "no drop pair lists: the last shbim_set_drops failed");
   int rc;
   if (far && (rc = far_expand(ctx, *far, KIND, s))) return rc;
   if (plan.direct_pairs == 0.0) {
