@@ -698,6 +698,8 @@ int shbim_eval_electric(shbim_ctx* ctx, int which, const double* dens_dev, doubl
   int rc;
   ctx->applications++;
   double* vals = out_kind == SHBIM_OUT_GRID ? out_dev : ctx->grid_out;
+  // may read back from the device (once per geometry): not between the events of a timed range
+  const double work = timed(ctx, s) ? pairs_work(ctx, which == SHBIM_LAPLACE_SL ? 1 : 0) : 0.0;
   Branches br;
   if ((rc = fork_branches(ctx, s, &br))) return rc;
   {
@@ -722,7 +724,7 @@ int shbim_eval_electric(shbim_ctx* ctx, int which, const double* dens_dev, doubl
   if (br.join) SHBIM_CUDA(ctx, cudaEventRecord(br.join, br.side));
   {
     TimeScope ts(ctx, pair_class(ctx), s);
-    if (ts.b) ts.work = pairs_work(ctx, which == SHBIM_LAPLACE_SL ? 1 : 0);
+    ts.work = work;
     if ((rc = pairs_laplace(ctx, which, vals, s, br.join))) return rc;
   }
   if (out_kind == SHBIM_OUT_COEF) {
@@ -751,6 +753,7 @@ int shbim_eval_stokes(shbim_ctx* ctx, const double* f_dev, const double* u_dev, 
   int rc;
   ctx->applications++;
   double* vals = out_kind == SHBIM_OUT_GRID ? out_dev : ctx->grid_out;
+  const double work = timed(ctx, s) ? pairs_work(ctx, f_dev && u_dev ? 2 : (f_dev ? 3 : 4)) : 0.0;
   Branches br;
   if ((rc = fork_branches(ctx, s, &br))) return rc;
   {
@@ -784,7 +787,7 @@ int shbim_eval_stokes(shbim_ctx* ctx, const double* f_dev, const double* u_dev, 
   if (br.join) SHBIM_CUDA(ctx, cudaEventRecord(br.join, br.side));
   {
     TimeScope ts(ctx, pair_class(ctx), s);
-    if (ts.b) ts.work = pairs_work(ctx, f_dev && u_dev ? 2 : (f_dev ? 3 : 4));
+    ts.work = work;
     if ((rc = pairs_stokes(ctx, f_dev != nullptr, u_dev != nullptr, vals, s, br.join))) return rc;
   }
   if (out_kind == SHBIM_OUT_COEF) {
@@ -805,11 +808,14 @@ int shbim_eval_stokes(shbim_ctx* ctx, const double* f_dev, const double* u_dev, 
 
 namespace shbim {
 
-TimeScope::TimeScope(shbim_ctx* c, int k, cudaStream_t st) : ctx(c), cls(k), s(st) {
-  if (!ctx->timing) return;
-  // launches being captured into a graph are not timed (their replays run as one graph launch)
+// launches being captured into a graph are not timed (their replays run as one graph launch)
+bool timed(const shbim_ctx* ctx, cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return;
+  return ctx->timing && cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+}
+
+TimeScope::TimeScope(shbim_ctx* c, int k, cudaStream_t st) : ctx(c), cls(k), s(st) {
+  if (!timed(ctx, s)) return;
   cudaEvent_t a;
   if (ctx->event_pool.empty()) {
     cudaEventCreate(&a);

@@ -1615,6 +1615,8 @@ NearList far_near(const shbim_ctx* ctx, const FarPlan& P, int kind) {
 }
 
 double far_direct_pairs(const shbim_ctx* ctx, const FarPlan& P, int kind) {
+  const int pr = ctx->opts.precision;
+  if (P.counted[pr][kind]) return P.count[pr][kind];
   const NearList nl = far_near(ctx, P, kind);
   if (!nl.order) return P.direct_pairs;
   std::vector<unsigned char> L((size_t)P.ngroup);
@@ -1630,7 +1632,8 @@ double far_direct_pairs(const shbim_ctx* ctx, const FarPlan& P, int kind) {
       if (L[f] == kNoReach || !nl.reach.worth(L[f], ns))
         n += (double)ns * std::min<int64_t>(kFarGroup, nt - (f - P.h_goff[en]) * kFarGroup);
   }
-  return n;
+  P.counted[pr][kind] = true;
+  return P.count[pr][kind] = n;
 }
 
 namespace {

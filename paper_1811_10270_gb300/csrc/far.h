@@ -102,6 +102,9 @@ struct FarPlan {
   unsigned char* order = nullptr;     // [ngroup]
   std::vector<int> h_drop, h_tgt;     // host copies of the lists
   std::vector<int64_t> h_goff;
+  // pairs summed directly, by [precision][kind], once they have been asked for
+  mutable bool counted[3][5] = {};
+  mutable double count[3][5] = {};
 };
 
 struct FarState {
@@ -135,7 +138,7 @@ const FarPlan& far_all(const shbim_ctx* ctx);
 bool far_ready(const shbim_ctx* ctx);
 // the plan's lists with the rule of a kind at the context's precision
 NearList far_near(const shbim_ctx* ctx, const FarPlan& P, int kind);
-// target-source pairs of the plan that the kind sums directly (reads the orders back)
+// target-source pairs of the plan that the kind sums directly (reads the orders back, once per geometry)
 double far_direct_pairs(const shbim_ctx* ctx, const FarPlan& P, int kind);
 // moments, translations and local expansions from the strengths in dens_up*; then their values at the targets
 int far_expand(shbim_ctx* ctx, const FarPlan& P, int kind, cudaStream_t s);

@@ -402,6 +402,8 @@ int cuda_fail(shbim_ctx* ctx, cudaError_t e, const char* what);
     if (e_ != cudaSuccess) return ::shbim::cuda_fail((ctx), e_, #call);\
   } while (0)
 
+// whether launches on the stream are timed now
+bool timed(const shbim_ctx* ctx, cudaStream_t s);
 // ---- timing: bracket a launch of class `cls` on stream s (no-op unless timing is on)
 struct TimeScope {
   shbim_ctx* ctx;
