@@ -627,7 +627,7 @@ int analysis_fourier_tc(shbim_ctx* ctx, const DegreeTables& T, const float2* W, 
     if (!dft_tc_fits(p) || !T.dft_digits || !rexp || !omajor)
       return fail(ctx, SHBIM_ERR_ARG, "folded tensor-core Fourier stage: needs row exponents and order-major output");
     const int sm4 = dft4_smem(p);
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_dft4_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, sm4));
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_dft4_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, dft4_smem(64)));
     int dev = 0, nsm = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -638,7 +638,7 @@ int analysis_fourier_tc(shbim_ctx* ctx, const DegreeTables& T, const float2* W, 
     return SHBIM_OK;
   }
   const int smem = dft_tc_smem(p);
-  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_dft_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_dft_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, dft_tc_smem(kNT / 2 - 1)));
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);

@@ -1685,7 +1685,8 @@ int expand(shbim_ctx* ctx, const FarPlan& P, int kind, cudaStream_t s) {
     mom = static_cast<T*>(F.mom);
   }
   const int sm = (2 * ncm + 6 * (P.lmax + 1)) * 8;
-  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_far_m2l<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+  constexpr int sm_max = (2 * (kFarCap64 + 1) * (kFarCap64 + 1) + 6 * (kFarCap64 + 1)) * 8;
+  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_far_m2l<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_max));
   k_far_m2l<T><<<dim3((unsigned)P.npairs, npot), 256, sm, s>>>(P.pairs, npot, P.sd, P.Lsrc, P.ang_dev, tab, mom, lp);
   SHBIM_CHECK_LAUNCH(ctx, "k_far_m2l");
   k_far_lsum<T><<<dim3((unsigned)((npot * ncm + 127) / 128), nd), 128, 0, s>>>(P.td, P.pairs, ctx->drops_dev, npot, lp, loc);

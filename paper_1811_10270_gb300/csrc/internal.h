@@ -415,6 +415,11 @@ struct TimeScope {
   ~TimeScope();
 };
 
+// Largest dynamic shared memory of a CTA whose kernel has no static shared memory. A kernel's opt-in belongs to the
+// kernel, not to a context or a launch: every call sets the largest value that any launch of the kernel needs, for set
+// to a launch's own need it could be lowered by a context in another host thread before that launch.
+constexpr int kSharedMax = 227 * 1024;
+
 // ---- tables (tables.cu)
 int build_degree_tables(shbim_ctx* ctx, int p, DegreeTables** out);
 void free_degree_tables(DegreeTables* t);

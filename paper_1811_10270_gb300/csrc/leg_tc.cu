@@ -303,7 +303,8 @@ template <int KS, int ND>
 int launch(shbim_ctx* ctx, const DegreeTables& T, const float2* FT, int64_t nitems, float2* coef, int64_t coef_stride,
            cudaStream_t s) {
   const int smem = leg_tc_smem(T.p);
-  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_leg_tc<KS, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_leg_tc<KS, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       leg_tc_smem(std::min(64, KS * kKS / 2 - 1))));
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);

@@ -390,14 +390,16 @@ k_gemv_bf16(int B, int N, int K, const float* __restrict__ x, const __nv_bfloat1
   }
 }
 
+constexpr int kGemvSmem = 200 * 1024;
+
 int forward(shbim_mlp* net, int B, const float* x, cudaStream_t s) {
   const float* in = x;
   for (int l = 0; l < net->L; ++l) {
     const int K = net->w[l], N = net->w[l + 1];
     const size_t smem = (size_t)B * K * sizeof(float);
-    if (B <= kGemvRows && smem <= 200 * 1024) {
+    if (B <= kGemvRows && smem <= kGemvSmem) {
       if (smem > 48 * 1024 &&
-          cudaFuncSetAttribute(k_gemv_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+          cudaFuncSetAttribute(k_gemv_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemvSmem) != cudaSuccess)
         return SHBIM_ERR_CUDA;
       k_gemv_bf16<<<(unsigned)((N + kGemvOut - 1) / kGemvOut), 256, smem, s>>>(B, N, K, in, net->Wh[l], net->b[l],
                                                                               l < net->L - 1 ? 1 : 0, net->H[l + 1]);

@@ -527,8 +527,8 @@ int rotate_tc(shbim_ctx* ctx, const DegreeTables& T, bool adjoint, const float2*
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const uint4* tdig = reinterpret_cast<const uint4*>(T.rot_digits);
   const int nmax = rot_tc_nmax(p);
-  auto launch = [&](auto kernel, int smem) -> int {
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  auto launch = [&](auto kernel, int smem, int smem_max) -> int {
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
     const Items I(p, nmax, ncomp, t_begin, ct);
     kernel<<<(unsigned)std::min<int64_t>(I.total, nsm), kThreads, smem, s>>>(
         vin, in_stride, nc, p, nmax, t_begin, ct, ncomp, T.cs_phi_df, tdig, T.rot_toff, T.rot_exp, vout, rows_lap,
@@ -537,10 +537,10 @@ int rotate_tc(shbim_ctx* ctx, const DegreeTables& T, bool adjoint, const float2*
     return SHBIM_OK;
   };
   if (p >= kSplitFirst)
-    return adjoint ? launch(k_rotate_tc<true, true>, rot_split_smem(nmax))
-                   : launch(k_rotate_tc<false, true>, rot_split_smem(nmax));
-  return adjoint ? launch(k_rotate_tc<true, false>, rot_tc_smem(p, ncomp))
-                 : launch(k_rotate_tc<false, false>, rot_tc_smem(p, ncomp));
+    return adjoint ? launch(k_rotate_tc<true, true>, rot_split_smem(nmax), rot_split_smem(kSplitLast))
+                   : launch(k_rotate_tc<false, true>, rot_split_smem(nmax), rot_split_smem(kSplitLast));
+  return adjoint ? launch(k_rotate_tc<true, false>, rot_tc_smem(p, ncomp), rot_tc_smem(kSplitFirst - 1, ncomp))
+                 : launch(k_rotate_tc<false, false>, rot_tc_smem(p, ncomp), rot_tc_smem(kSplitFirst - 1, ncomp));
 }
 
 }  // namespace shbim

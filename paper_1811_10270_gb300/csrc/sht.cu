@@ -169,9 +169,9 @@ __global__ void k_synth(const double* __restrict__ coef, int64_t coef_stride, in
 // Dynamic shared memory above the 48 KB default needs the kernel's opt-in (up to 227 KB per CTA).
 int synth_smem_ok(shbim_ctx* ctx, size_t smem) {
   if (smem <= 48 * 1024) return SHBIM_OK;
-  if (smem > 227 * 1024) return fail(ctx, SHBIM_ERR_ARG, "synthesis grid too large for shared memory");
-  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_synth<DropList>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_synth<FieldList>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > kSharedMax) return fail(ctx, SHBIM_ERR_ARG, "synthesis grid too large for shared memory");
+  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_synth<DropList>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedMax));
+  SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_synth<FieldList>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedMax));
   return SHBIM_OK;
 }
 

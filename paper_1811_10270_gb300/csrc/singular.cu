@@ -369,8 +369,8 @@ int build_singular_rows(shbim_ctx* ctx, const double* xcoef, cudaStream_t s) {
       return rc;
     const double* xc = xcoef + 3 * d.coef_off;
     const int rot_smem = (2 * nc + 4 * (d.p + 1)) * (int)sizeof(double);
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, rot_smem));
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, rot_smem));
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedMax));
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedMax));
     for (int t0 = 0; t0 < d.nt; t0 += CT) {
       const int ct = std::min(CT, d.nt - t0);
       k_rotate_fwd<<<dim3(ct, 3), 128, rot_smem, s>>>(

@@ -198,6 +198,8 @@ __host__ __device__ __forceinline__ int weights_set(int p) {
   return (w + ((12 - w) % 32 + 32) % 32) / 2;
 }
 
+inline int weights_smem(int p) { return (6 * weights_set(p) + 80 * (p + 1)) * (int)sizeof(float2); }
+
 // For target blockIdx.x (chunk-local) and the up-grid latitudes j = blockIdx.y and q - j: synthesise the rotated
 // position and tangents, then the 14 kernel weights of every node of the two latitudes.
 // FP32-pipe bound. The two latitudes mirror each other, P_n^m(-t) = (-1)^(n+m) P_n^m(t): sums over even and odd
@@ -561,11 +563,11 @@ int build_singular_rows_df(shbim_ctx* ctx, cudaStream_t s, const double* xcoef) 
     const int tpb14 = std::max(1, std::min({8, (100 * 1024 - dq_bytes) / per_t14, occ}));
     const int deg_smem3 = dq_bytes + tpb3 * per_t3;
     const int deg_smem14 = dq_bytes + tpb14 * per_t14;
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_deg_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, deg_smem3));
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_deg_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, deg_smem14));
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_deg_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedMax));
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_rotate_deg_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedMax));
     const int w_threads = (N + 31) / 32 * 32;   // one node of a latitude per thread (N <= 260)
-    const size_t w_smem = (size_t)(6 * weights_set(d.p) + 20 * N) * sizeof(float2);
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_self_weights_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w_smem));
+    const size_t w_smem = weights_smem(d.p);
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_self_weights_df, cudaFuncAttributeMaxDynamicSharedMemorySize, weights_smem(64)));
     const int budget = 46 * 1024 / (int)sizeof(float2) - 2 * N;
     const int rows = std::max(1, std::min(8, budget / (2 * N)));
     const size_t f_smem = (size_t)(2 * N + rows * 2 * N) * sizeof(float2);
@@ -574,7 +576,7 @@ int build_singular_rows_df(shbim_ctx* ctx, cudaStream_t s, const double* xcoef) 
     const bool rot_tc = rot_n >= 0;
     const int df_n0 = rot_n + 1;
     const int leg_smem = (d.q + 1) * 2 * (d.p + 1) * (int)sizeof(float2);
-    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_analysis_leg_item_df, cudaFuncAttributeMaxDynamicSharedMemorySize, leg_smem));
+    SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_analysis_leg_item_df, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedMax));
     const bool leg_fits = ctx->tc_leg && leg_tc_fits(d.p);
     const bool dft_tc = ctx->tc_rows && dft_tc_fits(d.p) && (leg_fits || !dft_tc_omajor_only(d.p));
     const bool leg_tc = dft_tc && leg_fits;   // reads the order-major Fourier output
