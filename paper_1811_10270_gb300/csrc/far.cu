@@ -52,7 +52,7 @@ using dfl::df;
 
 constexpr int kP2mThreads = 256;
 constexpr int kP2mTiles = 4;                            // source tiles per CTA
-constexpr int kP2mSrc = kP2mThreads * kP2mTiles;        // sources per CTA
+static_assert(kP2mSrc == kP2mThreads * kP2mTiles, "a chunk is a CTA's sources");
 constexpr int kL2pWarps = 8;
 
 // ---- arithmetic: double or double-float
@@ -142,19 +142,6 @@ __device__ __forceinline__ T warp_total(T v) {
 
 __host__ __device__ __forceinline__ int tri_n(int L) { return (L + 1) * (L + 2) / 2; }
 __host__ __device__ __forceinline__ int tri_o(int L, int m) { return m * (L + 1) - m * (m - 1) / 2; }
-
-// the entry whose groups hold flat group f
-__device__ __forceinline__ int entry_of(const int64_t* __restrict__ goff, int nent, int64_t f) {
-  int a = 0, b = nent;                    // goff[a] <= f < goff[b]
-  while (b - a > 1) {
-    const int c = (a + b) >> 1;
-    if (goff[c] <= f)
-      a = c;
-    else
-      b = c;
-  }
-  return a;
-}
 
 // (x + i y)^m by binary powers
 template <class T>
@@ -530,31 +517,6 @@ __global__ void k_far_dipoles(const FarSrcDrop* __restrict__ sd, const int* __re
 }
 
 // ---- 2. translation of one potential of one far pair
-// cos / sin of m phi and m theta, and the powers (2A/D)^n, (2B/D)^l, of every far pair (once per geometry)
-__global__ void k_far_angles(const FarPair* __restrict__ pairs, const DropDev* __restrict__ drops,
-                             const float* __restrict__ inv_src, const float* __restrict__ inv_tgt,
-                             double* __restrict__ ang) {
-  const FarPair p = pairs[blockIdx.x];
-  const DropDev Di = drops[p.i], Dj = drops[p.j];
-  const double tx = Di.cx - Dj.cx, ty = Di.cy - Dj.cy, tz = Di.cz - Dj.cz;
-  const double D = sqrt(tx * tx + ty * ty + tz * tz);
-  const double th = acos(fmin(1.0, fmax(-1.0, tz / D))), ph = atan2(ty, tx);
-  double* a = ang + p.ang;
-  const int n1 = p.L + 1;
-  for (int m = threadIdx.x; m < n1; m += blockDim.x) {
-    double s, c;
-    sincos(m * ph, &s, &c);
-    a[m] = c;
-    a[n1 + m] = s;
-    sincos(m * th, &s, &c);
-    a[2 * n1 + m] = c;
-    a[3 * n1 + m] = s;
-    const double w = 12.566370614359172954 / sqrt(2.0 * m + 1.0);
-    a[4 * n1 + m] = w * pow(2.0 / (D * (double)inv_src[p.j]), (double)m);
-    a[5 * n1 + m] = pow(2.0 / (D * (double)inv_tgt[p.i]), (double)m) / (sqrt(2.0 * m + 1.0) * D);
-  }
-}
-
 // Dz by -+alpha in place on all degrees of X: (x[m], x[-m]) turned by m alpha
 template <class T>
 __device__ __forceinline__ void far_dz(T* X, int nc, const T* c, const T* s, bool neg) {
@@ -909,32 +871,6 @@ k_far_l2p(const FarTgtDrop* __restrict__ td, const int2* __restrict__ blocks, co
 // their targets beyond 1.7 to 2 radii, and a value of order 45 costs a seventh to a thirtieth of a sum over the
 // 5e3 to 2e4 sources of a drop of degree 24 to 48.
 
-// order at which the targets of a group may take the expansion of an entry's drop: a warp per group
-__global__ void k_far_reach(int nent, const int* __restrict__ ent_tgt, NearList nl, int64_t ngroup,
-                            const DropDev* __restrict__ drops, const unsigned* __restrict__ ext,
-                            const int* __restrict__ Lsrc, const float* __restrict__ rho_max,
-                            const double* __restrict__ tgt, int64_t ntarget, unsigned char* __restrict__ order) {
-  const int64_t f = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (f >= ngroup) return;
-  const int en = entry_of(nl.goff, nent, f), lane = threadIdx.x & 31;
-  const int j = nl.drop[en];
-  const DropDev Di = drops[ent_tgt[en]], Dj = drops[j];
-  const int64_t sl = (f - nl.goff[en]) * kFarGroup + lane;
-  double d2 = INFINITY;
-  if (sl < Di.nt) {
-    const int64_t t = nl.tgt[Di.tgt_off + sl];
-    const double dx = tgt[t] - Dj.cx, dy = tgt[ntarget + t] - Dj.cy, dz = tgt[2 * ntarget + t] - Dj.cz;
-    d2 = dx * dx + dy * dy + dz * dz;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) d2 = fmin(d2, __shfl_xor_sync(0xffffffffu, d2, o));
-  if (lane) return;
-  const float rho = (float)((double)__uint_as_float(ext[j]) / sqrt(d2)) * 1.000001f;
-  int L = 2;
-  while (L <= Lsrc[j] && !(rho <= rho_max[L])) ++L;
-  order[f] = (unsigned char)(L <= Lsrc[j] ? L : kNoReach);
-}
-
 // coefficient (n, mm) of the derivative along axis ax of the multipole expansion v, times -A (a dipole along ax)
 template <class T>
 __device__ T multi_grad(const T* __restrict__ v, int n, int mm, int ax, const T* __restrict__ la,
@@ -1065,7 +1001,7 @@ __global__ void k_far_msum(NearList nl, const DropDev* __restrict__ drops, const
   double s[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) s[c] = 0.0;
-  for (int en = nl.off[i]; en < nl.off[i + 1] - 1; ++en) {
+  for (int en = nl.begin(i); en < nl.end(i); ++en) {
     if (nl.direct(en, g, drops[nl.drop[en]].ns)) continue;
     const double* p = part + (nl.goff[en] + g) * NC * 32 + (sl & 31);
 #pragma unroll
@@ -1232,6 +1168,8 @@ const FarHost& far_host() {
   return H;
 }
 
+}  // namespace
+
 int far_grow(shbim_ctx* ctx, void** p, size_t* cap, size_t bytes, const char* what) {
   if (bytes <= *cap) return SHBIM_OK;
   cudaFree(*p);
@@ -1245,7 +1183,7 @@ int far_grow(shbim_ctx* ctx, void** p, size_t* cap, size_t bytes, const char* wh
   return SHBIM_OK;
 }
 
-int upload_tables(shbim_ctx* ctx) {
+int far_tables(shbim_ctx* ctx) {
   FarState& F = *ctx->far;
   if (F.tables) return SHBIM_OK;
   const FarHost& H = far_host();
@@ -1296,344 +1234,6 @@ int upload_tables(shbim_ctx* ctx) {
   }
   F.tables = dev;
   return SHBIM_OK;
-}
-
-// FP32 instructions of a direct pair and of the expansions' inner steps (double-float 12 per multiply-add, FP64 64
-// issue slots per instruction), by kind DL, SL, S + D, S, D
-constexpr double kDirect32[5] = {25.0, 18.0, 45.0, 35.0, 37.0};
-constexpr double kDirectDf[5] = {121.0, 78.0, 260.0, 187.0, 195.0};
-constexpr double kDirect64[5] = {1060.0, 740.0, 1980.0, 1540.0, 1470.0};
-constexpr int kSets[5] = {3, 1, 12, 12, 12};
-constexpr int kCharges[5] = {1, 1, 13, 4, 9};
-// derivatives taken of 1/r in the truncation bound
-constexpr int kDerivs[5] = {1, 0, 2, 1, 2};
-
-}  // namespace
-
-void far_free(shbim_ctx* ctx) {
-  if (!ctx->far) return;
-  FarState& F = *ctx->far;
-  cudaFree(F.tables);
-  cudaFree(F.blob);
-  cudaFree(F.ang);
-  cudaFree(F.q);
-  cudaFree(F.part);
-  cudaFree(F.v);
-  cudaFree(F.mom);
-  cudaFree(F.lpair);
-  cudaFree(F.loc);
-  cudaFree(F.set);
-  cudaFree(F.mset);
-  cudaFree(F.order);
-  cudaFree(F.mpart);
-  delete ctx->far;
-  ctx->far = nullptr;
-}
-
-void far_forget(shbim_ctx* ctx) {
-  if (!ctx->far) return;
-  for (auto& P : ctx->far->plan) P = FarPlan{};
-}
-
-// Lists of direct and far drop pairs of the current geometry, per truncation level and number of
-// derivatives, and the workspaces of their expansions. ext holds per drop the largest |x - c| of the
-// sources, then of the targets.
-int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
-  if (!ctx->far) ctx->far = new FarState();
-  FarState& F = *ctx->far;
-  const int nd = ctx->n_drops;
-  std::vector<unsigned char> blob;
-  auto put = [&](const void* p, size_t bytes) {
-    const size_t o = (blob.size() + 15) / 16 * 16;
-    blob.resize(o + bytes);
-    if (bytes) std::memcpy(blob.data() + o, p, bytes);
-    return o;
-  };
-  struct Offsets {
-    size_t nb_off, nb_drop, nb_pre, pairs, lsrc, sd, td, chunks, blocks, goff, ent_tgt, rho;
-  } off[kFarPlans + 1] = {};
-  std::vector<float> inv(2 * nd, 1.f);
-  for (int i = 0; i < 2 * nd; ++i) {
-    int e = 0;
-    std::frexp(ext[i], &e);                 // ext < 2^e
-    inv[i] = (float)std::ldexp(1.0, -e);
-  }
-  const size_t inv_off = put(inv.data(), inv.size() * sizeof(float));
-  size_t max_part = 0, max_v = 0, max_mom = 0, max_lp = 0, max_loc = 0, max_set = 0, max_ang = 0, max_mset = 0, max_mpart = 0;
-  bool any = false;
-  for (int pl = 0; pl <= kFarPlans; ++pl) {
-    FarPlan& P = F.plan[pl];
-    P = FarPlan{};
-    const bool all = pl == kFarPlans;       // the list of every other drop
-    const int level = pl / 3, g = pl % 3;
-    const double eps = level == 0 ? kFarEps32 : kFarEps64;
-    const int cap = level == 0 ? kFarCap32 : kFarCap64;
-    // rho_max[L]: largest ratio order L serves
-    std::vector<double> rho_max(cap + 1);
-    for (int L = 0; L <= cap; ++L) rho_max[L] = std::pow(eps / std::pow(L + 1.0, g), 1.0 / (L + 1));
-    std::vector<int> Lsrc(nd, -1), nb_off(nd + 1, 0), nb_drop, ent_tgt;
-    std::vector<int64_t> nb_pre, goff;
-    std::vector<float> rho_f(cap + 1);
-    for (int L = 0; L <= cap; ++L) rho_f[L] = std::nextafterf((float)rho_max[L], 0.f);
-    std::vector<FarPair> pairs;
-    std::vector<FarTgtDrop> td(nd);
-    for (int i = 0; i < nd; ++i) {
-      td[i] = FarTgtDrop{-1, (int)pairs.size(), (int)pairs.size(), 0, 0};
-      int64_t pre = 0;
-      for (int j = 0; j < nd; ++j) {
-        if (j == i) continue;
-        int L = -1;
-        if (!all) {
-          double d2 = 0.0;
-          for (int k = 0; k < 3; ++k) {
-            const double c = ctx->drops[i].centre[k] - ctx->drops[j].centre[k];
-            d2 += c * c;
-          }
-          const double D = std::sqrt(d2), a = ext[j], b = ext[nd + i];
-          if (D > a + b) {
-            const double rho = std::max(a / (D - b), b / (D - a));
-            if (rho <= rho_max[cap]) {
-              L = (int)(std::lower_bound(rho_max.begin(), rho_max.end(), rho) - rho_max.begin());
-              L = std::max(L, 2);
-            }
-          }
-        }
-        if (L < 0) {
-          nb_drop.push_back(j);
-          nb_pre.push_back(pre);
-          ent_tgt.push_back(i);
-          goff.push_back(P.ngroup);
-          P.ngroup += (ctx->drops[i].nt + kFarGroup - 1) / kFarGroup;
-          pre += ctx->drops[j].ns;
-          P.direct_pairs += (double)ctx->drops[i].nt * ctx->drops[j].ns;
-        } else {
-          pairs.push_back(FarPair{i, j, L, 0, 0, 0});
-          P.far_pairs += (double)ctx->drops[i].nt * ctx->drops[j].ns;
-          Lsrc[j] = std::max(Lsrc[j], L);
-          td[i].L = std::max(td[i].L, L);
-          P.lmax = std::max(P.lmax, L);
-        }
-      }
-      nb_drop.push_back(-1);                // end of the list, with the total
-      nb_pre.push_back(pre);
-      ent_tgt.push_back(-1);
-      goff.push_back(P.ngroup);
-      nb_off[i + 1] = (int)nb_drop.size();
-      td[i].pair1 = (int)pairs.size();
-    }
-    P.npairs = (int)pairs.size();
-    std::vector<FarSrcDrop> sd(nd);
-    std::vector<FarChunk> chunks;
-    std::vector<int2> blocks;
-    int64_t part = 0, coef = 0, lout = 0, ang = 0, loc = 0, tri = 0;
-    for (int j = 0; j < nd; ++j) {
-      sd[j] = FarSrcDrop{part, coef, P.stri, 0};
-      if (Lsrc[j] < 0) continue;
-      const int L = Lsrc[j];
-      for (int f = 0; f < ctx->drops[j].ns; f += kP2mSrc) {
-        chunks.push_back(FarChunk{j, f, std::min(kP2mSrc, ctx->drops[j].ns - f), 0, part});
-        part += tri_n(L);
-        sd[j].nchunk++;
-      }
-      coef += (int64_t)(L + 1) * (L + 1);
-      P.stri += tri_n(L);
-      P.src_work += (double)ctx->drops[j].ns * tri_n(L);
-    }
-    for (auto& p : pairs) {
-      p.out = lout;
-      p.ang = ang;
-      lout += (int64_t)(p.L + 1) * (p.L + 1);
-      ang += 6 * (p.L + 1);
-      P.pair_work += 2.0 * p.L * (double)p.L * p.L;
-    }
-    for (int i = 0; i < nd; ++i) {
-      if (td[i].L < 0) continue;
-      td[i].coef = loc;
-      td[i].tri = tri;
-      loc += (int64_t)(td[i].L + 1) * (td[i].L + 1);
-      tri += tri_n(td[i].L);
-      for (int t = 0; t < ctx->drops[i].nt; t += 32) blocks.push_back(make_int2(i, t));
-      P.tgt_work += (double)ctx->drops[i].nt * tri_n(td[i].L);
-    }
-    P.nchunks = (int)chunks.size();
-    P.nblocks = (int)blocks.size();
-    P.part = part;
-    P.coef = coef;
-    P.loc = loc;
-    P.lout = lout;
-    P.tri = tri;
-    P.ang = ang;
-    // which kinds are worth it at which precision
-    for (int pr = 0; pr < 3; ++pr)
-      for (int k = 0; k < 5; ++k) {
-        const bool mine = !all && kDerivs[k] == g && (level == 0) == (pr == SHBIM_PREC_FP32_COMP);
-        P.use[pr][k] = mine && far_worth(P, pr, k);
-        any = any || P.use[pr][k];
-        if (!P.use[pr][k]) continue;
-        const size_t npot = stokes_like(k) ? 4 : 1;
-        max_part = std::max(max_part, (size_t)2 * kCharges[k] * part);
-        max_v = std::max(max_v, (size_t)kCharges[k] * coef);
-        if (k == 2 || k == 4) max_mom = std::max(max_mom, (size_t)4 * coef);
-        max_lp = std::max(max_lp, npot * (size_t)lout);
-        max_loc = std::max(max_loc, npot * (size_t)loc);
-        max_set = std::max(max_set, (size_t)2 * kSets[k] * tri);
-        max_ang = std::max(max_ang, (size_t)ang);
-        max_mset = std::max(max_mset, (size_t)2 * kSets[k] * P.stri);
-        max_mpart = std::max(max_mpart, (size_t)(stokes_like(k) ? 96 : 32) * P.ngroup);
-        F.max_charges = std::max(F.max_charges, kCharges[k]);
-      }
-    Offsets& o = off[pl];
-    o.nb_off = put(nb_off.data(), nb_off.size() * sizeof(int));
-    o.nb_drop = put(nb_drop.data(), nb_drop.size() * sizeof(int));
-    o.nb_pre = put(nb_pre.data(), nb_pre.size() * sizeof(int64_t));
-    o.pairs = put(pairs.data(), pairs.size() * sizeof(FarPair));
-    o.lsrc = put(Lsrc.data(), Lsrc.size() * sizeof(int));
-    o.sd = put(sd.data(), sd.size() * sizeof(FarSrcDrop));
-    o.td = put(td.data(), td.size() * sizeof(FarTgtDrop));
-    o.chunks = put(chunks.data(), chunks.size() * sizeof(FarChunk));
-    o.blocks = put(blocks.data(), blocks.size() * sizeof(int2));
-    goff.push_back(P.ngroup);
-    P.nent = (int)nb_drop.size();
-    o.goff = put(goff.data(), goff.size() * sizeof(int64_t));
-    o.ent_tgt = put(ent_tgt.data(), ent_tgt.size() * sizeof(int));
-    o.rho = put(rho_f.data(), rho_f.size() * sizeof(float));
-    P.h_drop = std::move(nb_drop);
-    P.h_tgt = std::move(ent_tgt);
-    P.h_goff = std::move(goff);
-  }
-  int rc;
-  if ((rc = far_grow(ctx, (void**)&F.blob, &F.blob_cap, blob.size(), "expansion plans"))) return rc;
-  SHBIM_CUDA(ctx, cudaMemcpyAsync(F.blob, blob.data(), blob.size(), cudaMemcpyHostToDevice, s));
-  SHBIM_CUDA(ctx, cudaStreamSynchronize(s));   // the host copy goes away
-  F.inv_src = reinterpret_cast<const float*>(F.blob + inv_off);
-  F.inv_tgt = F.inv_src + nd;
-  for (int pl = 0; pl <= kFarPlans; ++pl) {
-    FarPlan& P = F.plan[pl];
-    const Offsets& o = off[pl];
-    P.near = NearList{reinterpret_cast<const int*>(F.blob + o.nb_off), reinterpret_cast<const int*>(F.blob + o.nb_drop),
-                      reinterpret_cast<const int64_t*>(F.blob + o.nb_pre), ctx->tgt_order,
-                      reinterpret_cast<const int64_t*>(F.blob + o.goff), nullptr, FarReach{}};
-    P.ent_tgt = reinterpret_cast<const int*>(F.blob + o.ent_tgt);
-    P.rho_max = reinterpret_cast<const float*>(F.blob + o.rho);
-    P.pairs = reinterpret_cast<const FarPair*>(F.blob + o.pairs);
-    P.Lsrc = reinterpret_cast<const int*>(F.blob + o.lsrc);
-    P.sd = reinterpret_cast<const FarSrcDrop*>(F.blob + o.sd);
-    P.td = reinterpret_cast<const FarTgtDrop*>(F.blob + o.td);
-    P.chunks = reinterpret_cast<const FarChunk*>(F.blob + o.chunks);
-    P.blocks = reinterpret_cast<const int2*>(F.blob + o.blocks);
-  }
-  if (!any) return SHBIM_OK;
-  size_t ang_total = 0, group_total = 0;
-  for (int pl = 0; pl < kFarPlans; ++pl) {
-    ang_total += (size_t)F.plan[pl].ang;
-    group_total += (size_t)F.plan[pl].ngroup;
-  }
-  if ((rc = upload_tables(ctx)) ||
-      (rc = far_grow(ctx, (void**)&F.ang, &F.ang_cap, ang_total * 8, "expansion angles")) ||
-      (rc = far_grow(ctx, &F.q, &F.q_cap, (size_t)F.max_charges * ctx->nsource * 8, "expansion charges")) ||
-      (rc = far_grow(ctx, &F.part, &F.part_cap, max_part * 8, "expansion partial moments")) ||
-      (rc = far_grow(ctx, &F.v, &F.v_cap, max_v * 8, "expansion moments")) ||
-      (rc = far_grow(ctx, &F.mom, &F.mom_cap, max_mom * 8, "expansion dipole moments")) ||
-      (rc = far_grow(ctx, &F.lpair, &F.lpair_cap, max_lp * 8, "expansion pair terms")) ||
-      (rc = far_grow(ctx, &F.loc, &F.loc_cap, max_loc * 8, "local expansions")) ||
-      (rc = far_grow(ctx, &F.set, &F.set_cap, max_set * 8, "local expansions of derivatives")) ||
-      (rc = far_grow(ctx, &F.order, &F.order_cap, std::max<size_t>(group_total, 1), "orders of close pairs")) ||
-      (rc = far_grow(ctx, &F.mset, &F.mset_cap, max_mset * 8, "multipole expansions of derivatives")) ||
-      (rc = far_grow(ctx, &F.mpart, &F.mpart_cap, max_mpart * 8, "values of multipole expansions"))) {
-    // no room for the expansions: every pair directly
-    for (auto& P : F.plan) std::memset(P.use, 0, sizeof(P.use));
-    ctx->err.clear();
-    return SHBIM_OK;
-  }
-  size_t ao = 0, go = 0;
-  for (int pl = 0; pl < kFarPlans; ++pl) {
-    FarPlan& P = F.plan[pl];
-    P.ang_dev = F.ang + ao;
-    ao += (size_t)P.ang;
-    P.order = static_cast<unsigned char*>(F.order) + go;
-    go += (size_t)P.ngroup;
-    bool used = false;
-    for (auto& r : P.use)
-      for (bool u : r) used = used || u;
-    if (!used || P.npairs == 0) continue;
-    k_far_angles<<<P.npairs, 64, 0, s>>>(P.pairs, ctx->drops_dev, F.inv_src, F.inv_tgt, P.ang_dev);
-    SHBIM_CHECK_LAUNCH(ctx, "k_far_angles");
-    if (P.ngroup == 0) continue;
-    k_far_reach<<<(unsigned)((P.ngroup * 32 + 255) / 256), 256, 0, s>>>(
-        P.nent, P.ent_tgt, P.near, P.ngroup, ctx->drops_dev, ctx->dq_ext_dev, P.Lsrc, P.rho_max, ctx->geo.tgt,
-        ctx->ntarget, P.order);
-    SHBIM_CHECK_LAUNCH(ctx, "k_far_reach");
-    P.near.order = P.order;
-  }
-  return SHBIM_OK;
-}
-
-// The estimate in FP32 instructions of the expansions' inner steps (half as much again for latency and reads, twice
-// in FP64, plus 75 us of launches and short kernels) against the direct sums they replace. 40 drops of degree 11,
-// single layer in double-float (5.2e8 pairs): 1.48 ms directly, 1.03 with expansions; six drops of degree 16 in
-// FP64 (4e7 pairs, a third far), eight applications: 14.2 ms directly, 15.7 with expansions, and left direct; two
-// drops, or 1e8 pairs in FP32, stay direct.
-bool far_worth(const FarPlan& P, int precision, int kind) {
-  const double* direct = precision == SHBIM_PREC_FP32_COMP ? kDirect32 : (precision == SHBIM_PREC_DF64 ? kDirectDf : kDirect64);
-  const double unit = precision == SHBIM_PREC_FP64 ? 64.0 / 12.0 : 1.0;
-  const int npot = stokes_like(kind) ? 4 : 1;
-  const double cost = unit * (P.src_work * (45.0 + 26.0 * kCharges[kind]) + P.tgt_work * (30.0 + 26.0 * kSets[kind]) +
-                              P.pair_work * npot * 30.0);
-  return P.npairs > 0 && (precision == SHBIM_PREC_FP64 ? 2.0 : 1.5) * cost + 3e9 < P.far_pairs * direct[kind];
-}
-
-const FarPlan* far_plan(const shbim_ctx* ctx, int kind) {
-  if (!ctx->far) return nullptr;
-  const int level = ctx->opts.precision == SHBIM_PREC_FP32_COMP ? 0 : 1;
-  const FarPlan& P = ctx->far->plan[3 * level + kDerivs[kind]];
-  return P.use[ctx->opts.precision][kind] ? &P : nullptr;
-}
-
-const FarPlan& far_all(const shbim_ctx* ctx) { return ctx->far->plan[kFarPlans]; }
-
-bool far_ready(const shbim_ctx* ctx) { return ctx->n_drops < 2 || (ctx->far && far_all(ctx).near.off); }
-
-// Instructions of an expansion's value: recurrence and 2 NS multiply-adds per (n, m), half as much again for reads
-// and orders of uneven length; `base` for the powers of x + iy and the sums over warps. In FP64 four times that: six
-// drops of degree 16, double layer, solve of eight applications: 16.9 ms without these expansions, 16.3 at one
-// time, 15.7 at four. 64 drops of degree 16 to 48, without and with them: Stokeslet in double-float 35.5 and 24.2 ms,
-// stresslet FP32 10.2 and 9.0, double layer FP32 3.83 and 2.88; twice the instructions here change nothing. Below 0.1 ms
-// of direct sums the three launches cost more than they give (40 drops of degree 11, 3e9: 1.00 and 1.03 ms).
-NearList far_near(const shbim_ctx* ctx, const FarPlan& P, int kind) {
-  NearList nl = P.near;
-  const int ns = kSets[kind], pr = ctx->opts.precision;
-  const double direct = (pr == SHBIM_PREC_FP64 ? kDirect64 : (pr == SHBIM_PREC_DF64 ? kDirectDf : kDirect32))[kind];
-  if (P.direct_pairs * direct < 4e9) nl.order = nullptr;
-  FarReach& r = nl.reach;
-  if (pr == SHBIM_PREC_FP64) {
-    r = FarReach{kFarLmax, 384 * (3 + 2 * ns), 0, 120000, (int)direct};
-  } else {
-    const bool fp32 = pr == SHBIM_PREC_FP32_COMP;
-    r = FarReach{fp32 ? 12 : 36, 50 + 36 * ns, 9 + 6 * ns, 15000, (int)direct};
-  }
-  return nl;
-}
-
-double far_direct_pairs(const shbim_ctx* ctx, const FarPlan& P, int kind) {
-  const int pr = ctx->opts.precision;
-  if (P.counted[pr][kind]) return P.count[pr][kind];
-  const NearList nl = far_near(ctx, P, kind);
-  if (!nl.order) return P.direct_pairs;
-  std::vector<unsigned char> L((size_t)P.ngroup);
-  if (cudaMemcpy(L.data(), nl.order, L.size(), cudaMemcpyDeviceToHost) != cudaSuccess) {
-    cudaGetLastError();
-    return P.direct_pairs;
-  }
-  double n = 0.0;
-  for (int en = 0; en < P.nent; ++en) {
-    if (P.h_drop[en] < 0) continue;
-    const int ns = ctx->drops[P.h_drop[en]].ns, nt = ctx->drops[P.h_tgt[en]].nt;
-    for (int64_t f = P.h_goff[en]; f < P.h_goff[en + 1]; ++f)
-      if (L[f] == kNoReach || !nl.reach.worth(L[f], ns))
-        n += (double)ns * std::min<int64_t>(kFarGroup, nt - (f - P.h_goff[en]) * kFarGroup);
-  }
-  P.counted[pr][kind] = true;
-  return P.count[pr][kind] = n;
 }
 
 namespace {

@@ -1,4 +1,4 @@
-// Plans and workspaces of the expansions between well-separated drops (far.cu).
+// Plans (far_plan.cu) and workspaces of the expansions between well-separated drops (far.cu).
 #pragma once
 
 #include <cstdint>
@@ -15,6 +15,12 @@ constexpr double kFarEps64 = 3e-15; // ... and FP64-class sums
 constexpr int kFarCap32 = 36;       // largest order of a far pair, FP32 sums
 constexpr int kFarCap64 = 60;       // ... and FP64-class sums
 constexpr int kFarPlans = 6;        // [truncation level 2][derivatives 3]
+constexpr int kP2mSrc = 1024;       // sources of a chunk of the moments (a CTA of k_far_p2m)
+// by kind (0 DL, 1 SL, 2 S + D, 3 S, 4 D): expansions the targets evaluate, charges of a source, derivatives taken of
+// 1/r in the truncation bound
+constexpr int kSets[5] = {3, 1, 12, 12, 12};
+constexpr int kCharges[5] = {1, 1, 13, 4, 9};
+constexpr int kDerivs[5] = {1, 0, 2, 1, 2};
 
 // charge sets of the moments: Laplace strengths; f, y.f; dipole tensor and vector; both
 enum FarMode { kFarLap = 0, kFarS = 1, kFarD = 2, kFarSD = 3 };
@@ -37,6 +43,7 @@ struct FarSrcDrop {
 struct FarTgtDrop {
   int L, pair0, pair1;
   int64_t coef, tri;
+  int64_t out, ang, group;            // where its pairs' local terms and angles and its entries' groups start
 };
 
 // What a target's value of a multipole expansion of order L costs against the direct sum over ns sources, in
@@ -54,11 +61,15 @@ struct FarReach {
 constexpr int kFarGroup = 32;       // targets that share a decision
 constexpr int kNoReach = 255;
 
-// Per target drop i the drops that no local expansion covers, entries [off[i], off[i+1]): drop index and the number
-// of sources before it in the list; the last entry of a drop has index -1 and the total. The targets of a drop are
-// taken in the order tgt[] (patches of the surface); group g of 32 of them reaches the multipole expansion of the
-// entry's drop at order order[goff[entry] + g] (kNoReach: at none), and is summed directly where that is not worth it.
+// Per target drop i the drops that no local expansion covers, entries [begin(i), end(i)): drop and the number of sources
+// before it in the list. Without lists (drop null) those are all others in the order of the layout, entry e being drop e,
+// or e + 1 from drop i on; with lists off[] holds where a drop's entries start, and the last entry of a drop has index -1
+// and the total of sources. The targets of a drop are taken in the order tgt[] (patches of the surface); group g of 32
+// of them reaches the multipole expansion of the entry's drop at order order[goff[entry] + g] (kNoReach: at none), and is
+// summed directly where that is not worth it.
 struct NearList {
+  int n = 0;                        // drops
+  int64_t nsource = 0;
   const int* off = nullptr;
   const int* drop = nullptr;
   const int64_t* pre = nullptr;
@@ -66,12 +77,34 @@ struct NearList {
   const int64_t* goff = nullptr;    // [entries + 1]
   const unsigned char* order = nullptr;   // null: every group directly
   FarReach reach;
+  __device__ __forceinline__ int begin(int i) const { return drop ? off[i] : 0; }
+  __device__ __forceinline__ int end(int i) const { return drop ? off[i + 1] - 1 : n - 1; }
+  __device__ __forceinline__ int source(int entry, int i) const { return drop ? drop[entry] : entry + (entry >= i ? 1 : 0); }
+  __device__ __forceinline__ int64_t before(int entry, int i, const DropDev& Di, const DropDev& Dj) const {
+    return drop ? pre[entry] : Dj.src_off - (entry >= i ? (int64_t)Di.ns : 0);
+  }
+  __device__ __forceinline__ int64_t total(int i, const DropDev& Di) const {
+    return drop ? pre[off[i + 1] - 1] : nsource - Di.ns;
+  }
   __host__ __device__ bool direct(int entry, int group, int ns) const {
     if (!order) return true;
     const int L = order[goff[entry] + group];
     return L == kNoReach || !reach.worth(L, ns);
   }
 };
+
+// the entry whose groups hold flat group f
+__device__ __forceinline__ int entry_of(const int64_t* __restrict__ goff, int nent, int64_t f) {
+  int a = 0, b = nent;                    // goff[a] <= f < goff[b]
+  while (b - a > 1) {
+    const int c = (a + b) >> 1;
+    if (goff[c] <= f)
+      a = c;
+    else
+      b = c;
+  }
+  return a;
+}
 
 template <class T>
 struct FarTab {
@@ -98,19 +131,30 @@ struct FarPlan {
   int nent = 0;
   int64_t ngroup = 0, stri = 0;
   const int* ent_tgt = nullptr;       // target drop of an entry (-1: end of a list)
-  const float* rho_max = nullptr;     // [cap + 1]
   unsigned char* order = nullptr;     // [ngroup]
-  std::vector<int> h_drop, h_tgt;     // host copies of the lists
-  std::vector<int64_t> h_goff;
   // pairs summed directly, by [precision][kind], once they have been asked for
   mutable bool counted[3][5] = {};
   mutable double count[3][5] = {};
 };
 
+// What a target drop's row of the drop pairs comes to under one plan (k_far_count)
+struct FarRow {
+  int64_t out;                        // sum of (L + 1)^2 over its far drops
+  int64_t pairs;                      // targets times sources of its far drops
+  double cubes;                       // sum of 2 L^3
+  int far, lmax, ang, pad;            // far drops, largest order, sum of 6 (L + 1)
+};
+
 struct FarState {
   FarPlan plan[kFarPlans + 1];        // the last one: every other drop directly
-  unsigned char* blob = nullptr;      // device copies of the lists of all plans
+  unsigned char* blob = nullptr;      // per-drop lists of the plans in use, written by the host
   size_t blob_cap = 0;
+  unsigned char* lists = nullptr;     // per-pair lists of the plans in use, written by k_far_fill
+  size_t lists_cap = 0;
+  unsigned char* count = nullptr;     // [plans][n_drops] FarRow, [plans][n_drops] largest order of a source drop, a sum
+  unsigned char* count_host = nullptr;   // page-locked, the same
+  size_t count_cap = 0, count_host_cap = 0;
+  double* sum = nullptr;              // in count: pairs summed directly, when asked for
   void* tables = nullptr;
   FarTab<double> td{};
   FarTab<dfl::df> tf{};
@@ -122,10 +166,16 @@ struct FarState {
   size_t q_cap = 0, part_cap = 0, v_cap = 0, mom_cap = 0, lpair_cap = 0, loc_cap = 0, set_cap = 0;
   void *mset = nullptr, *order = nullptr, *mpart = nullptr;
   size_t mset_cap = 0, order_cap = 0, mpart_cap = 0;
-  int max_charges = 0;
 };
 
+// Lists of direct and far drop pairs of the current geometry. far_count queues the classification of all pairs under
+// every plan behind the extents (ctx->dq_ext_dev) and their read-back; after a synchronisation build_far decides which
+// plans are used and makes their lists, ext holding per drop the largest |x - c| of the sources, then of the targets.
+int far_count(shbim_ctx* ctx, cudaStream_t s);
 int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s);
+// expansion tables on the device (far.cu)
+int far_tables(shbim_ctx* ctx);
+int far_grow(shbim_ctx* ctx, void** p, size_t* cap, size_t bytes, const char* what);
 void far_free(shbim_ctx* ctx);
 // empties every plan (the workspaces stay): what comes before build_far may fail
 void far_forget(shbim_ctx* ctx);

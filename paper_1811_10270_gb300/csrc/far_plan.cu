@@ -1,0 +1,593 @@
+// Plans of the expansions between well-separated drops (far.cu): which pairs of drops are far and at what order, which
+// kinds of sums the expansions pay for, and the lists the kernels work through.
+//
+// The pairs of drops are classified on the GPU, a warp per target drop: k_far_count sums up what every plan would come
+// to, per drop, and k_far_fill writes the lists of the plans in use. The host sees O(drops) numbers only. One after
+// the other on the host, with lists for all plans copied to the device, set_drops took 1.8 s for 2048 drops of degree 4
+// (0.42 without expansions in the library), 0.37 so; 64 drops 5.9 and 5.1 ms. The sums without expansions need no lists.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <vector>
+
+#include "far.h"
+#include "internal.h"
+
+namespace shbim {
+
+namespace {
+
+// largest ratio rho that order L serves, per plan; the reach of close pairs takes the FP32 number below it
+struct RhoTab {
+  double r[kFarPlans][kFarCap64 + 1];
+};
+struct RhoReach {
+  float r[kFarCap64 + 1];
+};
+
+int plan_cap(int pl) { return pl < 3 ? kFarCap32 : kFarCap64; }
+
+const RhoTab& rho_tab() {
+  static const RhoTab T = [] {
+    RhoTab t{};
+    for (int pl = 0; pl < kFarPlans; ++pl)
+      for (int L = 0; L <= plan_cap(pl); ++L)
+        t.r[pl][L] = std::pow((pl < 3 ? kFarEps32 : kFarEps64) / std::pow(L + 1.0, pl % 3), 1.0 / (L + 1));
+    return t;
+  }();
+  return T;
+}
+
+// rho of a pair of drops, sources of j and targets of i; infinite where their spheres overlap
+__device__ __forceinline__ double far_ratio(const double* __restrict__ centres, const unsigned* __restrict__ ext, int nd, int i,
+                                            int j) {
+  double d2 = 0.0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double c = centres[3 * i + k] - centres[3 * j + k];
+    d2 = fma(c, c, d2);
+  }
+  const double D = sqrt(d2), a = (double)__uint_as_float(ext[j]), b = (double)__uint_as_float(ext[nd + i]);
+  if (!(D > a + b)) return INFINITY;
+  return fmax(a / (D - b), b / (D - a));
+}
+
+// smallest order that serves rho under plan pl, at least 2; -1: none
+__device__ __forceinline__ int far_order(const RhoTab& T, int pl, double rho) {
+  const int cap = pl < 3 ? kFarCap32 : kFarCap64;
+  if (!(rho <= T.r[pl][cap])) return -1;
+  int a = 0, b = cap;
+  while (a < b) {
+    const int c = (a + b) >> 1;
+    if (T.r[pl][c] < rho)
+      a = c + 1;
+    else
+      b = c;
+  }
+  return max(a, 2);
+}
+
+template <class V>
+__device__ __forceinline__ V warp_add(V v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// a warp per target drop: its row under every plan, and the largest orders of the source drops
+__global__ void k_far_count(const __grid_constant__ RhoTab T, const double* __restrict__ centres,
+                            const unsigned* __restrict__ ext, const DropDev* __restrict__ drops, int nd,
+                            FarRow* __restrict__ rows, int* __restrict__ lsrc) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= nd) return;
+  int far[kFarPlans], lmax[kFarPlans], ang[kFarPlans];
+  int64_t out[kFarPlans], src[kFarPlans];
+  double cubes[kFarPlans];
+#pragma unroll
+  for (int pl = 0; pl < kFarPlans; ++pl) {
+    far[pl] = ang[pl] = 0;
+    lmax[pl] = -1;
+    out[pl] = src[pl] = 0;
+    cubes[pl] = 0.0;
+  }
+  for (int j = lane; j < nd; j += 32) {
+    if (j == i) continue;
+    const double rho = far_ratio(centres, ext, nd, i, j);
+    const int ns = drops[j].ns;
+#pragma unroll
+    for (int pl = 0; pl < kFarPlans; ++pl) {
+      const int L = far_order(T, pl, rho);
+      if (L < 0) continue;
+      far[pl]++;
+      lmax[pl] = max(lmax[pl], L);
+      ang[pl] += 6 * (L + 1);
+      out[pl] += (L + 1) * (L + 1);
+      src[pl] += ns;
+      cubes[pl] += 2.0 * L * L * L;
+      if (lsrc[pl * nd + j] < L) atomicMax(lsrc + pl * nd + j, L);
+    }
+  }
+  const int64_t nt = drops[i].nt;
+#pragma unroll
+  for (int pl = 0; pl < kFarPlans; ++pl) {
+    FarRow r;
+    r.far = warp_add(far[pl]);
+    r.ang = warp_add(ang[pl]);
+    r.out = warp_add(out[pl]);
+    r.pairs = nt * warp_add(src[pl]);
+    r.cubes = warp_add(cubes[pl]);
+    r.lmax = lmax[pl];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r.lmax = max(r.lmax, __shfl_xor_sync(0xffffffffu, r.lmax, o));
+    r.pad = 0;
+    if (lane == 0) rows[(int64_t)pl * nd + i] = r;
+  }
+}
+
+struct FillPlan {
+  int pl;
+  const FarTgtDrop* td;
+  const int* off;
+  FarPair* pairs;
+  int *drop, *ent_tgt;
+  int64_t *pre, *goff;
+};
+struct FillPlans {
+  FillPlan p[kFarPlans];
+};
+
+__device__ __forceinline__ int scan_before(int v, int lane) {
+  int s = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += t;
+  }
+  return s - v;
+}
+
+// the same warp writes its drop's far pairs and its list of the others, in the order of the drops
+__global__ void k_far_fill(const __grid_constant__ RhoTab T, const __grid_constant__ FillPlans plans,
+                           const double* __restrict__ centres, const unsigned* __restrict__ ext,
+                           const DropDev* __restrict__ drops, int nd) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= nd) return;
+  const FillPlan& P = plans.p[blockIdx.y];
+  const FarTgtDrop d = P.td[i];
+  const int groups = (drops[i].nt + kFarGroup - 1) / kFarGroup;
+  const unsigned below = (1u << lane) - 1u;
+  int64_t pair = d.pair0, out = d.out, ang = d.ang, goff = d.group, pre = 0;
+  int entry = P.off[i];
+  for (int j0 = 0; j0 < nd; j0 += 32) {
+    const int j = j0 + lane;
+    const bool other = j < nd && j != i;
+    const int L = other ? far_order(T, P.pl, far_ratio(centres, ext, nd, i, j)) : -1;
+    const bool far = L >= 0, near = other && !far;
+    const unsigned fm = __ballot_sync(0xffffffffu, far), nm = __ballot_sync(0xffffffffu, near);
+    const int o = far ? (L + 1) * (L + 1) : 0, g = far ? 6 * (L + 1) : 0, ns = near ? drops[j].ns : 0;
+    const int ob = scan_before(o, lane), gb = scan_before(g, lane), nb = scan_before(ns, lane);
+    if (far) P.pairs[pair + __popc(fm & below)] = FarPair{i, j, L, 0, out + ob, ang + gb};
+    if (near) {
+      const int k = __popc(nm & below);
+      P.drop[entry + k] = j;
+      P.ent_tgt[entry + k] = i;
+      P.pre[entry + k] = pre + nb;
+      P.goff[entry + k] = goff + (int64_t)k * groups;
+    }
+    pair += __popc(fm);
+    out += __shfl_sync(0xffffffffu, ob + o, 31);
+    ang += __shfl_sync(0xffffffffu, gb + g, 31);
+    pre += __shfl_sync(0xffffffffu, nb + ns, 31);
+    entry += __popc(nm);
+    goff += (int64_t)__popc(nm) * groups;
+  }
+  if (lane) return;
+  P.drop[entry] = P.ent_tgt[entry] = -1;      // end of the list, with the total
+  P.pre[entry] = pre;
+  P.goff[entry] = goff;
+  if (i == nd - 1) P.goff[entry + 1] = goff;
+}
+
+// 1 / sqrt(2 m + 1)
+struct AngTab {
+  double r[kFarCap64 + 1];
+};
+
+// cos / sin of m phi and m theta, and the powers (2A/D)^n, (2B/D)^l, of every far pair (once per geometry). A thread per
+// pair and one product per value: FP64 instructions bound it: sine, cosine and power of every value apart, 100 to
+// 200 of them each, took 160 ms for the six plans of 1024 drops of degree 4, the products 4.9. The rounding of m factors
+// is that of an angle m phi.
+__global__ void k_far_angles(const FarPair* __restrict__ pairs, int npairs, const DropDev* __restrict__ drops,
+                             const float* __restrict__ inv_src, const float* __restrict__ inv_tgt,
+                             const __grid_constant__ AngTab T, double* __restrict__ ang) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= npairs) return;
+  const FarPair p = pairs[k];
+  const DropDev Di = drops[p.i], Dj = drops[p.j];
+  const double tx = Di.cx - Dj.cx, ty = Di.cy - Dj.cy, tz = Di.cz - Dj.cz;
+  const double h2 = tx * tx + ty * ty, h = sqrt(h2), iD = 1.0 / sqrt(h2 + tz * tz);
+  const double cp = h > 0.0 ? tx / h : 1.0, sp = h > 0.0 ? ty / h : 0.0, ct = tz * iD, st = h * iD;
+  const double gs = 2.0 * iD / (double)inv_src[p.j], gt = 2.0 * iD / (double)inv_tgt[p.i];
+  double* a = ang + p.ang;
+  const int n1 = p.L + 1;
+  double c1 = 1.0, s1 = 0.0, c2 = 1.0, s2 = 0.0, ps = 12.566370614359172954, pt = iD;
+  for (int m = 0; m < n1; ++m) {
+    a[m] = c1;
+    a[n1 + m] = s1;
+    a[2 * n1 + m] = c2;
+    a[3 * n1 + m] = s2;
+    a[4 * n1 + m] = T.r[m] * ps;
+    a[5 * n1 + m] = T.r[m] * pt;
+    const double u = c1 * cp - s1 * sp, v = c2 * ct - s2 * st;
+    s1 = c1 * sp + s1 * cp;
+    s2 = c2 * st + s2 * ct;
+    c1 = u;
+    c2 = v;
+    ps *= gs;
+    pt *= gt;
+  }
+}
+
+// order at which the targets of a group may take the expansion of an entry's drop: a warp per group
+__global__ void k_far_reach(int nent, const int* __restrict__ ent_tgt, NearList nl, int64_t ngroup,
+                            const DropDev* __restrict__ drops, const unsigned* __restrict__ ext,
+                            const int* __restrict__ Lsrc, const __grid_constant__ RhoReach R,
+                            const double* __restrict__ tgt, int64_t ntarget, unsigned char* __restrict__ order) {
+  const int64_t f = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (f >= ngroup) return;
+  const int en = entry_of(nl.goff, nent, f), lane = threadIdx.x & 31;
+  const int j = nl.drop[en];
+  const DropDev Di = drops[ent_tgt[en]], Dj = drops[j];
+  const int64_t sl = (f - nl.goff[en]) * kFarGroup + lane;
+  double d2 = INFINITY;
+  if (sl < Di.nt) {
+    const int64_t t = nl.tgt[Di.tgt_off + sl];
+    const double dx = tgt[t] - Dj.cx, dy = tgt[ntarget + t] - Dj.cy, dz = tgt[2 * ntarget + t] - Dj.cz;
+    d2 = dx * dx + dy * dy + dz * dz;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) d2 = fmin(d2, __shfl_xor_sync(0xffffffffu, d2, o));
+  if (lane) return;
+  const float rho = (float)((double)__uint_as_float(ext[j]) / sqrt(d2)) * 1.000001f;
+  int L = 2;
+  while (L <= Lsrc[j] && !(rho <= R.r[L])) ++L;
+  order[f] = (unsigned char)(L <= Lsrc[j] ? L : kNoReach);
+}
+
+// target-source pairs of the groups that are summed directly
+__global__ void k_far_direct(int nent, const int* __restrict__ ent_tgt, NearList nl, int64_t ngroup,
+                             const DropDev* __restrict__ drops, double* __restrict__ sum) {
+  double n = 0.0;
+  for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < ngroup; f += (int64_t)gridDim.x * blockDim.x) {
+    const int en = entry_of(nl.goff, nent, f), g = (int)(f - nl.goff[en]);
+    const int ns = drops[nl.drop[en]].ns, nt = drops[ent_tgt[en]].nt;
+    if (nl.direct(en, g, ns)) n += (double)ns * min(kFarGroup, nt - g * kFarGroup);
+  }
+  n = warp_add(n);
+  if ((threadIdx.x & 31) == 0 && n != 0.0) atomicAdd(sum, n);   // whole numbers: exact in any order
+}
+
+// FP32 instructions of a direct pair and of the expansions' inner steps (double-float 12 per multiply-add, FP64 64
+// issue slots per instruction), by kind DL, SL, S + D, S, D
+constexpr double kDirect32[5] = {25.0, 18.0, 45.0, 35.0, 37.0};
+constexpr double kDirectDf[5] = {121.0, 78.0, 260.0, 187.0, 195.0};
+constexpr double kDirect64[5] = {1060.0, 740.0, 1980.0, 1540.0, 1470.0};
+
+}  // namespace
+
+void far_free(shbim_ctx* ctx) {
+  if (!ctx->far) return;
+  FarState& F = *ctx->far;
+  cudaFree(F.tables);
+  cudaFree(F.blob);
+  cudaFree(F.lists);
+  cudaFree(F.count);
+  cudaFreeHost(F.count_host);
+  cudaFree(F.ang);
+  cudaFree(F.q);
+  cudaFree(F.part);
+  cudaFree(F.v);
+  cudaFree(F.mom);
+  cudaFree(F.lpair);
+  cudaFree(F.loc);
+  cudaFree(F.set);
+  cudaFree(F.mset);
+  cudaFree(F.order);
+  cudaFree(F.mpart);
+  delete ctx->far;
+  ctx->far = nullptr;
+}
+
+void far_forget(shbim_ctx* ctx) {
+  if (!ctx->far) return;
+  for (auto& P : ctx->far->plan) P = FarPlan{};
+}
+
+int far_count(shbim_ctx* ctx, cudaStream_t s) {
+  if (!ctx->far) ctx->far = new FarState();
+  FarState& F = *ctx->far;
+  const size_t n = (size_t)kFarPlans * ctx->n_drops;
+  const size_t lsrc_off = n * sizeof(FarRow), sum_off = (lsrc_off + n * sizeof(int) + 15) / 16 * 16;
+  if (int rc = far_grow(ctx, (void**)&F.count, &F.count_cap, sum_off + sizeof(double), "drop pair counts")) return rc;
+  if (F.count_host_cap < sum_off) {
+    cudaFreeHost(F.count_host);
+    F.count_host = nullptr;
+    F.count_host_cap = 0;
+    if (cudaMallocHost((void**)&F.count_host, sum_off) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(ctx, SHBIM_ERR_NOMEM, "cudaMallocHost drop pair counts");
+    }
+    F.count_host_cap = sum_off;
+  }
+  F.sum = reinterpret_cast<double*>(F.count + sum_off);
+  FarRow* rows = reinterpret_cast<FarRow*>(F.count);
+  int* lsrc = reinterpret_cast<int*>(F.count + lsrc_off);
+  SHBIM_CUDA(ctx, cudaMemsetAsync(lsrc, 0xff, n * sizeof(int), s));   // -1
+  k_far_count<<<(unsigned)((ctx->n_drops * 32 + 127) / 128), 128, 0, s>>>(rho_tab(), ctx->centres_dev, ctx->dq_ext_dev,
+                                                                         ctx->drops_dev, ctx->n_drops, rows, lsrc);
+  SHBIM_CHECK_LAUNCH(ctx, "k_far_count");
+  SHBIM_CUDA(ctx, cudaMemcpyAsync(F.count_host, F.count, sum_off, cudaMemcpyDeviceToHost, s));
+  return SHBIM_OK;
+}
+
+// Plans in use: their per-drop lists (uploaded), per-pair lists (k_far_fill) and the workspaces of their expansions.
+int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
+  FarState& F = *ctx->far;
+  const int nd = ctx->n_drops;
+  std::vector<unsigned char> blob;
+  auto put = [&](const void* p, size_t bytes) {
+    const size_t o = (blob.size() + 15) / 16 * 16;
+    blob.resize(o + bytes);
+    if (bytes) std::memcpy(blob.data() + o, p, bytes);
+    return o;
+  };
+  size_t lists = 0;
+  auto room = [&](size_t bytes) {
+    const size_t o = lists;
+    lists = (o + bytes + 15) / 16 * 16;
+    return o;
+  };
+  struct Offsets {
+    size_t off, lsrc, sd, td, chunks, blocks, pairs, drop, ent_tgt, pre, goff;
+  } off[kFarPlans] = {};
+  double cross = 0.0;
+  for (const Drop& d : ctx->drops) cross += (double)d.nt * (double)(ctx->nsource - d.ns);
+  F.plan[kFarPlans].near.n = nd;               // every other drop: no lists
+  F.plan[kFarPlans].near.nsource = ctx->nsource;
+  F.plan[kFarPlans].near.tgt = ctx->tgt_order;
+  F.plan[kFarPlans].direct_pairs = cross;
+  std::vector<float> inv(2 * nd, 1.f);
+  for (int i = 0; i < 2 * nd; ++i) {
+    int e = 0;
+    std::frexp(ext[i], &e);                 // ext < 2^e
+    inv[i] = (float)std::ldexp(1.0, -e);
+  }
+  const size_t inv_off = put(inv.data(), inv.size() * sizeof(float));
+  size_t max_part = 0, max_v = 0, max_mom = 0, max_lp = 0, max_loc = 0, max_set = 0, max_mset = 0, max_mpart = 0;
+  size_t ang_total = 0, group_total = 0;
+  int max_charges = 0;
+  bool used[kFarPlans] = {};
+  for (int pl = 0; pl < kFarPlans; ++pl) {
+    FarPlan& P = F.plan[pl];
+    const FarRow* row = reinterpret_cast<const FarRow*>(F.count_host) + (size_t)pl * nd;
+    const int* Lsrc = reinterpret_cast<const int*>(F.count_host + (size_t)kFarPlans * nd * sizeof(FarRow)) + (size_t)pl * nd;
+    int64_t npairs = 0, nent = 0;
+    for (int i = 0; i < nd; ++i) {
+      npairs += row[i].far;
+      nent += nd - row[i].far;                // the others and the end of the list
+      P.far_pairs += (double)row[i].pairs;
+      P.pair_work += row[i].cubes;
+      P.lmax = std::max(P.lmax, row[i].lmax);
+      P.tgt_work += (double)ctx->drops[i].nt * (row[i].lmax < 0 ? 0 : FarReach::tri(row[i].lmax));
+      P.src_work += (double)ctx->drops[i].ns * (Lsrc[i] < 0 ? 0 : FarReach::tri(Lsrc[i]));
+    }
+    P.direct_pairs = cross - P.far_pairs;
+    if (npairs == 0 || npairs > INT32_MAX || nent > INT32_MAX) continue;
+    P.npairs = (int)npairs;
+    P.nent = (int)nent;
+    // which kinds are worth it at which precision
+    for (int pr = 0; pr < 3; ++pr)
+      for (int k = 0; k < 5; ++k) {
+        P.use[pr][k] = kDerivs[k] == pl % 3 && (pl < 3) == (pr == SHBIM_PREC_FP32_COMP) && far_worth(P, pr, k);
+        used[pl] = used[pl] || P.use[pr][k];
+      }
+    if (!used[pl]) continue;
+    std::vector<int> nb_off(nd + 1, 0);
+    std::vector<FarSrcDrop> sd(nd);
+    std::vector<FarTgtDrop> td(nd);
+    std::vector<FarChunk> chunks;
+    std::vector<int2> blocks;
+    int pair = 0;
+    for (int i = 0; i < nd; ++i) {
+      const Drop& d = ctx->drops[i];
+      const int near = nd - 1 - row[i].far;
+      nb_off[i + 1] = nb_off[i] + near + 1;
+      td[i] = FarTgtDrop{row[i].lmax, pair, pair + row[i].far, P.loc, P.tri, P.lout, P.ang, P.ngroup};
+      pair += row[i].far;
+      P.lout += row[i].out;
+      P.ang += row[i].ang;
+      P.ngroup += (int64_t)near * ((d.nt + kFarGroup - 1) / kFarGroup);
+      if (row[i].lmax >= 0) {
+        P.loc += (int64_t)(row[i].lmax + 1) * (row[i].lmax + 1);
+        P.tri += FarReach::tri(row[i].lmax);
+        for (int t = 0; t < d.nt; t += 32) blocks.push_back(make_int2(i, t));
+      }
+      sd[i] = FarSrcDrop{P.part, P.coef, P.stri, 0};
+      if (Lsrc[i] < 0) continue;
+      for (int f = 0; f < d.ns; f += kP2mSrc) {
+        chunks.push_back(FarChunk{i, f, std::min(kP2mSrc, d.ns - f), 0, P.part});
+        P.part += FarReach::tri(Lsrc[i]);
+        sd[i].nchunk++;
+      }
+      P.coef += (int64_t)(Lsrc[i] + 1) * (Lsrc[i] + 1);
+      P.stri += FarReach::tri(Lsrc[i]);
+    }
+    P.nchunks = (int)chunks.size();
+    P.nblocks = (int)blocks.size();
+    for (int pr = 0; pr < 3; ++pr)
+      for (int k = 0; k < 5; ++k) {
+        if (!P.use[pr][k]) continue;
+        const size_t npot = stokes_like(k) ? 4 : 1;
+        max_part = std::max(max_part, (size_t)2 * kCharges[k] * P.part);
+        max_v = std::max(max_v, (size_t)kCharges[k] * P.coef);
+        if (k == 2 || k == 4) max_mom = std::max(max_mom, (size_t)4 * P.coef);
+        max_lp = std::max(max_lp, npot * (size_t)P.lout);
+        max_loc = std::max(max_loc, npot * (size_t)P.loc);
+        max_set = std::max(max_set, (size_t)2 * kSets[k] * P.tri);
+        max_mset = std::max(max_mset, (size_t)2 * kSets[k] * P.stri);
+        max_mpart = std::max(max_mpart, (size_t)(stokes_like(k) ? 96 : 32) * P.ngroup);
+        max_charges = std::max(max_charges, kCharges[k]);
+      }
+    ang_total += (size_t)P.ang;
+    group_total += (size_t)P.ngroup;
+    Offsets& o = off[pl];
+    o.off = put(nb_off.data(), nb_off.size() * sizeof(int));
+    o.lsrc = put(Lsrc, nd * sizeof(int));
+    o.sd = put(sd.data(), sd.size() * sizeof(FarSrcDrop));
+    o.td = put(td.data(), td.size() * sizeof(FarTgtDrop));
+    o.chunks = put(chunks.data(), chunks.size() * sizeof(FarChunk));
+    o.blocks = put(blocks.data(), blocks.size() * sizeof(int2));
+    o.pairs = room((size_t)npairs * sizeof(FarPair));
+    o.drop = room((size_t)nent * sizeof(int));
+    o.ent_tgt = room((size_t)nent * sizeof(int));
+    o.pre = room((size_t)nent * sizeof(int64_t));
+    o.goff = room((size_t)(nent + 1) * sizeof(int64_t));
+  }
+  if (std::none_of(used, used + kFarPlans, [](bool u) { return u; })) return SHBIM_OK;
+  int rc;
+  if ((rc = far_tables(ctx)) ||
+      (rc = far_grow(ctx, (void**)&F.blob, &F.blob_cap, blob.size(), "expansion plans")) ||
+      (rc = far_grow(ctx, (void**)&F.lists, &F.lists_cap, lists, "drop pair lists")) ||
+      (rc = far_grow(ctx, (void**)&F.ang, &F.ang_cap, ang_total * 8, "expansion angles")) ||
+      (rc = far_grow(ctx, &F.q, &F.q_cap, (size_t)max_charges * ctx->nsource * 8, "expansion charges")) ||
+      (rc = far_grow(ctx, &F.part, &F.part_cap, max_part * 8, "expansion partial moments")) ||
+      (rc = far_grow(ctx, &F.v, &F.v_cap, max_v * 8, "expansion moments")) ||
+      (rc = far_grow(ctx, &F.mom, &F.mom_cap, max_mom * 8, "expansion dipole moments")) ||
+      (rc = far_grow(ctx, &F.lpair, &F.lpair_cap, max_lp * 8, "expansion pair terms")) ||
+      (rc = far_grow(ctx, &F.loc, &F.loc_cap, max_loc * 8, "local expansions")) ||
+      (rc = far_grow(ctx, &F.set, &F.set_cap, max_set * 8, "local expansions of derivatives")) ||
+      (rc = far_grow(ctx, &F.order, &F.order_cap, std::max<size_t>(group_total, 1), "orders of close pairs")) ||
+      (rc = far_grow(ctx, &F.mset, &F.mset_cap, max_mset * 8, "multipole expansions of derivatives")) ||
+      (rc = far_grow(ctx, &F.mpart, &F.mpart_cap, max_mpart * 8, "values of multipole expansions"))) {
+    // no room for the expansions: every pair directly
+    for (int pl = 0; pl < kFarPlans; ++pl) std::memset(F.plan[pl].use, 0, sizeof(F.plan[pl].use));
+    ctx->err.clear();
+    return SHBIM_OK;
+  }
+  SHBIM_CUDA(ctx, cudaMemcpyAsync(F.blob, blob.data(), blob.size(), cudaMemcpyHostToDevice, s));
+  SHBIM_CUDA(ctx, cudaStreamSynchronize(s));   // the host copy goes away
+  F.inv_src = reinterpret_cast<const float*>(F.blob + inv_off);
+  F.inv_tgt = F.inv_src + nd;
+  FillPlans fill{};
+  int nfill = 0;
+  size_t ao = 0, go = 0;
+  for (int pl = 0; pl < kFarPlans; ++pl) {
+    if (!used[pl]) continue;
+    FarPlan& P = F.plan[pl];
+    const Offsets& o = off[pl];
+    P.near = F.plan[kFarPlans].near;
+    P.near.off = reinterpret_cast<const int*>(F.blob + o.off);
+    P.near.drop = reinterpret_cast<const int*>(F.lists + o.drop);
+    P.near.pre = reinterpret_cast<const int64_t*>(F.lists + o.pre);
+    P.near.goff = reinterpret_cast<const int64_t*>(F.lists + o.goff);
+    P.ent_tgt = reinterpret_cast<const int*>(F.lists + o.ent_tgt);
+    P.pairs = reinterpret_cast<const FarPair*>(F.lists + o.pairs);
+    P.Lsrc = reinterpret_cast<const int*>(F.blob + o.lsrc);
+    P.sd = reinterpret_cast<const FarSrcDrop*>(F.blob + o.sd);
+    P.td = reinterpret_cast<const FarTgtDrop*>(F.blob + o.td);
+    P.chunks = reinterpret_cast<const FarChunk*>(F.blob + o.chunks);
+    P.blocks = reinterpret_cast<const int2*>(F.blob + o.blocks);
+    P.ang_dev = F.ang + ao;
+    ao += (size_t)P.ang;
+    P.order = static_cast<unsigned char*>(F.order) + go;
+    go += (size_t)P.ngroup;
+    fill.p[nfill++] = FillPlan{pl, P.td, P.near.off, const_cast<FarPair*>(P.pairs), const_cast<int*>(P.near.drop),
+                               const_cast<int*>(P.ent_tgt), const_cast<int64_t*>(P.near.pre),
+                               const_cast<int64_t*>(P.near.goff)};
+  }
+  k_far_fill<<<dim3((unsigned)((nd * 32 + 127) / 128), (unsigned)nfill), 128, 0, s>>>(
+      rho_tab(), fill, ctx->centres_dev, ctx->dq_ext_dev, ctx->drops_dev, nd);
+  SHBIM_CHECK_LAUNCH(ctx, "k_far_fill");
+  AngTab A;
+  for (int m = 0; m <= kFarCap64; ++m) A.r[m] = 1.0 / std::sqrt(2.0 * m + 1.0);
+  for (int pl = 0; pl < kFarPlans; ++pl) {
+    if (!used[pl]) continue;
+    FarPlan& P = F.plan[pl];
+    k_far_angles<<<(unsigned)((P.npairs + 63) / 64), 64, 0, s>>>(P.pairs, P.npairs, ctx->drops_dev, F.inv_src, F.inv_tgt, A,
+                                                               P.ang_dev);
+    SHBIM_CHECK_LAUNCH(ctx, "k_far_angles");
+    if (P.ngroup == 0) continue;
+    RhoReach R{};
+    for (int L = 0; L <= plan_cap(pl); ++L) R.r[L] = std::nextafterf((float)rho_tab().r[pl][L], 0.f);
+    k_far_reach<<<(unsigned)((P.ngroup * 32 + 255) / 256), 256, 0, s>>>(
+        P.nent, P.ent_tgt, P.near, P.ngroup, ctx->drops_dev, ctx->dq_ext_dev, P.Lsrc, R, ctx->geo.tgt, ctx->ntarget, P.order);
+    SHBIM_CHECK_LAUNCH(ctx, "k_far_reach");
+    P.near.order = P.order;
+  }
+  return SHBIM_OK;
+}
+
+// The estimate in FP32 instructions of the expansions' inner steps (half as much again for latency and reads, twice
+// in FP64, plus 75 us of launches and short kernels) against the direct sums they replace. 40 drops of degree 11,
+// single layer in double-float (5.2e8 pairs): 1.48 ms directly, 1.03 with expansions; six drops of degree 16 in
+// FP64 (4e7 pairs, a third far), eight applications: 14.2 ms directly, 15.7 with expansions, and left direct; two
+// drops, or 1e8 pairs in FP32, stay direct.
+bool far_worth(const FarPlan& P, int precision, int kind) {
+  const double* direct = precision == SHBIM_PREC_FP32_COMP ? kDirect32 : (precision == SHBIM_PREC_DF64 ? kDirectDf : kDirect64);
+  const double unit = precision == SHBIM_PREC_FP64 ? 64.0 / 12.0 : 1.0;
+  const int npot = stokes_like(kind) ? 4 : 1;
+  const double cost = unit * (P.src_work * (45.0 + 26.0 * kCharges[kind]) + P.tgt_work * (30.0 + 26.0 * kSets[kind]) +
+                              P.pair_work * npot * 30.0);
+  return P.npairs > 0 && (precision == SHBIM_PREC_FP64 ? 2.0 : 1.5) * cost + 3e9 < P.far_pairs * direct[kind];
+}
+
+const FarPlan* far_plan(const shbim_ctx* ctx, int kind) {
+  if (!ctx->far) return nullptr;
+  const int level = ctx->opts.precision == SHBIM_PREC_FP32_COMP ? 0 : 1;
+  const FarPlan& P = ctx->far->plan[3 * level + kDerivs[kind]];
+  return P.use[ctx->opts.precision][kind] ? &P : nullptr;
+}
+
+const FarPlan& far_all(const shbim_ctx* ctx) { return ctx->far->plan[kFarPlans]; }
+
+bool far_ready(const shbim_ctx* ctx) { return ctx->n_drops < 2 || (ctx->far && far_all(ctx).near.tgt); }
+
+// Instructions of an expansion's value: recurrence and 2 NS multiply-adds per (n, m), half as much again for reads
+// and orders of uneven length; `base` for the powers of x + iy and the sums over warps. In FP64 four times that: six
+// drops of degree 16, double layer, solve of eight applications: 16.9 ms without these expansions, 16.3 at one
+// time, 15.7 at four. 64 drops of degree 16 to 48, without and with them: Stokeslet in double-float 35.5 and 24.2 ms,
+// stresslet FP32 10.2 and 9.0, double layer FP32 3.83 and 2.88; twice the instructions here change nothing. Below 0.1 ms
+// of direct sums the three launches cost more than they give (40 drops of degree 11, 3e9: 1.00 and 1.03 ms).
+NearList far_near(const shbim_ctx* ctx, const FarPlan& P, int kind) {
+  NearList nl = P.near;
+  const int ns = kSets[kind], pr = ctx->opts.precision;
+  const double direct = (pr == SHBIM_PREC_FP64 ? kDirect64 : (pr == SHBIM_PREC_DF64 ? kDirectDf : kDirect32))[kind];
+  if (P.direct_pairs * direct < 4e9) nl.order = nullptr;
+  FarReach& r = nl.reach;
+  if (pr == SHBIM_PREC_FP64) {
+    r = FarReach{kFarLmax, 384 * (3 + 2 * ns), 0, 120000, (int)direct};
+  } else {
+    const bool fp32 = pr == SHBIM_PREC_FP32_COMP;
+    r = FarReach{fp32 ? 12 : 36, 50 + 36 * ns, 9 + 6 * ns, 15000, (int)direct};
+  }
+  return nl;
+}
+
+double far_direct_pairs(const shbim_ctx* ctx, const FarPlan& P, int kind) {
+  const int pr = ctx->opts.precision;
+  if (P.counted[pr][kind]) return P.count[pr][kind];
+  const NearList nl = far_near(ctx, P, kind);
+  if (!nl.order) return P.direct_pairs;
+  double n = 0.0;
+  if (cudaDeviceSynchronize() != cudaSuccess || cudaMemset(ctx->far->sum, 0, sizeof(double)) != cudaSuccess) return P.direct_pairs;
+  k_far_direct<<<(unsigned)std::min<int64_t>((P.ngroup + 255) / 256, 1024), 256>>>(P.nent, P.ent_tgt, nl, P.ngroup,
+                                                                                  ctx->drops_dev, ctx->far->sum);
+  if (cudaMemcpy(&n, ctx->far->sum, sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) {
+    cudaGetLastError();
+    return P.direct_pairs;
+  }
+  P.counted[pr][kind] = true;
+  return P.count[pr][kind] = n;
+}
+
+}  // namespace shbim

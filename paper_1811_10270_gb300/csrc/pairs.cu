@@ -79,11 +79,11 @@ struct ListSplit {
   int64_t v0, v1;
 };
 
-__device__ __forceinline__ ListSplit list_split(const NearList& nl, int i, int by, int nsplit) {
+__device__ __forceinline__ ListSplit list_split(const NearList& nl, int i, const DropDev& Di, int by, int nsplit) {
   ListSplit r;
-  r.e0 = nl.off[i];
-  r.e1 = nl.off[i + 1] - 1;
-  const int64_t total = nl.pre[r.e1];
+  r.e0 = nl.begin(i);
+  r.e1 = nl.end(i);
+  const int64_t total = nl.total(i, Di);
   const int64_t chunk = (total + nsplit - 1) / nsplit;
   r.v0 = (int64_t)by * chunk;
   r.v1 = min(total, r.v0 + chunk);
@@ -130,7 +130,7 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
   if (!sub_tile<kTPT>(tiles, tile, bx)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const ListSplit ls = list_split(nl, i, by, nsplit);
+  const ListSplit ls = list_split(nl, i, Di, by, nsplit);
 
   // a warp's targets are neighbours: groups of 32 side by side
   const int s0 = (threadIdx.x >> 5) * 32 * kTPT;
@@ -156,9 +156,9 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
     for (int c = 0; c < NC; ++c) hi[k][c] = lo[k][c] = 0.f;
 
   for (int en = ls.e0; en < ls.e1; ++en) {
-    const int j = nl.drop[en];
+    const int j = nl.source(en, i);
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
+    const SrcRange rg = drop_range(Dj, nl.before(en, i, Di, Dj), ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     bool nr[kTPT];
     const bool mine = warp_near<kTPT>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
@@ -337,7 +337,7 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   if (!sub_tile<1>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
+  const ListSplit ls = list_split(nl, i, Di, (int)blockIdx.y, nsplit);
   const int s0 = (int)threadIdx.x & ~31;
   const bool ok = (int)threadIdx.x < tile.nt;
   const int64_t tg = nl.tgt[tile.t0 + (ok ? (int)threadIdx.x : 0)], t = tg;
@@ -350,9 +350,9 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   }
   dfl::acc A[NC];
   for (int en = ls.e0; en < ls.e1; ++en) {
-    const int j = nl.drop[en];
+    const int j = nl.source(en, i);
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
+    const SrcRange rg = drop_range(Dj, nl.before(en, i, Di, Dj), ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     bool nr[1];
     const bool mine = warp_near<1>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
@@ -429,7 +429,7 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   if (!sub_tile<1>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
+  const ListSplit ls = list_split(nl, i, Di, (int)blockIdx.y, nsplit);
   const int s0 = (int)threadIdx.x & ~31;
   const bool ok = (int)threadIdx.x < tile.nt;
   const int64_t tg = nl.tgt[tile.t0 + (ok ? (int)threadIdx.x : 0)], t = tg;
@@ -442,9 +442,9 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   }
   dfl::acc A[NC];
   for (int en = ls.e0; en < ls.e1; ++en) {
-    const int j = nl.drop[en];
+    const int j = nl.source(en, i);
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
+    const SrcRange rg = drop_range(Dj, nl.before(en, i, Di, Dj), ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     bool nr[1];
     const bool mine = warp_near<1>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
@@ -532,7 +532,7 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
   if (!sub_tile<kTPT>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
+  const ListSplit ls = list_split(nl, i, Di, (int)blockIdx.y, nsplit);
   const int s0 = (threadIdx.x >> 5) * 32 * kTPT;
   int64_t tg[kTPT];
   bool ok[kTPT];
@@ -551,9 +551,9 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
     for (int c = 0; c < NC; ++c) acc[k][c] = 0.0;
   }
   for (int en = ls.e0; en < ls.e1; ++en) {
-    const int j = nl.drop[en];
+    const int j = nl.source(en, i);
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
+    const SrcRange rg = drop_range(Dj, nl.before(en, i, Di, Dj), ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     bool nr[kTPT];
     const bool mine = warp_near<kTPT>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
@@ -888,6 +888,7 @@ int build_pair_lists(shbim_ctx* ctx, cudaStream_t s) {
   k_extent<<<dim3(grid.x, grid.y, 2), 256, 0, s>>>(ctx->geo.src, ctx->nsource, ctx->geo.tgt, ctx->ntarget,
                                                   ctx->drops_dev, ctx->dq_ext_dev);
   SHBIM_CHECK_LAUNCH(ctx, "k_extent");
+  if (int rc = far_count(ctx, s)) return rc;
   std::vector<unsigned> bits(2 * nd);
   SHBIM_CUDA(ctx, cudaMemcpyAsync(bits.data(), ctx->dq_ext_dev, (size_t)2 * nd * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
   SHBIM_CUDA(ctx, cudaStreamSynchronize(s));
