@@ -55,8 +55,9 @@ extern "C" {
 
 /* Arithmetic of the all-pairs sums (the singular self rows, the transforms and GMRES are
  * always FP64). Where it pays, the sums between drops far enough apart go through multipole and local
- * expansions of the same quadrature rule, in FP64 or double-float arithmetic, truncated below the rounding of
- * the mode (3e-15 of a pair's sum of magnitudes, 1e-8 in FP32 mode); the others are formed pair by pair. */
+ * expansions of the same quadrature rule (shbim_set_expansions), in FP64 or double-float arithmetic, the others are
+ * formed pair by pair. The truncation is bounded by 3e-15 (FP32 mode 1e-8) of the sum of a pair's strengths over the
+ * gap between the two drops. */
 #define SHBIM_PREC_FP64 0           /* FP64 sums */
 #define SHBIM_PREC_FP32_COMP 1      /* FP32 pair arithmetic, positions relative to the drop
                                        centres, compensated (two-sum) accumulation */
@@ -169,6 +170,11 @@ int shbim_set_field_shape(shbim_ctx* ctx, const double* G_host);
  * arithmetic (about 2^-42 relative per term, fewer instructions per pair); closer pairs, and every
  * pair when off, use the general double-float form (about 2^-45 per term). */
 int shbim_set_quantized_pairs(shbim_ctx* ctx, int on);
+
+/* Sums between drops through multipole and local expansions. On (default): the pairs of drops, and the groups of
+ * targets of close pairs, that are far enough apart take them where they cost less than the direct sums. Off: every
+ * pair of nodes is summed directly, as a reference for the expansions. */
+int shbim_set_expansions(shbim_ctx* ctx, int on);
 
 /* Equation of state of the surfactant (Section 1) used by shbim_rates, shbim_stokes_rhs and
  * shbim_step: SHBIM_EOS_LANGMUIR (default), the Langmuir law of Eq. langmuir normalised so that

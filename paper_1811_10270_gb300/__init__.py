@@ -52,7 +52,7 @@ EXPORTS = [
     "shbim_near_min_distance", "shbim_set_wait_limit", "shbim_check_wait", "shbim_set_self_precision", "shbim_set_oneshot_precision",
     "shbim_kernel_work", "shbim_warm_start_feature_count", "shbim_warm_start_features", "shbim_learned_guess",
     "shbim_set_warm_start", "shbim_stokes_rhs", "shbim_set_device_gmres", "shbim_reparametrize",
-    "shbim_set_field_shape", "shbim_set_equation_of_state", "shbim_set_quantized_pairs",
+    "shbim_set_field_shape", "shbim_set_equation_of_state", "shbim_set_quantized_pairs", "shbim_set_expansions",
     "shbim_set_stokes_preconditioner",
 ]
 PROBE_FFMA = 0
@@ -176,6 +176,7 @@ def lib():
         "shbim_set_field_shape": (i32, [vp, P(dp)]),
         "shbim_set_equation_of_state": (i32, [vp, i32]),
         "shbim_set_quantized_pairs": (i32, [vp, i32]),
+        "shbim_set_expansions": (i32, [vp, i32]),
         "shbim_set_stokes_preconditioner": (i32, [vp, i32]),
     }
     for name, (res, args) in sig.items():
@@ -400,6 +401,10 @@ class Context:
     def set_quantized_pairs(self, on: bool):
         """shbim_set_quantized_pairs: FP64-class pair sums on quantised positions (True) or general double-float."""
         self._check(self._L.shbim_set_quantized_pairs(self._h, 1 if on else 0), "shbim_set_quantized_pairs")
+
+    def set_expansions(self, on: bool):
+        """shbim_set_expansions: expansions between drops far enough apart where they pay (True) or direct sums only."""
+        self._check(self._L.shbim_set_expansions(self._h, 1 if on else 0), "shbim_set_expansions")
 
     def set_equation_of_state(self, law: int):
         """shbim_set_equation_of_state: EOS_LANGMUIR (beta, x_s) or EOS_LINEAR (gamma = 1 + beta (1 - Gamma))."""

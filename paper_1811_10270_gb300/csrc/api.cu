@@ -942,6 +942,15 @@ int shbim_set_quantized_pairs(shbim_ctx* ctx, int on) {
   return SHBIM_OK;
 }
 
+int shbim_set_expansions(shbim_ctx* ctx, int on) {
+  if (!ctx) return SHBIM_ERR_ARG;
+  ctx->expansions = on != 0;
+  // launch shapes and captured operator graphs are those of the other lists
+  for (auto& c : ctx->pair_cfg) c = shbim_ctx::PairCfg{1, ctx->pair_splits, !ctx->autotune};
+  ctx->geom_version++;
+  return SHBIM_OK;
+}
+
 int shbim_set_equation_of_state(shbim_ctx* ctx, int law) {
   if (!ctx) return SHBIM_ERR_ARG;
   if (law != SHBIM_EOS_LANGMUIR && law != SHBIM_EOS_LINEAR) return fail(ctx, SHBIM_ERR_ARG, "unknown equation of state");

@@ -542,7 +542,7 @@ bool far_worth(const FarPlan& P, int precision, int kind) {
 }
 
 const FarPlan* far_plan(const shbim_ctx* ctx, int kind) {
-  if (!ctx->far) return nullptr;
+  if (!ctx->far || !ctx->expansions) return nullptr;
   const int level = ctx->opts.precision == SHBIM_PREC_FP32_COMP ? 0 : 1;
   const FarPlan& P = ctx->far->plan[3 * level + kDerivs[kind]];
   return P.use[ctx->opts.precision][kind] ? &P : nullptr;

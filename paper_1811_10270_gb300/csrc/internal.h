@@ -227,6 +227,7 @@ struct shbim_ctx {
   unsigned* dq_ext_dev = nullptr; // [n_drops] largest |x - c| over each drop's sources (float bits)
   unsigned char* dq_far = nullptr; // [n_drops][n_drops]: the drop pair uses the quantised form
   int dq_cap = 0;                 // drops the two tables above hold
+  bool expansions = true;         // between drops far enough apart (shbim_set_expansions)
   shbim::FarState* far = nullptr; // lists of direct and far drop pairs, workspaces of the expansions
   int eos = SHBIM_EOS_LANGMUIR;      // tension law of shbim_rates / shbim_step (shbim_set_equation_of_state)
   bool refine_direct[2] = {true, true};     // refined solves (electric, Stokes): first inner solve aims at the end
