@@ -116,6 +116,7 @@ struct FarTab {
 struct FarPlan {
   NearList near;
   double direct_pairs = 0.0, far_pairs = 0.0;
+  double far_warps = 0.0, far_ctas = 0.0;   // far pairs with the targets of a drop rounded up to warps, to 128
   double src_work = 0.0, tgt_work = 0.0, pair_work = 0.0;
   int npairs = 0, nchunks = 0, nblocks = 0, lmax = 0;
   int64_t part = 0, coef = 0, loc = 0, lout = 0, tri = 0, ang = 0;

@@ -35,3 +35,23 @@ def test_set_drops_grows_with_the_drops_not_with_their_pairs():
         ctx.close()
         took.append(best)
     assert took[1] < 8.0 * took[0], took
+
+
+@pytest.mark.parametrize("n,p,precision,kind,expanded", [
+    (1024, 4, "FP32_COMP", "f", False), (1024, 4, "FP32_COMP", "fu", False), (128, 6, "FP32_COMP", "f", False),
+    (1024, 4, "DF64", "fu", True), (256, 8, "FP32_COMP", "f", True), (64, 8, "DF64", "f", True)])
+def test_expansions_are_taken_where_they_pay(n, p, precision, kind, expanded):
+    """The direct work of an application against that of every pair: many small drops whose translations cost more
+    than the sums they replace (2.6 times at the first size) are summed directly."""
+    import paper_1811_10270_gb300 as S
+    ctx = S.Context(precision=getattr(S, precision))
+    ctx.set_near(False)
+    ctx.set_drops([p] * n, lattice(n, p))
+    nc, nt, ns = ctx.sizes()
+    a, out = (torch.ones(3 * k, device="cuda", dtype=torch.float64) for k in (nc, nt))
+    ctx.set_timing(True)
+    ctx.eval_stokes(a, a if "u" in kind else None, out, S.OUT_GRID)
+    work = sum(ctx.kernel_work(c) for c in (S.K_PAIRS, S.K_PAIRS_FP64CLASS))
+    every = {"f": 29.0, "fu": 42.0}[kind] * (nt // n) * (ns // n) * n * (n - 1.0)
+    assert (work < 0.5 * every) if expanded else (work == every)
+    ctx.close()
