@@ -558,7 +558,7 @@ __device__ __forceinline__ void far_dq(const T* X, T* Y, int nc, const T* __rest
 template <class T>
 __global__ void __launch_bounds__(256)
 k_far_m2l(const FarPair* __restrict__ pairs, int npot, const FarSrcDrop* __restrict__ sd, const int* __restrict__ Lsrc,
-          const double* __restrict__ ang, FarTab<T> tab, const T* __restrict__ mom, T* __restrict__ out) {
+          const double* __restrict__ ang, FarTab<T> tab, const T* __restrict__ mom, int64_t out0, T* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char far_smem[];
   const FarPair p = pairs[blockIdx.x];
   const int L = p.L, n1 = L + 1, nc = n1 * n1;
@@ -607,7 +607,7 @@ k_far_m2l(const FarPair* __restrict__ pairs, int npot, const FarSrcDrop* __restr
   __syncthreads();
   far_dz(Y, nc, a, a + n1, false);
   __syncthreads();
-  T* dst = out + npot * p.out + (int64_t)blockIdx.y * nc;
+  T* dst = out + npot * (p.out - out0) + (int64_t)blockIdx.y * nc;
   for (int i = threadIdx.x; i < nc; i += blockDim.x) t_st(dst, i, t_ld(Y, i));
 }
 
@@ -615,8 +615,9 @@ k_far_m2l(const FarPair* __restrict__ pairs, int npot, const FarSrcDrop* __restr
 // sum over the far drops of a target drop, in order; psi is moved to the target drop's centre
 template <class T>
 __global__ void k_far_lsum(const FarTgtDrop* __restrict__ td, const FarPair* __restrict__ pairs,
-                           const DropDev* __restrict__ drops, int npot, const T* __restrict__ lp, T* __restrict__ loc) {
-  const int i = blockIdx.y;
+                           const DropDev* __restrict__ drops, int npot, int drop0, int64_t out0,
+                           const T* __restrict__ lp, T* __restrict__ loc) {
+  const int i = drop0 + blockIdx.y;
   const FarTgtDrop d = td[i];
   if (d.L < 0) return;
   const int nc = (d.L + 1) * (d.L + 1);
@@ -627,7 +628,7 @@ __global__ void k_far_lsum(const FarTgtDrop* __restrict__ td, const FarPair* __r
       const FarPair q = pairs[p];
       const int64_t ncp = (int64_t)(q.L + 1) * (q.L + 1);
       if (c >= ncp) continue;
-      const T* l = lp + npot * q.out;
+      const T* l = lp + npot * (q.out - out0);
       s.add(t_ld(l, k * ncp + c));
       if (k == 3) {
         const DropDev Di = drops[q.i], Dj = drops[q.j];
@@ -1287,10 +1288,16 @@ int expand(shbim_ctx* ctx, const FarPlan& P, int kind, cudaStream_t s) {
   const int sm = (2 * ncm + 6 * (P.lmax + 1)) * 8;
   constexpr int sm_max = (2 * (kFarCap64 + 1) * (kFarCap64 + 1) + 6 * (kFarCap64 + 1)) * 8;
   SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_far_m2l<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_max));
-  k_far_m2l<T><<<dim3((unsigned)P.npairs, npot), 256, sm, s>>>(P.pairs, npot, P.sd, P.Lsrc, P.ang_dev, tab, mom, lp);
-  SHBIM_CHECK_LAUNCH(ctx, "k_far_m2l");
-  k_far_lsum<T><<<dim3((unsigned)((npot * ncm + 127) / 128), nd), 128, 0, s>>>(P.td, P.pairs, ctx->drops_dev, npot, lp, loc);
-  SHBIM_CHECK_LAUNCH(ctx, "k_far_lsum");
+  for (const FarBatch& b : P.batches) {
+    if (b.pair1 > b.pair0) {
+      k_far_m2l<T><<<dim3((unsigned)(b.pair1 - b.pair0), npot), 256, sm, s>>>(P.pairs + b.pair0, npot, P.sd, P.Lsrc,
+                                                                            P.ang_dev, tab, mom, b.out0, lp);
+      SHBIM_CHECK_LAUNCH(ctx, "k_far_m2l");
+    }
+    k_far_lsum<T><<<dim3((unsigned)((npot * ncm + 127) / 128), (unsigned)(b.drop1 - b.drop0)), 128, 0, s>>>(
+        P.td, P.pairs, ctx->drops_dev, npot, b.drop0, b.out0, lp, loc);
+    SHBIM_CHECK_LAUNCH(ctx, "k_far_lsum");
+  }
   const unsigned lb = (unsigned)((tri_n(P.lmax) * 2 * kSets[kind] + 127) / 128);
   if (kind == 1)
     k_far_lset<T, 1><<<dim3(lb, nd), 128, 0, s>>>(P.td, F.inv_tgt, tab, npot, loc, set);

@@ -113,6 +113,13 @@ struct FarTab {
   const int2 *pat_r, *pat_c;
 };
 
+// target drops whose pair terms are held at once: their pairs and the terms' place
+struct FarBatch {
+  int drop0, drop1, pair0, pair1;
+  int64_t out0, out1;
+};
+constexpr int64_t kFarBatch = int64_t(1) << 25;   // coefficients per potential (1 GB for the four of a Stokes sum)
+
 struct FarPlan {
   NearList near;
   double direct_pairs = 0.0, far_pairs = 0.0;
@@ -133,6 +140,7 @@ struct FarPlan {
   int64_t ngroup = 0, stri = 0;
   const int* ent_tgt = nullptr;       // target drop of an entry (-1: end of a list)
   unsigned char* order = nullptr;     // [ngroup]
+  std::vector<FarBatch> batches;
   // pairs summed directly, by [precision][kind], once they have been asked for
   mutable bool counted[3][5] = {};
   mutable double count[3][5] = {};
@@ -178,6 +186,8 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s);
 int far_tables(shbim_ctx* ctx);
 int far_grow(shbim_ctx* ctx, void** p, size_t* cap, size_t bytes, const char* what);
 void far_free(shbim_ctx* ctx);
+// gives the lists and workspaces back
+void far_release(shbim_ctx* ctx);
 // empties every plan (the workspaces stay): what comes before build_far may fail
 void far_forget(shbim_ctx* ctx);
 // whether the expansions pay for this kind of sum at this precision

@@ -275,25 +275,35 @@ constexpr double kDirect64[5] = {1060.0, 740.0, 1980.0, 1540.0, 1470.0};
 
 }  // namespace
 
+void far_release(shbim_ctx* ctx) {
+  FarState& F = *ctx->far;
+  auto drop = [](auto*& p, size_t& cap) {
+    cudaFree(p);
+    p = nullptr;
+    cap = 0;
+  };
+  drop(F.blob, F.blob_cap);
+  drop(F.lists, F.lists_cap);
+  drop(F.ang, F.ang_cap);
+  drop(F.q, F.q_cap);
+  drop(F.part, F.part_cap);
+  drop(F.v, F.v_cap);
+  drop(F.mom, F.mom_cap);
+  drop(F.lpair, F.lpair_cap);
+  drop(F.loc, F.loc_cap);
+  drop(F.set, F.set_cap);
+  drop(F.mset, F.mset_cap);
+  drop(F.order, F.order_cap);
+  drop(F.mpart, F.mpart_cap);
+}
+
 void far_free(shbim_ctx* ctx) {
   if (!ctx->far) return;
   FarState& F = *ctx->far;
+  far_release(ctx);
   cudaFree(F.tables);
-  cudaFree(F.blob);
-  cudaFree(F.lists);
   cudaFree(F.count);
   cudaFreeHost(F.count_host);
-  cudaFree(F.ang);
-  cudaFree(F.q);
-  cudaFree(F.part);
-  cudaFree(F.v);
-  cudaFree(F.mom);
-  cudaFree(F.lpair);
-  cudaFree(F.loc);
-  cudaFree(F.set);
-  cudaFree(F.mset);
-  cudaFree(F.order);
-  cudaFree(F.mpart);
   delete ctx->far;
   ctx->far = nullptr;
 }
@@ -406,8 +416,13 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
       const int near = nd - 1 - row[i].far;
       nb_off[i + 1] = nb_off[i] + near + 1;
       td[i] = FarTgtDrop{row[i].lmax, pair, pair + row[i].far, P.loc, P.tri, P.lout, P.ang, P.ngroup};
+      if (P.batches.empty() || P.lout + row[i].out - P.batches.back().out0 > kFarBatch)
+        P.batches.push_back(FarBatch{i, i, pair, pair, P.lout, P.lout});
       pair += row[i].far;
       P.lout += row[i].out;
+      P.batches.back().drop1 = i + 1;
+      P.batches.back().pair1 = pair;
+      P.batches.back().out1 = P.lout;
       P.ang += row[i].ang;
       P.ngroup += (int64_t)near * ((d.nt + kFarGroup - 1) / kFarGroup);
       if (row[i].lmax >= 0) {
@@ -434,7 +449,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
         max_part = std::max(max_part, (size_t)2 * kCharges[k] * P.part);
         max_v = std::max(max_v, (size_t)kCharges[k] * P.coef);
         if (k == 2 || k == 4) max_mom = std::max(max_mom, (size_t)4 * P.coef);
-        max_lp = std::max(max_lp, npot * (size_t)P.lout);
+        for (const FarBatch& b : P.batches) max_lp = std::max(max_lp, npot * (size_t)(b.out1 - b.out0));
         max_loc = std::max(max_loc, npot * (size_t)P.loc);
         max_set = std::max(max_set, (size_t)2 * kSets[k] * P.tri);
         max_mset = std::max(max_mset, (size_t)2 * kSets[k] * P.stri);
@@ -457,26 +472,49 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     o.goff = room((size_t)(nent + 1) * sizeof(int64_t));
   }
   if (std::none_of(used, used + kFarPlans, [](bool u) { return u; })) return SHBIM_OK;
-  int rc;
-  if ((rc = far_tables(ctx)) ||
-      (rc = far_grow(ctx, (void**)&F.blob, &F.blob_cap, blob.size(), "expansion plans")) ||
-      (rc = far_grow(ctx, (void**)&F.lists, &F.lists_cap, lists, "drop pair lists")) ||
-      (rc = far_grow(ctx, (void**)&F.ang, &F.ang_cap, ang_total * 8, "expansion angles")) ||
-      (rc = far_grow(ctx, &F.q, &F.q_cap, (size_t)max_charges * ctx->nsource * 8, "expansion charges")) ||
-      (rc = far_grow(ctx, &F.part, &F.part_cap, max_part * 8, "expansion partial moments")) ||
-      (rc = far_grow(ctx, &F.v, &F.v_cap, max_v * 8, "expansion moments")) ||
-      (rc = far_grow(ctx, &F.mom, &F.mom_cap, max_mom * 8, "expansion dipole moments")) ||
-      (rc = far_grow(ctx, &F.lpair, &F.lpair_cap, max_lp * 8, "expansion pair terms")) ||
-      (rc = far_grow(ctx, &F.loc, &F.loc_cap, max_loc * 8, "local expansions")) ||
-      (rc = far_grow(ctx, &F.set, &F.set_cap, max_set * 8, "local expansions of derivatives")) ||
-      (rc = far_grow(ctx, &F.order, &F.order_cap, std::max<size_t>(group_total, 1), "orders of close pairs")) ||
-      (rc = far_grow(ctx, &F.mset, &F.mset_cap, max_mset * 8, "multipole expansions of derivatives")) ||
-      (rc = far_grow(ctx, &F.mpart, &F.mpart_cap, max_mpart * 8, "values of multipole expansions"))) {
-    // no room for the expansions: every pair directly
-    for (int pl = 0; pl < kFarPlans; ++pl) std::memset(F.plan[pl].use, 0, sizeof(F.plan[pl].use));
+  // The expansions take at most half of the memory that is free: near grids, the row build's lanes and the solvers'
+  // vectors come after them. Where that, or an allocation, falls short, they give everything back and every pair is
+  // summed directly.
+  struct Want {
+    void** p;
+    size_t* cap;
+    size_t bytes;
+    const char* what;
+  };
+  const Want want[] = {{(void**)&F.blob, &F.blob_cap, blob.size(), "expansion plans"},
+                       {(void**)&F.lists, &F.lists_cap, lists, "drop pair lists"},
+                       {(void**)&F.ang, &F.ang_cap, ang_total * 8, "expansion angles"},
+                       {&F.q, &F.q_cap, (size_t)max_charges * ctx->nsource * 8, "expansion charges"},
+                       {&F.part, &F.part_cap, max_part * 8, "expansion partial moments"},
+                       {&F.v, &F.v_cap, max_v * 8, "expansion moments"},
+                       {&F.mom, &F.mom_cap, max_mom * 8, "expansion dipole moments"},
+                       {&F.lpair, &F.lpair_cap, max_lp * 8, "expansion pair terms"},
+                       {&F.loc, &F.loc_cap, max_loc * 8, "local expansions"},
+                       {&F.set, &F.set_cap, max_set * 8, "local expansions of derivatives"},
+                       {&F.order, &F.order_cap, std::max<size_t>(group_total, 1), "orders of close pairs"},
+                       {&F.mset, &F.mset_cap, max_mset * 8, "multipole expansions of derivatives"},
+                       {&F.mpart, &F.mpart_cap, max_mpart * 8, "values of multipole expansions"}};
+  size_t more = 0, held = 0;
+  for (const Want& w : want) {
+    held += *w.cap;
+    more += w.bytes > *w.cap ? w.bytes : 0;
+  }
+  int rc = SHBIM_OK;
+  if (more > 0) {
+    size_t free_bytes = 0, total = 0;
+    SHBIM_CUDA(ctx, cudaMemGetInfo(&free_bytes, &total));
+    if (more > (free_bytes + held) / 2) rc = SHBIM_ERR_NOMEM;
+  }
+  if (!rc) rc = far_tables(ctx);
+  for (const Want& w : want)
+    if (!rc) rc = far_grow(ctx, w.p, w.cap, w.bytes, w.what);
+  if (rc == SHBIM_ERR_NOMEM) {
+    far_release(ctx);
+    for (int pl = 0; pl < kFarPlans; ++pl) F.plan[pl] = FarPlan{};
     ctx->err.clear();
     return SHBIM_OK;
   }
+  if (rc) return rc;
   SHBIM_CUDA(ctx, cudaMemcpyAsync(F.blob, blob.data(), blob.size(), cudaMemcpyHostToDevice, s));
   SHBIM_CUDA(ctx, cudaStreamSynchronize(s));   // the host copy goes away
   F.inv_src = reinterpret_cast<const float*>(F.blob + inv_off);

@@ -55,3 +55,60 @@ def test_expansions_are_taken_where_they_pay(n, p, precision, kind, expanded):
     every = {"f": 29.0, "fu": 42.0}[kind] * (nt // n) * (ns // n) * n * (n - 1.0)
     assert (work < 0.5 * every) if expanded else (work == every)
     ctx.close()
+
+
+def test_pair_terms_are_held_in_parts():
+    """1024 drops of degree 4 with their expansions in 8 GB (13.5 where every pair's terms lie side by side)."""
+    import paper_1811_10270_gb300 as S
+    n, p = 1024, 4
+    x = lattice(n, p)
+    before = torch.cuda.mem_get_info()[0]
+    ctx = S.Context(precision=S.DF64)
+    ctx.set_drops([p] * n, x)
+    assert before - torch.cuda.mem_get_info()[0] < 8 * 2 ** 30
+    ctx.close()
+
+
+def test_parts_add_up():
+    """Sums whose pair terms take several parts, against direct sums: 2^-42 of the sum of magnitudes, which is below
+    the sum of the 1/r^2 of a lattice of unit drops, times strengths of which the largest is taken."""
+    import paper_1811_10270_gb300 as S
+    n, p = 700, 5
+    ctx = S.Context(precision=S.DF64)
+    ctx.set_near(False)
+    ctx.set_drops([p] * n, lattice(n, p))
+    nc, nt, ns = ctx.sizes()
+    rng = np.random.default_rng(8)
+    d = torch.tensor(np.concatenate([inputs.random_density(p, rng)[0] for _ in range(n)]), device="cuda")
+    a, b = (torch.empty(nt, device="cuda", dtype=torch.float64) for _ in range(2))
+    for which in (S.LAPLACE_DL, S.LAPLACE_SL):
+        ctx.set_expansions(True)
+        ctx.eval_electric(which, d, a, S.OUT_GRID)
+        ctx.set_expansions(False)
+        ctx.eval_electric(which, d, b, S.OUT_GRID)
+        # |density| < 5; 700 unit spheres at distances from 2.6: sum 4 pi / r / (4 pi) < 700 / 2.6
+        assert (a - b).abs().max().item() < 2.0 ** -42 * 5.0 * n / 2.6
+    ctx.close()
+
+
+def test_without_memory_for_the_expansions_every_pair_is_direct():
+    """With 2.5 GB left the expansions of 512 drops (3.9 GB where all terms lie side by side) leave the near grids and
+    the row build their room, and give back what they took."""
+    import paper_1811_10270_gb300 as S
+    n, p = 512, 4
+    x = lattice(n, p)
+    nc = n * (p + 1) ** 2
+    d = torch.ones(nc, device="cuda", dtype=torch.float64)
+    ctx = S.Context(precision=S.DF64)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - int(2.5 * 2 ** 30), device="cuda", dtype=torch.uint8)
+    try:
+        ctx.set_drops([p] * n, x)
+        out = torch.empty(ctx.sizes()[1], device="cuda", dtype=torch.float64)
+        ctx.eval_electric(S.LAPLACE_DL, d, out, S.OUT_GRID)
+        assert torch.isfinite(out).all()
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+        ctx.close()
