@@ -25,8 +25,13 @@
 //
 // Orders: the truncation error of a pair with source radius a, target radius b and centre distance D is at
 // most sum|q| (L+1)^g rho^(L+1) / (D-a-b), rho = max(a/(D-b), b/(D-a)), g the number of derivatives taken; L is
-// the smallest order that puts it below 3e-15 (FP64 and double-float sums) or 1e-8 (FP32 sums, whose own
-// error is 3e-8). A pair that would need more than the level's largest order is summed directly.
+// the smallest order that puts it below 2e-16 (FP64 sums), 3e-15 (double-float sums) or 1e-8 (FP32 sums). A pair that
+// would need more than the level's largest order is summed directly.
+//
+// Errors against sums in 128 bits on the same sources, of a target's sum of magnitudes, expansions and direct sums
+// (24 drops of degree 16 to 32, all five kinds, worst of 120 values): FP64 2e-16 and 7e-16, double-float 2.4e-14 and
+// 1.4e-12. At a drop 57 radii away from twelve others the FP64 double layer has 8.8e-16 directly; with 3e-15, as for
+// double-float sums, the expansions had 1.4e-15 there.
 //
 // Arithmetic: native FP64 in FP64 mode, double-float on the FP32 pipe otherwise (a multiply-add costs 12
 // FP32 instructions against 64 issue slots), the same code through a template. Harmonics are the real
@@ -251,7 +256,7 @@ __global__ void k_far_charges(SrcView V, const DropDev* __restrict__ drops, T* _
 // L - g (together L + 2 columns, so every CTA of a drop has the same work), sums over the chunk of
 // q Q_nm (Re|Im (x+iy)^m). Threads first advance the recurrence of their own sources by eight degrees and leave
 // Q C and Q S of the tile in shared memory; then warp w sums degree n0 + w over the tile for every charge.
-// Degrees above nfull go on in FP32, 16 at a time and two per warp: a far pair's ratio rho is at most 0.61, so
+// Degrees above nfull go on in FP32, 16 at a time and two per warp: a far pair's ratio rho is at most 0.608, so
 // degree n is rho^n of the result and the FP32 rounding (about n 2^-24, independent from source to source) of
 // what nfull leaves out stays below the level's truncation error.
 // Bound by the FP32 pipe up to nfull (about 35 + 24 NQ instructions per source and (n, m) in double-float), by
@@ -565,7 +570,7 @@ k_far_m2l(const FarPair* __restrict__ pairs, int npot, const FarSrcDrop* __restr
   T* X = reinterpret_cast<T*>(far_smem);
   T* Y = X + nc;
   T* a = Y + nc;                            // [6][n1]
-  for (int i = threadIdx.x; i < 6 * n1; i += blockDim.x) t_st(a, i, from_d<T>(ang[p.ang + i]));
+  for (int i = threadIdx.x; i < 6 * n1; i += blockDim.x) t_st(a, i, from_d<T>(ang[p.ang + i / n1 * p.na + i % n1]));
   const int Ls = Lsrc[p.j];
   const int64_t ncs = (int64_t)(Ls + 1) * (Ls + 1);
   const T* M = mom + npot * sd[p.j].coef + blockIdx.y * ncs;
@@ -1239,8 +1244,9 @@ int far_tables(shbim_ctx* ctx) {
 
 namespace {
 
-// degrees carried in full precision: above it rho^n (rho <= 0.61) has taken the term below what FP32 loses. FP32
-// sums 12 (0.55^12 12 2^-24 = 6e-10), double-float 36 (0.56^36 36 2^-24 = 2e-15), FP64 all
+// degrees carried in full precision: above it rho^n has taken the term below what FP32 loses, whose rounding (about
+// n 2^-24, independent from source to source) leaves at the largest ratios of a level 0.608^13 13 2^-24 = 1.2e-9 above
+// degree 12 of FP32 sums and 0.578^37 37 2^-24 = 3.4e-15 above degree 36 of double-float ones; FP64 carries all
 int far_full(const shbim_ctx* ctx) {
   return ctx->opts.precision == SHBIM_PREC_FP32_COMP ? 12 : (ctx->opts.precision == SHBIM_PREC_DF64 ? 36 : kFarLmax);
 }
@@ -1286,12 +1292,12 @@ int expand(shbim_ctx* ctx, const FarPlan& P, int kind, cudaStream_t s) {
     mom = static_cast<T*>(F.mom);
   }
   const int sm = (2 * ncm + 6 * (P.lmax + 1)) * 8;
-  constexpr int sm_max = (2 * (kFarCap64 + 1) * (kFarCap64 + 1) + 6 * (kFarCap64 + 1)) * 8;
+  constexpr int sm_max = (2 * (kFarCapMax + 1) * (kFarCapMax + 1) + 6 * (kFarCapMax + 1)) * 8;
   SHBIM_CUDA(ctx, cudaFuncSetAttribute(k_far_m2l<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_max));
   for (const FarBatch& b : P.batches) {
     if (b.pair1 > b.pair0) {
       k_far_m2l<T><<<dim3((unsigned)(b.pair1 - b.pair0), npot), 256, sm, s>>>(P.pairs + b.pair0, npot, P.sd, P.Lsrc,
-                                                                            P.ang_dev, tab, mom, b.out0, lp);
+                                                                            F.ang, tab, mom, b.out0, lp);
       SHBIM_CHECK_LAUNCH(ctx, "k_far_m2l");
     }
     k_far_lsum<T><<<dim3((unsigned)((npot * ncm + 127) / 128), (unsigned)(b.drop1 - b.drop0)), 128, 0, s>>>(

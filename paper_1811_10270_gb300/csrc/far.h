@@ -10,11 +10,14 @@
 namespace shbim {
 
 constexpr int kFarLmax = 63;        // orders the constant tables hold
-constexpr double kFarEps32 = 1e-8;  // truncation of a pair, FP32 sums
-constexpr double kFarEps64 = 3e-15; // ... and FP64-class sums
-constexpr int kFarCap32 = 36;       // largest order of a far pair, FP32 sums
-constexpr int kFarCap64 = 60;       // ... and FP64-class sums
-constexpr int kFarPlans = 6;        // [truncation level 2][derivatives 3]
+// Levels of truncation by precision (FP64, FP32, double-float: the order of SHBIM_PREC_*): bound of a pair's error
+// relative to strengths over gap, and largest order of a far pair. In each case below the rounding of the direct sums:
+// 2e-16 of a target's sum of magnitudes in FP64 and more (measured 9e-16), 2^-44 in double-float, 2^-24 in FP32.
+constexpr double kFarEps[3] = {2e-16, 1e-8, 3e-15};
+__host__ __device__ constexpr int far_cap(int precision) { return precision == 0 ? 63 : (precision == 1 ? 36 : 60); }
+constexpr int kFarPlans = 9;        // [precision][derivatives]
+constexpr int kFarCapMax = 63;
+static_assert(kFarCapMax <= kFarLmax, "the tables hold every order");
 constexpr int kP2mSrc = 1024;       // sources of a chunk of the moments (a CTA of k_far_p2m)
 // by kind (0 DL, 1 SL, 2 S + D, 3 S, 4 D): expansions the targets evaluate, charges of a source, derivatives taken of
 // 1/r in the truncation bound
@@ -28,7 +31,8 @@ enum FarMode { kFarLap = 0, kFarS = 1, kFarD = 2, kFarSD = 3 };
 inline bool stokes_like(int kind) { return kind >= 2; }
 
 struct FarPair {
-  int i, j, L, pad;
+  int i, j, L;
+  int na;             // rows of its angles and powers, six of them (they serve every plan)
   int64_t out;        // offset of the pair's local terms (coefficients, per potential)
   int64_t ang;        // offset of its angles and powers
 };
@@ -126,33 +130,34 @@ struct FarPlan {
   double far_warps = 0.0, far_ctas = 0.0;   // far pairs with the targets of a drop rounded up to warps, to 128
   double src_work = 0.0, tgt_work = 0.0, pair_work = 0.0;
   int npairs = 0, nchunks = 0, nblocks = 0, lmax = 0;
-  int64_t part = 0, coef = 0, loc = 0, lout = 0, tri = 0, ang = 0;
-  bool use[3][5] = {};                // [precision][kind]
+  int64_t part = 0, coef = 0, loc = 0, lout = 0, tri = 0;
+  bool use[5] = {};                   // [kind]
   const FarPair* pairs = nullptr;
   const int* Lsrc = nullptr;
   const FarSrcDrop* sd = nullptr;
   const FarTgtDrop* td = nullptr;
   const FarChunk* chunks = nullptr;
   const int2* blocks = nullptr;
-  double* ang_dev = nullptr;
   // close pairs: groups of targets far enough for the source drop's own expansion
   int nent = 0;
   int64_t ngroup = 0, stri = 0;
   const int* ent_tgt = nullptr;       // target drop of an entry (-1: end of a list)
   unsigned char* order = nullptr;     // [ngroup]
   std::vector<FarBatch> batches;
-  // pairs summed directly, by [precision][kind], once they have been asked for
-  mutable bool counted[3][5] = {};
-  mutable double count[3][5] = {};
+  // pairs summed directly, by kind, once they have been asked for
+  mutable bool counted[5] = {};
+  mutable double count[5] = {};
 };
 
-// What a target drop's row of the drop pairs comes to under one plan (k_far_count)
+// What a target drop's row of the drop pairs comes to under one plan, or (the last row) where a pair has the largest
+// order that any plan gives it (k_far_count)
 struct FarRow {
   int64_t out;                        // sum of (L + 1)^2 over its far drops
   int64_t pairs;                      // targets times sources of its far drops
   double cubes;                       // sum of 2 L^3
   int far, lmax, ang, pad;            // far drops, largest order, sum of 6 (L + 1)
 };
+constexpr int kFarRows = kFarPlans + 1;
 
 struct FarState {
   FarPlan plan[kFarPlans + 1];        // the last one: every other drop directly
@@ -160,7 +165,7 @@ struct FarState {
   size_t blob_cap = 0;
   unsigned char* lists = nullptr;     // per-pair lists of the plans in use, written by k_far_fill
   size_t lists_cap = 0;
-  unsigned char* count = nullptr;     // [plans][n_drops] FarRow, [plans][n_drops] largest order of a source drop, a sum
+  unsigned char* count = nullptr;     // [kFarRows][n_drops] FarRow, [kFarPlans][n_drops] largest order of a source drop, a sum
   unsigned char* count_host = nullptr;   // page-locked, the same
   size_t count_cap = 0, count_host_cap = 0;
   double* sum = nullptr;              // in count: pairs summed directly, when asked for

@@ -19,20 +19,20 @@ namespace {
 
 // largest ratio rho that order L serves, per plan; the reach of close pairs takes the FP32 number below it
 struct RhoTab {
-  double r[kFarPlans][kFarCap64 + 1];
+  double r[kFarPlans][kFarCapMax + 1];
 };
 struct RhoReach {
-  float r[kFarCap64 + 1];
+  float r[kFarCapMax + 1];
 };
 
-int plan_cap(int pl) { return pl < 3 ? kFarCap32 : kFarCap64; }
+__host__ __device__ constexpr int plan_cap(int pl) { return far_cap(pl / 3); }
 
 const RhoTab& rho_tab() {
   static const RhoTab T = [] {
     RhoTab t{};
     for (int pl = 0; pl < kFarPlans; ++pl)
       for (int L = 0; L <= plan_cap(pl); ++L)
-        t.r[pl][L] = std::pow((pl < 3 ? kFarEps32 : kFarEps64) / std::pow(L + 1.0, pl % 3), 1.0 / (L + 1));
+        t.r[pl][L] = std::pow(kFarEps[pl / 3] / std::pow(L + 1.0, pl % 3), 1.0 / (L + 1));
     return t;
   }();
   return T;
@@ -54,7 +54,7 @@ __device__ __forceinline__ double far_ratio(const double* __restrict__ centres, 
 
 // smallest order that serves rho under plan pl, at least 2; -1: none
 __device__ __forceinline__ int far_order(const RhoTab& T, int pl, double rho) {
-  const int cap = pl < 3 ? kFarCap32 : kFarCap64;
+  const int cap = plan_cap(pl);
   if (!(rho <= T.r[pl][cap])) return -1;
   int a = 0, b = cap;
   while (a < b) {
@@ -65,6 +65,14 @@ __device__ __forceinline__ int far_order(const RhoTab& T, int pl, double rho) {
       b = c;
   }
   return max(a, 2);
+}
+
+// largest order that any plan gives the pair
+__device__ __forceinline__ int far_order_any(const RhoTab& T, double rho) {
+  int L = -1;
+#pragma unroll
+  for (int pl = 0; pl < kFarPlans; ++pl) L = max(L, far_order(T, pl, rho));
+  return L;
 }
 
 template <class V>
@@ -80,12 +88,12 @@ __global__ void k_far_count(const __grid_constant__ RhoTab T, const double* __re
                             FarRow* __restrict__ rows, int* __restrict__ lsrc) {
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= nd) return;
-  int far[kFarPlans], lmax[kFarPlans], ang[kFarPlans];
+  int far[kFarPlans], lmax[kFarPlans], ang = 0, pairs = 0;
   int64_t out[kFarPlans], src[kFarPlans];
   double cubes[kFarPlans];
 #pragma unroll
   for (int pl = 0; pl < kFarPlans; ++pl) {
-    far[pl] = ang[pl] = 0;
+    far[pl] = 0;
     lmax[pl] = -1;
     out[pl] = src[pl] = 0;
     cubes[pl] = 0.0;
@@ -94,25 +102,28 @@ __global__ void k_far_count(const __grid_constant__ RhoTab T, const double* __re
     if (j == i) continue;
     const double rho = far_ratio(centres, ext, nd, i, j);
     const int ns = drops[j].ns;
+    int top = -1;
 #pragma unroll
     for (int pl = 0; pl < kFarPlans; ++pl) {
       const int L = far_order(T, pl, rho);
       if (L < 0) continue;
+      top = max(top, L);
       far[pl]++;
       lmax[pl] = max(lmax[pl], L);
-      ang[pl] += 6 * (L + 1);
       out[pl] += (L + 1) * (L + 1);
       src[pl] += ns;
       cubes[pl] += 2.0 * L * L * L;
       if (lsrc[pl * nd + j] < L) atomicMax(lsrc + pl * nd + j, L);
     }
+    pairs += top >= 0;
+    ang += 6 * (top + 1);
   }
   const int64_t nt = drops[i].nt;
 #pragma unroll
   for (int pl = 0; pl < kFarPlans; ++pl) {
     FarRow r;
     r.far = warp_add(far[pl]);
-    r.ang = warp_add(ang[pl]);
+    r.ang = 0;
     r.out = warp_add(out[pl]);
     r.pairs = nt * warp_add(src[pl]);
     r.cubes = warp_add(cubes[pl]);
@@ -122,8 +133,13 @@ __global__ void k_far_count(const __grid_constant__ RhoTab T, const double* __re
     r.pad = 0;
     if (lane == 0) rows[(int64_t)pl * nd + i] = r;
   }
+  FarRow r{};
+  r.far = warp_add(pairs);
+  r.ang = warp_add(ang);
+  if (lane == 0) rows[(int64_t)kFarPlans * nd + i] = r;
 }
 
+// lists of a plan; pl kFarPlans: every pair that is far under some plan, with the order its angles need
 struct FillPlan {
   int pl;
   const FarTgtDrop* td;
@@ -133,7 +149,7 @@ struct FillPlan {
   int64_t *pre, *goff;
 };
 struct FillPlans {
-  FillPlan p[kFarPlans];
+  FillPlan p[kFarRows];
 };
 
 __device__ __forceinline__ int scan_before(int v, int lane) {
@@ -157,17 +173,18 @@ __global__ void k_far_fill(const __grid_constant__ RhoTab T, const __grid_consta
   const int groups = (drops[i].nt + kFarGroup - 1) / kFarGroup;
   const unsigned below = (1u << lane) - 1u;
   int64_t pair = d.pair0, out = d.out, ang = d.ang, goff = d.group, pre = 0;
-  int entry = P.off[i];
+  int entry = P.drop ? P.off[i] : 0;
   for (int j0 = 0; j0 < nd; j0 += 32) {
     const int j = j0 + lane;
     const bool other = j < nd && j != i;
-    const int L = other ? far_order(T, P.pl, far_ratio(centres, ext, nd, i, j)) : -1;
+    const double rho = other ? far_ratio(centres, ext, nd, i, j) : INFINITY;
+    const int top = far_order_any(T, rho), L = P.pl < kFarPlans ? far_order(T, P.pl, rho) : top;
     const bool far = L >= 0, near = other && !far;
     const unsigned fm = __ballot_sync(0xffffffffu, far), nm = __ballot_sync(0xffffffffu, near);
-    const int o = far ? (L + 1) * (L + 1) : 0, g = far ? 6 * (L + 1) : 0, ns = near ? drops[j].ns : 0;
+    const int o = far ? (L + 1) * (L + 1) : 0, g = 6 * (top + 1), ns = near ? drops[j].ns : 0;
     const int ob = scan_before(o, lane), gb = scan_before(g, lane), nb = scan_before(ns, lane);
-    if (far) P.pairs[pair + __popc(fm & below)] = FarPair{i, j, L, 0, out + ob, ang + gb};
-    if (near) {
+    if (far) P.pairs[pair + __popc(fm & below)] = FarPair{i, j, L, top + 1, out + ob, ang + gb};
+    if (near && P.drop) {
       const int k = __popc(nm & below);
       P.drop[entry + k] = j;
       P.ent_tgt[entry + k] = i;
@@ -181,7 +198,7 @@ __global__ void k_far_fill(const __grid_constant__ RhoTab T, const __grid_consta
     entry += __popc(nm);
     goff += (int64_t)__popc(nm) * groups;
   }
-  if (lane) return;
+  if (lane || !P.drop) return;
   P.drop[entry] = P.ent_tgt[entry] = -1;      // end of the list, with the total
   P.pre[entry] = pre;
   P.goff[entry] = goff;
@@ -190,13 +207,13 @@ __global__ void k_far_fill(const __grid_constant__ RhoTab T, const __grid_consta
 
 // 1 / sqrt(2 m + 1)
 struct AngTab {
-  double r[kFarCap64 + 1];
+  double r[kFarCapMax + 1];
 };
 
 // cos / sin of m phi and m theta, and the powers (2A/D)^n, (2B/D)^l, of every far pair (once per geometry). A thread per
 // pair and one product per value: FP64 instructions bound it: sine, cosine and power of every value apart, 100 to
-// 200 of them each, took 160 ms for the six plans of 1024 drops of degree 4, the products 4.9. The rounding of m factors
-// is that of an angle m phi.
+// 200 of them each, took 160 ms for 1024 drops of degree 4 and six plans, the products 4.9 (the plans share them now). The
+// rounding of m factors is that of an angle m phi.
 __global__ void k_far_angles(const FarPair* __restrict__ pairs, int npairs, const DropDev* __restrict__ drops,
                              const float* __restrict__ inv_src, const float* __restrict__ inv_tgt,
                              const __grid_constant__ AngTab T, double* __restrict__ ang) {
@@ -317,7 +334,7 @@ int far_count(shbim_ctx* ctx, cudaStream_t s) {
   if (!ctx->far) ctx->far = new FarState();
   FarState& F = *ctx->far;
   const size_t n = (size_t)kFarPlans * ctx->n_drops;
-  const size_t lsrc_off = n * sizeof(FarRow), sum_off = (lsrc_off + n * sizeof(int) + 15) / 16 * 16;
+  const size_t lsrc_off = (size_t)kFarRows * ctx->n_drops * sizeof(FarRow), sum_off = (lsrc_off + n * sizeof(int) + 15) / 16 * 16;
   if (int rc = far_grow(ctx, (void**)&F.count, &F.count_cap, sum_off + sizeof(double), "drop pair counts")) return rc;
   if (F.count_host_cap < sum_off) {
     cudaFreeHost(F.count_host);
@@ -360,6 +377,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
   struct Offsets {
     size_t off, lsrc, sd, td, chunks, blocks, pairs, drop, ent_tgt, pre, goff;
   } off[kFarPlans] = {};
+  size_t all_off = 0;                          // every pair with angles
   double cross = 0.0;
   for (const Drop& d : ctx->drops) cross += (double)d.nt * (double)(ctx->nsource - d.ns);
   F.plan[kFarPlans].near.n = nd;               // every other drop: no lists
@@ -374,13 +392,20 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
   }
   const size_t inv_off = put(inv.data(), inv.size() * sizeof(float));
   size_t max_part = 0, max_v = 0, max_mom = 0, max_lp = 0, max_loc = 0, max_set = 0, max_mset = 0, max_mpart = 0;
-  size_t ang_total = 0, group_total = 0;
+  size_t group_total = 0;
+  const FarRow* all = reinterpret_cast<const FarRow*>(F.count_host) + (size_t)kFarPlans * nd;
+  int64_t all_pairs = 0, ang_total = 0;
+  for (int i = 0; i < nd; ++i) {
+    all_pairs += all[i].far;
+    ang_total += all[i].ang;
+  }
+  if (all_pairs > INT32_MAX) return SHBIM_OK;
   int max_charges = 0;
   bool used[kFarPlans] = {};
   for (int pl = 0; pl < kFarPlans; ++pl) {
     FarPlan& P = F.plan[pl];
     const FarRow* row = reinterpret_cast<const FarRow*>(F.count_host) + (size_t)pl * nd;
-    const int* Lsrc = reinterpret_cast<const int*>(F.count_host + (size_t)kFarPlans * nd * sizeof(FarRow)) + (size_t)pl * nd;
+    const int* Lsrc = reinterpret_cast<const int*>(F.count_host + (size_t)kFarRows * nd * sizeof(FarRow)) + (size_t)pl * nd;
     int64_t npairs = 0, nent = 0;
     for (int i = 0; i < nd; ++i) {
       npairs += row[i].far;
@@ -398,12 +423,11 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     if (npairs == 0 || npairs > INT32_MAX || nent > INT32_MAX) continue;
     P.npairs = (int)npairs;
     P.nent = (int)nent;
-    // which kinds are worth it at which precision
-    for (int pr = 0; pr < 3; ++pr)
-      for (int k = 0; k < 5; ++k) {
-        P.use[pr][k] = kDerivs[k] == pl % 3 && (pl < 3) == (pr == SHBIM_PREC_FP32_COMP) && far_worth(P, pr, k);
-        used[pl] = used[pl] || P.use[pr][k];
-      }
+    // which kinds are worth it
+    for (int k = 0; k < 5; ++k) {
+      P.use[k] = kDerivs[k] == pl % 3 && far_worth(P, pl / 3, k);
+      used[pl] = used[pl] || P.use[k];
+    }
     if (!used[pl]) continue;
     std::vector<int> nb_off(nd + 1, 0);
     std::vector<FarSrcDrop> sd(nd);
@@ -411,11 +435,12 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     std::vector<FarChunk> chunks;
     std::vector<int2> blocks;
     int pair = 0;
+    int64_t ang = 0;
     for (int i = 0; i < nd; ++i) {
       const Drop& d = ctx->drops[i];
       const int near = nd - 1 - row[i].far;
       nb_off[i + 1] = nb_off[i] + near + 1;
-      td[i] = FarTgtDrop{row[i].lmax, pair, pair + row[i].far, P.loc, P.tri, P.lout, P.ang, P.ngroup};
+      td[i] = FarTgtDrop{row[i].lmax, pair, pair + row[i].far, P.loc, P.tri, P.lout, ang, P.ngroup};
       if (P.batches.empty() || P.lout + row[i].out - P.batches.back().out0 > kFarBatch)
         P.batches.push_back(FarBatch{i, i, pair, pair, P.lout, P.lout});
       pair += row[i].far;
@@ -423,7 +448,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
       P.batches.back().drop1 = i + 1;
       P.batches.back().pair1 = pair;
       P.batches.back().out1 = P.lout;
-      P.ang += row[i].ang;
+      ang += all[i].ang;
       P.ngroup += (int64_t)near * ((d.nt + kFarGroup - 1) / kFarGroup);
       if (row[i].lmax >= 0) {
         P.loc += (int64_t)(row[i].lmax + 1) * (row[i].lmax + 1);
@@ -442,9 +467,8 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     }
     P.nchunks = (int)chunks.size();
     P.nblocks = (int)blocks.size();
-    for (int pr = 0; pr < 3; ++pr)
       for (int k = 0; k < 5; ++k) {
-        if (!P.use[pr][k]) continue;
+        if (!P.use[k]) continue;
         const size_t npot = stokes_like(k) ? 4 : 1;
         max_part = std::max(max_part, (size_t)2 * kCharges[k] * P.part);
         max_v = std::max(max_v, (size_t)kCharges[k] * P.coef);
@@ -456,7 +480,6 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
         max_mpart = std::max(max_mpart, (size_t)(stokes_like(k) ? 96 : 32) * P.ngroup);
         max_charges = std::max(max_charges, kCharges[k]);
       }
-    ang_total += (size_t)P.ang;
     group_total += (size_t)P.ngroup;
     Offsets& o = off[pl];
     o.off = put(nb_off.data(), nb_off.size() * sizeof(int));
@@ -472,6 +495,20 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     o.goff = room((size_t)(nent + 1) * sizeof(int64_t));
   }
   if (std::none_of(used, used + kFarPlans, [](bool u) { return u; })) return SHBIM_OK;
+  // where a drop's pairs with angles start
+  size_t all_td;
+  {
+    std::vector<FarTgtDrop> td(nd);
+    int pair = 0;
+    int64_t ang = 0;
+    for (int i = 0; i < nd; ++i) {
+      td[i] = FarTgtDrop{-1, pair, pair + all[i].far, 0, 0, 0, ang, 0};
+      pair += all[i].far;
+      ang += all[i].ang;
+    }
+    all_td = put(td.data(), td.size() * sizeof(FarTgtDrop));
+    all_off = room((size_t)all_pairs * sizeof(FarPair));
+  }
   // The expansions take at most half of the memory that is free: near grids, the row build's lanes and the solvers'
   // vectors come after them. Where that, or an allocation, falls short, they give everything back and every pair is
   // summed directly.
@@ -483,7 +520,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
   };
   const Want want[] = {{(void**)&F.blob, &F.blob_cap, blob.size(), "expansion plans"},
                        {(void**)&F.lists, &F.lists_cap, lists, "drop pair lists"},
-                       {(void**)&F.ang, &F.ang_cap, ang_total * 8, "expansion angles"},
+                       {(void**)&F.ang, &F.ang_cap, (size_t)ang_total * 8, "expansion angles"},
                        {&F.q, &F.q_cap, (size_t)max_charges * ctx->nsource * 8, "expansion charges"},
                        {&F.part, &F.part_cap, max_part * 8, "expansion partial moments"},
                        {&F.v, &F.v_cap, max_v * 8, "expansion moments"},
@@ -521,7 +558,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
   F.inv_tgt = F.inv_src + nd;
   FillPlans fill{};
   int nfill = 0;
-  size_t ao = 0, go = 0;
+  size_t go = 0;
   for (int pl = 0; pl < kFarPlans; ++pl) {
     if (!used[pl]) continue;
     FarPlan& P = F.plan[pl];
@@ -538,25 +575,26 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     P.td = reinterpret_cast<const FarTgtDrop*>(F.blob + o.td);
     P.chunks = reinterpret_cast<const FarChunk*>(F.blob + o.chunks);
     P.blocks = reinterpret_cast<const int2*>(F.blob + o.blocks);
-    P.ang_dev = F.ang + ao;
-    ao += (size_t)P.ang;
     P.order = static_cast<unsigned char*>(F.order) + go;
     go += (size_t)P.ngroup;
     fill.p[nfill++] = FillPlan{pl, P.td, P.near.off, const_cast<FarPair*>(P.pairs), const_cast<int*>(P.near.drop),
                                const_cast<int*>(P.ent_tgt), const_cast<int64_t*>(P.near.pre),
                                const_cast<int64_t*>(P.near.goff)};
   }
+  FarPair* all_dev = reinterpret_cast<FarPair*>(F.lists + all_off);
+  fill.p[nfill++] = FillPlan{kFarPlans, reinterpret_cast<const FarTgtDrop*>(F.blob + all_td), nullptr, all_dev,
+                             nullptr, nullptr, nullptr, nullptr};
   k_far_fill<<<dim3((unsigned)((nd * 32 + 127) / 128), (unsigned)nfill), 128, 0, s>>>(
       rho_tab(), fill, ctx->centres_dev, ctx->dq_ext_dev, ctx->drops_dev, nd);
   SHBIM_CHECK_LAUNCH(ctx, "k_far_fill");
   AngTab A;
-  for (int m = 0; m <= kFarCap64; ++m) A.r[m] = 1.0 / std::sqrt(2.0 * m + 1.0);
+  for (int m = 0; m <= kFarCapMax; ++m) A.r[m] = 1.0 / std::sqrt(2.0 * m + 1.0);
+  k_far_angles<<<(unsigned)((all_pairs + 63) / 64), 64, 0, s>>>(all_dev, (int)all_pairs, ctx->drops_dev, F.inv_src, F.inv_tgt,
+                                                              A, F.ang);
+  SHBIM_CHECK_LAUNCH(ctx, "k_far_angles");
   for (int pl = 0; pl < kFarPlans; ++pl) {
     if (!used[pl]) continue;
     FarPlan& P = F.plan[pl];
-    k_far_angles<<<(unsigned)((P.npairs + 63) / 64), 64, 0, s>>>(P.pairs, P.npairs, ctx->drops_dev, F.inv_src, F.inv_tgt, A,
-                                                               P.ang_dev);
-    SHBIM_CHECK_LAUNCH(ctx, "k_far_angles");
     if (P.ngroup == 0) continue;
     RhoReach R{};
     for (int L = 0; L <= plan_cap(pl); ++L) R.r[L] = std::nextafterf((float)rho_tab().r[pl][L], 0.f);
@@ -592,9 +630,8 @@ bool far_worth(const FarPlan& P, int precision, int kind) {
 
 const FarPlan* far_plan(const shbim_ctx* ctx, int kind) {
   if (!ctx->far || !ctx->expansions) return nullptr;
-  const int level = ctx->opts.precision == SHBIM_PREC_FP32_COMP ? 0 : 1;
-  const FarPlan& P = ctx->far->plan[3 * level + kDerivs[kind]];
-  return P.use[ctx->opts.precision][kind] ? &P : nullptr;
+  const FarPlan& P = ctx->far->plan[3 * ctx->opts.precision + kDerivs[kind]];
+  return P.use[kind] ? &P : nullptr;
 }
 
 const FarPlan& far_all(const shbim_ctx* ctx) { return ctx->far->plan[kFarPlans]; }
@@ -623,8 +660,7 @@ NearList far_near(const shbim_ctx* ctx, const FarPlan& P, int kind) {
 }
 
 double far_direct_pairs(const shbim_ctx* ctx, const FarPlan& P, int kind) {
-  const int pr = ctx->opts.precision;
-  if (P.counted[pr][kind]) return P.count[pr][kind];
+  if (P.counted[kind]) return P.count[kind];
   const NearList nl = far_near(ctx, P, kind);
   if (!nl.order) return P.direct_pairs;
   double n = 0.0;
@@ -635,8 +671,8 @@ double far_direct_pairs(const shbim_ctx* ctx, const FarPlan& P, int kind) {
     cudaGetLastError();
     return P.direct_pairs;
   }
-  P.counted[pr][kind] = true;
-  return P.count[pr][kind] = n;
+  P.counted[kind] = true;
+  return P.count[kind] = n;
 }
 
 }  // namespace shbim

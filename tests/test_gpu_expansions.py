@@ -193,3 +193,48 @@ def test_expansions_follow_the_shapes_through_captured_graphs(made):
     np.testing.assert_array_equal(first, solve(used, [x for _, x, _ in drops]))
     used.close()
     fresh.close()
+
+
+def in_long_double(kind, drops, dens, i, targets):
+    """Sums over the other drops at targets of drop i, in long double on the oracle's sources."""
+    from oracle import operators, sh
+    LD = np.longdouble
+    geo = [operators.DropGeom(x, p, lam) for p, x, lam in drops]
+    out = []
+    for t in targets:
+        x0, n0, v = geo[i].x0[:, t].astype(LD), geo[i].n0[:, t].astype(LD), np.zeros(1 if kind == "dl" else 3, LD)
+        for j, d in enumerate(geo):
+            if j == i:
+                continue
+            r = [x0[c] - d.xs[c].astype(LD) for c in range(3)]
+            ri = 1 / np.sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2])
+            if kind == "dl":
+                q = (sh.sht_inverse(dens["scalar"][j], d.p, d.q) * d.ws).astype(LD)
+                v[0] += (q * ri ** 3 * sum(r[c] * n0[c] for c in range(3))).sum()
+            else:
+                q = sh.sht_inverse(dens["u"][j], d.p, d.q).astype(LD) * d.ws.astype(LD)
+                w = ri ** 5 * sum(r[c] * q[c] for c in range(3)) * sum(r[c] * d.ns[c].astype(LD) for c in range(3))
+                v += np.array([(w * r[c]).sum() for c in range(3)]) * (-6 * (LD(d.lam) - 1))
+        out.append(v * LD("0.0795774715459476678844418816862571810"))
+    return np.stack(out, 1)
+
+
+@pytest.mark.parametrize("kind", ["dl", "u"])
+def test_fp64_sums_at_a_distant_drop_are_rounded_not_truncated(made, kind):
+    """At a drop 57 radii away every source lies in one direction and the truncation's bound is nearly reached. Allowed:
+    1e-15 of the sum of magnitudes, five roundings (the oracle's positions there are rounded to 1e-16 of the distance)."""
+    import paper_1811_10270_gb300 as S
+    drops, dens, mags = made("suspension")
+    degrees = [p for p, _, _ in drops]
+    nt = [(p + 1) * (2 * p + 2) for p in degrees]
+    ctx = S.Context(precision=S.FP64)
+    ctx.set_near(False)
+    ctx.set_drops(degrees, device([x for _, x, _ in drops]), [l for _, _, l in drops])
+    assert made_of_expansions(S, ctx, kind, dens, nt, degrees)
+    got = others(S, ctx, kind, dens, nt)[2]
+    ctx.close()
+    targets = np.arange(7, nt[2], nt[2] // 24)
+    ref = in_long_double(kind, drops, dens, 2, targets)
+    err = np.abs(got[:, targets] - ref).max(0).astype(float) / mags[kind][2][targets]
+    print(kind, "%.2e" % err.max())
+    assert err.max() < 1e-15
