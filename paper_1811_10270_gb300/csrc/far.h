@@ -122,7 +122,7 @@ struct FarBatch {
   int drop0, drop1, pair0, pair1;
   int64_t out0, out1;
 };
-constexpr int64_t kFarBatch = int64_t(1) << 25;   // coefficients per potential (1 GB for the four of a Stokes sum)
+constexpr int64_t kFarBatch = int64_t(1) << 26;   // coefficients per potential (2 GB for the four of a Stokes sum)
 
 struct FarPlan {
   NearList near;
