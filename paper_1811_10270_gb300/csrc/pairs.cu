@@ -519,8 +519,13 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   }
 }
 
+// CTAs per SM of the FP64 kernel: the FP64 pipe is busy with fewer warps than the registers would allow, and CTAs that
+// wait let the near sums of the side stream in between. A solve of eight double-layer applications to six drops of
+// degree 16: 14.9 ms with seven CTAs per SM, 15.7 with eight (all CTAs of the grid resident, the near sums after them).
+constexpr int pairs64_ctas(int kind) { return kind == LDL ? 7 : (kind == LSL ? 8 : 6); }
+
 template <int KIND, int kTPT>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, kTPT == 2 ? pairs64_ctas(KIND) : 1)
 k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, NearList nl,
           const double* __restrict__ tgt, int64_t ntarget, const double* __restrict__ src,
           int64_t nsource, const double* __restrict__ dens, int nsplit, int has_f, int has_u,
