@@ -56,8 +56,9 @@ extern "C" {
 /* Arithmetic of the all-pairs sums (the singular self rows, the transforms and GMRES are
  * always FP64). Where it pays, the sums between drops far enough apart go through multipole and local
  * expansions of the same quadrature rule (shbim_set_expansions), in FP64 or double-float arithmetic, the others are
- * formed pair by pair. The truncation is bounded by 2e-16 (FP64), 3e-15 (double-float) or 1e-8 (FP32) of the sum of a
- * pair's strengths over the gap between the two drops, below the rounding of the mode's direct sums. */
+ * formed pair by pair. The truncation is bounded by 3e-15 (FP64 and double-float; FP64 sums take an order more for
+ * distant drops) or 1e-8 (FP32) of the sum of a pair's strengths over the gap between the two drops; what it comes to
+ * is below the rounding of the mode's direct sums. */
 #define SHBIM_PREC_FP64 0           /* FP64 sums */
 #define SHBIM_PREC_FP32_COMP 1      /* FP32 pair arithmetic, positions relative to the drop
                                        centres, compensated (two-sum) accumulation */

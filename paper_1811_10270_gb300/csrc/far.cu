@@ -25,13 +25,13 @@
 //
 // Orders: the truncation error of a pair with source radius a, target radius b and centre distance D is at
 // most sum|q| (L+1)^g rho^(L+1) / (D-a-b), rho = max(a/(D-b), b/(D-a)), g the number of derivatives taken; L is
-// the smallest order that puts it below 2e-16 (FP64 sums), 3e-15 (double-float sums) or 1e-8 (FP32 sums). A pair that
-// would need more than the level's largest order is summed directly.
+// the smallest order that puts it below 3e-15 (FP64 and double-float sums) or 1e-8 (FP32 sums), one more up to order 24
+// in FP64. A pair that would need more than the level's largest order is summed directly.
 //
 // Errors against sums in 128 bits on the same sources, of a target's sum of magnitudes, expansions and direct sums
 // (24 drops of degree 16 to 32, all five kinds, worst of 120 values): FP64 2e-16 and 7e-16, double-float 2.4e-14 and
-// 1.4e-12. At a drop 57 radii away from twelve others the FP64 double layer has 8.8e-16 directly; with 3e-15, as for
-// double-float sums, the expansions had 1.4e-15 there.
+// 1.4e-12. At the targets where the two differ most, close, elongated and distant drops among them, the expansions'
+// error is the smaller one in every kind: FP64 at most 3.8e-16 and 2.2e-15, double-float 6.2e-14 and 1.2e-12.
 //
 // Arithmetic: native FP64 in FP64 mode, double-float on the FP32 pipe otherwise (a multiply-add costs 12
 // FP32 instructions against 64 issue slots), the same code through a template. Harmonics are the real

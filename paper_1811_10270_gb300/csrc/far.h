@@ -11,12 +11,16 @@ namespace shbim {
 
 constexpr int kFarLmax = 63;        // orders the constant tables hold
 // Levels of truncation by precision (FP64, FP32, double-float: the order of SHBIM_PREC_*): bound of a pair's error
-// relative to strengths over gap, and largest order of a far pair. In each case below the rounding of the direct sums:
-// 2e-16 of a target's sum of magnitudes in FP64 and more (measured 9e-16), 2^-44 in double-float, 2^-24 in FP32.
-constexpr double kFarEps[3] = {2e-16, 1e-8, 3e-15};
-__host__ __device__ constexpr int far_cap(int precision) { return precision == 0 ? 63 : (precision == 1 ? 36 : 60); }
+// relative to strengths over gap, and largest order of a far pair. What they come to is below the rounding of the direct
+// sums, 7e-16 to 2e-15 of a target's sum of magnitudes in FP64, 1e-12 in double-float, 1e-7 in FP32; FP64 sums take one
+// order more up to kFarTight, where the sources of a distant drop lie in one direction and the bound is nearly reached:
+// 57 radii away the double layer was 1.4e-15 off without it, 8.8e-16 summed directly. One bound of 1e-15 for every pair
+// made solves of six drops of degree 16 3 % slower: the order of the closest pair sets the time of k_far_m2l there.
+constexpr double kFarEps[3] = {3e-15, 1e-8, 3e-15};
+constexpr int kFarTight = 24;
+__host__ __device__ constexpr int far_cap(int precision) { return precision == 1 ? 36 : 60; }
 constexpr int kFarPlans = 9;        // [precision][derivatives]
-constexpr int kFarCapMax = 63;
+constexpr int kFarCapMax = 60;
 static_assert(kFarCapMax <= kFarLmax, "the tables hold every order");
 constexpr int kP2mSrc = 1024;       // sources of a chunk of the moments (a CTA of k_far_p2m)
 // by kind (0 DL, 1 SL, 2 S + D, 3 S, 4 D): expansions the targets evaluate, charges of a source, derivatives taken of

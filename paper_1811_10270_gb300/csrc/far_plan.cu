@@ -33,6 +33,8 @@ const RhoTab& rho_tab() {
     for (int pl = 0; pl < kFarPlans; ++pl)
       for (int L = 0; L <= plan_cap(pl); ++L)
         t.r[pl][L] = std::pow(kFarEps[pl / 3] / std::pow(L + 1.0, pl % 3), 1.0 / (L + 1));
+    for (int pl = 0; pl < 3; ++pl)             // FP64
+      for (int L = kFarTight; L > 0; --L) t.r[pl][L] = t.r[pl][L - 1];
     return t;
   }();
   return T;
@@ -609,14 +611,15 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
 // What the expansions of a plan cost against the direct sums they replace, in FP32 instructions of the whole GPU (37 per
 // ns): their inner steps, half as much again for latency and reads (twice in FP64); a term per pair of drops and potential
 // for the short loops and barriers of k_far_m2l and k_far_lsum (9.4 to 10.4 ns in FP32 sums and 19 to 23 in double-float
-// at 1024 drops, inner steps included); the launches and the chain of dependent kernels, 80 to 320 us. A direct sum pays
+// at 1024 drops, inner steps included); the launches and the chain of dependent kernels, 80 to 220 us. A direct sum pays
 // for whole warps of targets (FP32) or whole CTAs of 128, of which at most 2.5 lanes per target were seen to count.
 // Both sides were measured on lattices of 6 to 1024 drops of degree 3 to 24, every kind and precision: the rule picks
 // the faster one beyond 10 % of its crossings but for a few sums of drops of degree 3. Without the term per pair, FP32
 // Stokes sums took the expansions for 1024 drops of degree 4 (40.4 ms, 15.8 directly) and 128 of degree 6 (1.31, 0.84).
 // 64 drops of degree 8, double layer, with expansions and directly: FP32 0.31 and 0.46 ms, double-float 0.86 and 2.40,
-// FP64 3.8 and 27.5. 16 drops of degree 11, Stokeslet in double-float: 0.63 and 0.56 ms, six drops of degree 16, double
-// layer in FP64 (a third of 4e7 pairs far), a solve of eight applications: 14.6 and 13.7; both are left direct.
+// FP64 3.8 and 27.5. 16 drops of degree 11, Stokeslet in double-float: 0.63 and 0.56 ms, left direct. Solves of eight
+// FP64 applications to six drops of degree 16 in boxes lie at the crossing: 12.0 to 14.4 ms where the rule takes the
+// expansions, 14.0 to 14.9 directly.
 bool far_worth(const FarPlan& P, int precision, int kind) {
   const bool fp64 = precision == SHBIM_PREC_FP64, fp32 = precision == SHBIM_PREC_FP32_COMP;
   const double* direct = fp32 ? kDirect32 : (fp64 ? kDirect64 : kDirectDf);
@@ -624,7 +627,7 @@ bool far_worth(const FarPlan& P, int precision, int kind) {
   const double inner = P.src_work * (45.0 + 26.0 * kCharges[kind]) + P.tgt_work * (30.0 + 26.0 * kSets[kind]) +
                        P.pair_work * npot * 30.0;
   const double unit = fp64 ? 2.0 * 64.0 / 12.0 : 1.5, pair = fp32 ? 3.2e5 : (fp64 ? 1.1e6 : 4.5e5);
-  const double launches = npot == 1 ? (fp32 ? 3e9 : (fp64 ? 12e9 : 5e9)) : (fp32 ? 5.5e9 : 8e9);
+  const double launches = npot == 1 ? (fp32 ? 3e9 : 5e9) : (fp32 ? 5.5e9 : 8e9);
   return P.npairs > 0 &&
          unit * inner + pair * npot * P.npairs + launches < (fp32 ? P.far_warps : P.far_ctas) * direct[kind];
 }
