@@ -82,7 +82,7 @@ namespace {
 
 void free_drop_state(shbim_ctx* ctx) {
   ctx->geom_version++;   // captured operator graphs, drop pair lists and near pairs refer to the buffers freed here
-  far_forget(ctx);
+  far_forget(ctx, true);
   ctx->near.npairs = 0;
   for (auto& d : ctx->drops) {
     cudaFree(d.rows_lap);

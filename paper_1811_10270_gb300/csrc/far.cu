@@ -1044,7 +1044,7 @@ __global__ void k_far_msum(NearList nl, const DropDev* __restrict__ drops, const
   double s[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) s[c] = 0.0;
-  for (int en = nl.begin(i); en < nl.end(i); ++en) {
+  for (unsigned en = nl.off[i]; en < nl.off[i + 1] - 1; ++en) {
     if (nl.direct(en, g, drops[nl.drop[en]].ns)) continue;
     const double* p = part + (nl.goff[en] + g) * NC * 32 + (sl & 31);
 #pragma unroll

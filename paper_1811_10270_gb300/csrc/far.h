@@ -69,32 +69,20 @@ struct FarReach {
 constexpr int kFarGroup = 32;       // targets that share a decision
 constexpr int kNoReach = 255;
 
-// Per target drop i the drops that no local expansion covers, entries [begin(i), end(i)): drop and the number of sources
-// before it in the list. Without lists (drop null) those are all others in the order of the layout, entry e being drop e,
-// or e + 1 from drop i on; with lists off[] holds where a drop's entries start, and the last entry of a drop has index -1
-// and the total of sources. The targets of a drop are taken in the order tgt[] (patches of the surface); group g of 32
-// of them reaches the multipole expansion of the entry's drop at order order[goff[entry] + g] (kNoReach: at none), and is
-// summed directly where that is not worth it.
+// Per target drop i the drops that no local expansion covers (or all others), entries [off[i], off[i+1]): drop index and
+// the number of sources before it in the list; the last entry of a drop has index -1 and the total. The targets of a drop
+// are taken in the order tgt[] (patches of the surface); group g of 32 of them reaches the multipole expansion of the
+// entry's drop at order order[goff[entry] + g] (kNoReach: at none), and is summed directly where that is not worth it.
+// Entries are unsigned: the list of all others holds the square of up to 65535 drops.
 struct NearList {
-  int n = 0;                        // drops
-  int64_t nsource = 0;
-  const int* off = nullptr;
+  const unsigned* off = nullptr;
   const int* drop = nullptr;
   const int64_t* pre = nullptr;
   const int* tgt = nullptr;
   const int64_t* goff = nullptr;    // [entries + 1]
   const unsigned char* order = nullptr;   // null: every group directly
   FarReach reach;
-  __device__ __forceinline__ int begin(int i) const { return drop ? off[i] : 0; }
-  __device__ __forceinline__ int end(int i) const { return drop ? off[i + 1] - 1 : n - 1; }
-  __device__ __forceinline__ int source(int entry, int i) const { return drop ? drop[entry] : entry + (entry >= i ? 1 : 0); }
-  __device__ __forceinline__ int64_t before(int entry, int i, const DropDev& Di, const DropDev& Dj) const {
-    return drop ? pre[entry] : Dj.src_off - (entry >= i ? (int64_t)Di.ns : 0);
-  }
-  __device__ __forceinline__ int64_t total(int i, const DropDev& Di) const {
-    return drop ? pre[off[i + 1] - 1] : nsource - Di.ns;
-  }
-  __host__ __device__ bool direct(int entry, int group, int ns) const {
+  __host__ __device__ bool direct(unsigned entry, int group, int ns) const {
     if (!order) return true;
     const int L = order[goff[entry] + group];
     return L == kNoReach || !reach.worth(L, ns);
@@ -169,6 +157,9 @@ struct FarState {
   size_t blob_cap = 0;
   unsigned char* lists = nullptr;     // per-pair lists of the plans in use, written by k_far_fill
   size_t lists_cap = 0;
+  unsigned char* all = nullptr;       // list of all others: [n_drops^2] int64 and int, [n_drops + 1] offsets
+  size_t all_cap = 0;
+  int all_drops = 0;                  // drops of the layout it was made for (0: none)
   unsigned char* count = nullptr;     // [kFarRows][n_drops] FarRow, [kFarPlans][n_drops] largest order of a source drop, a sum
   unsigned char* count_host = nullptr;   // page-locked, the same
   size_t count_cap = 0, count_host_cap = 0;
@@ -197,8 +188,9 @@ int far_grow(shbim_ctx* ctx, void** p, size_t* cap, size_t bytes, const char* wh
 void far_free(shbim_ctx* ctx);
 // gives the lists and workspaces back
 void far_release(shbim_ctx* ctx);
-// empties every plan (the workspaces stay): what comes before build_far may fail
-void far_forget(shbim_ctx* ctx);
+// empties every plan (the workspaces stay): what comes before build_far may fail; with the layout the list of all
+// others too
+void far_forget(shbim_ctx* ctx, bool layout = false);
 // whether the expansions pay for this kind of sum at this precision
 bool far_worth(const FarPlan& P, int precision, int kind);
 // the plan of a kind (0 DL, 1 SL, 2 S + D, 3 S, 4 D) at the context's precision, null: all pairs directly

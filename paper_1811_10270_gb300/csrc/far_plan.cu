@@ -4,7 +4,9 @@
 // The pairs of drops are classified on the GPU, a warp per target drop: k_far_count sums up what every plan would come
 // to, per drop, and k_far_fill writes the lists of the plans in use. The host sees O(drops) numbers only. One after
 // the other on the host, with lists for all plans copied to the device, set_drops took 1.8 s for 2048 drops of degree 4
-// (0.42 without expansions in the library), 0.37 so; 64 drops 5.9 and 5.1 ms. The sums without expansions need no lists.
+// (0.42 without expansions in the library), 0.37 so; 64 drops 5.9 and 5.1 ms. The list of every other drop, for the sums
+// without expansions, belongs to the layout; implied in the pair sums instead of read, it made the FP32 double layer
+// 2 to 6 % slower.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -145,7 +147,7 @@ __global__ void k_far_count(const __grid_constant__ RhoTab T, const double* __re
 struct FillPlan {
   int pl;
   const FarTgtDrop* td;
-  const int* off;
+  const unsigned* off;
   FarPair* pairs;
   int *drop, *ent_tgt;
   int64_t *pre, *goff;
@@ -175,7 +177,7 @@ __global__ void k_far_fill(const __grid_constant__ RhoTab T, const __grid_consta
   const int groups = (drops[i].nt + kFarGroup - 1) / kFarGroup;
   const unsigned below = (1u << lane) - 1u;
   int64_t pair = d.pair0, out = d.out, ang = d.ang, goff = d.group, pre = 0;
-  int entry = P.drop ? P.off[i] : 0;
+  unsigned entry = P.drop ? P.off[i] : 0;
   for (int j0 = 0; j0 < nd; j0 += 32) {
     const int j = j0 + lane;
     const bool other = j < nd && j != i;
@@ -273,6 +275,20 @@ __global__ void k_far_reach(int nent, const int* __restrict__ ent_tgt, NearList 
   order[f] = (unsigned char)(L <= Lsrc[j] ? L : kNoReach);
 }
 
+// every other drop, in the order of the layout
+__global__ void k_far_all(const DropDev* __restrict__ drops, int nd, int64_t nsource, int64_t* __restrict__ pre,
+                          int* __restrict__ drop, unsigned* __restrict__ off) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+  if (e >= nd) return;
+  const bool end = e == nd - 1;
+  const int j = e + (e >= i ? 1 : 0);
+  const int64_t at = (int64_t)i * nd + e, before = end ? nsource : drops[j].src_off;
+  drop[at] = end ? -1 : j;
+  pre[at] = before - (end || j > i ? (int64_t)drops[i].ns : 0);
+  if (e == 0) off[i] = (unsigned)i * (unsigned)nd;
+  if (end && i == nd - 1) off[nd] = (unsigned)nd * (unsigned)nd;
+}
+
 // target-source pairs of the groups that are summed directly
 __global__ void k_far_direct(int nent, const int* __restrict__ ent_tgt, NearList nl, int64_t ngroup,
                              const DropDev* __restrict__ drops, double* __restrict__ sum) {
@@ -321,14 +337,16 @@ void far_free(shbim_ctx* ctx) {
   FarState& F = *ctx->far;
   far_release(ctx);
   cudaFree(F.tables);
+  cudaFree(F.all);
   cudaFree(F.count);
   cudaFreeHost(F.count_host);
   delete ctx->far;
   ctx->far = nullptr;
 }
 
-void far_forget(shbim_ctx* ctx) {
+void far_forget(shbim_ctx* ctx, bool layout) {
   if (!ctx->far) return;
+  if (layout) ctx->far->all_drops = 0;
   for (auto& P : ctx->far->plan) P = FarPlan{};
 }
 
@@ -382,9 +400,23 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
   size_t all_off = 0;                          // every pair with angles
   double cross = 0.0;
   for (const Drop& d : ctx->drops) cross += (double)d.nt * (double)(ctx->nsource - d.ns);
-  F.plan[kFarPlans].near.n = nd;               // every other drop: no lists
-  F.plan[kFarPlans].near.nsource = ctx->nsource;
-  F.plan[kFarPlans].near.tgt = ctx->tgt_order;
+  // every other drop: once per layout
+  const size_t n2 = (size_t)nd * nd;
+  if (F.all_drops != nd) {
+    if (int rc = far_grow(ctx, (void**)&F.all, &F.all_cap, n2 * (sizeof(int64_t) + sizeof(int)) + (nd + 1) * sizeof(unsigned),
+                          "list of all drop pairs"))
+      return rc;
+    k_far_all<<<dim3((unsigned)((nd + 127) / 128), (unsigned)nd), 128, 0, s>>>(
+        ctx->drops_dev, nd, ctx->nsource, reinterpret_cast<int64_t*>(F.all), reinterpret_cast<int*>(F.all + n2 * sizeof(int64_t)),
+        reinterpret_cast<unsigned*>(F.all + n2 * (sizeof(int64_t) + sizeof(int))));
+    SHBIM_CHECK_LAUNCH(ctx, "k_far_all");
+    F.all_drops = nd;
+  }
+  NearList& others = F.plan[kFarPlans].near;
+  others.pre = reinterpret_cast<const int64_t*>(F.all);
+  others.drop = reinterpret_cast<const int*>(F.all + n2 * sizeof(int64_t));
+  others.off = reinterpret_cast<const unsigned*>(F.all + n2 * (sizeof(int64_t) + sizeof(int)));
+  others.tgt = ctx->tgt_order;
   F.plan[kFarPlans].direct_pairs = cross;
   std::vector<float> inv(2 * nd, 1.f);
   for (int i = 0; i < 2 * nd; ++i) {
@@ -431,7 +463,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
       used[pl] = used[pl] || P.use[k];
     }
     if (!used[pl]) continue;
-    std::vector<int> nb_off(nd + 1, 0);
+    std::vector<unsigned> nb_off(nd + 1, 0);
     std::vector<FarSrcDrop> sd(nd);
     std::vector<FarTgtDrop> td(nd);
     std::vector<FarChunk> chunks;
@@ -484,7 +516,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
       }
     group_total += (size_t)P.ngroup;
     Offsets& o = off[pl];
-    o.off = put(nb_off.data(), nb_off.size() * sizeof(int));
+    o.off = put(nb_off.data(), nb_off.size() * sizeof(unsigned));
     o.lsrc = put(Lsrc, nd * sizeof(int));
     o.sd = put(sd.data(), sd.size() * sizeof(FarSrcDrop));
     o.td = put(td.data(), td.size() * sizeof(FarTgtDrop));
@@ -566,7 +598,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
     FarPlan& P = F.plan[pl];
     const Offsets& o = off[pl];
     P.near = F.plan[kFarPlans].near;
-    P.near.off = reinterpret_cast<const int*>(F.blob + o.off);
+    P.near.off = reinterpret_cast<const unsigned*>(F.blob + o.off);
     P.near.drop = reinterpret_cast<const int*>(F.lists + o.drop);
     P.near.pre = reinterpret_cast<const int64_t*>(F.lists + o.pre);
     P.near.goff = reinterpret_cast<const int64_t*>(F.lists + o.goff);

@@ -75,15 +75,15 @@ __device__ __forceinline__ SrcRange drop_range(const DropDev& Dj, int64_t pre, i
 
 // split `by` of `nsplit` of the target drop's list: [v0, v1) and the list's entries
 struct ListSplit {
-  int e0, e1;
+  unsigned e0, e1;
   int64_t v0, v1;
 };
 
-__device__ __forceinline__ ListSplit list_split(const NearList& nl, int i, const DropDev& Di, int by, int nsplit) {
+__device__ __forceinline__ ListSplit list_split(const NearList& nl, int i, int by, int nsplit) {
   ListSplit r;
-  r.e0 = nl.begin(i);
-  r.e1 = nl.end(i);
-  const int64_t total = nl.total(i, Di);
+  r.e0 = nl.off[i];
+  r.e1 = nl.off[i + 1] - 1;
+  const int64_t total = nl.pre[r.e1];
   const int64_t chunk = (total + nsplit - 1) / nsplit;
   r.v0 = (int64_t)by * chunk;
   r.v1 = min(total, r.v0 + chunk);
@@ -92,7 +92,7 @@ __device__ __forceinline__ ListSplit list_split(const NearList& nl, int i, const
 
 // which of the warp's groups of 32 targets (slots s0 + 32 k of a drop of nt targets) entry en is summed for directly
 template <int TPT>
-__device__ __forceinline__ bool warp_near(const NearList& nl, int en, int ns, int s0, int nt, bool (&nr)[TPT]) {
+__device__ __forceinline__ bool warp_near(const NearList& nl, unsigned en, int ns, int s0, int nt, bool (&nr)[TPT]) {
   bool any = false;
 #pragma unroll
   for (int k = 0; k < TPT; ++k) {
@@ -130,7 +130,7 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
   if (!sub_tile<kTPT>(tiles, tile, bx)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const ListSplit ls = list_split(nl, i, Di, by, nsplit);
+  const ListSplit ls = list_split(nl, i, by, nsplit);
 
   // a warp's targets are neighbours: groups of 32 side by side
   const int s0 = (threadIdx.x >> 5) * 32 * kTPT;
@@ -155,10 +155,10 @@ __device__ __forceinline__ void pairs32_unit(int bx, int by, const PairTile* __r
 #pragma unroll
     for (int c = 0; c < NC; ++c) hi[k][c] = lo[k][c] = 0.f;
 
-  for (int en = ls.e0; en < ls.e1; ++en) {
-    const int j = nl.source(en, i);
+  for (unsigned en = ls.e0; en < ls.e1; ++en) {
+    const int j = nl.drop[en];
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Dj, nl.before(en, i, Di, Dj), ls.v0, ls.v1);
+    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     bool nr[kTPT];
     const bool mine = warp_near<kTPT>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
@@ -337,7 +337,7 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   if (!sub_tile<1>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const ListSplit ls = list_split(nl, i, Di, (int)blockIdx.y, nsplit);
+  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
   const int s0 = (int)threadIdx.x & ~31;
   const bool ok = (int)threadIdx.x < tile.nt;
   const int64_t tg = nl.tgt[tile.t0 + (ok ? (int)threadIdx.x : 0)], t = tg;
@@ -349,10 +349,10 @@ k_pairs_df(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
     N0[c] = dfl::from_double(tgt[(3 + c) * ntarget + t]);
   }
   dfl::acc A[NC];
-  for (int en = ls.e0; en < ls.e1; ++en) {
-    const int j = nl.source(en, i);
+  for (unsigned en = ls.e0; en < ls.e1; ++en) {
+    const int j = nl.drop[en];
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Dj, nl.before(en, i, Di, Dj), ls.v0, ls.v1);
+    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     bool nr[1];
     const bool mine = warp_near<1>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
@@ -429,7 +429,7 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   if (!sub_tile<1>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const ListSplit ls = list_split(nl, i, Di, (int)blockIdx.y, nsplit);
+  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
   const int s0 = (int)threadIdx.x & ~31;
   const bool ok = (int)threadIdx.x < tile.nt;
   const int64_t tg = nl.tgt[tile.t0 + (ok ? (int)threadIdx.x : 0)], t = tg;
@@ -441,10 +441,10 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
     N0[c] = dfl::from_double(tgt[(3 + c) * ntarget + t]);
   }
   dfl::acc A[NC];
-  for (int en = ls.e0; en < ls.e1; ++en) {
-    const int j = nl.source(en, i);
+  for (unsigned en = ls.e0; en < ls.e1; ++en) {
+    const int j = nl.drop[en];
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Dj, nl.before(en, i, Di, Dj), ls.v0, ls.v1);
+    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     bool nr[1];
     const bool mine = warp_near<1>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
@@ -519,13 +519,8 @@ k_pairs_dq(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops
   }
 }
 
-// CTAs per SM of the FP64 kernel: the FP64 pipe is busy with fewer warps than the registers would allow, and CTAs that
-// wait let the near sums of the side stream in between. A solve of eight double-layer applications to six drops of
-// degree 16: 14.9 ms with seven CTAs per SM, 15.7 with eight (all CTAs of the grid resident, the near sums after them).
-constexpr int pairs64_ctas(int kind) { return kind == LDL ? 7 : (kind == LSL ? 8 : 6); }
-
 template <int KIND, int kTPT>
-__global__ void __launch_bounds__(kThreads, kTPT == 2 ? pairs64_ctas(KIND) : 1)
+__global__ void __launch_bounds__(kThreads)
 k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops, NearList nl,
           const double* __restrict__ tgt, int64_t ntarget, const double* __restrict__ src,
           int64_t nsource, const double* __restrict__ dens, int nsplit, int has_f, int has_u,
@@ -537,7 +532,7 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
   if (!sub_tile<kTPT>(tiles, tile, blockIdx.x)) return;
   const int i = tile.drop;
   const DropDev Di = drops[i];
-  const ListSplit ls = list_split(nl, i, Di, (int)blockIdx.y, nsplit);
+  const ListSplit ls = list_split(nl, i, (int)blockIdx.y, nsplit);
   const int s0 = (threadIdx.x >> 5) * 32 * kTPT;
   int64_t tg[kTPT];
   bool ok[kTPT];
@@ -555,10 +550,10 @@ k_pairs64(const PairTile* __restrict__ tiles, const DropDev* __restrict__ drops,
 #pragma unroll
     for (int c = 0; c < NC; ++c) acc[k][c] = 0.0;
   }
-  for (int en = ls.e0; en < ls.e1; ++en) {
-    const int j = nl.source(en, i);
+  for (unsigned en = ls.e0; en < ls.e1; ++en) {
+    const int j = nl.drop[en];
     const DropDev Dj = drops[j];
-    const SrcRange rg = drop_range(Dj, nl.before(en, i, Di, Dj), ls.v0, ls.v1);
+    const SrcRange rg = drop_range(Dj, nl.pre[en], ls.v0, ls.v1);
     if (rg.a >= rg.b) continue;
     bool nr[kTPT];
     const bool mine = warp_near<kTPT>(nl, en, Dj.ns, (int)(tile.t0 - Di.tgt_off) + s0, Di.nt, nr);
