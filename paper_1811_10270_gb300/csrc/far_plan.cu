@@ -642,7 +642,7 @@ int build_far(shbim_ctx* ctx, const std::vector<double>& ext, cudaStream_t s) {
 
 // What the expansions of a plan cost against the direct sums they replace, in FP32 instructions of the whole GPU (37 per
 // ns): their inner steps, half as much again for latency and reads (twice in FP64); a term per pair of drops and potential
-// for the short loops and barriers of k_far_m2l and k_far_lsum (9.4 to 10.4 ns in FP32 sums and 19 to 23 in double-float
+// for the short loops and barriers of k_far_m2l and k_far_lsum (8 to 10 ns in FP32 sums and 19 to 22 in double-float
 // at 1024 drops, inner steps included); the launches and the chain of dependent kernels, 80 to 220 us. A direct sum pays
 // for whole warps of targets (FP32) or whole CTAs of 128, of which at most 2.5 lanes per target were seen to count.
 // Both sides were measured on lattices of 6 to 1024 drops of degree 3 to 24, every kind and precision: the rule picks
@@ -658,7 +658,7 @@ bool far_worth(const FarPlan& P, int precision, int kind) {
   const int npot = stokes_like(kind) ? 4 : 1;
   const double inner = P.src_work * (45.0 + 26.0 * kCharges[kind]) + P.tgt_work * (30.0 + 26.0 * kSets[kind]) +
                        P.pair_work * npot * 30.0;
-  const double unit = fp64 ? 2.0 * 64.0 / 12.0 : 1.5, pair = fp32 ? 3.2e5 : (fp64 ? 1.1e6 : 4.5e5);
+  const double unit = fp64 ? 2.0 * 64.0 / 12.0 : 1.5, pair = fp32 ? (npot == 1 ? 2e5 : 3.2e5) : (fp64 ? 1.1e6 : 4.5e5);
   const double launches = npot == 1 ? (fp32 ? 3e9 : 5e9) : (fp32 ? 5.5e9 : 8e9);
   return P.npairs > 0 &&
          unit * inner + pair * npot * P.npairs + launches < (fp32 ? P.far_warps : P.far_ctas) * direct[kind];
