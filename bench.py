@@ -159,11 +159,20 @@ def weights_flops_per_unit(p: int) -> float:
     return 2 * (18 * ntri + 9 * (N // 4 + 1) * 2 * p) / N + 70
 
 
+# FP64-class flops of the row build's analysis per target of a degree-p drop: for each of the 14 weights and every
+# latitude of the degree q = 2p + 1 grid the four-fold Fourier analysis (folding 2 N additions, 2p + 1 outputs of N / 4
+# FMAs, N = 2q + 2 longitudes), then the Legendre sums, an FMA per latitude and coefficient (cosine and sine).
+def analysis_flops_per_target(p: int) -> float:
+    q = 2 * p + 1
+    N = 2 * q + 2
+    return 14.0 * (q + 1) * (2 * N + (2 * p + 1) * (N // 4) * 2 + 2 * (p + 1) * (p + 2))
+
+
 def roofline(cls_ms, cls_n, cls_work, cfg, peaks, dom=None):
     """Roofline of the dominant kernel class of one step (largest summed duration in the timing pass), or
     of class `dom`, from the method's own work: the all-pairs classes count the flops of the kernel
-    formulas per target-source pair (shbim_kernel_work), the row build the FP64 flops of the weights
-    stage."""
+    formulas per target-source pair (shbim_kernel_work), the row build the FP64 flops of the weights and of
+    the analysis stage."""
     if dom is None:
         dom = max(cls_ms, key=lambda k: cls_ms[k])
     ms, n = cls_ms[dom], cls_n[dom]
@@ -194,6 +203,16 @@ def roofline(cls_ms, cls_n, cls_work, cfg, peaks, dom=None):
                     "kernel": "k_self_weights_df (double-float on the FP32 pipe)",
                     "work": "FP64 flops of the weights stage per (target, rotated node) x units",
                     "peak_source": "measured FP32 FMA rate (the pipe the double-float arithmetic runs on)",
+                    "frac_of_fp64_nominal": ach / FP64_NOMINAL_TFLOPS})
+        return out
+    if dom == "self_analysis":
+        units = sum((d.p + 1) * (2 * d.p + 2) * analysis_flops_per_target(d.p) for d in cfg.drops) * 2
+        ach = units / (ms / 1e3) / 1e12
+        out.update({"bound": "alu", "achieved": ach, "peak": ffma, "unit": "TFLOP/s", "frac": ach / ffma,
+                    "kernel": "k_dft_tc, k_dft4_tc, k_leg_tc (bfloat16 digit products on the tensor cores; folding, "
+                              "splitting and joining digits on the FP32 and integer pipes, which bound them)",
+                    "work": "FP64 flops of the folded Fourier and Legendre sums of the rows, two geometries",
+                    "peak_source": "measured FP32 FMA rate",
                     "frac_of_fp64_nominal": ach / FP64_NOMINAL_TFLOPS})
         return out
     out.update({"bound": "alu", "achieved": None, "peak": None, "unit": None, "frac": None,
