@@ -173,8 +173,9 @@ int shbim_set_field_shape(shbim_ctx* ctx, const double* G_host);
 int shbim_set_quantized_pairs(shbim_ctx* ctx, int on);
 
 /* Sums between drops through multipole and local expansions. On (default): the pairs of drops, and the groups of
- * targets of close pairs, that are far enough apart take them where they cost less than the direct sums. Off: every
- * pair of nodes is summed directly, as a reference for the expansions. */
+ * targets of close pairs, that are far enough apart take them where they cost less than the direct sums and half of the
+ * free device memory holds their workspaces. Off: every pair of nodes is summed directly, as a reference for the
+ * expansions. */
 int shbim_set_expansions(shbim_ctx* ctx, int on);
 
 /* Equation of state of the surfactant (Section 1) used by shbim_rates, shbim_stokes_rhs and
@@ -515,11 +516,11 @@ int shbim_set_self_precision(shbim_ctx* ctx, int precision);
 /* Tensor-core stages of the double-float row build (at the next shbim_set_drops), a bit mask:
  * SHBIM_TC_FOURIER, the GEMM of the rows' weights with the DFT table; SHBIM_TC_LEGENDRE, the
  * Legendre stage that follows it (used only together with SHBIM_TC_FOURIER); SHBIM_TC_ROTATION,
- * the pole rotations, one GEMM per latitude and degree (all degrees up
- * to 63; degree 64 on the FP32 pipe). They split their operands into bfloat16 digits whose products accumulate
- * exactly: six digits for drops up to degree 39 (error ~2^-40 of the sum of magnitudes per output), seven above (2^-47;
- * the Fourier stage of those degrees is used only together with the Legendre stage). A stage that is off, or does not fit, runs as the double-float FP32-pipe kernel. Default
- * SHBIM_TC_ALL (the tensor-core Legendre stage measures as fast as the FP32-pipe one); any other bit is
+ * the pole rotations, one GEMM per latitude and degree (all degrees up to 63; degree 64 on the FP32
+ * pipe). They split their operands into bfloat16 digits whose products accumulate exactly: six digits
+ * for drops up to degree 39 (error ~2^-40 of the sum of magnitudes per output), seven above (2^-47; the
+ * Fourier stage of those degrees is used only together with the Legendre stage). A stage that is off, or
+ * does not fit, runs as the double-float FP32-pipe kernel. Default SHBIM_TC_ALL; any other bit is
  * SHBIM_ERR_ARG. */
 #define SHBIM_TC_FOURIER 1
 #define SHBIM_TC_ROTATION 2

@@ -18,10 +18,9 @@
 //      centre take its multipole expansion itself; the direct sums of pairs.cu leave those targets out.
 // What it costs: O(L^2) per source and target and O(L^3) per pair of drops instead of the product of
 // their node counts. Whole operator applications at 64 drops of degree 16 to 48 (6.6e10 pairs, 95 % of them far), every
-// pair directly -> expansions: Laplace double layer FP32 50.4 -> 3.2 ms, stresslet FP32 73.7 -> 9.7 ms, Stokeslet
-// double-float 432 -> 27.6 ms; what remains is the direct sums (10.7 ms of the 27.6, 1.8 of the 9.7), the singular
-// rows (2.2) and k_far_p2m (4.6, 2.6). Against native FP64 direct sums the double-float results are 4 to 60
-// times closer than the direct double-float sums, the FP32 ones as close or closer.
+// pair directly -> expansions: Laplace double layer FP32 50.4 -> 3.1 ms, stresslet FP32 73.7 -> 9.3 ms, Stokeslet
+// double-float 432 -> 27.0 ms; what remains is the direct sums (13.0 ms of the 27.0, 2.2 of the 9.3), the singular
+// rows (2.2) and k_far_p2m (4.6, 2.5).
 //
 // Orders: the truncation error of a pair with source radius a, target radius b and centre distance D is at
 // most sum|q| (L+1)^g rho^(L+1) / (D-a-b), rho = max(a/(D-b), b/(D-a)), g the number of derivatives taken; L is
@@ -259,8 +258,10 @@ __global__ void k_far_charges(SrcView V, const DropDev* __restrict__ drops, T* _
 // Degrees above nfull go on in FP32, 16 at a time and two per warp: a far pair's ratio rho is at most 0.608, so
 // degree n is rho^n of the result and the FP32 rounding (about n 2^-24, independent from source to source) of
 // what nfull leaves out stays below the level's truncation error.
-// Bound by the FP32 pipe up to nfull (about 35 + 24 NQ instructions per source and (n, m) in double-float), by
-// shared-memory and L1 reads above it (2 NQ + 6); four tiles share one cross-lane reduction.
+// Bound by instruction issue up to nfull (about 35 + 24 NQ instructions per source and (n, m) in double-float; Stokeslet
+// of 24 drops of degree 16 to 32: 2.9 of 4 a cycle, FMA pipe 47 %), above it, where FP32 sums spend most degrees, by the
+// latency of the charges' reads at sixteen warps per SM (stresslet: 2.2 a cycle, L1 29 %, 2.3 cycles of waiting for
+// memory per issue). Four tiles share one cross-lane reduction.
 template <class T, int NQ>
 __global__ void __launch_bounds__(kP2mThreads, 2)
 k_far_p2m(SrcView V, const DropDev* __restrict__ drops, const FarChunk* __restrict__ chunks, const int* __restrict__ Lsrc,
@@ -559,7 +560,8 @@ __device__ __forceinline__ void far_dq(const T* X, T* Y, int nc, const T* __rest
 }
 
 // One CTA per (far pair, potential): all in shared memory; O(2 L^3) multiply-adds. Rotations cost as much as the
-// translation (Dq has a quarter of its entries); tables are read from L1 along consecutive rows.
+// translation (Dq has a quarter of its entries); tables are read from L1 along consecutive rows. Bound by L1 (46 to 52 %)
+// and waiting: 1.9 to 2.5 instructions a cycle, barriers between short loops 1.4 to 4.5 cycles per issue, memory 4.
 template <class T>
 __global__ void __launch_bounds__(256)
 k_far_m2l(const FarPair* __restrict__ pairs, int npot, const FarSrcDrop* __restrict__ sd, const int* __restrict__ Lsrc,
@@ -752,8 +754,9 @@ __global__ void k_far_lset(const FarTgtDrop* __restrict__ td, const float* __res
 // m = w, w + 8, ... The coefficients of the next degrees are read by the lanes side by side while the present ones
 // are used from a slot of shared memory, as broadcasts (read where they are used, they cost two L2 latencies per
 // degree: 4.7 ms instead of 1.0 for the Stokes sets at 1.4e5 targets). Degrees above nfull in FP32, as for the
-// moments. Up to nfull FP32-pipe bound (35 + 24 NS instructions per target and (n, m) in double-float); splitting
-// the orders keeps every SM busy from a few thousand targets on.
+// moments. Bound by issue and the latency of the recurrence's chain (35 + 24 NS instructions per target and (n, m) in
+// double-float; 2.6 of 4 a cycle, FMA pipe 50 %, for FP32 sums 1.9 and 33 %); splitting the orders keeps every SM busy
+// from a few thousand targets on.
 template <class T, int NS>
 __device__ __forceinline__ void eval_sets(T x, T y, T z, int L, int Ls, int nfull, const T* __restrict__ rec,
                                           const T* __restrict__ set, T* __restrict__ red, unsigned char* slot_raw) {

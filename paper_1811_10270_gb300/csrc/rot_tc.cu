@@ -20,11 +20,13 @@
 // accumulators in double-float. Every wait is bounded; a timeout sets the error flag and the CTA
 // stops.
 //
-// Drops of degree 40 and more (SPLIT), degrees up to 63: M couples neither cosine orders with sine orders nor the reverse (a rotation about y commutes
-// with the reflection y -> -y), so the block is two blocks of n (sine) and n + 1 (cosine) rows, contiguous in the
-// coefficient order: two GEMMs of half the size each, a quarter of the products, that fit tensor memory with seven
-// digits (2^-47: as close as the double-float kernel). Angles come from L1 there: the value block
-// takes the shared memory. Degree 64 (65 cosine rows) stays on the FP32-pipe kernel (singular_df.cu).
+// Drops of degree 40 and more (SPLIT), degrees up to 63: M couples neither cosine orders with sine orders nor
+// the reverse (a rotation about y commutes with the reflection y -> -y), so the block is two blocks of n (sine)
+// and n + 1 (cosine) rows, contiguous in the coefficient order: two GEMMs of half the size each, a quarter of the
+// products, that fit tensor memory with seven digits (2^-47: closer to the FP64 rows than the double-float kernel
+// at every degree measured from 40 to 64, but for the double layer of degree 52, 9.7e-13 and 9.5e-13). Angles come
+// from L1 there: the value block takes the shared memory. Degree 64 (65 cosine rows) stays on the FP32-pipe kernel
+// (singular_df.cu).
 #include <algorithm>
 #include <climits>
 #include <cmath>
