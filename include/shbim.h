@@ -116,7 +116,7 @@ int shbim_set_R(shbim_ctx* ctx, double R);
  * transform tables per distinct degree, target and source geometry (x, outward normal n,
  * area element; Section 1 and Eq. reg_quadrature) and the singular self rows of every
  * kernel (rotated-pole rule, Section 2.1).
- *   n_drops      number of drops (>= 1)
+ *   n_drops      number of drops, 1 to 65535 (the list of every other drop takes 12 bytes per pair of drops)
  *   p_host       degree of each drop, 1 <= p <= 64
  *   lambda_host  viscosity ratio of each drop (Eq. main_eq); may be NULL (all 1)
  *   xcoef_dev    position coefficients, per drop 3 (p+1)^2 doubles (x, y, z component-major)

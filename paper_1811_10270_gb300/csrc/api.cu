@@ -387,6 +387,8 @@ int shbim_set_drops(shbim_ctx* ctx, int n_drops, const int32_t* p_host, const do
                     const double* xcoef_dev, void* stream) {
   if (!ctx) return SHBIM_ERR_ARG;
   if (n_drops < 1 || !p_host || !xcoef_dev) return fail(ctx, SHBIM_ERR_ARG, "need n_drops >= 1, p and x");
+  // drops are the second dimension of launch grids, and entries of the drop pair lists count in 32 bits
+  if (n_drops > 65535) return fail(ctx, SHBIM_ERR_ARG, "at most 65535 drops");
   for (int i = 0; i < n_drops; ++i) {
     if (p_host[i] < 1 || p_host[i] > 64) return fail(ctx, SHBIM_ERR_ARG, "degree p must be in [1, 64]");
     if (lambda_host && (!std::isfinite(lambda_host[i]) || lambda_host[i] <= 0.0))

@@ -86,3 +86,15 @@ def test_refused_shapes_of_the_same_layout_are_not_summed(S):
     for call in operators(S, ctx, 25 + 16):
         call()
     ctx.close()
+
+
+def test_more_drops_than_the_lists_hold_are_refused(S):
+    """Before anything is allocated: the drop set of before stays."""
+    ctx = S.Context(precision=S.FP64)
+    ctx.set_drops([4, 3], device(drops([4, 3])))
+    n = 65536
+    with pytest.raises(S.ShbimError, match="65535"):
+        ctx.set_drops([1] * n, torch.zeros(n * 3 * 4, device="cuda", dtype=torch.float64))
+    for call in operators(S, ctx, 25 + 16):
+        call()
+    ctx.close()
